@@ -276,7 +276,8 @@ typedef struct {
     int64_t fallback_lookups;        /* hashtable lookups of the flux update (0: every stencil cell is linked) */
     /* persistent kernel (GBEES_LAUNCH_PERSISTENT / AUTO): microseconds that its
      * block 0 spent per phase, measured with the SM clock between grid
-     * barriers -- grow, halo, link, faces, apply, prune, step scalars, unused --
+     * barriers -- grow (with the waves), 0, 0, faces (with the new halo cells'
+     * keys), apply (with their links), prune, step scalars, unused --
      * and the steps covered (accumulated since the last init, not reset by
      * reset) */
     double persist_us[8];

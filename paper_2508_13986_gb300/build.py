@@ -15,10 +15,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libgbees_gb300.so")
-# (source, extra defines, object name): update_inst.cu once per precision and model family
+# (source, extra defines, object name): update_inst.cu once per precision and dimension
 SOURCES = [("api.cu", [], "api.o")] + [
-    ("update_inst.cu", [f"-DGBEES_PREC={p}", f"-DGBEES_FAMILY={f}"], f"update_p{p}_f{f}.o")
-    for p in (64, 32) for f in range(6)]
+    ("update_inst.cu", [f"-DGBEES_PREC={p}", f"-DGBEES_DIM={n}"], f"update_p{p}_n{n}.o")
+    for p in (64, 32) for n in (6, 5, 4, 3, 2, 1)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
          "-I", os.path.join(ROOT, "include")]
@@ -64,7 +64,7 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
 
     workers = max(1, min(len(SOURCES), os.cpu_count() or 1))
     # the longest jobs first
-    order = sorted(SOURCES, key=lambda s: (s[0] != "update_inst.cu", s[2]))
+    order = sorted(SOURCES, key=lambda s: (s[2][-3:-2] if s[0] == "update_inst.cu" else "5"), reverse=True)
     with cf.ThreadPoolExecutor(max_workers=workers) as ex:
         objs = list(ex.map(compile_one, order))
     tmp = LIB + f".tmp{os.getpid()}"

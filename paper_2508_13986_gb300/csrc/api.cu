@@ -16,29 +16,29 @@
 #include "gbees_misc_kernels.cuh"
 
 namespace gbees {
-// update_inst.cu, one object per precision and model family
-#define GBEES_DECL(p, fam) bool update_kernels_p##p##_f##fam(int n, int dyn, Kernels* k);
-GBEES_DECL(64, 0) GBEES_DECL(64, 1) GBEES_DECL(64, 2) GBEES_DECL(64, 3) GBEES_DECL(64, 4) GBEES_DECL(64, 5)
-GBEES_DECL(32, 0) GBEES_DECL(32, 1) GBEES_DECL(32, 2) GBEES_DECL(32, 3) GBEES_DECL(32, 4) GBEES_DECL(32, 5)
+// update_inst.cu, one object per precision and dimension
+#define GBEES_DECL(p) \
+    void update_kernels_p##p##_n1(Kernels* k); \
+    void update_kernels_p##p##_n2(Kernels* k); \
+    void update_kernels_p##p##_n3(Kernels* k); \
+    void update_kernels_p##p##_n4(Kernels* k); \
+    void update_kernels_p##p##_n5(Kernels* k); \
+    void update_kernels_p##p##_n6(Kernels* k);
+GBEES_DECL(64)
+GBEES_DECL(32)
 #undef GBEES_DECL
 
 // The kernels of one time step of a model (before and after the link phase)
-// and its persistent step-loop kernel.
+// and its step-loop kernels.
 bool update_kernels(const Model& m, bool f32, Kernels* k) {
-    int fam;
-    switch (m.dyn) {
-        case DYN_LORENZ63:
-        case DYN_LORENZ63_SHIFTED: fam = 0; break;
-        case DYN_LORENZ96: fam = 1; break;
-        case DYN_LINEAR: fam = m.n <= 3 ? 2 : 3; break;
-        default: fam = m.n <= 3 ? 4 : 5; break;
-    }
-    typedef bool (*Entry)(int, int, Kernels*);
-    static const Entry e64[6] = {update_kernels_p64_f0, update_kernels_p64_f1, update_kernels_p64_f2,
-                                 update_kernels_p64_f3, update_kernels_p64_f4, update_kernels_p64_f5};
-    static const Entry e32[6] = {update_kernels_p32_f0, update_kernels_p32_f1, update_kernels_p32_f2,
-                                 update_kernels_p32_f3, update_kernels_p32_f4, update_kernels_p32_f5};
-    return (f32 ? e32 : e64)[fam](m.n, m.dyn, k);
+    typedef void (*Entry)(Kernels*);
+    static const Entry e64[6] = {update_kernels_p64_n1, update_kernels_p64_n2, update_kernels_p64_n3,
+                                 update_kernels_p64_n4, update_kernels_p64_n5, update_kernels_p64_n6};
+    static const Entry e32[6] = {update_kernels_p32_n1, update_kernels_p32_n2, update_kernels_p32_n3,
+                                 update_kernels_p32_n4, update_kernels_p32_n5, update_kernels_p32_n6};
+    if (m.n < 1 || m.n > 6) return false;
+    (f32 ? e32 : e64)[m.n - 1](k);
+    return true;
 }
 }  // namespace gbees
 
@@ -436,7 +436,8 @@ void resolve_update_kernels(gbees_ctx* ctx) {
     int dev = 0, sms = 0, per_sm = 0;
     if (ctx->kern_ok && cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ctx->kern.persist, THREADS, 0) == cudaSuccess &&
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ctx->kern.persist, PERSIST_THREADS, 0) ==
+                cudaSuccess &&
             per_sm >= 1)
             ctx->persist_grid = std::min(GRID_MAX, sms);
         for (int i = 0; i < ctx->kern.npre; ++i) ctx->pre_grid[i] = resident_grid(ctx, ctx->kern.pre[i], sms);
@@ -993,7 +994,7 @@ int gbees_propagate(gbees_ctx* ctx, double t_end, gbees_stats* stats) {
             // the kernel's barriers count arrivals from zero
             if (!cuda_ok(ctx, cudaMemsetAsync(&ctx->b.sc->bar_seq, 0, sizeof(unsigned long long), s), "propagate"))
                 return ctx->status;
-            if (!cuda_ok(ctx, cudaLaunchCooperativeKernel(ctx->kern.persist, dim3(pg), dim3(THREADS), args, 0, s),
+            if (!cuda_ok(ctx, cudaLaunchCooperativeKernel(ctx->kern.persist, dim3(pg), dim3(PERSIST_THREADS), args, 0, s),
                          "propagate"))
                 return ctx->status;
             cudaEventRecord(ctx->pev[1], s);
@@ -1180,14 +1181,10 @@ int gbees_batch_propagate(gbees_ctx* const* ctxs, int32_t count, const double* t
     const int cap_blocks = c0->batch_blocks > 0 ? c0->batch_blocks : GRID_MAX;
     int G = std::max(1, std::min({count, sms * std::max(per_sm, 1), cap_blocks}));
     // teams: every grid resident at once with blocks in proportion to its work
-    int per_sm_team = 0;
-    bool teams = c0->kern.batch_teams &&
-                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_team, c0->kern.batch_teams, THREADS, 0) ==
-                     cudaSuccess &&
-                 per_sm_team >= 1 && count <= std::min({GRID_MAX, sms * per_sm_team, cap_blocks});
+    const bool teams = per_sm >= 1 && count <= std::min({GRID_MAX, sms * per_sm, cap_blocks});
     cudaGetLastError();
     if (teams) {
-        const int Gt = std::min({GRID_MAX, sms * per_sm_team, cap_blocks});
+        const int Gt = std::min({GRID_MAX, sms * per_sm, cap_blocks});
         const std::vector<int> k = team_sizes(ctxs, count, t_end, Gt, max_steps > 0);
         std::vector<TeamSlot> h_slots;
         for (int32_t i = 0; i < count; ++i)
@@ -1205,10 +1202,11 @@ int gbees_batch_propagate(gbees_ctx* const* ctxs, int32_t count, const double* t
         if (!e && !cuda_ok(c0, cudaEventCreate(&e), "batch_propagate")) return c0->status;
     for (int round = 0;; ++round) {
         if (!cuda_ok(c0, cudaMemsetAsync(next, 0, sizeof(unsigned int), s), "batch_propagate")) return c0->status;
-        void* args[] = {&items, &count, &next, &launch_steps};
-        void* targs[] = {&items, &slots, &launch_steps};
+        const TeamSlot* team_slots = teams ? slots : nullptr;
+        void* args[] = {&items, &count, &next, &team_slots, &launch_steps};
+        if (round > 0) k_batch_again<<<(count + THREADS - 1) / THREADS, THREADS, 0, s>>>(items, count);
         cudaEventRecord(c0->pev[0], s);
-        const cudaError_t le = teams ? cudaLaunchCooperativeKernel(c0->kern.batch_teams, dim3(G), dim3(THREADS), targs, 0, s)
+        const cudaError_t le = teams ? cudaLaunchCooperativeKernel(c0->kern.batch, dim3(G), dim3(THREADS), args, 0, s)
                                      : cudaLaunchKernel(c0->kern.batch, dim3(G), dim3(THREADS), args, 0, s);
         if (!cuda_ok(c0, le, "batch_propagate")) return c0->status;
         cudaEventRecord(c0->pev[1], s);

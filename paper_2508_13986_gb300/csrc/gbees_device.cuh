@@ -6,6 +6,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "gbees_keys.cuh"
 
@@ -16,6 +17,8 @@ namespace cg = cooperative_groups;
 constexpr int MAXN = 6;
 constexpr int THREADS = 256;
 constexpr int WARPS = THREADS / 32;
+constexpr int PERSIST_THREADS = 512;                 // block of the persistent step loop
+constexpr int MAX_WARPS = PERSIST_THREADS / 32;      // warps of the largest block that uses the block helpers
 constexpr int GRID_MAX = 8192;                       // blocks of the fixed launch grid (upper bound)
 constexpr unsigned long long EMPTY_KEY = ~0ull;      // free hashtable slot
 
@@ -77,11 +80,8 @@ struct alignas(256) DevScalars {
     unsigned long long tmp_ord;  // scratch maximum (init)
     long long loop_iter;  // iterations of the device-side step loop in the current graph launch
     long long graph_kernels;  // kernels executed by graph launches (counted on the device)
-    // grid barrier of a team of a batched launch: arrivals in the low 32 bits,
-    // generation in the high 32 bits
-    unsigned long long bar_word;
-    // grid barrier of the persistent kernel: arrivals since the launch began
-    // (cleared by the host before every persistent launch)
+    // grid barrier of the persistent kernel and of a team of a batched launch:
+    // arrivals since the launch began (cleared before every such launch)
     unsigned long long bar_seq;
     // the step loop's running reductions, in global atomics: the largest CFL
     // rate of the current prune epoch (two epochs by parity), and the exact
@@ -99,7 +99,6 @@ struct alignas(256) DevScalars {
     int step_last;        // the step lands on t_target
     int step_pad;
     double coef_dth[MAXN];  // dt / h_j
-    double coef_ch[MAXN];   // dt / (2 h_j)
     long long mom[28][NDIG];     // exact sums for moments
     double mom_mean[MAXN];       // mean, input of the covariance pass
     double mom_out[28];          // moments times prod h
@@ -163,7 +162,9 @@ struct alignas(64) Partial {
 // flow leaves through the upper j-face, bit 2j: through the lower j-face),
 // fixed at creation because the drift does not depend on time; bit 14 marks a
 // halo cell; bit 15 marks an active cell whose downwind set is known to be
-// active (cleared by every prune).
+// active (cleared by every prune). Bits 12 and 13 mark a halo cell that a step
+// of a persistent or batched step loop made active (by the step's parity in the
+// launch; cleared by the next step or at the end of the launch).
 //
 // Face velocities (storage type, dimension-major: u[g][j * cap + c]): f_j at
 // the centre of the lower j-face of entry c (Eq. 7), evaluated once in FP64 when
@@ -200,8 +201,9 @@ struct Bufs {
 
 constexpr unsigned short OM_COMPLETE = 0x8000;
 constexpr unsigned short OM_GHOST = 0x4000;
+constexpr unsigned short OM_NEW = 0x1000;  // two bits, by the parity of the loop's step
 
-// The kernels of one time step for one model and precision: those before the
+// The kernels of one time step for one dimension and precision: those before the
 // link phase, those after it, and the persistent step-loop kernel.
 struct Kernels {
     void* pre[3];
@@ -210,7 +212,6 @@ struct Kernels {
     int npost;
     void* persist;
     void* batch;
-    void* batch_teams;
 };
 
 // One grid of a batched propagation (k_batch): its model, its buffers (in its
@@ -221,7 +222,7 @@ struct BatchItem {
     double t_end;
 };
 
-// Block of a team launch (k_batch_teams): the grid it works on (-1: none), the
+// Block of a team launch (k_batch with slots): the grid it works on (-1: none), the
 // team's size and this block's index in the team.
 struct TeamSlot {
     int item, nb, bi;
@@ -251,6 +252,30 @@ struct WarpRuns {
     }
 };
 
+// The same for the step loop of a small grid, in 32-bit numbers (a pool has
+// fewer than 2^31 entries): run k of n_runs, handed out from the block's first
+// warp up (FIRST), or for the few runs that go beside a phase's many from its
+// last warp down (LAST) or from its middle (MIDDLE).
+enum { FIRST, MIDDLE, LAST };
+struct Runs {
+    int k, step, n;
+    __device__ __forceinline__ Runs(int n_runs, int nb, int bi, int place = FIRST) {
+        const int nw = (int)(blockDim.x >> 5);
+        int w = (int)(threadIdx.x >> 5);
+        if (place == LAST) w = nw - 1 - w;
+        if (place == MIDDLE) w = w >= nw / 2 ? w - nw / 2 : w + nw - nw / 2;
+        step = nb * nw;
+        k = bi + nb * w - step;
+        n = n_runs;
+    }
+    __device__ __forceinline__ bool next() {
+        k += step;
+        return k < n;
+    }
+    __device__ __forceinline__ int cell() const { return k * 32 + (int)(threadIdx.x & 31); }
+};
+__device__ __forceinline__ int runs_of(long long entries) { return (int)((entries + 31) >> 5); }
+
 // ------------------------------------------------------------------ keys
 
 template <int N>
@@ -269,6 +294,7 @@ __device__ __forceinline__ void unpack_key(const Model& m, unsigned long long k,
 
 __device__ __forceinline__ int table_find(const Model& m, const Slot* __restrict__ T, unsigned long long key) {
     unsigned long long h = mix64(key) & m.tmask;
+#pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
         ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(T + h));
         if (s.x == key) return (int)(long long)s.y;
@@ -286,6 +312,7 @@ __device__ __forceinline__ int table_find_tile(const Model& m, const Slot* __res
                                                cg::thread_block_tile<W> tile) {
     unsigned long long base = mix64(key) & m.tmask;
     const int lane = tile.thread_rank();
+#pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; probe += W) {
         unsigned long long h = (base + probe + lane) & m.tmask;
         ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(T + h));
@@ -308,6 +335,7 @@ __device__ __forceinline__ int table_find_tile(const Model& m, const Slot* __res
 // slot, 0 when the key is present, -1 when the table is full.
 __device__ __forceinline__ int table_claim(const Model& m, Slot* T, unsigned long long key, unsigned long long* slot) {
     unsigned long long h = mix64(key) & m.tmask;
+#pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
         unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&T[h].key);
         if (k == key) return 0;
@@ -584,65 +612,65 @@ __device__ __forceinline__ void acc_add(long long (&d)[NDIG], float x, int& err)
     }
 }
 
-// Round the exact value sum_q D[q] 2^(32 q + ACC_LSB) once to the nearest double.
-__device__ inline double acc_to_double(const long long* D) {
-    long long c[8];
+// Round the exact value sum_q D[q] 2^(32 q + ACC_LSB) once to the nearest double
+// (ties to even). Straight-line code on registers: one thread of each block
+// runs it once per time step, on the critical path of a small grid's step.
+static __host__ __device__ __noinline__ double acc_to_double(const long long* D) {
+    // carries: base-2^32 digits below a signed top word
+    unsigned int c[NDIG];
+    long long carry = 0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) c[q] = q < NDIG ? D[q] : 0;
-    for (int q = 0; q < 7; ++q) {
-        long long carry = c[q] >> 32;  // floor division by 2^32
-        c[q] -= carry * 4294967296ll;
-        c[q + 1] += carry;
+    for (int q = 0; q < NDIG; ++q) {
+        const long long v = D[q] + carry;
+        c[q] = (unsigned int)(unsigned long long)v;
+        carry = v >> 32;  // floor division by 2^32
     }
-    const bool neg = c[7] < 0;
-    unsigned long long W[4];
-    {
-        unsigned int mag[8];
-        unsigned long long carry = 1;
-        for (int q = 0; q < 8; ++q) {
-            unsigned int v = (unsigned int)(unsigned long long)c[q];
-            if (neg) {
-                unsigned long long s = (unsigned long long)(~v) + carry;
-                mag[q] = (unsigned int)s;
-                carry = s >> 32;
-            } else {
-                mag[q] = v;
-            }
-        }
-        for (int q = 0; q < 4; ++q) W[q] = (unsigned long long)mag[2 * q] | ((unsigned long long)mag[2 * q + 1] << 32);
+    unsigned long long w0 = (unsigned long long)c[0] | ((unsigned long long)c[1] << 32);
+    unsigned long long w1 = (unsigned long long)c[2] | ((unsigned long long)c[3] << 32);
+    unsigned long long w2 = (unsigned long long)c[4] | ((unsigned long long)c[5] << 32);
+    unsigned long long w3 = (unsigned long long)carry;
+    const bool neg = carry < 0;
+    if (neg) {  // the magnitude
+        w0 = ~w0 + 1ull;
+        w1 = ~w1 + (w0 == 0 ? 1ull : 0ull);
+        w2 = ~w2 + (w0 == 0 && w1 == 0 ? 1ull : 0ull);
+        w3 = ~w3 + (w0 == 0 && w1 == 0 && w2 == 0 ? 1ull : 0ull);
     }
-    int top = -1;
-    for (int q = 3; q >= 0; --q)
-        if (W[q]) { top = q; break; }
-    if (top < 0) return 0.0;
-    const int msb = 64 * top + 63 - __clzll((long long)W[top]);
-    auto extract = [&](int shift) -> unsigned long long {  // bits [shift, shift + 64)
-        if (shift < 0) return W[0] << (-shift);
-        int wq = shift >> 6, r = shift & 63;
-        unsigned long long lo = wq < 4 ? W[wq] >> r : 0ull;
-        unsigned long long hi = (r && wq + 1 < 4) ? W[wq + 1] << (64 - r) : 0ull;
-        return lo | hi;
-    };
-    double result;
-    if (msb < 53) {
-        result = ldexp((double)W[0], ACC_LSB);
-    } else {
-        const int sh = msb - 53;  // the 54 bits [sh, msb] hold mantissa + round bit
-        unsigned long long v54 = extract(sh) & ((1ull << 54) - 1);
-        unsigned long long v = v54 >> 1;
-        const unsigned long long round = v54 & 1ull;
-        bool sticky = false;
-        for (int q = 0; q < 4 && !sticky; ++q) {
-            int lo_bit = 64 * q;
-            if (lo_bit >= sh) break;
-            int nb = sh - lo_bit;
-            unsigned long long mask = nb >= 64 ? ~0ull : ((1ull << nb) - 1);
-            sticky = (W[q] & mask) != 0;
-        }
-        if (round && (sticky || (v & 1ull))) v += 1;
-        result = ldexp((double)v, msb - 52 + ACC_LSB);
+    // the top non-zero word, the word below it, and whether anything lies below that
+    unsigned long long hi = w0, lo = 0ull;
+    bool rest = false;
+    int base = 0;
+    if (w3) {
+        hi = w3; lo = w2; rest = (w1 | w0) != 0; base = 192;
+    } else if (w2) {
+        hi = w2; lo = w1; rest = w0 != 0; base = 128;
+    } else if (w1) {
+        hi = w1; lo = w0; base = 64;
     }
-    return neg ? -result : result;
+    if (hi == 0) return 0.0;
+#if defined(__CUDA_ARCH__)
+    const int z = __clzll((long long)hi);
+#else
+    const int z = __builtin_clzll(hi);
+#endif
+    // 64 significant bits and a sticky bit, then 53 bits
+    const unsigned long long m = z ? (hi << z) | (lo >> (64 - z)) : hi;
+    const bool sticky = rest || (z ? (lo << z) : lo) != 0;
+    unsigned long long v = m >> 11;
+    const unsigned int cut = (unsigned int)(m & 0x7FFull);
+    if (cut > 0x400u || (cut == 0x400u && (sticky || (v & 1ull)))) v += 1;
+    // v in [2^52, 2^53]: the exponent field takes a carry out of the mantissa;
+    // the exponent is within [ACC_LSB, ACC_LSB + 255], far inside the normal range
+    const int ex = base + 63 - z + ACC_LSB + 1023;
+    unsigned long long bits = ((unsigned long long)ex << 52) + (v - (1ull << 52));
+    if (neg) bits |= 1ull << 63;
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double((long long)bits);
+#else
+    double r;
+    memcpy(&r, &bits, sizeof r);
+    return r;
+#endif
 }
 
 // Order-preserving map of doubles onto unsigned 64-bit keys (for atomicMax).
@@ -659,8 +687,8 @@ __device__ __forceinline__ double ord_val(unsigned long long k) {
 // digit into global memory. All threads of the block must call it.
 __device__ __forceinline__ void block_reduce_acc_max(long long (&d)[NDIG], double mx, long long* g_acc,
                                                      unsigned long long* g_ord) {
-    __shared__ long long s_acc[WARPS][NDIG];
-    __shared__ double s_mx[WARPS];
+    __shared__ long long s_acc[MAX_WARPS][NDIG];
+    __shared__ double s_mx[MAX_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < NDIG; ++q) {
@@ -677,11 +705,13 @@ __device__ __forceinline__ void block_reduce_acc_max(long long (&d)[NDIG], doubl
     __syncthreads();
     if (threadIdx.x < NDIG) {
         long long v = 0;
+#pragma unroll 4
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += s_acc[w][threadIdx.x];
         if (v) atomicAdd((unsigned long long*)&g_acc[threadIdx.x], (unsigned long long)v);
     }
     if (threadIdx.x == 32 && g_ord) {
         double m = -INFINITY;
+#pragma unroll 4
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, s_mx[w]);
         if (m > -INFINITY) atomicMax(g_ord, ord_key(m));
     }
@@ -689,12 +719,13 @@ __device__ __forceinline__ void block_reduce_acc_max(long long (&d)[NDIG], doubl
 }
 
 __device__ __forceinline__ double block_max(double mx) {
-    __shared__ double s_m[WARPS];
+    __shared__ double s_m[MAX_WARPS];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
     if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mx;
     __syncthreads();
     double m = -INFINITY;
+#pragma unroll 4
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, s_m[w]);
     __syncthreads();
     return m;
@@ -748,8 +779,8 @@ __device__ __forceinline__ void finalise_norm(const Model& m, DevScalars* sc, in
 // maxima are reduced as order-preserving integer keys (integer pipe).
 __device__ __forceinline__ void block_partial(Partial* part, long long (&d)[NDIG], double mx, double rate,
                                               int bi) {
-    __shared__ long long s_acc[WARPS][NDIG];
-    __shared__ unsigned long long s_mx[WARPS], s_rt[WARPS];
+    __shared__ long long s_acc[MAX_WARPS][NDIG];
+    __shared__ unsigned long long s_mx[MAX_WARPS], s_rt[MAX_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long mk = mx > -INFINITY ? ord_key(mx) : 0ull;
     unsigned long long rk = rate > 0.0 ? (unsigned long long)__double_as_longlong(rate) : 0ull;
@@ -774,14 +805,17 @@ __device__ __forceinline__ void block_partial(Partial* part, long long (&d)[NDIG
     const int q = threadIdx.x, nw = (int)(blockDim.x >> 5);
     if (q < NDIG) {
         long long a = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) a += s_acc[w][q];
         part[bi].acc[q] = a;
     } else if (q == NDIG) {
         unsigned long long mm = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) mm = max(mm, s_mx[w]);
         part[bi].maxq_ord = mm;
     } else if (q == NDIG + 1) {
         unsigned long long rr = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) rr = max(rr, s_rt[w]);
         part[bi].rate_bits = rr;
     }
@@ -791,56 +825,56 @@ __device__ __forceinline__ void block_partial(Partial* part, long long (&d)[NDIG
     block_partial(part, d, mx, rate, blockIdx.x);
 }
 
-// The block's digits, maximum value and maximum rate folded into global
-// accumulators with atomics (acc may be null: rate only). Integer sums and
-// maxima: the totals do not depend on the order of the blocks.
-__device__ __forceinline__ void block_atomics(long long* acc, unsigned long long* maxq, unsigned long long* rate,
-                                              long long (&d)[NDIG], double mx, double r) {
-    __shared__ long long s_acc[WARPS][NDIG];
-    __shared__ unsigned long long s_mx[WARPS], s_rt[WARPS];
+// The block's digits and maximum value folded into global accumulators with
+// atomics. Integer sums and maxima: the totals do not depend on the order of
+// the blocks. Within a warp the six digits (padded to eight) are summed
+// together: each exchange halves the values a lane carries, 9 shuffles of 64
+// bits instead of 30.
+__device__ __forceinline__ void block_atomics(long long* acc, unsigned long long* maxq, const long long (&d)[NDIG],
+                                              double mx) {
+    __shared__ long long s_acc[MAX_WARPS][8];
+    __shared__ unsigned long long s_mx[MAX_WARPS];
+    const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long mk = mx > -INFINITY ? ord_key(mx) : 0ull;
-    unsigned long long rk = r > 0.0 ? (unsigned long long)__double_as_longlong(r) : 0ull;
-    if (acc) {
+    long long a[4];
+    {
+        const bool up = lane & 16;
+        const long long hi[4] = {d[4], d[5], 0, 0};
 #pragma unroll
-        for (int q = 0; q < NDIG; ++q) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) d[q] += __shfl_down_sync(0xffffffffu, d[q], off);
+        for (int i = 0; i < 4; ++i) {
+            const long long got = __shfl_xor_sync(full, up ? d[i] : hi[i], 16);
+            a[i] = (up ? hi[i] : d[i]) + got;
         }
-    }
+        const bool up2 = lane & 8;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        mk = max(mk, __shfl_down_sync(0xffffffffu, mk, off));
-        rk = max(rk, __shfl_down_sync(0xffffffffu, rk, off));
+        for (int i = 0; i < 2; ++i) {
+            const long long got = __shfl_xor_sync(full, up2 ? a[i] : a[i + 2], 8);
+            a[i] = (up2 ? a[i + 2] : a[i]) + got;
+        }
+        const bool up4 = lane & 4;
+        const long long got = __shfl_xor_sync(full, up4 ? a[0] : a[1], 4);
+        a[0] = (up4 ? a[1] : a[0]) + got;
+        a[0] += __shfl_xor_sync(full, a[0], 2);
+        a[0] += __shfl_xor_sync(full, a[0], 1);
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < NDIG; ++q) s_acc[wid][q] = d[q];
-        s_mx[wid] = mk;
-        s_rt[wid] = rk;
-    }
+    const unsigned long long mk = mx > -INFINITY ? ord_key(mx) : 0ull;
+    const unsigned top = __reduce_max_sync(full, (unsigned)(mk >> 32));
+    const unsigned low = __reduce_max_sync(full, (unsigned)(mk >> 32) == top ? (unsigned)mk : 0u);
+    if ((lane & 3) == 0) s_acc[wid][lane >> 2] = a[0];
+    if (lane == 0) s_mx[wid] = ((unsigned long long)top << 32) | low;
     __syncthreads();
     const int q = threadIdx.x, nw = (int)(blockDim.x >> 5);
     if (q < NDIG) {
-        if (acc) {
-            long long a = 0;
-            for (int w = 0; w < nw; ++w) a += s_acc[w][q];
-            if (a) atomicAdd((unsigned long long*)&acc[q], (unsigned long long)a);
-        }
+        long long t = 0;
+#pragma unroll 4
+        for (int w = 0; w < nw; ++w) t += s_acc[w][q];
+        if (t) atomicAdd((unsigned long long*)&acc[q], (unsigned long long)t);
     } else if (q == NDIG) {
-        if (maxq) {
-            unsigned long long mm = 0;
-            for (int w = 0; w < nw; ++w) mm = max(mm, s_mx[w]);
-            if (mm) atomicMax(maxq, mm);
-        }
-    } else if (q == NDIG + 1) {
-        if (rate) {
-            unsigned long long rr = 0;
-            for (int w = 0; w < nw; ++w) rr = max(rr, s_rt[w]);
-            if (rr) atomicMax(rate, rr);
-        }
+        unsigned long long mm = 0;
+#pragma unroll 4
+        for (int w = 0; w < nw; ++w) mm = max(mm, s_mx[w]);
+        if (mm) atomicMax(maxq, mm);
     }
-    __syncthreads();
 }
 
 // Combine the partials of blocks [0, nblk) in every thread of the calling
@@ -851,10 +885,11 @@ struct Combined {
     unsigned long long rate_bits;
 };
 __device__ __forceinline__ Combined combine_partials(const Partial* part, int nblk) {
-    __shared__ long long s_acc[WARPS][NDIG];
-    __shared__ unsigned long long s_mo[WARPS], s_rt[WARPS];
+    __shared__ long long s_acc[MAX_WARPS][NDIG];
+    __shared__ unsigned long long s_mo[MAX_WARPS], s_rt[MAX_WARPS];
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
     unsigned long long mo = 0, rt = 0;
+#pragma unroll 1
     for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
         const Partial* p = part + i;
 #pragma unroll
@@ -885,14 +920,17 @@ __device__ __forceinline__ Combined combine_partials(const Partial* part, int nb
     const int q = threadIdx.x, nw = (int)(blockDim.x >> 5);
     if (q < NDIG) {
         long long a = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) a += s_acc[w][q];
         s_fin[q] = (unsigned long long)a;
     } else if (q == NDIG) {
         unsigned long long mm = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) mm = max(mm, s_mo[w]);
         s_fin[q] = mm;
     } else if (q == NDIG + 1) {
         unsigned long long rr = 0;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) rr = max(rr, s_rt[w]);
         s_fin[q] = rr;
     }
@@ -924,70 +962,62 @@ __device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long
     return v;
 }
 
-// Barrier of the nb blocks that share the grid whose scalars are sc (the whole
-// launch, or a team of a batched launch); every block of the team must be
-// resident (cooperative launch). Bounded: gives up with ST_ETIMEOUT.
-__device__ __forceinline__ bool grid_barrier(DevScalars* sc, int nb, long long spin_limit = BARRIER_SPIN_LIMIT) {
-    __shared__ int s_ok;
-    unsigned long long* word = &sc->bar_word;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // one release-acquire add per block: it publishes the block's writes
-        // and counts the arrival; the last to arrive clears the count and opens
-        // the next generation with a second add on the same word (a count of
-        // nb plus 2^32 - nb carries into the generation), so the waiters'
-        // acquire loads see every block's writes once the generation moves
-        const unsigned long long old = atom_add_acq_rel_gpu(word, 1ull);
-        const unsigned int gen = (unsigned int)(old >> 32);
-        int ok = 1;
-        if ((unsigned int)old == (unsigned int)nb - 1u) {
-            atom_add_acq_rel_gpu(word, (1ull << 32) - (unsigned long long)(unsigned int)nb);
-        } else {
-            long long spins = 0;
-            while ((unsigned int)(ld_acquire_gpu(word) >> 32) == gen) {
-                if (*(volatile int*)&sc->error) { ok = 0; break; }
-                if (++spins > spin_limit) {
-                    set_error(sc, ST_ETIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
-            }
+// Barrier k (1, 2, ...) of a launch whose nb blocks all take part in every
+// barrier of the grid with scalars sc (the whole launch, or a team of a batched
+// launch), on a counter that was zero when the launch began: the barrier is
+// complete once k * nb arrivals are counted. One release-acquire add per block
+// publishes the block's writes and counts the arrival; there is no reset, so the
+// last arrival releases the waiters directly. All blocks must be resident
+// (cooperative launch). Bounded: gives up with ST_ETIMEOUT.
+// fetch runs in thread 0 after the barrier is complete, before the block goes
+// on: it reads the scalars that the phase before produced, one reader per
+// block, its loads in flight together with the error word's (read from every
+// thread, the same few words queue up at one L2 slice).
+__device__ __noinline__ static int barrier_wait(DevScalars* sc, unsigned long long target, long long spin_limit) {
+    unsigned long long* cnt = &sc->bar_seq;
+    if (atom_add_acq_rel_gpu(cnt, 1ull) + 1ull >= target) return 1;
+    long long spins = 0;
+    while (ld_acquire_gpu(cnt) < target) {
+        ++spins;
+        // the error word is read now and then: a second load per poll would
+        // double the time until a waiter sees the barrier open
+        if ((spins & 31) == 0) {
+            if (*(volatile int*)&sc->error) return 0;
+            __nanosleep(32);
         }
-        s_ok = ok && !*(volatile int*)&sc->error;
+        if (spins > spin_limit) {
+            set_error(sc, ST_ETIMEOUT);
+            return 0;
+        }
+    }
+    return 1;
+}
+template <typename F>
+__device__ __forceinline__ bool grid_barrier_seq(DevScalars* sc, int nb, unsigned long long& k, long long spin_limit,
+                                                 F&& fetch) {
+    __shared__ int s_ok;
+    __syncthreads();
+    k += 1;
+    if (threadIdx.x == 0) {
+        const int ok = barrier_wait(sc, k * (unsigned long long)(unsigned int)nb, spin_limit);
+        const int e = *(volatile int*)&sc->error;
+        fetch();
+        s_ok = ok && !e;
     }
     __syncthreads();
     return s_ok != 0;
 }
 
-// Barrier k (1, 2, ...) of a launch whose nb blocks all take part in every
-// barrier, on a counter that was zero when the launch began: the barrier is
-// complete once k * nb arrivals are counted. One release-acquire add per block
-// and no reset, so the last arrival releases the waiters directly. Bounded like
-// grid_barrier.
-__device__ __forceinline__ bool grid_barrier_seq(DevScalars* sc, int nb, unsigned long long& k,
-                                                 long long spin_limit = BARRIER_SPIN_LIMIT) {
+// The same for a block that works alone: a block barrier, the error word read
+// by one thread.
+template <typename F>
+__device__ __forceinline__ bool block_barrier(DevScalars* sc, F&& fetch) {
     __shared__ int s_ok;
-    unsigned long long* cnt = &sc->bar_seq;
     __syncthreads();
-    k += 1;
     if (threadIdx.x == 0) {
-        const unsigned long long target = k * (unsigned long long)(unsigned int)nb;
-        const unsigned long long old = atom_add_acq_rel_gpu(cnt, 1ull);
-        int ok = 1;
-        if (old + 1ull < target) {
-            long long spins = 0;
-            while (ld_acquire_gpu(cnt) < target) {
-                if (*(volatile int*)&sc->error) { ok = 0; break; }
-                if (++spins > spin_limit) {
-                    set_error(sc, ST_ETIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
-            }
-        }
-        s_ok = ok && !*(volatile int*)&sc->error;
+        const int e = *(volatile int*)&sc->error;
+        fetch();
+        s_ok = !e;
     }
     __syncthreads();
     return s_ok != 0;
@@ -995,13 +1025,14 @@ __device__ __forceinline__ bool grid_barrier_seq(DevScalars* sc, int nb, unsigne
 
 // Exclusive prefix of a 0/1 flag over the block (in thread order) and the total.
 __device__ __forceinline__ int block_exclusive_scan(int flag, int& total) {
-    __shared__ int s_w[WARPS];
+    __shared__ int s_w[MAX_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned bal = __ballot_sync(0xffffffffu, flag);
     int in_warp = __popc(bal & ((1u << lane) - 1u));
     if (lane == 0) s_w[wid] = __popc(bal);
     __syncthreads();
     int before = 0, tot = 0;
+#pragma unroll 4
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
         int v = s_w[w];
         if (w < wid) before += v;

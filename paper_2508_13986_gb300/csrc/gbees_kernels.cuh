@@ -21,7 +21,7 @@ __device__ __forceinline__ void finish_link(const Model& m, DevScalars* sc, cons
     unsigned long long r = max(sc->maxrate_bits, cr.rate_bits);
     sc->maxrate_bits = r;
     if (step) {
-        StepTime st = step_time(m, __longlong_as_double((long long)r), sc->t, sc->t_target, sc->coef_dth, sc->coef_ch);
+        StepTime st = step_time(m, __longlong_as_double((long long)r), sc->t, sc->t_target, sc->coef_dth);
         if (!(st.dt > 0.0)) set_error(sc, ST_EDEGENERATE);  // no progress possible
         sc->step_dt = st.dt;
         sc->step_t_new = st.t_new;
@@ -264,12 +264,12 @@ __device__ __forceinline__ void finish_step(const Model& m, DevScalars* sc, cons
 // The first phase of a step of a large grid in two kernels: the waves of the
 // existing entries, listing the cells that grow (no block-wide rounds over the
 // whole pool), then every (listed cell, candidate) pair over the grid.
-template <int N, int DYN, typename T>
+template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_waves_list(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
     const StepView v = view_of(m, sc);
-    waves_body<N, DYN, T, true>(m, b, v, v.N_prev);
+    waves_body<N, T, true>(m, b, v, v.N_prev);
 }
 
 template <int N, typename T>
@@ -283,11 +283,11 @@ __global__ void __launch_bounds__(THREADS) k_grow_list(const Model m, Bufs b) {
 // Flux update, pass 2: the flux through every face that touches an active
 // cell: donor cell (Eq. 7), the transverse terms of Algorithm 1 read from the
 // upwind cell's wave row, and the limited high-resolution term.
-template <int N, int DYN, typename T>
+template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_faces(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    faces_body<N, DYN, T>(m, b, view_of(m, sc));
+    faces_body<N, T>(m, b, view_of(m, sc));
 }
 
 // Flux update, pass 3: the conservative update of every active cell from the

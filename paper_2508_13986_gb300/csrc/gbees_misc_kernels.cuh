@@ -27,7 +27,14 @@ __global__ void k_batch_begin(const BatchItem* items, int count) {
         sc->done = !(sc->t < tt) || sc->error != 0;
         sc->steps_call = 0;
         sc->updates_call = 0;
+        sc->bar_seq = 0;
     }
+}
+
+// A further launch of the same batch: the teams' barriers count from zero.
+__global__ void k_batch_again(const BatchItem* items, int count) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
+        items[i].b.sc->bar_seq = 0;
 }
 
 // Copy the scalars of every grid of a batch into one array (one read-back).
@@ -131,7 +138,6 @@ __global__ void k_reset(DevScalars* sc, double t0) {
     sc->tmp_ord = 0;
     sc->loop_iter = 0;
     sc->graph_kernels = 0;
-    sc->bar_word = 0;
     sc->bar_seq = 0;
     for (int e = 0; e < 2; ++e) {
         sc->loop_rate[e] = 0;

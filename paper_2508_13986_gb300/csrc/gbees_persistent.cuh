@@ -4,42 +4,51 @@
 // time step is a few microseconds of work split into dependent phases; kernel
 // launches and their drain would dominate. This cooperative kernel keeps one
 // block per SM resident and separates the phases by a bounded grid barrier
-// (the cooperative-kernel structure of Sec. 4, with GB300's block count).
+// (the cooperative-kernel structure of Sec. 4, with GB300's block count). 512
+// threads: a pool of 7.8 * 10^4 entries has one entry per thread.
+// What bounds a step is the longest chain of its phases and the instruction
+// fetch (L1 instruction cache 32 KB, beyond it straight code runs at a third of
+// the rate): the phases' code is kept small, rare work out of line. Lorenz '63,
+// h = 0.25, 5 * 10^3 to 5 * 10^4 pool entries: 26.0 us per FP64 step and 25.3 us per FP32
+// step (38.2 and 35.4 us with five phases, each work item's chain in one
+// thread, in 214 KB of code); h = 0.5, 7 * 10^3 entries: 23.0 us (35.3 us).
 //
-// k_batch: many independent grids in one launch. Each block takes a grid from
-// a queue and runs its whole step loop alone, the phases separated by block
-// barriers; blocks never wait on each other, so the launch needs no
+// k_batch: many independent grids in one launch. With a team of blocks per grid
+// (all grids resident, a cooperative launch), or as a queue: each block takes a
+// grid and runs its whole step loop alone, the phases separated by block
+// barriers; blocks never wait on each other then, so the launch needs no
 // co-residency and ragged grids balance over the SMs.
 //
 // Every block computes the step's scalars (dt, normalisation, maximum) itself
-// from the same per-block partials, so the scalars need no extra barrier;
-// block 0 of the grid writes them back.
+// from the same sums, so the scalars need no extra barrier; block 0 of the grid
+// writes them back at the end.
 //
-// Barriers per step: grow + waves | halo | link | faces | apply (halo and link
-// are skipped in a step whose grow added and activated nothing); a prune adds
-// mark | scatter | status | compact | relink.
+// Barriers per step: waves + grow | new halo cells + fluxes | update; a prune
+// adds mark | scatter | status | compact | relink. The normalisation of a step
+// and the next dt are formed by one warp beside the grow of the next step.
 #pragma once
 
 #include "gbees_kernels.cuh"
 
 namespace gbees {
 
-// The step's scalars, computed by one thread of each block (FP64 divisions are
-// expensive on this chip) and read by the others from shared memory.
+// What one thread of each block reads or computes for the others.
 struct StepShared {
     double dt, t_new, scale, maxq, w;
-    double dth[MAXN], ch[MAXN];
-    unsigned long long maxrate;
+    double dth[MAXN];
+    unsigned long long maxrate;           // largest CFL rate of the active cells
+    long long n_ins, n_act, n_halo;  // counts after the grow, after the halo
     int last, bad;
 };
 
-// w = (prod h) sum, 1 / w and the maximum from combined partials (one thread).
-__device__ __forceinline__ void normalisation(const Model& m, const Combined& c, StepShared& ss) {
-    const double w = m.prod_h * acc_to_double(c.acc);
+// w = (prod h) sum, 1 / w and the maximum from combined sums (one thread).
+static __device__ __noinline__ void normalisation(const Model& m, const long long* acc, unsigned long long maxq_ord,
+                                              StepShared& ss) {
+    const double w = m.prod_h * acc_to_double(acc);
     ss.w = w;
     ss.bad = !(w > 0.0) || !isfinite(w);
     ss.scale = ss.bad ? 0.0 : 1.0 / w;
-    ss.maxq = c.maxq_ord ? ord_val(c.maxq_ord) : 0.0;
+    ss.maxq = maxq_ord ? ord_val(maxq_ord) : 0.0;
 }
 
 // Up to max_steps steps of the grid (m, b) by the nb blocks of index bi that
@@ -48,23 +57,23 @@ __device__ __forceinline__ void normalisation(const Model& m, const Combined& c,
 // max_pool: the loop also stops after a step that leaves more pool entries
 // than that (the persistent kernel hands a grown grid to the graph path; every
 // block sees the same count, so all leave together).
-// seq: the nb blocks are the whole launch and sc->bar_seq was zero when it
-// began (the persistent kernel), so the barriers count arrivals without reset.
-template <int N, int DYN, typename T>
+// sc->bar_seq was zero when the launch began.
+template <int N, typename T>
 __device__ __forceinline__ void step_loop(const Model& m, const Bufs& b, long long max_steps, int nb, int bi,
-                                          long long max_pool = 0x7fffffffffffffffll, bool seq = false) {
+                                          long long max_pool = 0x7fffffffffffffffll) {
     __shared__ StepShared ss;
+    __shared__ GrowQueue gq;
     DevScalars* sc = b.sc;
     // The result is the same for every thread of the block: a warp that read
     // the error flag after another warp of the block had already raised it in
     // the next phase must not return while the others go on (their block
     // barriers would then pair with the wrong ones).
     unsigned long long n_bar = 0;
-    auto barrier = [&]() -> bool {
-        if (nb == 1) return __syncthreads_and(!*(volatile int*)&sc->error) != 0;
-        if (seq) return grid_barrier_seq(sc, nb + m.bar_extra, n_bar, m.spin_limit);
-        return grid_barrier(sc, nb + m.bar_extra, m.spin_limit);
+    auto barrier = [&](auto&& fetch) -> bool {
+        if (nb == 1) return block_barrier(sc, fetch);
+        return grid_barrier_seq(sc, nb + m.bar_extra, n_bar, m.spin_limit, fetch);
     };
+    auto nothing = [] {};
     StepView v = view_of(m, sc);
     v.nb = nb;
     v.bi = bi;
@@ -75,153 +84,186 @@ __device__ __forceinline__ void step_loop(const Model& m, const Bufs& b, long lo
     unsigned long long maxrate = *(volatile unsigned long long*)&sc->maxrate_bits;
     double w = *(volatile double*)&sc->w;
     double last_dt = *(volatile double*)&sc->dt;
+    long long n_active = *(volatile long long*)&sc->NA;
     long long nsteps = 0, nupd = 0;
+    const bool lead = bi == 0 && threadIdx.x == 0;
     // the running reductions start from the state (before the first barrier,
     // which orders these writes before every use)
     int ep = 0;  // parity of the prune epoch in loop_rate
-    if (bi == 0 && threadIdx.x == 0 && !done) {
+    if (lead && !done) {
         sc->loop_rate[0] = maxrate;
         for (int e = 0; e < 2; ++e) {
             sc->loop_maxq[e] = 0;
             for (int q = 0; q < NDIG; ++q) sc->loop_acc[e][q] = 0;
         }
     }
+    if (threadIdx.x == 0) {
+        ss.maxrate = maxrate;
+        ss.bad = 0;
+    }
     // every block has read the state before anyone changes it
-    if (done || *(volatile int*)&sc->error || !barrier()) return;
+    if (done || *(volatile int*)&sc->error || !barrier(nothing)) return;
     // phase timing by block 0 (cycles between the barriers it passes)
     long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     long long t_mark = clock64();
     auto mark = [&](int ph) {
-        if (bi == 0 && threadIdx.x == 0) {
+        if (lead) {
             const long long now = clock64();
             pc[ph] += now - t_mark;
             t_mark = now;
         }
     };
+    // The normalisation of the step before is still to be formed from its sums
+    // (slot `from` of loop_acc), by one thread: beside the grow of the next step
+    // in the block's last warp (the grow needs the maximum alone), or at once
+    // before a prune and at the end.
+    bool pending = false;
+    auto normalise = [&](int from) {
+        long long acc[NDIG];
+#pragma unroll
+        for (int q = 0; q < NDIG; ++q) acc[q] = *(volatile long long*)&sc->loop_acc[from][q];
+        normalisation(m, acc, *(volatile unsigned long long*)&sc->loop_maxq[from], ss);
+    };
+    auto take = [&] {  // every thread, after a block barrier
+        w = ss.w;
+        v.scale = ss.scale;
+        v.maxq = ss.maxq;
+        pending = false;
+    };
+    bool marks = false;      // the last step's activated cells still carry their marks
+    double free_dt = 0.0;    // thread 0: cfl / rate of free_rate
+    unsigned long long free_rate = 0;
 
     for (long long it = 0; it < max_steps && !done; ++it) {
-        // grow (appends active cells to sc->N, activates halo cells) and the
-        // waves of the existing entries alongside
-        const double rg = grow_body<N, T>(m, b, v);
-        waves_body<N, DYN, T>(m, b, v, v.N_prev);
-        if (!barrier()) return;
-        mark(0);
-        // every block read the other apply slot in the previous step: clear it
-        // for the next one
-        if (bi == 0 && threadIdx.x == 0) {
-            sc->loop_maxq[(it + 1) & 1] = 0;
-            for (int q = 0; q < NDIG; ++q) sc->loop_acc[(it + 1) & 1][q] = 0;
+        // 1: waves of the existing entries; the grow
+        v.fresh = (it & 1) ? 2u * OM_NEW : 1u * OM_NEW;
+        if (threadIdx.x == 0) gq.n = 0;
+        if (pending && threadIdx.x == blockDim.x - 64) {
+            const unsigned long long o = *(volatile unsigned long long*)&sc->loop_maxq[(it - 1) & 1];
+            ss.maxq = o ? ord_val(o) : 0.0;
         }
-        // halo cells around the newly active cells (appended after sc->N, which
-        // stays put until the link phase)
-        const long long n_ins = min(*(volatile long long*)&sc->N, m.cap);
-        const long long n_active = *(volatile long long*)&sc->NA;
-        const long long n_act = *(volatile long long*)&sc->n_act;
-        if (n_ins == v.N_prev && n_act == 0) {
-            // the grow added and activated nothing (every block reads the same
-            // counts): no halo to make, no entry to link, no new CFL rate
-            v.N = n_ins;
-            mark(1);
-            mark(2);
-        } else {
-            halo_body<N, T>(m, b, v, v.N_prev, n_ins, n_act);
-            if (!barrier()) return;
-            mark(1);
-            v.N = min(n_ins + *(volatile long long*)&sc->n_halo, m.cap);
-            // link the new entries; CFL rates of the new active cells
-            {
-                const double r = fmax(rg, link_body<N, T>(m, b, v.N_prev, v.N, v.g, nb, bi));
-                long long zero[NDIG] = {0, 0, 0, 0, 0, 0};
-                block_atomics(nullptr, nullptr, &sc->loop_rate[ep], zero, -INFINITY, r);
-            }
-            if (bi == 0 && threadIdx.x == 0) sc->N = v.N;  // read again only after the next grow
-            if (!barrier()) return;
-            mark(2);
-            // everyone has read the halo and activation counts: reset them
-            if (bi == 0 && threadIdx.x == 0) {
-                sc->n_halo = 0;
-                sc->n_act = 0;
-            }
-            // the epoch's largest rate, every block's included (thread 0 uses it)
-            if (threadIdx.x == 0) maxrate = max(maxrate, *(volatile unsigned long long*)&sc->loop_rate[ep]);
-        }
-        if (threadIdx.x == 0) {
-            const StepTime st0 = step_time(m, __longlong_as_double((long long)maxrate), t, tt, ss.dth, ss.ch);
-            ss.dt = st0.dt;
-            ss.t_new = st0.t_new;
-            ss.last = st0.last;
-        }
+        waves_small_body<N, T>(m, b, v);
         __syncthreads();
-        StepTime st;
-        st.dt = ss.dt;
-        st.t_new = ss.t_new;
-        st.last = ss.last;
-        v.dt = ss.dt;
-#pragma unroll
-        for (int k = 0; k < MAXN; ++k) {
-            v.dth[k] = ss.dth[k];
-            v.ch[k] = ss.ch[k];
+        if (pending) v.maxq = ss.maxq;
+        // dt of Eq. 8 needs the new active cells' rates. They rarely exceed the
+        // largest one known: the step's time is formed for that before the
+        // barrier and again only if it does
+        auto set_time = [&](unsigned long long r) {
+            if (r != free_rate || free_dt == 0.0) {
+                free_rate = r;
+                const double rate = __longlong_as_double((long long)r);
+                free_dt = rate > 0.0 ? __ddiv_rn(m.cfl, rate) : (double)INFINITY;
+            }
+            const StepTime st = step_time_of(m, free_dt, t, tt, ss.dth);
+            ss.dt = st.dt;
+            ss.t_new = st.t_new;
+            ss.last = st.last;
+            if (r != ss.maxrate) ss.maxrate = r;
+        };
+        if (threadIdx.x == blockDim.x - 32) {
+            if (pending) normalise((int)((it - 1) & 1));
+            set_time(ss.maxrate);
         }
+        grow_detect<N, T>(m, b, v, gq, ss.maxrate, &sc->loop_rate[ep]);
         __syncthreads();
-        if (!(st.dt > 0.0)) {
-            set_error(sc, ST_EDEGENERATE);
+        grow_drain<N, T>(m, b, v, gq, ss.maxrate, &sc->loop_rate[ep]);
+        if (!barrier([&] {
+                const long long n_ins = *(volatile long long*)&sc->N;
+                ss.n_act = *(volatile long long*)&sc->n_act;
+                const unsigned long long r =
+                    max(ss.maxrate, *(volatile unsigned long long*)&sc->loop_rate[ep]);
+                ss.n_ins = min(n_ins, m.cap);
+                if (r != ss.maxrate) set_time(r);
+            }))
             return;
-        }
-        mark(6);
-        // flux update
-        long long d[NDIG] = {0, 0, 0, 0, 0, 0};
-        double mx = -INFINITY;
-        int err = 0;
-        faces_body<N, DYN, T, true>(m, b, v);
-        if (!barrier()) return;
-        mark(3);
-        apply_body<N, T, true>(m, b, v, d, mx, err);
-        if (err) set_error(sc, ST_EDEGENERATE);
-        block_atomics(sc->loop_acc[it & 1], &sc->loop_maxq[it & 1], nullptr, d, mx, 0.0);
-        if (!barrier()) return;
-        mark(4);
-        {
-            if (threadIdx.x == 0) {
-                Combined cs;
-#pragma unroll
-                for (int q = 0; q < NDIG; ++q) cs.acc[q] = *(volatile long long*)&sc->loop_acc[it & 1][q];
-                cs.maxq_ord = *(volatile unsigned long long*)&sc->loop_maxq[it & 1];
-                cs.rate_bits = 0;
-                normalisation(m, cs, ss);
-            }
-            __syncthreads();
-            w = ss.w;
-            v.scale = ss.scale;
-            v.maxq = ss.maxq;
-            const int bad = ss.bad;
-            __syncthreads();
-            if (bad) {
+        if (pending) {
+            take();
+            if (ss.bad) {
                 set_error(sc, ST_EDEGENERATE);
                 return;
             }
         }
-        t = st.t_new;
-        last_dt = st.dt;
-        done = st.last;
+        const long long n_ins = ss.n_ins, n_act = ss.n_act;
+        n_active += n_ins - v.N_prev + n_act;
+        const double t_new = ss.t_new;
+        const int last = ss.last;
+        maxrate = ss.maxrate;
+        v.dt = ss.dt;
+#pragma unroll
+        for (int k = 0; k < N; ++k) v.dth[k] = ss.dth[k];
+        if (!(v.dt > 0.0)) {
+            set_error(sc, ST_EDEGENERATE);
+            return;
+        }
+        mark(0);
+        // every block has read the other slot of the sums: clear it for the next step
+        if (lead) {
+            sc->loop_maxq[(it + 1) & 1] = 0;
+            for (int q = 0; q < NDIG; ++q) sc->loop_acc[(it + 1) & 1][q] = 0;
+        }
+        // 2: new halo cells; fluxes between existing entries
+        halo_claim_body<N, T>(m, b, v, n_ins, n_act);
+        faces_old_body<N, T>(m, b, v);
+        if (!barrier([&] { ss.n_halo = *(volatile long long*)&sc->n_halo; })) return;
+        v.N = min(n_ins + ss.n_halo, m.cap);
+        mark(3);
+        // the counts have been read by all: the next grow starts from them
+        if (lead) {
+            sc->N = v.N;
+            sc->n_act = 0;
+        }
+        // 3: the update; the new halo cells
+        halo_complete_body<N, T>(m, b, v, n_ins);
+        {
+            long long d[NDIG] = {0, 0, 0, 0, 0, 0};
+            T mx = -INFINITY;
+            int err = 0;
+            apply_small_body<N, T>(m, b, v, n_ins, n_act, d, mx, err);
+            if (err) set_error(sc, ST_EDEGENERATE);
+            block_atomics(sc->loop_acc[it & 1], &sc->loop_maxq[it & 1], d, (double)mx);
+        }
+        if (!barrier(nothing)) return;
+        mark(4);
+        if (lead) sc->n_halo = 0;  // read by all before this barrier, added to after the next
+        pending = true;
+        marks = n_act > 0;
+        t = t_new;
+        last_dt = v.dt;
+        done = last;
         step += 1;
         nsteps += 1;
         nupd += n_active;
         v.pb ^= 1;
+        const bool prune = m.prune_interval > 0 && step % m.prune_interval == 0;
+        const bool leave = done || it + 1 == max_steps || v.N > max_pool;
+        if (prune || leave) {
+            if (threadIdx.x == 0) normalise((int)(it & 1));
+            __syncthreads();
+            take();
+            if (ss.bad) {
+                set_error(sc, ST_EDEGENERATE);
+                return;
+            }
+            mark(6);
+        }
+        if (leave && !prune && marks) clear_marks(b, v, n_act);
         v.N_prev = v.N;
-        mark(6);
         // prune (Algorithm 3) every prune_interval steps
-        if (m.prune_interval > 0 && step % m.prune_interval == 0) {
+        if (prune) {
             prune_mark_body<T>(m, b, v);
-            if (!barrier()) return;
+            if (!barrier(nothing)) return;
             prune_scatter_body<N, T>(m, b, v);
-            if (!barrier()) return;
+            if (!barrier(nothing)) return;
             prune_count_body<N>(m, b, v);
-            if (!barrier()) return;
+            if (!barrier(nothing)) return;
             const Survivors sv = block_offsets(b, v.nb, v.bi);
             const long long total = sv.total_a + sv.total_g;
-            if (bi == 0 && threadIdx.x == 0) {  // before the next grow appends
+            n_active = sv.total_a;
+            if (lead) {  // before the next grow appends
                 sc->N = total;
-                sc->NA = sv.total_a;
+                // a new epoch of the running rate: the new cells' largest, beside
+                // the survivors' (in ss.maxrate)
+                sc->loop_rate[ep ^ 1] = 0;
             }
             {
                 long long dp[NDIG] = {0, 0, 0, 0, 0, 0};
@@ -231,25 +273,22 @@ __device__ __forceinline__ void step_loop(const Model& m, const Bufs& b, long lo
                 if (errp) set_error(sc, ST_EDEGENERATE);
                 block_partial(b.part, dp, mxp, rmax, bi);
             }
-            if (!barrier()) return;
+            if (!barrier(nothing)) return;
             prune_relink_body<N>(m, b, v);
-            if (!barrier()) return;
-            Combined cp = combine_partials(b.part, nb);
-            if (threadIdx.x == 0) normalisation(m, cp, ss);
+            if (!barrier(nothing)) return;
+            const Combined cp = combine_partials(b.part, nb);
+            if (threadIdx.x == 0) {
+                normalisation(m, cp.acc, cp.maxq_ord, ss);
+                ss.maxrate = cp.rate_bits;
+            }
             __syncthreads();
-            w = ss.w;
-            v.scale = ss.scale;
-            v.maxq = ss.maxq;
-            const int bad = ss.bad || sv.total_a == 0;
-            __syncthreads();
-            if (bad) {
+            take();
+            if (ss.bad || sv.total_a == 0) {
                 set_error(sc, ST_EDEGENERATE);
                 return;
             }
             maxrate = cp.rate_bits;
-            // a new epoch of the running rate starts from the survivors' largest
             ep ^= 1;
-            if (bi == 0 && threadIdx.x == 0) sc->loop_rate[ep] = maxrate;
             mark(5);
             v.N = total;
             v.N_prev = total;
@@ -258,8 +297,9 @@ __device__ __forceinline__ void step_loop(const Model& m, const Bufs& b, long lo
         }
         if (v.N > max_pool) break;
     }
-    if (bi == 0 && threadIdx.x == 0) {
+    if (lead) {
         sc->N = v.N;
+        sc->NA = n_active;
         sc->N_prev = v.N_prev;
         sc->pbuf = v.pb;
         sc->gen = v.g;
@@ -274,18 +314,17 @@ __device__ __forceinline__ void step_loop(const Model& m, const Bufs& b, long lo
         sc->steps_call += nsteps;
         sc->updates_call += nupd;
         sc->prune_now = 0;
-    }
-    if (bi == 0 && threadIdx.x == 0) {
         for (int q = 0; q < 8; ++q) sc->phase_cycles[q] += pc[q];
         sc->phase_steps += nsteps;
     }
 }
 
 
-template <int N, int DYN, typename T>
-__global__ void __launch_bounds__(THREADS, 1) k_persistent(const Model m, Bufs b, long long max_steps,
-                                                           long long max_pool) {
-    step_loop<N, DYN, T>(m, b, max_steps, gridDim.x, blockIdx.x, max_pool, true);
+template <int N, typename T>
+__global__ void __launch_bounds__(PERSIST_THREADS, 1) k_persistent(const __grid_constant__ Model m,
+                                                                   const __grid_constant__ Bufs b, long long max_steps,
+                                                                   long long max_pool) {
+    step_loop<N, T>(m, b, max_steps, gridDim.x, blockIdx.x, max_pool);
 }
 
 // Resident blocks per SM of the batch kernels: the register cap (64) spills a
@@ -294,35 +333,38 @@ __global__ void __launch_bounds__(THREADS, 1) k_persistent(const Model m, Bufs b
 // two blocks per SM on 256 Lorenz '63 grids).
 constexpr int BATCH_BLOCKS_PER_SM = 4;
 
-// k_batch: block after block takes the next grid of the queue (next counts the
-// grids handed out) and runs up to max_steps of its steps. A grid that is done
-// or in error returns at once, so a launch can be repeated until all are done.
-template <int N, int DYN, typename T>
-__global__ void __launch_bounds__(THREADS, BATCH_BLOCKS_PER_SM) k_batch(const BatchItem* items, int count, unsigned int* next,
-                                                  long long max_steps) {
-    __shared__ int s_item;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
-        __syncthreads();
-        const int i = s_item;
-        __syncthreads();
-        if (i >= count) return;
-        const Bufs b = items[i].b;
-        step_loop<N, DYN, T>(items[i].m, b, max_steps, 1, 0);
-        __syncthreads();
-    }
-}
-
-// k_batch_teams: a cooperative launch in which every grid has a team of
+// Many grids in one launch, in one of two forms.
+// slots null (queue): block after block takes the next grid of the queue (next
+// counts the grids handed out) and runs up to max_steps of its steps. A grid
+// that is done or in error returns at once, so a launch can be repeated until
+// all are done.
+// slots given (teams): a cooperative launch in which every grid has a team of
 // blocks (slots[blockIdx.x]) sized to its work, the team's phases separated by
 // a barrier on the grid's own scalars.
-template <int N, int DYN, typename T>
-__global__ void __launch_bounds__(THREADS, BATCH_BLOCKS_PER_SM) k_batch_teams(const BatchItem* items, const TeamSlot* slots,
-                                                        long long max_steps) {
-    const TeamSlot ts = slots[blockIdx.x];
-    if (ts.item < 0) return;
-    const Bufs b = items[ts.item].b;
-    step_loop<N, DYN, T>(items[ts.item].m, b, max_steps, ts.nb, ts.bi);
+template <int N, typename T>
+__global__ void __launch_bounds__(THREADS, BATCH_BLOCKS_PER_SM) k_batch(const BatchItem* items, int count,
+                                                                        unsigned int* next, const TeamSlot* slots,
+                                                                        long long max_steps) {
+    __shared__ int s_item;
+    for (;;) {
+        int i, nb = 1, bi = 0;
+        if (slots) {
+            const TeamSlot ts = slots[blockIdx.x];
+            i = ts.item;
+            nb = ts.nb;
+            bi = ts.bi;
+            if (i < 0) return;
+        } else {
+            if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+            __syncthreads();
+            i = s_item;
+            __syncthreads();
+            if (i >= count) return;
+        }
+        step_loop<N, T>(items[i].m, items[i].b, max_steps, nb, bi);
+        if (slots) return;
+        __syncthreads();
+    }
 }
 
 }  // namespace gbees

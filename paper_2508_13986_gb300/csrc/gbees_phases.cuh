@@ -5,6 +5,10 @@
 // launch, so no pointer here is marked read-only (no non-coherent loads): the
 // grid barrier's fences make plain loads see the other blocks' writes.
 //
+// A large grid runs them one kernel each; the step loop of a small grid (one
+// resident launch, gbees_persistent.cuh) has forms of its own for grow, halo,
+// link, faces and apply (below, "step loop of a small grid").
+//
 //   grow       directional grow of the significant cells (Sec. 3.3, Algorithm 2)
 //   halo       the missing face neighbours of the newly active cells, as halo cells
 //   link       neighbour links, outward mask and CFL rate of the new entries (Sec. 4.1)
@@ -31,9 +35,9 @@ struct StepView {
     double maxq;       // max stored value (threshold p* = thr_rel * maxq)
     double scale;      // 1 / w of the previous normalisation
     double dth[MAXN];  // dt / h_j of this step
-    double ch[MAXN];   // dt / (2 h_j)
     double dt;         // dt of this step
     int nb, bi;        // the blocks that share this grid's work, and this block's index among them
+    unsigned fresh;    // flag of the halo cells that this step makes active (step loop of a small grid)
 };
 
 __device__ __forceinline__ StepView view_of(const Model& m, DevScalars* sc) {
@@ -44,32 +48,28 @@ __device__ __forceinline__ StepView view_of(const Model& m, DevScalars* sc) {
     v.g = *(volatile int*)&sc->gen;
     v.maxq = *(volatile double*)&sc->maxq;
     v.scale = *(volatile double*)&sc->scale;
-    for (int j = 0; j < MAXN; ++j) {
-        v.dth[j] = *(volatile double*)&sc->coef_dth[j];
-        v.ch[j] = *(volatile double*)&sc->coef_ch[j];
-    }
+    for (int j = 0; j < MAXN; ++j) v.dth[j] = *(volatile double*)&sc->coef_dth[j];
     v.dt = *(volatile double*)&sc->step_dt;
     v.nb = gridDim.x;
     v.bi = blockIdx.x;
+    v.fresh = OM_NEW;
     return v;
 }
 
 // dt of Eq. 8 (CFL over the maximum rate, clipped to land on the target) and
-// its coefficients; the same IEEE operations wherever it is evaluated.
+// its coefficients dt / h_j; the same IEEE operations wherever it is evaluated.
 struct StepTime {
     double dt, t_new;
     int last;
 };
-__device__ __forceinline__ StepTime step_time(const Model& m, double rate, double t, double tt, double* dth,
-                                              double* ch) {
-    double dt = rate > 0.0 ? __ddiv_rn(m.cfl, rate) : (double)INFINITY;
+// free_dt: cfl over the maximum rate (infinite when every rate is zero).
+__device__ __forceinline__ StepTime step_time_of(const Model& m, double free_dt, double t, double tt, double* dth) {
+    double dt = free_dt;
     const double rem = __dsub_rn(tt, t);
     const bool last = dt >= rem;
     if (last) dt = rem;
-    for (int j = 0; j < MAXN; ++j) {
-        dth[j] = j < m.n ? dt * m.inv_h[j] : 0.0;
-        ch[j] = j < m.n ? dt * m.inv_2h[j] : 0.0;
-    }
+#pragma unroll
+    for (int j = 0; j < MAXN; ++j) dth[j] = j < m.n ? dt * m.inv_h[j] : 0.0;
     StepTime s;
     s.dt = dt;
     s.last = last;
@@ -81,6 +81,9 @@ __device__ __forceinline__ StepTime step_time(const Model& m, double rate, doubl
         s.t_new = tt;
     }
     return s;
+}
+__device__ __forceinline__ StepTime step_time(const Model& m, double rate, double t, double tt, double* dth) {
+    return step_time_of(m, rate > 0.0 ? __ddiv_rn(m.cfl, rate) : (double)INFINITY, t, tt, dth);
 }
 
 // The outward directions of cell I: bit 2j+1 when the flow leaves through the
@@ -140,11 +143,12 @@ __device__ __forceinline__ void table_insert_new(const Model& m, const Bufs& b, 
 
 // ------------------------------------------------------------------ grow
 
-// Entry e is a halo cell: make it active. True for the one thread that does.
-__device__ __forceinline__ bool activate(unsigned short* om, long long e) {
+// Entry e is a halo cell: make it active (mark: flags to set with it). True for
+// the one thread that does.
+__device__ __forceinline__ bool activate(unsigned short* om, long long e, unsigned short mark = 0) {
     unsigned short old = *(volatile unsigned short*)&om[e];
     while (old & OM_GHOST) {
-        const unsigned short prev = atomicCAS(&om[e], old, (unsigned short)(old & ~OM_GHOST));
+        const unsigned short prev = atomicCAS(&om[e], old, (unsigned short)((old & ~OM_GHOST) | mark));
         if (prev == old) return true;
         old = prev;
     }
@@ -206,14 +210,26 @@ __device__ __forceinline__ long long insert_cell(const Model& m, const Bufs& b, 
 //
 // The candidates of a cell (2n faces, 4 C(n,2) edges, those that are not
 // downwind skipped at once) are independent chains of dependent loads and
-// atomics, spread over many threads: grow_body gathers a block's qualifying
-// cells in shared memory (the persistent and batch step loops); for large
-// grids the wave pass lists them (grow_list_mark) and a kernel of its own
-// spreads every (cell, candidate) pair of the list over the grid
-// (grow_list_body).
+// atomics, spread over many threads: for large grids the wave pass lists the
+// growing cells (grow_list_mark) and a kernel of its own spreads every (cell,
+// candidate) pair of the list over the grid (grow_list_body); the step loop of
+// a small grid has grow_detect and grow_act.
 struct GrowWork {
     double rmax = 0.0;  // largest CFL rate of the halo cells this thread activated
 };
+
+// The two directions d1 < d2 (of different dimensions) of edge candidate k >= 2N.
+template <int N>
+__device__ __forceinline__ void edge_dirs(int k, int& d1, int& d2) {
+    const int e = k - 2 * N;
+    int rem = e >> 2, j = 0;
+    while (rem >= N - 1 - j) {
+        rem -= N - 1 - j;
+        ++j;
+    }
+    d1 = 2 * j + (e & 1);
+    d2 = 2 * (j + 1 + rem) + ((e >> 1) & 1);
+}
 
 // Candidate k of cell cc with downwind directions out.
 template <int N, typename T>
@@ -223,19 +239,8 @@ __device__ __forceinline__ void grow_candidate(const Model& m, const Bufs& b, co
     const long long cap = m.cap;
     const int* link = b.link[v.g];
     unsigned short* om = b.om[v.g];
-    int d1, d2 = -1;
-    if (k < 2 * N) {
-        d1 = k;
-    } else {
-        const int e = k - 2 * N;
-        int rem = e >> 2, j = 0;
-        while (rem >= N - 1 - j) {
-            rem -= N - 1 - j;
-            ++j;
-        }
-        d1 = 2 * j + (e & 1);
-        d2 = 2 * (j + 1 + rem) + ((e >> 1) & 1);
-    }
+    int d1 = k, d2 = -1;
+    if (k >= 2 * N) edge_dirs<N>(k, d1, d2);
     if (!((out >> d1) & 1u) || (d2 >= 0 && !((out >> d2) & 1u))) return;
     const int a = link[(long long)d1 * cap + cc];
     long long e;
@@ -279,47 +284,7 @@ __device__ __forceinline__ bool grows(const unsigned short* om, const T* Q, cons
     return !(f & (OM_COMPLETE | OM_GHOST)) && out;
 }
 
-// The block-gathered form (all threads of the block must call it).
-template <int N, typename T>
-__device__ __forceinline__ double grow_body(const Model& m, const Bufs& b, const StepView& v) {
-    constexpr int K = GROW_K<N>;
-    const long long ncell = v.N_prev;
-    const Above<T> above(m.thr_rel * v.maxq);
-    const T* Q = static_cast<const T*>(b.q[v.pb]);
-    unsigned short* om = b.om[v.g];
-    __shared__ long long s_cell[THREADS];
-    __shared__ unsigned s_out[THREADS];
-    GrowWork gw;
-    // rounds of one run of 32 cells per warp; the block's first warp has the most
-    const long long runs = (ncell + 31) / 32;
-    const long long stride = (long long)v.nb * (blockDim.x >> 5);
-    const long long rounds = runs > v.bi ? (runs - v.bi + stride - 1) / stride : 0;
-    const int wid = threadIdx.x >> 5;
-    for (long long rd = 0; rd < rounds; ++rd) {
-        const long long k = v.bi + (long long)v.nb * wid + stride * rd;
-        const long long c = k * 32 + (threadIdx.x & 31);
-        unsigned out = 0;
-        const bool q = k < runs && c < ncell && grows<T>(om, Q, above, c, out);
-        int nq;
-        const int pos = block_exclusive_scan(q, nq);
-        if (nq == 0) continue;
-        if (q) {
-            s_cell[pos] = c;
-            s_out[pos] = out;
-        }
-        __syncthreads();
-        const int pairs = nq * K;
-        for (int t = threadIdx.x; t < pairs; t += blockDim.x) {
-            const int rank = t / K;
-            grow_candidate<N, T>(m, b, v, s_cell[rank], s_out[rank], t - rank * K, gw);
-        }
-        __syncthreads();
-        if (q) om[c] = (unsigned short)(om[c] | OM_COMPLETE);
-    }
-    return gw.rmax;
-}
-
-// The listed form, first half: cell c (of the wave pass's sweep) joins the
+// First half: cell c (of the wave pass's sweep) joins the
 // step's grow list (in the flux scratch, free until the flux pass) when it
 // grows.
 template <typename T>
@@ -332,7 +297,7 @@ __device__ __forceinline__ void grow_list_mark(const Bufs& b, const StepView& v,
     }
 }
 
-// The listed form, second half: every (listed cell, candidate) pair, over all
+// Second half: every (listed cell, candidate) pair, over all
 // threads of the grid; the thread of a cell's first candidate marks it
 // complete (only its own flag bit, and nothing else writes that word now).
 template <int N, typename T>
@@ -373,6 +338,7 @@ __device__ __forceinline__ void halo_body(const Model& m, const Bufs& b, const S
     const long long items = (ni + nact) * 2 * N;
     // runs of 32 items, one per warp, the warps of consecutive runs on
     // different SMs: a few hundred items of a small grid spread over the GPU
+#pragma unroll 1
     for (WarpRuns wr(items, v.nb, v.bi); wr.next();) {
         const long long it = wr.c;
         if (it >= items) continue;
@@ -394,39 +360,50 @@ __device__ __forceinline__ void halo_body(const Model& m, const Bufs& b, const S
 
 // ------------------------------------------------------------------ link
 
+// Face velocities, outward mask and CFL rate of entry c of generation g (cell
+// I; Eq. 7 and Eq. 8, the same IEEE operations as outward_mask and cfl_rate64);
+// the velocities and the rate are stored, the mask and the rate returned.
+template <int N, typename T>
+__device__ __forceinline__ double entry_velocities(const Model& m, const Bufs& b, int g, long long c, const int* I,
+                                                   unsigned& msk) {
+    T* U = static_cast<T*>(b.u[g]);
+    double r = 0.0;
+    msk = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        int J[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) J[k] = I[k] + (k == j ? 1 : 0);
+        const double ul = face_velocity64<N>(m, I, j);
+        if (face_velocity64<N>(m, J, j) > 0.0) msk |= 1u << (2 * j + 1);
+        if (ul < 0.0) msk |= 1u << (2 * j);
+        U[j * m.cap + c] = (T)ul;
+        r = __dadd_rn(r, div_h(m, fabs(ul), j));
+    }
+    b.rate[g][c] = r;
+    return r;
+}
+
 // Face velocities and outward masks of the new entries [lo, hi) (the mask is
 // added to the flags their inserter wrote), and the largest CFL rate among the
-// active ones (Eq. 8: the same IEEE operations as cfl_rate64).
+// active ones.
 template <int N, typename T>
 __device__ __forceinline__ double link_masks(const Model& m, const Bufs& b, long long lo, long long hi, int g,
                                               int nb, int bi) {
     const unsigned long long* key = b.key[g];
-    T* U = static_cast<T*>(b.u[g]);
-    const long long cap = m.cap;
     double rmax = 0.0;
     // runs of 32 entries, one per warp, consecutive runs on different SMs (the
     // FP64 drift evaluations of a few hundred new entries spread over the GPU)
+#pragma unroll 1
     for (WarpRuns wr(hi - lo, nb, bi); wr.next();) {
         const long long c = lo + wr.c;
         if (c >= hi) continue;
         int I[N];
         unpack_key<N>(m, key[c], I);
         const unsigned short f = b.om[g][c];
-        unsigned msk = 0;
-        double r = 0.0;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            int J[N];
-#pragma unroll
-            for (int k = 0; k < N; ++k) J[k] = I[k] + (k == j ? 1 : 0);
-            const double ul = face_velocity64<N>(m, I, j);
-            if (face_velocity64<N>(m, J, j) > 0.0) msk |= 1u << (2 * j + 1);
-            if (ul < 0.0) msk |= 1u << (2 * j);
-            U[j * cap + c] = (T)ul;
-            r = __dadd_rn(r, div_h(m, fabs(ul), j));
-        }
+        unsigned msk;
+        const double r = entry_velocities<N, T>(m, b, g, c, I, msk);
         b.om[g][c] = (unsigned short)(f | msk);
-        b.rate[g][c] = r;
         if (!(f & OM_GHOST)) rmax = fmax(rmax, r);
     }
     return rmax;
@@ -443,6 +420,7 @@ __device__ __forceinline__ double link_body(const Model& m, const Bufs& b, long 
     int* link = b.link[g];
     const long long cap = m.cap;
     const long long work = (hi - lo) * 2 * N;
+#pragma unroll 1
     for (WarpRuns wr(work, nb, bi); wr.next();) {
         const long long wi = wr.c;
         if (wi >= work) continue;
@@ -561,7 +539,7 @@ __device__ __forceinline__ T wave_of_halo(const T* Q, const T* U, long long cap,
 // are left out: they have p = 0, and their waves are formed on the spot. Runs
 // beside grow: a cell that grow or halo adds has p = 0 like the missing cell it
 // replaces, so these waves do not change.
-template <int N, int DYN, typename T, bool LIST_GROW = false>
+template <int N, typename T, bool LIST_GROW = false>
 __device__ __forceinline__ void waves_body(const Model& m, const Bufs& b, const StepView& v, long long ncell) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
     const int* link = b.link[v.g];
@@ -576,6 +554,7 @@ __device__ __forceinline__ void waves_body(const Model& m, const Bufs& b, const 
 #pragma unroll
     for (int d = 0; d < N; ++d) i2h[d] = (T)m.inv_2h[d];
     const Above<T> above(m.thr_rel * v.maxq);
+#pragma unroll 1
     for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
         const long long c = wr.c;
         if (c >= ncell) continue;
@@ -609,6 +588,56 @@ __device__ __forceinline__ void waves_body(const Model& m, const Bufs& b, const 
     }
 }
 
+// The same for the step loop of a small grid, in less code: one form for active
+// and halo entries, 32-bit indices.
+template <int N, typename T>
+__device__ __forceinline__ void waves_small_body(const Model& m, const Bufs& b, const StepView& v) {
+    const T* Q = static_cast<const T*>(b.q[v.pb]);
+    const long long cap = m.cap;
+    const int ncell = (int)v.N_prev;
+#pragma unroll 1
+    for (Runs r(runs_of(ncell), v.nb, v.bi); r.next();) {
+        const int c = r.cell();
+        if (c >= ncell) continue;
+        const unsigned act = __activemask();
+        const T P0 = Q[c];
+        int dn[N], up[N];
+        T ul[N], Pm[N], Pp[N], uh[N];
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            dn[d] = (b.link[v.g] + (2 * d) * cap)[c];
+            up[d] = (b.link[v.g] + (2 * d + 1) * cap)[c];
+            ul[d] = (static_cast<const T*>(b.u[v.g]) + d * cap)[c];
+        }
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            Pm[d] = dn[d] >= 0 ? Q[dn[d]] : (T)0;
+            Pp[d] = (T)0;
+            uh[d] = (T)0;
+            if (up[d] >= 0) {
+                Pp[d] = Q[up[d]];
+                uh[d] = (static_cast<const T*>(b.u[v.g]) + d * cap)[up[d]];
+            }
+        }
+        T t = (T)0;
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            // wave_of with the warp's votes
+            const T wlo = P0 - Pm[d];
+            const bool in_lo = gt0(ul[d]), in_hi = lt0(uh[d]);
+            T G = (in_lo ? ul[d] : (T)0) * wlo;
+            if (__any_sync(act, in_hi)) {
+                const T whi = Pp[d] - P0;
+                if (in_hi) G = in_lo ? fmadd(uh[d], whi, G) : uh[d] * whi;
+            }
+            (static_cast<T*>(b.wl) + d * cap)[c] = wlo;
+            (static_cast<T*>(b.wg) + d * cap)[c] = G;
+            t = fmadd(G, (T)m.inv_2h[d], t);
+        }
+        static_cast<T*>(b.tg)[c] = t;
+    }
+}
+
 // sum_{d != j} G_d(y) / (2 h_d) of a new pool entry y (p = 0, no pass-1 values),
 // formed on the spot from its links.
 template <int N, typename T>
@@ -639,6 +668,36 @@ struct FaceCtx {
     int lim;
     T dt, i2h[N], dth[N];
 };
+
+// a[j] of a short array in registers, j known at run time only.
+template <int N, typename T, int M>
+__device__ __forceinline__ T pick_of(const T (&a)[M], int j) {
+    T x = a[0];
+#pragma unroll
+    for (int k = 1; k < N; ++k) x = j == k ? a[k] : x;
+    return x;
+}
+
+template <int N, typename T>
+__device__ __forceinline__ FaceCtx<N, T> face_ctx(const Model& m, const Bufs& b, const StepView& v) {
+    FaceCtx<N, T> fc;
+    fc.Q = static_cast<const T*>(b.q[v.pb]);
+    fc.link = b.link[v.g];
+    fc.U = static_cast<const T*>(b.u[v.g]);
+    fc.wl = static_cast<const T*>(b.wl);
+    fc.wg = static_cast<const T*>(b.wg);
+    fc.tg = static_cast<const T*>(b.tg);
+    fc.cap = m.cap;
+    fc.nold = v.N_prev;
+    fc.lim = m.limiter;
+    fc.dt = (T)v.dt;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {  // converted once
+        fc.i2h[j] = (T)m.inv_2h[j];
+        fc.dth[j] = (T)v.dth[j];
+    }
+    return fc;
+}
 
 // The flux through the lower j-face of pool entry X (Eq. 7, the corrections of
 // Algorithm 1 gathered onto the face, the limited HR term), X's value P0. The
@@ -724,31 +783,13 @@ __device__ __forceinline__ bool face_flux_old(const FaceCtx<N, T>& fc, long long
 // needs only the few faces it shares with active cells. The upper face of an active cell
 // is the lower face of its upper neighbour, which is in the pool (active or
 // halo).
-// LATENCY: the step loop of a small grid, bound by dependent loads, not by the
-// FP64 pipe: faces that touch a new entry are evaluated where they stand (a
-// second queue would add a flush to the critical path of every warp).
-template <int N, int DYN, typename T, bool LATENCY = false>
+template <int N, typename T>
 __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const StepView& v) {
     const long long ncell = v.N;
     const long long cap = m.cap;
     const unsigned short* om = b.om[v.g];
     T* __restrict__ fl = static_cast<T*>(b.fl);  // aliases no input
-    FaceCtx<N, T> fc;
-    fc.Q = static_cast<const T*>(b.q[v.pb]);
-    fc.link = b.link[v.g];
-    fc.U = static_cast<const T*>(b.u[v.g]);
-    fc.wl = static_cast<const T*>(b.wl);
-    fc.wg = static_cast<const T*>(b.wg);
-    fc.tg = static_cast<const T*>(b.tg);
-    fc.cap = cap;
-    fc.nold = v.N_prev;
-    fc.lim = m.limiter;
-    fc.dt = (T)v.dt;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {  // converted once
-        fc.i2h[j] = (T)m.inv_2h[j];
-        fc.dth[j] = (T)v.dth[j];
-    }
+    const FaceCtx<N, T> fc = face_ctx<N, T>(m, b, v);
     // The warp's needed faces wait in a queue in shared memory (entry, j) and
     // are evaluated 32 at a time once that many are queued, whatever runs
     // they come from; the rest at the end.
@@ -757,7 +798,7 @@ __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const 
     __shared__ unsigned char s_qj[WARPS][QCAP];
     // FP64 (the pipe bounds it): faces that touch a new entry wait in a second
     // queue, so that face_flux's longer path runs with all lanes too
-    constexpr bool DEFER = sizeof(T) == 8 && !LATENCY;
+    constexpr bool DEFER = sizeof(T) == 8;
     __shared__ int s_lx[WARPS][DEFER ? 64 : 1];
     __shared__ unsigned char s_lj[WARPS][DEFER ? 64 : 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -802,6 +843,7 @@ __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const 
             if (n_later >= 32) later_flush(32);
         }
     };
+#pragma unroll 1
     for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
         const long long c = wr.c;
         unsigned need = 0;
@@ -837,11 +879,11 @@ __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const 
 
 // Pass 3: the conservative update of the active cells with the previous
 // normalisation applied (halo cells stay 0); adds this thread's new values to
-// its digits and maximum. Large FP64 grids (not LATENCY): each warp queues the
-// active cells of its runs in shared memory and updates them 32 at a time, so
-// the FP64 lanes all work where halo and active entries mix (after growth);
-// FP32 and small grids are bound by load latency and update in place.
-template <int N, typename T, bool LATENCY = false>
+// its digits and maximum. FP64: each warp queues the active cells of its runs in
+// shared memory and updates them 32 at a time, so the FP64 lanes all work where
+// halo and active entries mix (after growth); FP32 is bound by load latency and
+// updates in place.
+template <int N, typename T>
 __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const StepView& v, long long (&dacc)[NDIG],
                                            double& mx, int& err) {
     const long long ncell = v.N;
@@ -871,7 +913,8 @@ __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const 
         acc_add(dacc, qn, err);
         tmax = vmax(tmax, qn);
     };
-    if constexpr (LATENCY || sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll 1
         for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
             const long long c = wr.c;
             if (c >= ncell) continue;
@@ -886,6 +929,7 @@ __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const 
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         const unsigned lt = (1u << lane) - 1u;
         int n_a = 0;  // the same in every lane
+#pragma unroll 1
         for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
             const long long c = wr.c;
             bool act = false;
@@ -908,6 +952,571 @@ __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const 
     if (tmax > -INFINITY) mx = fmax(mx, (double)tmax);
 }
 
+// ------------------------------------------------------------------ step loop of a small grid
+// A grid of 10^3 to 10^5 cells in one resident launch is bound by chains of
+// dependent operations and by its grid barriers, not by any pipe's throughput.
+// Measured on GB300 in SM cycles: a load from L2 290, an atomic that returns 690
+// (a 16-bit compare-and-swap 1380), a fence after a store 620, an FP64
+// instruction 64 per warp, a grid barrier of 152 blocks 2360; code that does not
+// stay in the instruction caches costs more than any of these. So these forms of
+// the phases keep one entry, face or neighbour per lane, leave no chain to a
+// single thread where lanes can share it, keep rare work out of line, and need
+// three barriers per step:
+//   1  waves of the existing entries; grow. A new active cell gets its
+//      velocities and rate from the warp that inserts it, so dt is known
+//      after this phase
+//   2  the keys of the missing face neighbours of the newly active cells are
+//      claimed (new halo cells); the fluxes of the faces between existing entries
+//   3  the update; velocities and links of the new halo cells
+// Only newly active cells have faces that touch a new entry (every face neighbour
+// of an active cell is in the pool), and few of those fluxes differ from zero
+// (apply_small_body).
+
+// The requests of the block's growing cells, in shared memory: the neighbour of
+// cell c in direction d1, or the edge neighbour in d1 and d2 (code d1 | d2 << 4;
+// d2 = 15: none), is to be made active.
+constexpr int GROW_QUEUE = 1024;
+struct GrowQueue {
+    int n;
+    int cell[GROW_QUEUE];
+    unsigned char code[GROW_QUEUE];
+};
+
+// f_j at the lower (up = 0) or upper (up = 1) j-face of the cell with packed
+// key k: face_velocity64 with j known at run time, out of line. The step loop's
+// code runs once per step and phase from the instruction caches, so what is not
+// a matter of a few instructions is kept in one place.
+template <int N>
+__device__ __noinline__ double face_velocity_key(const Model& m, unsigned long long k, int j, int up) {
+    using A = Ar<double>;
+    const int bits = m.key_bits;
+    const long long bias = 1ll << (bits - 1);
+    const unsigned long long mask = (1ull << bits) - 1;
+    auto y = [&](int a) -> double {
+        const int i = (int)((long long)((k >> (bits * (N - 1 - a))) & mask) - bias);
+        const double s = a == j ? __dsub_rn((double)(i + up), 0.5) : (double)i;
+        return __dadd_rn(m.x0[a], __dmul_rn(s, m.h[a]));
+    };
+    if (m.dyn == DYN_CONSTANT) return m.a[j];
+    if (m.dyn == DYN_LINEAR) {
+        double s = 0;
+#pragma unroll 1
+        for (int a = 0; a < N; ++a) s = A::add(s, A::mul(m.a[j * N + a], y(a)));
+        return A::add(s, m.a[N * N + j]);
+    }
+    if (m.dyn == DYN_LORENZ96) {
+        const int jp = j + 1 < N ? j + 1 : j + 1 - N, jm1 = j >= 1 ? j - 1 : j + N - 1, jm2 = j >= 2 ? j - 2 : j + N - 2;
+        return A::add(A::sub(A::mul(A::sub(y(jp % N), y(jm2 % N)), y(jm1 % N)), y(j)), m.a[0]);
+    }
+    if constexpr (N == 3) {
+        const double y0 = y(0), y1 = y(1), y2 = y(2);
+        if (m.dyn == DYN_LORENZ63) {
+            if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
+            if (j == 1) return A::sub(A::mul(y0, A::sub(m.a[1], y2)), y1);
+            return A::sub(A::mul(y0, y1), A::mul(m.a[2], y2));
+        }
+        if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
+        if (j == 1) return A::sub(-y1, A::mul(y0, y2));
+        return A::sub(A::add(A::mul(-m.a[1], y2), A::mul(y0, y1)), A::mul(m.a[1], m.a[2]));
+    }
+    return 0.0;
+}
+
+// New entries of a warp, 2N lanes per entry (on: this lane has one; index c, key
+// k and flags the same in its lanes), one face each: face velocities, outward
+// mask, CFL rate (an FP64 instruction holds a warp scheduler for 64 cycles
+// whatever its active lanes, so one lane with all faces of its entry takes 2N
+// times as long), and with look the links to the neighbours in the table, both
+// ways. All lanes must call it. Returns the entry's rate.
+template <int N, typename T>
+__device__ __noinline__ double complete_group(const Model& m, const Bufs& b, int g, bool on, int c,
+                                              unsigned long long k, unsigned flags, bool look) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int F = 2 * N;
+    const long long cap = m.cap;
+    const int lane = threadIdx.x & 31;
+    const int s = lane / F, e = lane - s * F;
+    double u = 0.0, term = 0.0;
+    if (on) {
+        // the neighbour in direction e: one field of the key up or down, unless
+        // at its end; its first probe is in flight beside the velocity
+        const int shift = m.key_bits * (N - 1 - (e >> 1));
+        const unsigned long long last = (1ull << m.key_bits) - 1, field = (k >> shift) & last;
+        const bool end = field == ((e & 1) ? last : 0ull);
+        const unsigned long long nk = (e & 1) ? k + (1ull << shift) : k - (1ull << shift);
+        ulonglong2 first = make_ulonglong2(EMPTY_KEY, ~0ull);
+        if (look && !end) first = __ldcg(reinterpret_cast<const ulonglong2*>(b.table + (mix64(nk) & m.tmask)));
+        u = face_velocity_key<N>(m, k, e >> 1, e & 1);
+        if (!(e & 1)) {
+            (static_cast<T*>(b.u[g]) + (e >> 1) * cap)[c] = (T)u;
+            term = div_h(m, abs_bits(u), e >> 1);
+        }
+        if (look) {
+            int nbr = -1;
+            if (first.x == nk) nbr = (int)(long long)first.y;
+            else if (first.x != EMPTY_KEY) nbr = table_find(m, b.table, nk);
+            (b.link[g] + e * cap)[c] = nbr;
+            if (nbr >= 0) (b.link[g] + (e ^ 1) * cap)[nbr] = c;
+        }
+    }
+    // outward: upper face and u > 0, lower face and u < 0
+    const unsigned out = __ballot_sync(full, on && ((e & 1) ? u : -u) > 0.0);
+    double r = 0.0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) r = __dadd_rn(r, __shfl_sync(full, term, (s * F + 2 * j) & 31));
+    if (on && e == 0) {
+        b.om[g][c] = (unsigned short)(flags | ((out >> lane) & ((1u << F) - 1u)));
+        b.rate[g][c] = r;
+    }
+    return r;
+}
+
+// A warp's grow requests: neighbour `code` of cell cc (made active as
+// grow_candidate does it, with the marks of the step loop, and the inserted
+// cells' velocities formed at once). rate_now: the largest CFL rate known; only a larger one is written (it
+// rarely is). All lanes must call it.
+template <int N, typename T>
+__device__ __noinline__ void grow_act(const Model& m, const Bufs& b, int g, int pb, unsigned fresh, bool has, int cc,
+                                      unsigned code, unsigned long long rate_now, unsigned long long* rate) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int F = 2 * N, G = 32 / F;
+    DevScalars* sc = b.sc;
+    const long long cap = m.cap;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int d1 = code & 15, d2 = code >> 4;
+    int e = -2;
+    if (has) {
+        e = (b.link[g] + d1 * cap)[cc];
+        if (d2 < F && e >= 0) e = (b.link[g] + d2 * cap)[e];
+    }
+    // a halo cell: the one lane that clears its flag activates it (32-bit
+    // atomics: a 16-bit compare-and-swap is a loop around a 32-bit one)
+    bool act = false;
+    if (e >= 0) {
+        unsigned* word = reinterpret_cast<unsigned*>(b.om[g]) + (e >> 1);
+        const int sh = (e & 1) * 16;
+        act = (atomicAnd(word, ~((unsigned)OM_GHOST << sh)) >> sh) & OM_GHOST;
+        if (act) {
+            atomicOr(word, fresh << sh);
+            const unsigned long long rb = (unsigned long long)__double_as_longlong(b.rate[g][e]);
+            if (rb > rate_now) atomicMax(rate, rb);
+        }
+    }
+    const unsigned acts = __ballot_sync(full, act);
+    if (acts) {
+        long long base = 0;
+        if (lane == 0) base = (long long)atomicAdd((unsigned long long*)&sc->n_act, (unsigned long long)__popc(acts));
+        base = __shfl_sync(full, base, 0);
+        if (act) b.map[base + __popc(acts & lt)] = e;
+    }
+    if (!__any_sync(full, e == -1)) return;
+    // missing cells (rare): inserted as active
+    bool inserted = false;
+    long long c = 0;
+    unsigned long long key = 0;
+    if (e == -1) {
+        int J[N];
+        unpack_key<N>(m, b.key[g][cc], J);
+#pragma unroll
+        for (int x = 0; x < N; ++x) {
+            if ((d1 >> 1) == x) J[x] += (d1 & 1) ? 1 : -1;
+            if ((d2 >> 1) == x) J[x] += (d2 & 1) ? 1 : -1;  // (15: no dimension)
+        }
+        if (!interior<N>(m, J)) {
+            set_error(sc, ST_EKEYRANGE);
+        } else {
+            pack_key<N>(m, J, key);
+            unsigned long long slot;
+            const int claim = table_claim(m, b.table, key, &slot);
+            if (claim < 0) set_error(sc, ST_ETABLE);
+            if (claim > 0) {
+                c = (long long)atomicAdd((unsigned long long*)&sc->N, 1ull);
+                if (c >= cap) {
+                    set_error(sc, ST_ECAPACITY);
+                } else {
+                    inserted = true;
+                    b.table[slot].val = c;
+                    b.slot[g][c] = (unsigned int)slot;
+                    b.key[g][c] = key;
+                    static_cast<T*>(b.q[pb])[c] = (T)0;
+#pragma unroll 1
+                    for (int d = 0; d < F; ++d) b.link[g][(long long)d * cap + c] = -1;
+                }
+            }
+        }
+    }
+    const int s = lane / F;
+#pragma unroll 1
+    for (unsigned todo = __ballot_sync(full, inserted); todo;) {
+        unsigned rest = todo;  // lanes of slot s work on the s-th entry still to do
+#pragma unroll 1
+        for (int i = 0; i < s && rest; ++i) rest &= rest - 1;
+        const bool on = s < G && rest;
+        const int owner = on ? __ffs(rest) - 1 : 0;
+        const unsigned long long ko = __shfl_sync(full, key, owner);
+        const int co = __shfl_sync(full, (int)c, owner);
+        const double r = complete_group<N, T>(m, b, g, on, co, ko, 0u, false);
+        const unsigned long long rb = (unsigned long long)__double_as_longlong(r);
+        if (on && lane == s * F && rb > rate_now) atomicMax(rate, rb);
+#pragma unroll 1
+        for (int i = 0; i < G; ++i) todo &= todo - 1;
+    }
+}
+
+// Every growing cell of the existing entries looks at its downwind set: face
+// neighbours (in the pool, perhaps as halo cells) and edge neighbours (through
+// the link of the first face), four neighbours at a time with their loads in
+// flight together (links do not change in this phase). A cell's outward
+// directions are mostly one per dimension, so its list is short: N faces and
+// N (N - 1) / 2 edges. What is still to be made active goes to the block's list,
+// and from there to all its warps; a warp that finds the list full acts on its
+// own requests at once.
+template <int N, typename T>
+__device__ __forceinline__ void grow_detect(const Model& m, const Bufs& b, const StepView& v, GrowQueue& gq,
+                                            unsigned long long rate_now, unsigned long long* rate) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int C = 4;
+    const int ncell = (int)v.N_prev;
+    const long long cap = m.cap;
+    const Above<T> above(m.thr_rel * v.maxq);
+    const T* Q = static_cast<const T*>(b.q[v.pb]);
+    const int* link = b.link[v.g];
+    unsigned short* om = b.om[v.g];
+    const unsigned stale = v.fresh ^ (3u * OM_NEW);  // the mark of the step before
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (Runs r(runs_of(ncell), v.nb, v.bi); r.next();) {
+        const int c = r.cell();
+        unsigned out = 0;
+        if (c < ncell) {
+            const unsigned f = *(volatile unsigned short*)&om[c];
+            out = f & 0xfffu;
+            const bool grow = !(f & (OM_COMPLETE | OM_GHOST)) && out && above(Q[c]);
+            if (grow || (f & stale)) om[c] = (unsigned short)((f & ~stale) | (grow ? OM_COMPLETE : 0));
+            if (!grow) out = 0;
+        }
+        // (d1, d2) runs over the outward directions d1, alone and with each later d2
+        unsigned rem1 = out, rem2 = 0;
+        int d1 = 0;
+        bool face = false;  // d1 alone is next
+        auto next = [&]() -> unsigned {  // the next code, or 0xff
+            if (!face && !rem2) {
+                if (!rem1) return 0xffu;
+                d1 = __ffs(rem1) - 1;
+                rem1 &= rem1 - 1;
+                face = true;
+            }
+            if (face) {
+                face = false;
+                rem2 = out & (~0u << ((d1 | 1) + 1));
+                return (unsigned)d1 | 0xf0u;
+            }
+            const int d2 = __ffs(rem2) - 1;
+            rem2 &= rem2 - 1;
+            return (unsigned)(d1 | (d2 << 4));
+        };
+#pragma unroll 1
+        while (__any_sync(full, (rem1 | rem2) != 0 || face)) {
+            unsigned code[C];
+            int e[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                code[i] = next();
+                e[i] = code[i] != 0xffu ? (link + (code[i] & 15) * cap)[c] : -2;
+            }
+#pragma unroll
+            for (int i = 0; i < C; ++i)
+                if (e[i] >= 0 && (code[i] >> 4) != 15) e[i] = (link + (code[i] >> 4) * cap)[e[i]];
+            unsigned need = 0;  // four codes of eight bits
+            int n_need = 0;
+            unsigned f[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) f[i] = e[i] >= 0 ? *(volatile unsigned short*)&om[e[i]] : 0u;
+#pragma unroll
+            for (int i = 0; i < C; ++i)
+                if (e[i] == -1 || (f[i] & OM_GHOST)) {
+                    need = (need << 8) | code[i];
+                    ++n_need;
+                }
+#pragma unroll 1
+            for (unsigned bal; (bal = __ballot_sync(full, n_need > 0)) != 0; --n_need, need >>= 8) {
+                const bool want = n_need > 0;
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&gq.n, __popc(bal));
+                at = __shfl_sync(full, at, 0) + __popc(bal & ((1u << lane) - 1u));
+                if (want && at < GROW_QUEUE) {
+                    gq.cell[at] = c;
+                    gq.code[at] = (unsigned char)need;
+                }
+                const bool over = want && at >= GROW_QUEUE;
+                if (__any_sync(full, over))
+                    grow_act<N, T>(m, b, v.g, v.pb, v.fresh, over, c, need & 0xffu, rate_now, rate);
+            }
+        }
+    }
+}
+
+// The listed requests, 32 per warp and round (after a block barrier).
+template <int N, typename T>
+__device__ __forceinline__ void grow_drain(const Model& m, const Bufs& b, const StepView& v, const GrowQueue& gq,
+                                           unsigned long long rate_now, unsigned long long* rate) {
+    const int n = min(gq.n, GROW_QUEUE);
+#pragma unroll 1
+    for (int q0 = threadIdx.x & ~31; q0 < n; q0 += blockDim.x) {
+        const int q = q0 + (threadIdx.x & 31);
+        const bool has = q < n;
+        grow_act<N, T>(m, b, v.g, v.pb, v.fresh, has, has ? gq.cell[q] : 0, has ? gq.code[q] : 0u, rate_now, rate);
+    }
+}
+
+// The slot of key: claimed (1, was free), found (0) or the table is full (-1).
+// Compare-and-swap at once: most keys asked for here are new.
+__device__ __forceinline__ int table_claim_or_find(const Model& m, Slot* T, unsigned long long key,
+                                                   unsigned long long* slot) {
+    unsigned long long h = mix64(key) & m.tmask;
+#pragma unroll 1
+    for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
+        const unsigned long long k = atomicCAS(&T[h].key, EMPTY_KEY, key);
+        *slot = h;
+        if (k == EMPTY_KEY) return 1;
+        if (k == key) return 0;
+        h = (h + 1) & m.tmask;
+    }
+    return -1;
+}
+
+// The face neighbours of the newly active cells, one (cell, face) per lane: the
+// inserted cells [N_prev, n_ins) and the nact activated halo cells listed in map
+// (only their missing neighbours). A neighbour that was in the pool before this
+// phase is linked with the cell; a key that is not in the table is claimed for a
+// new halo cell, appended at n_ins + n_halo, whose links and velocities phase 3
+// makes (halo_complete_body), when all new cells have their indices in the table.
+template <int N, typename T>
+__device__ __forceinline__ void halo_claim_body(const Model& m, const Bufs& b, const StepView& v, long long n_ins,
+                                                long long nact) {
+    constexpr int F = 2 * N, G = 32 / F;  // cells per warp
+    DevScalars* sc = b.sc;
+    const long long cap = m.cap;
+    const int lo = (int)v.N_prev, ni = (int)(n_ins - lo), total = ni + (int)nact;
+    const int lane = threadIdx.x & 31;
+    const int s = lane / F, d = lane - s * F;
+#pragma unroll 1
+    for (Runs r((total + G - 1) / G, v.nb, v.bi, LAST); r.next();) {
+        const int q = r.k * G + s;
+        if (s >= G || q >= total) continue;
+        const int x = q < ni ? lo + q : b.map[q - ni];
+        unsigned long long k = b.key[v.g][x];
+        if (*(volatile int*)&(b.link[v.g] + d * cap)[x] >= 0) continue;
+        const int shift = m.key_bits * (N - 1 - (d >> 1));
+        const unsigned long long last = (1ull << m.key_bits) - 1, field = (k >> shift) & last;
+        // an activated halo cell at the end of the key range has a neighbour without a key
+        if (field == ((d & 1) ? last : 0ull)) {
+            set_error(sc, ST_EKEYRANGE);
+            continue;
+        }
+        k = (d & 1) ? k + (1ull << shift) : k - (1ull << shift);
+        unsigned long long slot;
+        const int claim = table_claim_or_find(m, b.table, k, &slot);
+        if (claim < 0) {
+            set_error(sc, ST_ETABLE);
+        } else if (claim == 0) {
+            const long long nbr = *(volatile long long*)&b.table[slot].val;
+            if (nbr >= 0 && nbr < n_ins) {
+                (b.link[v.g] + d * cap)[x] = (int)nbr;
+                (b.link[v.g] + (d ^ 1) * cap)[nbr] = x;
+            }
+        } else {
+            const long long c = n_ins + warp_aggregated_add(&sc->n_halo);
+            if (c >= cap) {
+                set_error(sc, ST_ECAPACITY);
+                continue;
+            }
+            *(volatile long long*)&b.table[slot].val = c;
+            b.slot[v.g][c] = (unsigned int)slot;
+            b.key[v.g][c] = k;
+        }
+    }
+}
+
+// Phase 3 of the new halo cells [n_ins, N): velocities, mask, rate, links, value 0.
+template <int N, typename T>
+__device__ __forceinline__ void halo_complete_body(const Model& m, const Bufs& b, const StepView& v,
+                                                   long long n_ins) {
+    constexpr int F = 2 * N, G = 32 / F;  // entries per warp
+    const int lo = (int)n_ins, total = (int)(v.N - n_ins);
+    const int lane = threadIdx.x & 31, s = lane / F;
+#pragma unroll 1
+    for (Runs r((total + G - 1) / G, v.nb, v.bi, LAST); r.next();) {
+        const int q = r.k * G + s;
+        const bool on = s < G && q < total;
+        const int c = on ? lo + q : 0;
+        const unsigned long long k = on ? b.key[v.g][c] : 0ull;
+        complete_group<N, T>(m, b, v.g, on, c, k, OM_GHOST, true);
+        if (on && lane == s * F) static_cast<T*>(b.q[v.pb ^ 1])[c] = (T)0;
+    }
+}
+
+// The fluxes of the faces between existing entries that touch an active cell
+// (both sides below nold: halo_claim_body meanwhile writes links to or from
+// entries beyond it only, so what it changes is not read here). One face per thread,
+// the runs of 32 entries of dimension after dimension.
+template <int N, typename T>
+__device__ __forceinline__ void faces_old_body(const Model& m, const Bufs& b, const StepView& v) {
+    const unsigned short* om = b.om[v.g];
+    const T* Q = static_cast<const T*>(b.q[v.pb]);
+    const T* tg = static_cast<const T*>(b.tg);
+    const long long cap = m.cap;
+    const int nold = (int)v.N_prev, runs = runs_of(nold);
+    const int lim = m.limiter;
+    const T dt = (T)v.dt;
+#pragma unroll 1
+    for (Runs r(runs * N, v.nb, v.bi); r.next();) {
+        int j = 0, k = r.k;
+#pragma unroll 1
+        while (k >= runs) {
+            k -= runs;
+            ++j;
+        }
+        const int X = k * 32 + (int)(threadIdx.x & 31);
+        if (X >= nold) continue;
+        const int* lo = b.link[v.g] + 2 * j * cap;
+        const T* wl = static_cast<const T*>(b.wl) + j * cap;
+        const int Llo = lo[X], Lup = (lo + cap)[X];
+        const T u = (static_cast<const T*>(b.u[v.g]) + j * cap)[X];
+        const unsigned short fX = om[X];
+        const T P0 = Q[X], W = wl[X];
+        if (Llo < 0 || Llo >= nold) continue;
+        if ((fX & OM_GHOST) && is_halo(om, Llo)) continue;
+        T f = (T)0;
+        if (gt0(u) || lt0(u)) {
+            const bool up = gt0(u);  // the upwind cell is Llo, else X
+            const int y = up ? Llo : X;
+            // the jump across the face beyond the upwind cell
+            const int z = up ? Llo : (Lup < nold ? Lup : -1);
+            const T Wb = z >= 0 ? wl[z] : zero_minus(P0);
+            const T Py = up ? Q[Llo] : P0;
+            const T S = fmadd(-(T)m.inv_2h[j], (static_cast<const T*>(b.wg) + j * cap)[y], tg[y]);
+            f = u * fmadd(-dt, S, Py);
+            if (lim != LIM_NONE && (gt0(W) || lt0(W))) {
+                const T au = abs_bits(u);
+                f = fmadd(half_nonneg(au) * fmadd(-(T)pick_of<N>(v.dth, j), au, (T)1), limited_wave<T>(lim, W, Wb), f);
+            }
+        }
+        (static_cast<T*>(b.fl) + j * cap)[X] = f;
+    }
+}
+
+// Phase 3: the update.
+// Newly active cells (density 0; the inserted ones and the nact listed in map):
+// 2N lanes of a warp per cell, one face each, and the update in the first of
+// them. Let x be the cell and z its neighbour across a face.
+//   both existing entries: the flux is there (faces_old_body);
+//   both new: nothing nearby has a density (a new entry is no face neighbour of
+//     a cell that was active before), the flux is 0;
+//   one of them new: both densities are 0, so neither the donor term nor the
+//     limited term contributes, and only the transverse sum of the existing one
+//     does, when it is upwind of the face.
+// (Zeros enter the update as +0 here where the general form may give -0; a sum
+// that starts from +0 is the same with either.)
+// The existing entries that were active before this step: one lane per cell, all
+// its faces lie between existing entries; existing halo entries get 0.
+// The new values add to the thread's digits and maximum.
+template <int N, typename T>
+__device__ __forceinline__ void apply_small_body(const Model& m, const Bufs& b, const StepView& v, long long n_ins,
+                                                 long long nact, long long (&dacc)[NDIG], T& mx, int& err) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int F = 2 * N, G = 32 / F;  // new cells per warp
+    const long long cap = m.cap;
+    const int nold = (int)v.N_prev, ni = (int)(n_ins - v.N_prev), total = ni + (int)nact;
+    const T* Q = static_cast<const T*>(b.q[v.pb]);
+    T* Qn = static_cast<T*>(b.q[v.pb ^ 1]);
+    const int* link = b.link[v.g];
+    const unsigned short* om = b.om[v.g];
+    const T* U = static_cast<const T*>(b.u[v.g]);
+    const T* fl = static_cast<const T*>(b.fl);
+    const T* wg = static_cast<const T*>(b.wg);
+    const T* tg = static_cast<const T*>(b.tg);
+    const T scale = (T)v.scale;
+    const int lane = threadIdx.x & 31;
+    const int s = lane / F, d = lane - s * F;
+    Runs fresh((total + G - 1) / G, v.nb, v.bi, MIDDLE);
+    Runs old(runs_of(nold), v.nb, v.bi);
+#pragma unroll 1
+    for (;;) {
+        int c = 0;
+        bool active = false;
+        T upd = (T)0;
+        if (fresh.next()) {
+            const int q = fresh.k * G + s;
+            const bool mine = s < G && q < total;
+            const int j = d >> 1;
+            T f = (T)0;
+            if (mine) {
+                c = q < ni ? nold + q : b.map[q - ni];
+                // (links to new halo cells appear while this runs: missing or new, it is the same)
+                const int z = (link + d * cap)[c];
+                const bool oldx = c < nold, oldz = z >= 0 && z < nold;
+                if (oldx && oldz) {
+                    f = (fl + j * cap)[(d & 1) ? z : c];
+                } else if (oldx || oldz) {
+                    const int y = oldx ? c : z;
+                    const T S = fmadd(-(T)m.inv_2h[j], (wg + j * cap)[y], tg[y]);
+                    T u;
+                    if (!(d & 1)) u = (U + j * cap)[c];
+                    else if (z >= 0 && z < n_ins) u = (U + j * cap)[z];
+                    else u = (T)face_velocity_key<N>(m, b.key[v.g][c], j, 1);
+                    // the existing one upwind: z below and the flow up, or z above and it down; c the other way round
+                    if ((oldz == !(d & 1)) ? gt0(u) : lt0(u)) f = u * fmadd(-(T)v.dt, S, (T)0);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const T lo = __shfl_sync(full, f, (lane + 2 * i) & 31);
+                const T hi = __shfl_sync(full, f, (lane + 2 * i + 1) & 31);
+                upd = fmadd((T)v.dth[i], hi - lo, upd);
+            }
+            active = mine && d == 0;
+        } else if (old.next()) {
+            c = old.cell();
+            const unsigned f = c < nold ? om[c] : v.fresh;
+            if (f & OM_GHOST) Qn[c] = (T)0;
+            active = !(f & (OM_GHOST | v.fresh));
+            if (active) {
+                T hi[N], lo[N];
+                int up[N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) up[j] = (link + (2 * j + 1) * cap)[c];
+#pragma unroll
+                for (int j = 0; j < N; ++j) lo[j] = (fl + j * cap)[c];
+#pragma unroll
+                for (int j = 0; j < N; ++j) hi[j] = up[j] >= 0 ? (fl + j * cap)[up[j]] : (T)0;
+#pragma unroll
+                for (int j = 0; j < N; ++j) upd = fmadd((T)v.dth[j], hi[j] - lo[j], upd);
+            }
+        } else {
+            break;
+        }
+        if (active) {
+            const T qn = (Q[c] - upd) * scale;
+            Qn[c] = qn;
+            acc_add(dacc, qn, err);
+            mx = vmax(mx, qn);
+        }
+    }
+}
+
+// The end of a launch: the marks of its last step's activated cells.
+__device__ __forceinline__ void clear_marks(const Bufs& b, const StepView& v, long long nact) {
+    unsigned short* om = b.om[v.g];
+#pragma unroll 1
+    for (WarpRuns wr(nact, v.nb, v.bi); wr.next();) {
+        if (wr.c >= nact) continue;
+        const int x = b.map[wr.c];
+        om[x] = (unsigned short)(om[x] & ~(3u * OM_NEW));
+    }
+}
+
 // ------------------------------------------------------------------ prune
 
 // keep[c] = (p_c > p*) for the active cells: the significant cells S.
@@ -917,6 +1526,7 @@ __device__ __forceinline__ void prune_mark_body(const Model& m, const Bufs& b, c
     const Above<T> above(pstar);
     const T* Q = static_cast<const T*>(b.q[v.pb]);
     const unsigned short* om = b.om[v.g];
+#pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
         if (c < v.N) b.keep[c] = !is_halo(om, c) && above(Q[c]);
@@ -933,6 +1543,7 @@ __device__ __forceinline__ void prune_scatter_body(const Model& m, const Bufs& b
     const int* link = b.link[v.g];
     const unsigned short* om = b.om[v.g];
     const long long cap = m.cap;
+#pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
         if (c >= v.N) continue;
@@ -971,7 +1582,7 @@ __device__ __forceinline__ void block_chunk(long long total, long long& c0, long
 
 // Sum of a per-thread count over the block (every thread gets it).
 __device__ __forceinline__ long long block_count(int cnt) {
-    __shared__ long long s[WARPS];
+    __shared__ long long s[MAX_WARPS];
     for (int off = 16; off > 0; off >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, off);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = cnt;
     __syncthreads();
@@ -993,6 +1604,7 @@ __device__ __forceinline__ void prune_count_body(const Model& m, const Bufs& b, 
     long long c0, c1;
     block_chunk(v.N, c0, c1, v.nb, v.bi);
     int na = 0, ng = 0;
+#pragma unroll 1
     for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
         int st = 0;
         if (b.keep[c] && !is_halo(om, c)) {
@@ -1025,8 +1637,9 @@ struct Survivors {
     long long base_a, base_g, total_a, total_g;
 };
 __device__ __forceinline__ Survivors block_offsets(const Bufs& b, int nb, int bi) {
-    __shared__ long long s[4][WARPS];
+    __shared__ long long s[4][MAX_WARPS];
     long long v[4] = {0, 0, 0, 0};  // offset a, total a, offset g, total g
+#pragma unroll 1
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
         const long long a = __ldcg(&b.blk[i]);
         const long long g = __ldcg(&b.blk2[i]);
@@ -1046,6 +1659,7 @@ __device__ __forceinline__ Survivors block_offsets(const Bufs& b, int nb, int bi
     long long t[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int k = 0; k < 4; ++k)
+#pragma unroll 1
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t[k] += s[k][w];
     __syncthreads();
     Survivors r;
@@ -1088,6 +1702,7 @@ __device__ __forceinline__ void prune_compact_body(const Model& m, const Bufs& b
     long long ba = sv.base_a, bg = sv.base_g;
     long long c0, c1;
     block_chunk(v.N, c0, c1, v.nb, v.bi);
+#pragma unroll 1
     for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
         const long long c = t0 + threadIdx.x;
         const int st = (c < c1) ? b.map[c] : 0;
@@ -1138,6 +1753,7 @@ __device__ __forceinline__ void prune_compact_sorted_body(const Model& m, const 
     unsigned short* omo = b.om[v.g ^ 1];
     const double mq = v.maxq;
     const double s2 = (mq > 0.0 && isfinite(mq)) ? ldexp(1.0, -ilogb(mq)) : 1.0;
+#pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
         if (c >= v.N) continue;
@@ -1168,6 +1784,7 @@ __device__ __forceinline__ void prune_relink_body(const Model& m, const Bufs& b,
     int* linko = b.link[v.g ^ 1];
     const unsigned long long* keyo = b.key[v.g ^ 1];
     const long long cap = m.cap;
+#pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
         if (c >= v.N) continue;
