@@ -846,6 +846,16 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         ctx->err = "initial box too large";
         return GBEES_EINVAL;
     }
+    {  // q of the cell nearest the mean: no cell with a larger one has the maximum
+        double dx[6], q = 0.0;
+        for (int k = 0; k < n; ++k) {
+            const double i = std::round((mean[k] - ctx->cfg.x0[k]) / ctx->cfg.h[k]);
+            dx[k] = ctx->cfg.x0[k] + i * ctx->cfg.h[k] - mean[k];
+        }
+        for (int a = 0; a < n; ++a)
+            for (int c = 0; c < n; ++c) q += dx[a] * bx.icov[a * n + c] * dx[c];
+        bx.qlim = (float)q;
+    }
     const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
     {
@@ -869,6 +879,7 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         return ctx->status;
     }
     bx.pstar = ctx->cfg.thr_rel * gmax;
+    bx.qlim = bx.pstar > 0.0 ? (float)(-2.0 * std::log(bx.pstar)) : INFINITY;
     if (!box_for(ctx, mean, cov, -2.0 * std::log(thr * gmax), &bx)) {
         ctx->err = "initial box too large";
         return GBEES_EINVAL;

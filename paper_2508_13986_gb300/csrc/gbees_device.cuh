@@ -442,15 +442,6 @@ __device__ __forceinline__ double div_h(const Model& m, double x, int j) {
     return ((m.h_pow2 >> j) & 1) ? __dmul_rn(x, m.inv_h[j]) : __ddiv_rn(x, m.h[j]);
 }
 
-// FP64 CFL rate sum_j |f_j(x_{i-e_j/2})| / h_j (Eq. 8 with |f|).
-template <int N>
-__device__ __forceinline__ double cfl_rate64(const Model& m, const int* I) {
-    double r = 0.0;
-#pragma unroll
-    for (int j = 0; j < N; ++j) r = __dadd_rn(r, div_h(m, fabs(face_velocity64<N>(m, I, j)), j));
-    return r;
-}
-
 // a * b + c rounded once, and the larger of two values, in the arithmetic
 // type itself (explicit single-precision forms for float, so that nothing is
 // widened to double).

@@ -58,6 +58,7 @@ struct InitBox {
     double mean[MAXN];
     double icov[MAXN * MAXN];
     double pstar;
+    float qlim;  // pass 1: q of the cell nearest the mean; then: -2 ln pstar
 };
 
 template <int N>
@@ -69,7 +70,8 @@ __device__ __forceinline__ void box_index(const InitBox& bx, long long lin, int*
     }
 }
 
-// exp(-1/2 (x - mean)^T icov (x - mean)) at the centre of cell I.
+// exp(-1/2 (x - mean)^T icov (x - mean)) at the centre of cell I. (A zero of icov
+// adds a zero to the sum: left out, a diagonal covariance takes N terms.)
 template <int N>
 __device__ __forceinline__ double gauss_at(const Model& m, const InitBox& bx, const int* I) {
     double dx[N];
@@ -79,20 +81,139 @@ __device__ __forceinline__ double gauss_at(const Model& m, const InitBox& bx, co
 #pragma unroll
     for (int a = 0; a < N; ++a)
 #pragma unroll
-        for (int c = 0; c < N; ++c) q = __dadd_rn(q, __dmul_rn(__dmul_rn(dx[a], bx.icov[a * N + c]), dx[c]));
+        for (int c = 0; c < N; ++c)
+            if (bx.icov[a * N + c] != 0.0)
+                q = __dadd_rn(q, __dmul_rn(__dmul_rn(dx[a], bx.icov[a * N + c]), dx[c]));
     return exp(__dmul_rn(-0.5, q));
 }
 
+// From three dimensions on, most of the box lies outside the ellipsoid of the
+// initial set (97 % of it in six), and FP64 is scarce: the box is swept by rows
+// along the last dimension, one thread per row, with the quadratic form q of each
+// cell in single precision and a bound of its error. Only a cell whose q lies
+// within that bound of the limit is decided in FP64, so the set is the one that
+// FP64 gives everywhere; the densities of the cells in the set are FP64. The
+// paper's 6-D case (2.0e6 cells in the set, a box of 6.4e7): 0.68 + 0.69 + 2.57 ms
+// for the three passes (81 ms with the FP64 density at every cell of the box in
+// each of them and a covariance's zeros multiplied out; the whole call 87.5 ->
+// 10.5 ms; Lorenz '96 6-D with h = 0.25 286 -> 69 ms).
+// Longer rows than INIT_ROW_MAX (a chain of that many steps per thread) and
+// fewer dimensions (the set fills most of the box) are swept cell by cell.
+constexpr int INIT_ROW_MAX = 1024;
+template <int N>
+__device__ __forceinline__ bool by_rows(const InitBox& bx) {
+    return N >= 3 && bx.dims[N - 1] <= INIT_ROW_MAX;
+}
+// Rows [c0, c1) of this block, as even as possible: a small box spreads over all blocks.
+__device__ __forceinline__ void row_chunk(long long rows, long long& c0, long long& c1) {
+    const long long per = (rows + gridDim.x - 1) / gridDim.x;
+    c0 = min(rows, per * blockIdx.x);
+    c1 = min(rows, c0 + per);
+}
+
+struct InitRow {
+    float A, B, C;     // q = A + B dx + C dx^2
+    float Aa, Ba;      // the same sums of absolute values
+    float dx0, h, err; // dx of the row's first cell, cell width, error bound of dx
+};
+
+template <int N>
+__device__ __forceinline__ void row_index(const InitBox& bx, long long row, int* I) {
+    I[N - 1] = bx.lo[N - 1];
+    if (bx.total <= 0x7fffffffll) {
+        unsigned r = (unsigned)row;
+#pragma unroll
+        for (int k = N - 2; k >= 0; --k) {
+            const unsigned d = (unsigned)bx.dims[k];
+            I[k] = bx.lo[k] + (int)(r % d);
+            r /= d;
+        }
+    } else {
+#pragma unroll
+        for (int k = N - 2; k >= 0; --k) {
+            I[k] = bx.lo[k] + (int)(row % bx.dims[k]);
+            row /= bx.dims[k];
+        }
+    }
+}
+
+template <int N>
+__device__ __forceinline__ InitRow row_form(const Model& m, const InitBox& bx, const int* I) {
+    float dx[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) dx[k] = (float)__dsub_rn(centre64(m, k, I[k]), bx.mean[k]);
+    InitRow r;
+    r.A = r.Aa = r.B = r.Ba = 0.0f;
+#pragma unroll
+    for (int a = 0; a < N - 1; ++a) {
+#pragma unroll
+        for (int c = 0; c < N - 1; ++c) {
+            const float t = dx[a] * (float)bx.icov[a * N + c] * dx[c];
+            r.A += t;
+            r.Aa += fabsf(t);
+        }
+        const float t = dx[a] * ((float)bx.icov[a * N + N - 1] + (float)bx.icov[(N - 1) * N + a]);
+        r.B += t;
+        r.Ba += fabsf(t);
+    }
+    r.C = (float)bx.icov[N * N - 1];
+    r.h = (float)m.h[N - 1];
+    r.dx0 = dx[N - 1];
+    // dx of a cell of the row as dx0 + i h: two roundings and those of dx0 and h
+    r.err = 5e-7f * (fabsf(r.dx0) + (float)bx.dims[N - 1] * r.h);
+    return r;
+}
+
+// q of cell i of the row and a bound of its error: fewer than 64 roundings of
+// relative size 2^-24 on sums of absolute value S (1e-5 is 2.5 times that), and
+// the error of dx.
+__device__ __forceinline__ float row_q(const InitRow& r, int i, float& e) {
+    const float dx = r.dx0 + (float)i * r.h, ad = fabsf(dx);
+    e = 1e-5f * (r.Aa + (r.Ba + r.C * ad) * ad) + (r.Ba + 2.0f * r.C * (ad + r.err)) * r.err + 1e-6f;
+    return r.A + (r.B + r.C * dx) * dx;
+}
+
+// Whether cell i of the row at I is in the set p > pstar (qlim: -2 ln pstar).
+template <int N>
+__device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const InitRow& r, int* I, int i) {
+    float e;
+    const float q = row_q(r, i, e), d = q - bx.qlim;
+    e += 1e-6f * fabsf(bx.qlim);
+    if (d > e) return false;
+    if (d < -e) return true;
+    I[N - 1] = bx.lo[N - 1] + i;  // too near the limit (or not a number)
+    return gauss_at<N>(m, bx, I) > bx.pstar;
+}
+
 // Initial Gaussian (Sec. 5.1), pass 1: the largest density over the box of
-// candidate cells, which fixes the threshold p* = thr_rel * max p.
+// candidate cells, which fixes the threshold p* = thr_rel * max p. By rows: the
+// cells whose q may be as small as that of the cell nearest the mean (bx.qlim).
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_init_max(const Model m, Bufs b, const InitBox bx) {
     double mx = 0.0;
-    for (long long lin = blockIdx.x * (long long)blockDim.x + threadIdx.x; lin < bx.total;
-         lin += (long long)gridDim.x * blockDim.x) {
-        int I[N];
-        box_index<N>(bx, lin, I);
-        mx = fmax(mx, gauss_at<N>(m, bx, I));
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    if (by_rows<N>(bx)) {
+        const int len = (int)bx.dims[N - 1];
+        const long long rows = bx.total / len;
+        for (long long row = first; row < rows; row += stride) {
+            int I[N];
+            row_index<N>(bx, row, I);
+            const InitRow r = row_form<N>(m, bx, I);
+            for (int i = 0; i < len; ++i) {
+                float e;
+                const float q = row_q(r, i, e);
+                if (q - bx.qlim > e + 1e-6f * fabsf(bx.qlim)) continue;
+                I[N - 1] = bx.lo[N - 1] + i;
+                mx = fmax(mx, gauss_at<N>(m, bx, I));
+            }
+        }
+    } else {
+        for (long long lin = first; lin < bx.total; lin += stride) {
+            int I[N];
+            box_index<N>(bx, lin, I);
+            mx = fmax(mx, gauss_at<N>(m, bx, I));
+        }
     }
     mx = block_max(mx);
     if (threadIdx.x == 0 && mx > 0.0) atomicMax(&b.sc->tmp_ord, ord_key(mx));
@@ -103,15 +224,26 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const Model m, Bufs b, con
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_init_count(const Model m, Bufs b, const InitBox bx) {
     long long c0, c1;
-    block_chunk(bx.total, c0, c1);
-    int cnt = 0;
-    for (long long lin = c0 + threadIdx.x; lin < c1; lin += blockDim.x) {
-        int I[N];
-        box_index<N>(bx, lin, I);
-        cnt += gauss_at<N>(m, bx, I) > bx.pstar;
+    long long cnt = 0;
+    if (by_rows<N>(bx)) {
+        const int len = (int)bx.dims[N - 1];
+        row_chunk(bx.total / len, c0, c1);
+        for (long long row = c0 + threadIdx.x; row < c1; row += blockDim.x) {
+            int I[N];
+            row_index<N>(bx, row, I);
+            const InitRow r = row_form<N>(m, bx, I);
+            for (int i = 0; i < len; ++i) cnt += row_in<N>(m, bx, r, I, i);
+        }
+    } else {
+        block_chunk(bx.total, c0, c1);
+        for (long long lin = c0 + threadIdx.x; lin < c1; lin += blockDim.x) {
+            int I[N];
+            box_index<N>(bx, lin, I);
+            cnt += gauss_at<N>(m, bx, I) > bx.pstar;
+        }
     }
     for (int off = 16; off > 0; off >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, off);
-    __shared__ int s[WARPS];
+    __shared__ long long s[WARPS];
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = cnt;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -122,63 +254,123 @@ __global__ void __launch_bounds__(THREADS) k_init_count(const Model m, Bufs b, c
 }
 
 // Write the kept cells of the box in lexicographic order, insert them in the
-// table, and reduce their sum, maximum and CFL rates.
+// table, and reduce their sum and maximum (their velocities, masks and rates
+// come with the links). By rows: a block takes a tile of one row per thread,
+// and its threads then share the tile's kept cells.
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, const InitBox bx) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->error) return;
     long long c0, c1;
-    block_chunk(bx.total, c0, c1);
     long long base = b.blk[blockIdx.x];
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
-    double mx = -INFINITY, rmax = 0.0;
+    double mx = -INFINITY;
     int err = 0;
-    for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
-        long long lin = t0 + threadIdx.x;
-        int I[N];
-        double g = 0.0;
-        int f = 0;
-        if (lin < c1) {
-            box_index<N>(bx, lin, I);
-            g = gauss_at<N>(m, bx, I);
-            f = g > bx.pstar;
+    auto write = [&](long long c, const int* I, double g) {
+        unsigned long long k;
+        if (c >= m.cap) {
+            set_error(sc, ST_ECAPACITY);
+        } else if (!interior<N>(m, I) || !pack_key<N>(m, I, k)) {
+            set_error(sc, ST_EKEYRANGE);
+        } else {
+            T v = (T)g;
+            b.key[0][c] = k;
+            static_cast<T*>(b.q[0])[c] = v;
+            b.om[0][c] = 0;
+            table_insert_new(m, b, k, c, b.slot[0]);
+            acc_add(d, (double)v, err);
+            mx = fmax(mx, (double)v);
         }
-        int total;
-        int pos = block_exclusive_scan(f, total);
-        if (f) {
-            long long c = base + pos;
-            unsigned long long k;
-            if (c >= m.cap) {
-                set_error(sc, ST_ECAPACITY);
-            } else if (!interior<N>(m, I) || !pack_key<N>(m, I, k)) {
-                set_error(sc, ST_EKEYRANGE);
-            } else {
-                T v = (T)g;
-                b.key[0][c] = k;
-                static_cast<T*>(b.q[0])[c] = v;
-                b.om[0][c] = (unsigned short)outward_mask<N>(m, I);
-                table_insert_new(m, b, k, c, b.slot[0]);
-                acc_add(d, (double)v, err);
-                mx = fmax(mx, (double)v);
-                rmax = fmax(rmax, cfl_rate64<N>(m, I));
+    };
+    if (by_rows<N>(bx)) {
+        __shared__ int s_first[THREADS], s_end[THREADS], s_w[WARPS];
+        const int len = (int)bx.dims[N - 1];
+        row_chunk(bx.total / len, c0, c1);
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
+            const long long row = t0 + threadIdx.x;
+            int n_in = 0, i_first = 0, i_last = -1;
+            if (row < c1) {
+                int I[N];
+                row_index<N>(bx, row, I);
+                const InitRow r = row_form<N>(m, bx, I);
+                for (int i = 0; i < len; ++i)
+                    if (row_in<N>(m, bx, r, I, i)) {
+                        if (n_in == 0) i_first = i;
+                        i_last = i;
+                        ++n_in;
+                    }
             }
+            // inclusive scan of the rows' counts
+            int x = n_in;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, off);
+                if (lane >= off) x += y;
+            }
+            if (lane == 31) s_w[wid] = x;
+            __syncthreads();
+            int before = 0, total = 0;
+            for (int w = 0; w < nw; ++w) {
+                if (w < wid) before += s_w[w];
+                total += s_w[w];
+            }
+            s_end[threadIdx.x] = before + x;
+            // a row with a gap (rounding at the limit) is walked again: negative first index
+            s_first[threadIdx.x] = i_last - i_first + 1 == n_in ? i_first : -1;
+            __syncthreads();
+            for (int q = threadIdx.x; q < total; q += blockDim.x) {
+                int lo = 0, hi = (int)blockDim.x - 1;  // the first row that ends beyond q
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (s_end[mid] > q) hi = mid;
+                    else lo = mid + 1;
+                }
+                int I[N];
+                row_index<N>(bx, t0 + lo, I);
+                int left = q - (lo > 0 ? s_end[lo - 1] : 0), i = s_first[lo] + left;
+                if (s_first[lo] < 0) {
+                    const InitRow r = row_form<N>(m, bx, I);
+                    for (i = 0; i < len; ++i)
+                        if (row_in<N>(m, bx, r, I, i) && left-- == 0) break;
+                }
+                I[N - 1] = bx.lo[N - 1] + i;
+                write(base + q, I, gauss_at<N>(m, bx, I));
+            }
+            base += total;
+            __syncthreads();
         }
-        base += total;
+    } else {
+        block_chunk(bx.total, c0, c1);
+        for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
+            long long lin = t0 + threadIdx.x;
+            int I[N];
+            double g = 0.0;
+            int f = 0;
+            if (lin < c1) {
+                box_index<N>(bx, lin, I);
+                g = gauss_at<N>(m, bx, I);
+                f = g > bx.pstar;
+            }
+            int total;
+            int pos = block_exclusive_scan(f, total);
+            if (f) write(base + pos, I, g);
+            base += total;
+        }
     }
     if (err) set_error(sc, ST_EDEGENERATE);
     block_reduce_acc_max(d, mx, sc->acc, &sc->maxq_ord);
-    double r = block_max(rmax);
-    if (threadIdx.x == 0 && r > 0.0) atomicMax(&sc->maxrate_bits, (unsigned long long)__double_as_longlong(r));
 }
 
 // ------------------------------------------------------------------ explicit cells
 
-// Load N cells given as int32 indices (staged in device memory) and doubles.
+// Load N cells given as int32 indices (staged in device memory) and doubles
+// (their velocities, masks and rates come with the links).
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_init_cells(const Model m, Bufs b, const int* __restrict__ idx,
                                                         const double* __restrict__ p, long long count) {
     DevScalars* sc = b.sc;
-    double mx = -INFINITY, rmax = 0.0;
+    double mx = -INFINITY;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < count;
          c += (long long)gridDim.x * blockDim.x) {
         int I[N];
@@ -192,17 +384,12 @@ __global__ void __launch_bounds__(THREADS) k_init_cells(const Model m, Bufs b, c
         T v = (T)p[c];
         b.key[0][c] = k;
         static_cast<T*>(b.q[0])[c] = v;
-        b.om[0][c] = (unsigned short)outward_mask<N>(m, I);
+        b.om[0][c] = 0;
         table_insert_new(m, b, k, c, b.slot[0]);
         mx = fmax(mx, (double)v);
-        rmax = fmax(rmax, cfl_rate64<N>(m, I));
     }
     mx = block_max(mx);
-    double r = block_max(rmax);
-    if (threadIdx.x == 0) {
-        if (mx > -INFINITY) atomicMax(&sc->maxq_ord, ord_key(mx));
-        if (r > 0.0) atomicMax(&sc->maxrate_bits, (unsigned long long)__double_as_longlong(r));
-    }
+    if (threadIdx.x == 0 && mx > -INFINITY) atomicMax(&sc->maxq_ord, ord_key(mx));
 }
 
 // ------------------------------------------------------------------ grow

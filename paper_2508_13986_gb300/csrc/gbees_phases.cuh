@@ -86,23 +86,6 @@ __device__ __forceinline__ StepTime step_time(const Model& m, double rate, doubl
     return step_time_of(m, rate > 0.0 ? __ddiv_rn(m.cfl, rate) : (double)INFINITY, t, tt, dth);
 }
 
-// The outward directions of cell I: bit 2j+1 when the flow leaves through the
-// upper j-face (f_j at the upper face > 0), bit 2j when it leaves through the
-// lower j-face (f_j at the lower face < 0). FP64, as in Eq. 7.
-template <int N>
-__device__ __forceinline__ unsigned outward_mask(const Model& m, const int* I) {
-    unsigned msk = 0;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        int J[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) J[k] = I[k] + (k == j ? 1 : 0);
-        if (face_velocity64<N>(m, J, j) > 0.0) msk |= 1u << (2 * j + 1);
-        if (face_velocity64<N>(m, I, j) < 0.0) msk |= 1u << (2 * j);
-    }
-    return msk;
-}
-
 // Index of cell c + s1 e_j + s2 e_d (j != d) through the links (L: the links
 // of c), -1 when it is not in the pool. For an active cell c the face
 // neighbour c + s1 e_j is in the pool, so its link decides; -2 only when both
@@ -361,8 +344,10 @@ __device__ __forceinline__ void halo_body(const Model& m, const Bufs& b, const S
 // ------------------------------------------------------------------ link
 
 // Face velocities, outward mask and CFL rate of entry c of generation g (cell
-// I; Eq. 7 and Eq. 8, the same IEEE operations as outward_mask and cfl_rate64);
-// the velocities and the rate are stored, the mask and the rate returned.
+// I; Eq. 7, Eq. 8 with |f|): bit 2j+1 of the mask when the flow leaves through the
+// upper j-face (f_j at the upper face > 0), bit 2j when it leaves through the lower
+// one (f_j < 0). The velocities and the rate are stored, the mask and the rate
+// returned.
 template <int N, typename T>
 __device__ __forceinline__ double entry_velocities(const Model& m, const Bufs& b, int g, long long c, const int* I,
                                                    unsigned& msk) {
