@@ -226,15 +226,15 @@ void bind_context(gbees_ctx* ctx, const gbees_config* cfg, const Layout& L, void
     m.thr_rel = cfg->thr_rel;
     m.cfl = cfg->cfl;
     m.h_pow2 = 0;
+    m.h_plain = 1;
+    for (int j = 0; j < cfg->n; ++j)
+        if (!(cfg->h[j] >= std::ldexp(1.0, -128) && cfg->h[j] <= std::ldexp(1.0, 128))) m.h_plain = 0;
     for (int j = 0; j < cfg->n; ++j) {
         m.inv_h[j] = 1.0 / cfg->h[j];
         m.inv_2h[j] = 1.0 / (2.0 * cfg->h[j]);
         int ex = 0;
         if (std::frexp(cfg->h[j], &ex) == 0.5 && std::isnormal(m.inv_h[j])) m.h_pow2 |= 1 << j;
-        m.hf[j] = (float)cfg->h[j];
-        m.x0f[j] = (float)cfg->x0[j];
     }
-    for (int i = 0; i < 48; ++i) m.af[i] = (float)cfg->params[i];
     char* base = (char*)workspace;
     Bufs& b = ctx->b;
     b.sc = (DevScalars*)(base + L.sc);
@@ -841,6 +841,10 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         ctx->err = "covariance is not symmetric positive definite";
         return GBEES_EINVAL;
     }
+    for (int k = 0; k < n * n; ++k) {
+        bx.icovf[k] = (float)bx.icov[k];
+        if (bx.icov[k] != 0.0) bx.nonzero |= 1ull << k;
+    }
     const double thr = ctx->cfg.thr_rel > 0.0 ? ctx->cfg.thr_rel : 1e-300;
     if (!box_for(ctx, mean, cov, -2.0 * std::log(thr), &bx)) {
         ctx->err = "initial box too large";
@@ -886,18 +890,22 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
     }
     {
         Phase ph(ctx, GBEES_PHASE_OTHER, 7);
+        // the set's rows lie in the middle of the box: smaller chunks than one per
+        // resident block even out a large one
+        const long long rows = bx.total / bx.dims[n - 1];
+        const int Gi = (int)std::max<long long>(G, std::min<long long>(std::min(8 * G, GRID_MAX), rows / 256));
         with_nt(ctx, [&](auto NN, auto TT) {
             constexpr int N = decltype(NN)::value;
             using T = decltype(TT);
-            k_init_count<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
-            k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap);
-            k_init_write<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
+            k_init_count<N><<<Gi, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
+            k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, Gi, ctx->m.cap);
+            k_init_write<N, T><<<Gi, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
         });
         k_set_count_from_new<<<1, 1, 0, s>>>(ctx->b.sc);
         with_nt(ctx, [&](auto NN, auto TT) {
             constexpr int N = decltype(NN)::value;
             using T = decltype(TT);
-            k_halo<N, T, 0><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+            k_halo<N, T, 0><<<std::min(2 * G, GRID_MAX), THREADS, 0, s>>>(ctx->m, ctx->b);
             launch_link<N, T>(ctx, 0);
         });
         k_finalise<<<1, 1, 0, s>>>(ctx->m, ctx->b.sc, 0);
@@ -944,7 +952,7 @@ int gbees_init_cells(gbees_ctx* ctx, const int32_t* idx, const double* p, int64_
     with_nt(ctx, [&](auto NN, auto TT) {
         constexpr int NC = decltype(NN)::value;
         using T = decltype(TT);
-        k_halo<NC, T, 0><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+        k_halo<NC, T, 0><<<std::min(2 * G, GRID_MAX), THREADS, 0, s>>>(ctx->m, ctx->b);
         launch_link<NC, T>(ctx, 0);
     });
     k_finalise<<<1, 1, 0, s>>>(ctx->m, ctx->b.sc, 2);
@@ -1285,6 +1293,8 @@ int gbees_correct_gaussian(gbees_ctx* ctx, const double* y, const double* R, con
         ctx->err = "measurement covariance is not symmetric positive definite";
         return GBEES_EINVAL;
     }
+    for (int k = 0; k < m * m; ++k)
+        if (ms.Rinv[k] != 0.0) ms.nonzero |= 1ull << k;
     const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
     {

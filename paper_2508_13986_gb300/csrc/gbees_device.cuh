@@ -126,19 +126,8 @@ struct Model {
     double inv_h[MAXN];    // 1 / h_j
     double inv_2h[MAXN];   // 1 / (2 h_j)
     int h_pow2;            // bit j: h_j is a power of two
-    // float copies for the FP32 update (no double-to-float conversion per use)
-    float af[48];
-    float hf[MAXN];
-    float x0f[MAXN];
+    int h_plain;           // every h_j lies within [2^-128, 2^128] (div_round's range)
 };
-
-// Model parameter i in the arithmetic type of the caller.
-template <typename R>
-__device__ __forceinline__ R par(const Model& m, int i);
-template <>
-__device__ __forceinline__ double par<double>(const Model& m, int i) { return m.a[i]; }
-template <>
-__device__ __forceinline__ float par<float>(const Model& m, int i) { return m.af[i]; }
 
 // One block's share of a grid-wide reduction, written without atomics and
 // combined by whoever finishes the step (deterministic: integer digits, max).
@@ -289,32 +278,32 @@ __device__ __forceinline__ void unpack_key(const Model& m, unsigned long long k,
 }
 
 // ------------------------------------------------------------------ hashtable
-// Open addressing with linear probing (Sec. 4.2); keys are claimed with
+// Open addressing (Sec. 4.2) along table_home and table_next; keys are claimed with
 // atomicCAS (the concurrent insertion of Algorithm 2 without staging).
 
 __device__ __forceinline__ int table_find(const Model& m, const Slot* __restrict__ T, unsigned long long key) {
-    unsigned long long h = mix64(key) & m.tmask;
+    unsigned long long h = table_home(key, m.tmask);
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
         ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(T + h));
         if (s.x == key) return (int)(long long)s.y;
         if (s.x == EMPTY_KEY) return -1;
-        h = (h + 1) & m.tmask;
+        h = table_next(h, probe, m.tmask);
     }
     return -1;
 }
 
-// Cooperative lookup: a tile of W lanes probes W consecutive slots per round
-// (one coalesced load) and the lowest lane that sees the key or an empty slot
+// Cooperative lookup: a tile of W lanes probes W slots of the sequence per round
+// and the lowest lane that sees the key or an empty slot
 // decides. All lanes of the tile must call it with the same key.
 template <int W>
 __device__ __forceinline__ int table_find_tile(const Model& m, const Slot* __restrict__ T, unsigned long long key,
                                                cg::thread_block_tile<W> tile) {
-    unsigned long long base = mix64(key) & m.tmask;
+    const unsigned long long home = table_home(key, m.tmask);
     const int lane = tile.thread_rank();
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; probe += W) {
-        unsigned long long h = (base + probe + lane) & m.tmask;
+        unsigned long long h = table_slot(home, (probe + lane) & m.tmask, m.tmask);
         ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(T + h));
         unsigned hit = tile.ballot(s.x == key);
         unsigned emp = tile.ballot(s.x == EMPTY_KEY);
@@ -334,7 +323,7 @@ __device__ __forceinline__ int table_find_tile(const Model& m, const Slot* __res
 // Insert key if absent. Returns 1 and the slot when this thread claimed a new
 // slot, 0 when the key is present, -1 when the table is full.
 __device__ __forceinline__ int table_claim(const Model& m, Slot* T, unsigned long long key, unsigned long long* slot) {
-    unsigned long long h = mix64(key) & m.tmask;
+    unsigned long long h = table_home(key, m.tmask);
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
         unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&T[h].key);
@@ -347,7 +336,7 @@ __device__ __forceinline__ int table_claim(const Model& m, Slot* T, unsigned lon
             }
             if (old == key) return 0;
         }
-        h = (h + 1) & m.tmask;
+        h = table_next(h, probe, m.tmask);
     }
     return -1;
 }
@@ -366,80 +355,28 @@ __device__ __forceinline__ long long warp_aggregated_add(long long* counter, int
 }
 
 // ------------------------------------------------------------------ drift models
+// f_j(y) is evaluated with the order of operations written out and no fused
+// multiply-add, so that the FP64 velocities that take the grow / prune / CFL
+// decisions are the IEEE values of the textbook expressions.
 
-template <typename R>
-struct Ar;  // IEEE operations without contraction into fused multiply-add
-
-template <>
-struct Ar<double> {
+struct Ar {
     static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 };
-template <>
-struct Ar<float> {
-    static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-    static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-    static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-};
 
-// f_j(y) with the evaluation order written out (no fused multiply-add), so that
-// the FP64 velocities that take the grow / prune / CFL decisions are the IEEE
-// values of the textbook expressions.
-template <typename R, int N>
-__device__ __forceinline__ R drift(const Model& m, int dyn, const R* y, int j) {
-    using A = Ar<R>;
-    switch (dyn) {
-        case DYN_CONSTANT:
-            return par<R>(m, j);
-        case DYN_LINEAR: {
-            R s = 0;
-#pragma unroll
-            for (int k = 0; k < N; ++k) s = A::add(s, A::mul(par<R>(m, j * N + k), y[k]));
-            return A::add(s, par<R>(m, N * N + j));
-        }
-        case DYN_LORENZ63:
-            if (N != 3) return 0;
-            if (j == 0) return A::mul(par<R>(m, 0), A::sub(y[1], y[0]));
-            if (j == 1) return A::sub(A::mul(y[0], A::sub(par<R>(m, 1), y[2 % N])), y[1]);
-            return A::sub(A::mul(y[0], y[1]), A::mul(par<R>(m, 2), y[2 % N]));
-        case DYN_LORENZ63_SHIFTED:
-            if (N != 3) return 0;
-            if (j == 0) return A::mul(par<R>(m, 0), A::sub(y[1], y[0]));
-            if (j == 1) return A::sub(-y[1], A::mul(y[0], y[2 % N]));
-            return A::sub(A::add(A::mul(-par<R>(m, 1), y[2 % N]), A::mul(y[0], y[1])),
-                          A::mul(par<R>(m, 1), par<R>(m, 2)));
-        case DYN_LORENZ96: {
-            const int jp = (j + 1) % N, jm2 = (j + N - 2) % N, jm1 = (j + N - 1) % N;
-            return A::add(A::sub(A::mul(A::sub(y[jp], y[jm2]), y[jm1]), y[j]), par<R>(m, 0));
-        }
-    }
-    return 0;
-}
-
-// Centre coordinate x0_k + i_k h_k and lower-face coordinate x0_k + (i_k - 1/2) h_k,
-// evaluated exactly as written (one rounded product, one rounded sum).
+// Centre coordinate x0_k + i_k h_k (one rounded product, one rounded sum).
 __device__ __forceinline__ double centre64(const Model& m, int k, int i) {
     return __dadd_rn(m.x0[k], __dmul_rn((double)i, m.h[k]));
 }
-__device__ __forceinline__ double lowface64(const Model& m, int k, int i) {
-    return __dadd_rn(m.x0[k], __dmul_rn((double)i - 0.5, m.h[k]));
-}
 
-// FP64 face velocity f_j at the lower face of cell I in dimension j (Eq. 7).
-template <int N>
-__device__ __forceinline__ double face_velocity64(const Model& m, const int* I, int j) {
-    double y[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) y[k] = (k == j) ? lowface64(m, k, I[k]) : centre64(m, k, I[k]);
-    return drift<double, N>(m, m.dyn, y, j);
-}
-
-// x / h_j as the IEEE division rounds it. For a width that is a power of two
-// the reciprocal is exact, so the product rounds the same real number: the
-// same result for one FP64 multiplication instead of a division sequence.
+// x / h_j for x >= 0 as the IEEE division rounds it. For a width that is a power
+// of two the reciprocal is exact, so the product rounds the same real number.
 __device__ __forceinline__ double div_h(const Model& m, double x, int j) {
-    return ((m.h_pow2 >> j) & 1) ? __dmul_rn(x, m.inv_h[j]) : __ddiv_rn(x, m.h[j]);
+    if ((m.h_pow2 >> j) & 1) return __dmul_rn(x, m.inv_h[j]);
+    const int e = (int)(__double_as_longlong(x) >> 52);
+    if (m.h_plain && e > 256 && e < 1792) return div_round(x, m.h[j], m.inv_h[j]);
+    return __ddiv_rn(x, m.h[j]);
 }
 
 // a * b + c rounded once, and the larger of two values, in the arithmetic

@@ -34,13 +34,21 @@ __device__ __forceinline__ void finish_link(const Model& m, DevScalars* sc, cons
 // masks and rates; with step != 0 the last block also fixes dt (Eq. 8).
 // W lanes probe the hashtable together (warp-cooperative probing).
 template <int N, int W, typename T>
-__global__ void __launch_bounds__(THREADS) k_link(const Model m, Bufs b, int step) {
+__global__ void __launch_bounds__(THREADS, 4) k_link(const __grid_constant__ Model m, const __grid_constant__ Bufs b,
+                                                     int step) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->error) return;
     if (step && *(volatile int*)&sc->done) return;
     const StepView v = view_of(m, sc);
-    const double r = (W == 1) ? link_body<N, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi)
-                              : link_body_tile<N, W, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi);
+    double r;
+    if constexpr (W == 1) {
+        // few: at most four rounds of all warps with one or a few entries each
+        const long long few = 4ll * v.nb * (blockDim.x >> 5) * (32 / (2 * N));
+        r = v.N - v.N_prev <= few ? link_few_body<N, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi)
+                                  : link_body<N, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi);
+    } else {
+        r = link_body_tile<N, W, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi);
+    }
     long long zero[NDIG] = {0, 0, 0, 0, 0, 0};
     block_partial(b.part, zero, -INFINITY, r);
     if (last_block(sc)) {
@@ -59,7 +67,42 @@ struct InitBox {
     double icov[MAXN * MAXN];
     double pstar;
     float qlim;  // pass 1: q of the cell nearest the mean; then: -2 ln pstar
+    float icovf[MAXN * MAXN];
+    unsigned long long nonzero;  // bit a N + c: icov[a][c] != 0 (a comparison would take the FP64 pipe)
 };
+
+// Distance of the cells' centres from the mean, per dimension and index of the
+// box, formed once per block (four FP64 instructions per look otherwise).
+constexpr int AXIS_MAX = 1024;  // entries; a box with longer axes forms them where they are used
+template <int N>
+struct Axes {
+    const double* tab;  // null: not tabulated
+    int at[N];          // place of index lo_k of axis k, less lo_k
+    __device__ __forceinline__ double dx(const Model& m, const InitBox& bx, int k, int i) const {
+        return tab ? tab[at[k] + i] : __dsub_rn(centre64(m, k, i), bx.mean[k]);
+    }
+};
+// (all threads of the block)
+template <int N>
+__device__ __forceinline__ Axes<N> make_axes(const Model& m, const InitBox& bx, double* s_tab) {
+    Axes<N> ax;
+    long long n = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) n += bx.dims[k];
+    ax.tab = n <= AXIS_MAX ? s_tab : nullptr;
+    int off = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        ax.at[k] = off - bx.lo[k];
+        if (ax.tab) {
+            for (int i = threadIdx.x; i < (int)bx.dims[k]; i += blockDim.x)
+                s_tab[off + i] = __dsub_rn(centre64(m, k, bx.lo[k] + i), bx.mean[k]);
+            off += (int)bx.dims[k];
+        }
+    }
+    __syncthreads();
+    return ax;
+}
 
 template <int N>
 __device__ __forceinline__ void box_index(const InitBox& bx, long long lin, int* I) {
@@ -73,16 +116,16 @@ __device__ __forceinline__ void box_index(const InitBox& bx, long long lin, int*
 // exp(-1/2 (x - mean)^T icov (x - mean)) at the centre of cell I. (A zero of icov
 // adds a zero to the sum: left out, a diagonal covariance takes N terms.)
 template <int N>
-__device__ __forceinline__ double gauss_at(const Model& m, const InitBox& bx, const int* I) {
+__device__ __noinline__ double gauss_at(const Model& m, const InitBox& bx, const Axes<N>& ax, const int* I) {
     double dx[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) dx[k] = __dsub_rn(centre64(m, k, I[k]), bx.mean[k]);
+    for (int k = 0; k < N; ++k) dx[k] = ax.dx(m, bx, k, I[k]);
     double q = 0.0;
 #pragma unroll
     for (int a = 0; a < N; ++a)
 #pragma unroll
         for (int c = 0; c < N; ++c)
-            if (bx.icov[a * N + c] != 0.0)
+            if ((bx.nonzero >> (a * N + c)) & 1ull)
                 q = __dadd_rn(q, __dmul_rn(__dmul_rn(dx[a], bx.icov[a * N + c]), dx[c]));
     return exp(__dmul_rn(-0.5, q));
 }
@@ -93,10 +136,10 @@ __device__ __forceinline__ double gauss_at(const Model& m, const InitBox& bx, co
 // cell in single precision and a bound of its error. Only a cell whose q lies
 // within that bound of the limit is decided in FP64, so the set is the one that
 // FP64 gives everywhere; the densities of the cells in the set are FP64. The
-// paper's 6-D case (2.0e6 cells in the set, a box of 6.4e7): 0.68 + 0.69 + 2.57 ms
+// paper's 6-D case (2.0e6 cells in the set, a box of 6.4e7): 0.11 + 0.13 + 0.6 ms
 // for the three passes (81 ms with the FP64 density at every cell of the box in
-// each of them and a covariance's zeros multiplied out; the whole call 87.5 ->
-// 10.5 ms; Lorenz '96 6-D with h = 0.25 286 -> 69 ms).
+// each of them); the whole call 87.5 -> 3.0 ms, Lorenz '96 6-D with h = 0.25
+// 286 -> 8.0 ms.
 // Longer rows than INIT_ROW_MAX (a chain of that many steps per thread) and
 // fewer dimensions (the set fills most of the box) are swept cell by cell.
 constexpr int INIT_ROW_MAX = 1024;
@@ -138,25 +181,25 @@ __device__ __forceinline__ void row_index(const InitBox& bx, long long row, int*
 }
 
 template <int N>
-__device__ __forceinline__ InitRow row_form(const Model& m, const InitBox& bx, const int* I) {
+__device__ __forceinline__ InitRow row_form(const Model& m, const InitBox& bx, const Axes<N>& ax, const int* I) {
     float dx[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) dx[k] = (float)__dsub_rn(centre64(m, k, I[k]), bx.mean[k]);
+    for (int k = 0; k < N; ++k) dx[k] = (float)ax.dx(m, bx, k, I[k]);
     InitRow r;
     r.A = r.Aa = r.B = r.Ba = 0.0f;
 #pragma unroll
     for (int a = 0; a < N - 1; ++a) {
 #pragma unroll
         for (int c = 0; c < N - 1; ++c) {
-            const float t = dx[a] * (float)bx.icov[a * N + c] * dx[c];
+            const float t = dx[a] * bx.icovf[a * N + c] * dx[c];
             r.A += t;
             r.Aa += fabsf(t);
         }
-        const float t = dx[a] * ((float)bx.icov[a * N + N - 1] + (float)bx.icov[(N - 1) * N + a]);
+        const float t = dx[a] * (bx.icovf[a * N + N - 1] + bx.icovf[(N - 1) * N + a]);
         r.B += t;
         r.Ba += fabsf(t);
     }
-    r.C = (float)bx.icov[N * N - 1];
+    r.C = bx.icovf[N * N - 1];
     r.h = (float)m.h[N - 1];
     r.dx0 = dx[N - 1];
     // dx of a cell of the row as dx0 + i h: two roundings and those of dx0 and h
@@ -175,21 +218,25 @@ __device__ __forceinline__ float row_q(const InitRow& r, int i, float& e) {
 
 // Whether cell i of the row at I is in the set p > pstar (qlim: -2 ln pstar).
 template <int N>
-__device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const InitRow& r, int* I, int i) {
+__device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const Axes<N>& ax, const InitRow& r, int* I,
+                                       int i) {
     float e;
     const float q = row_q(r, i, e), d = q - bx.qlim;
     e += 1e-6f * fabsf(bx.qlim);
     if (d > e) return false;
     if (d < -e) return true;
     I[N - 1] = bx.lo[N - 1] + i;  // too near the limit (or not a number)
-    return gauss_at<N>(m, bx, I) > bx.pstar;
+    return gauss_at<N>(m, bx, ax, I) > bx.pstar;
 }
 
 // Initial Gaussian (Sec. 5.1), pass 1: the largest density over the box of
 // candidate cells, which fixes the threshold p* = thr_rel * max p. By rows: the
 // cells whose q may be as small as that of the cell nearest the mean (bx.qlim).
 template <int N>
-__global__ void __launch_bounds__(THREADS) k_init_max(const Model m, Bufs b, const InitBox bx) {
+__global__ void __launch_bounds__(THREADS) k_init_max(const __grid_constant__ Model m, Bufs b,
+                                                        const __grid_constant__ InitBox bx) {
+    __shared__ double s_tab[AXIS_MAX];
+    const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     double mx = 0.0;
     const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -199,20 +246,20 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const Model m, Bufs b, con
         for (long long row = first; row < rows; row += stride) {
             int I[N];
             row_index<N>(bx, row, I);
-            const InitRow r = row_form<N>(m, bx, I);
+            const InitRow r = row_form<N>(m, bx, ax, I);
             for (int i = 0; i < len; ++i) {
                 float e;
                 const float q = row_q(r, i, e);
                 if (q - bx.qlim > e + 1e-6f * fabsf(bx.qlim)) continue;
                 I[N - 1] = bx.lo[N - 1] + i;
-                mx = fmax(mx, gauss_at<N>(m, bx, I));
+                mx = fmax(mx, gauss_at<N>(m, bx, ax, I));
             }
         }
     } else {
         for (long long lin = first; lin < bx.total; lin += stride) {
             int I[N];
             box_index<N>(bx, lin, I);
-            mx = fmax(mx, gauss_at<N>(m, bx, I));
+            mx = fmax(mx, gauss_at<N>(m, bx, ax, I));
         }
     }
     mx = block_max(mx);
@@ -222,7 +269,10 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const Model m, Bufs b, con
 // Initial Gaussian, pass 2: per-block counts of the box cells above p*, the
 // offsets of the write pass.
 template <int N>
-__global__ void __launch_bounds__(THREADS) k_init_count(const Model m, Bufs b, const InitBox bx) {
+__global__ void __launch_bounds__(THREADS) k_init_count(const __grid_constant__ Model m, Bufs b,
+                                                        const __grid_constant__ InitBox bx) {
+    __shared__ double s_tab[AXIS_MAX];
+    const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     long long c0, c1;
     long long cnt = 0;
     if (by_rows<N>(bx)) {
@@ -231,15 +281,15 @@ __global__ void __launch_bounds__(THREADS) k_init_count(const Model m, Bufs b, c
         for (long long row = c0 + threadIdx.x; row < c1; row += blockDim.x) {
             int I[N];
             row_index<N>(bx, row, I);
-            const InitRow r = row_form<N>(m, bx, I);
-            for (int i = 0; i < len; ++i) cnt += row_in<N>(m, bx, r, I, i);
+            const InitRow r = row_form<N>(m, bx, ax, I);
+            for (int i = 0; i < len; ++i) cnt += row_in<N>(m, bx, ax, r, I, i);
         }
     } else {
         block_chunk(bx.total, c0, c1);
         for (long long lin = c0 + threadIdx.x; lin < c1; lin += blockDim.x) {
             int I[N];
             box_index<N>(bx, lin, I);
-            cnt += gauss_at<N>(m, bx, I) > bx.pstar;
+            cnt += gauss_at<N>(m, bx, ax, I) > bx.pstar;
         }
     }
     for (int off = 16; off > 0; off >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, off);
@@ -258,13 +308,16 @@ __global__ void __launch_bounds__(THREADS) k_init_count(const Model m, Bufs b, c
 // come with the links). By rows: a block takes a tile of one row per thread,
 // and its threads then share the tile's kept cells.
 template <int N, typename T>
-__global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, const InitBox bx) {
+__global__ void __launch_bounds__(THREADS, 4) k_init_write(const __grid_constant__ Model m, Bufs b,
+                                                        const __grid_constant__ InitBox bx) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->error) return;
+    __shared__ double s_tab[AXIS_MAX];
+    const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     long long c0, c1;
     long long base = b.blk[blockIdx.x];
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
-    double mx = -INFINITY;
+    T mx = -INFINITY;
     int err = 0;
     auto write = [&](long long c, const int* I, double g) {
         unsigned long long k;
@@ -278,8 +331,8 @@ __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, c
             static_cast<T*>(b.q[0])[c] = v;
             b.om[0][c] = 0;
             table_insert_new(m, b, k, c, b.slot[0]);
-            acc_add(d, (double)v, err);
-            mx = fmax(mx, (double)v);
+            acc_add(d, v, err);
+            mx = vmax(mx, v);
         }
     };
     if (by_rows<N>(bx)) {
@@ -293,9 +346,9 @@ __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, c
             if (row < c1) {
                 int I[N];
                 row_index<N>(bx, row, I);
-                const InitRow r = row_form<N>(m, bx, I);
+                const InitRow r = row_form<N>(m, bx, ax, I);
                 for (int i = 0; i < len; ++i)
-                    if (row_in<N>(m, bx, r, I, i)) {
+                    if (row_in<N>(m, bx, ax, r, I, i)) {
                         if (n_in == 0) i_first = i;
                         i_last = i;
                         ++n_in;
@@ -319,23 +372,30 @@ __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, c
             // a row with a gap (rounding at the limit) is walked again: negative first index
             s_first[threadIdx.x] = i_last - i_first + 1 == n_in ? i_first : -1;
             __syncthreads();
-            for (int q = threadIdx.x; q < total; q += blockDim.x) {
-                int lo = 0, hi = (int)blockDim.x - 1;  // the first row that ends beyond q
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (s_end[mid] > q) hi = mid;
-                    else lo = mid + 1;
-                }
+            for (int q0 = threadIdx.x & ~31; q0 < total; q0 += blockDim.x) {
+                const int q = q0 + lane;
+                const bool on = q < total;
                 int I[N];
-                row_index<N>(bx, t0 + lo, I);
-                int left = q - (lo > 0 ? s_end[lo - 1] : 0), i = s_first[lo] + left;
-                if (s_first[lo] < 0) {
-                    const InitRow r = row_form<N>(m, bx, I);
-                    for (i = 0; i < len; ++i)
-                        if (row_in<N>(m, bx, r, I, i) && left-- == 0) break;
+                if (on) {
+                    int lo = 0, hi = (int)blockDim.x - 1;  // the first row that ends beyond q
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (s_end[mid] > q) hi = mid;
+                        else lo = mid + 1;
+                    }
+                    row_index<N>(bx, t0 + lo, I);
+                    int left = q - (lo > 0 ? s_end[lo - 1] : 0), i = s_first[lo] + left;
+                    if (s_first[lo] < 0) {
+                        const InitRow r = row_form<N>(m, bx, ax, I);
+                        for (i = 0; i < len; ++i)
+                            if (row_in<N>(m, bx, ax, r, I, i) && left-- == 0) break;
+                    }
+                    I[N - 1] = bx.lo[N - 1] + i;
                 }
-                I[N - 1] = bx.lo[N - 1] + i;
-                write(base + q, I, gauss_at<N>(m, bx, I));
+                __syncwarp();  // (the FP64 part with the warp in one piece)
+                const double g = on ? gauss_at<N>(m, bx, ax, I) : 0.0;
+                if (on) write(base + q, I, g);
+                __syncwarp();
             }
             base += total;
             __syncthreads();
@@ -349,7 +409,7 @@ __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, c
             int f = 0;
             if (lin < c1) {
                 box_index<N>(bx, lin, I);
-                g = gauss_at<N>(m, bx, I);
+                g = gauss_at<N>(m, bx, ax, I);
                 f = g > bx.pstar;
             }
             int total;
@@ -359,7 +419,7 @@ __global__ void __launch_bounds__(THREADS) k_init_write(const Model m, Bufs b, c
         }
     }
     if (err) set_error(sc, ST_EDEGENERATE);
-    block_reduce_acc_max(d, mx, sc->acc, &sc->maxq_ord);
+    block_reduce_acc_max(d, (double)mx, sc->acc, &sc->maxq_ord);
 }
 
 // ------------------------------------------------------------------ explicit cells
@@ -504,34 +564,45 @@ struct Meas {
     int H[MAXN];
     double y[MAXN];
     double Rinv[MAXN * MAXN];
+    unsigned long long nonzero;  // bit a m + e: Rinv[a][e] != 0
 };
 
 // p <- exp(-1/2 (y - x_H)^T R^-1 (y - x_H)) p at the cell centres (Eq. 4); the
 // maximum is reduced for the prune that follows.
 template <int N, typename T>
-__global__ void __launch_bounds__(THREADS) k_correct(const Model m, Bufs b, const Meas ms) {
+__global__ void __launch_bounds__(THREADS) k_correct(const __grid_constant__ Model m, Bufs b,
+                                                     const __grid_constant__ Meas ms) {
     DevScalars* sc = b.sc;
     if (*(volatile int*)&sc->error) return;
     const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
     const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
     T* Q = static_cast<T*>(b.q[pb]);
     const unsigned long long* key = b.key[g];
-    double mx = -INFINITY;
+    T tmax = -INFINITY;
     for (WarpRuns wr(ncell); wr.next();) {
         const long long c = wr.c;
         if (c >= ncell) continue;
+        const T q = Q[c];
+        // a density of 0 (a halo cell's) stays 0: FP64 bounds this pass
+        if (q == (T)0) {
+            tmax = vmax(tmax, q);
+            continue;
+        }
         int I[N];
         unpack_key<N>(m, key[c], I);
         double r[MAXN];
         for (int a = 0; a < ms.m; ++a) r[a] = __dsub_rn(ms.y[a], centre64(m, ms.H[a], I[ms.H[a]]));
         double qf = 0.0;
         for (int a = 0; a < ms.m; ++a)
-            for (int e = 0; e < ms.m; ++e) qf = __dadd_rn(qf, __dmul_rn(__dmul_rn(r[a], ms.Rinv[a * ms.m + e]), r[e]));
-        double L = exp(__dmul_rn(-0.5, qf));
-        T v = (T)__dmul_rn(L, (double)Q[c]);
+            for (int e = 0; e < ms.m; ++e)
+                if ((ms.nonzero >> (a * ms.m + e)) & 1ull)  // (a zero adds a zero)
+                    qf = __dadd_rn(qf, __dmul_rn(__dmul_rn(r[a], ms.Rinv[a * ms.m + e]), r[e]));
+        const double L = exp(__dmul_rn(-0.5, qf));
+        const T v = (T)__dmul_rn(L, (double)q);
         Q[c] = v;
-        mx = fmax(mx, (double)v);
+        tmax = vmax(tmax, v);
     }
+    const double mx = (double)tmax;
     long long zero[NDIG] = {0, 0, 0, 0, 0, 0};
     block_partial(b.part, zero, mx, 0.0);
     if (last_block(sc)) {

@@ -1,13 +1,15 @@
-// Packed cell keys and the hashtable's hash: pure integer functions that the
-// device code uses and that a host compiler can build too (the host tests pin
-// them: round trip, key order, range limits, and the probe lengths of linear
-// probing at load factor 1/2, Sec. 4.2).
+// Packed cell keys, the hashtable's hash and the rounded division by a cell
+// width: pure functions that the device code uses and that a host compiler can build too (the host tests pin
+// them: round trip, key order, range limits, the probe sequence, and the probe
+// lengths at load factor 1/2, Sec. 4.2).
 //
 // A cell index I (N signed ints) packs into one u64: each component biased by
 // 2^(b-1) into b bits, dimension 0 in the most significant position, so that
 // key order is the lexicographic order of the index vectors. A component
 // outside [-2^(b-1), 2^(b-1)) has no key.
 #pragma once
+
+#include <math.h>
 
 #if defined(__CUDACC__)
 #define GBEES_HD __host__ __device__ __forceinline__
@@ -67,8 +69,7 @@ GBEES_HD unsigned long long row_morton_code(unsigned long long k, int n, int b) 
     return (morton_code(k >> b, n - 1, b) << b) | last;
 }
 
-// murmur3 64-bit finaliser (a bijection of u64); the table slot of a key is
-// mix64(key) & (slots - 1)
+// murmur3 64-bit finaliser (a bijection of u64)
 GBEES_HD unsigned long long mix64(unsigned long long x) {
     x ^= x >> 33;
     x *= 0xff51afd7ed558ccdull;
@@ -76,6 +77,56 @@ GBEES_HD unsigned long long mix64(unsigned long long x) {
     x *= 0xc4ceb9fe1a85ec53ull;
     x ^= x >> 33;
     return x;
+}
+
+// Probe sequence of a key in a table of mask + 1 slots (a power of two, at
+// least 64). Cells whose keys differ in the low 4 bits alone (16 neighbours along
+// the last dimension) share a group of 16 consecutive slots: the group's place is
+// hashed from the other bits, and the order within it is permuted by an XOR with
+// bits of the same hash, so that a set that repeats with the period of a group
+// (one cell in each, say) does not fill one slot of every group. A collision
+// moves on to the same slot of the next group, so the sequences of 16 cells stay
+// side by side; each of the 16 interleaved subtables is an ordinary table with
+// linear probing at the same load. After all groups the sequence goes on with the
+// next slot of each: it visits every slot once.
+//
+// Why groups: a random probe costs a translation miss and a DRAM sector, and
+// translation misses bound the lookups of large pools. The cells of a warp follow
+// one another along the last dimension, and so do their neighbours in any
+// direction: a warp's 32 probes fall into 2 to 5 groups instead of 32 places.
+constexpr int TABLE_GROUP_BITS = 4;
+constexpr unsigned long long TABLE_GROUP = 1ull << TABLE_GROUP_BITS;
+
+GBEES_HD unsigned long long table_home(unsigned long long key, unsigned long long mask) {
+    const unsigned long long g = mix64(key >> TABLE_GROUP_BITS);
+    return ((g << TABLE_GROUP_BITS) | ((key ^ (g >> 60)) & (TABLE_GROUP - 1))) & mask;
+}
+
+// The slot after `slot`, the probe-th of the sequence (0, 1, ...).
+GBEES_HD unsigned long long table_next(unsigned long long slot, unsigned long long probe, unsigned long long mask) {
+    slot = (slot + TABLE_GROUP) & mask;
+    if (((probe + 1) & (mask >> TABLE_GROUP_BITS)) == 0)
+        slot = (slot & ~(TABLE_GROUP - 1)) | ((slot + 1) & (TABLE_GROUP - 1));
+    return slot;
+}
+
+// The probe-th slot of the sequence that starts at home.
+GBEES_HD unsigned long long table_slot(unsigned long long home, unsigned long long probe, unsigned long long mask) {
+    const unsigned long long groups = (mask >> TABLE_GROUP_BITS) + 1;
+    return ((home + probe * TABLE_GROUP) & mask & ~(TABLE_GROUP - 1)) |
+           ((home + probe / groups) & (TABLE_GROUP - 1));
+}
+
+// x / h for x >= 0 with y = RN(1 / h), x and h far from the ends of the exponent
+// range, as the IEEE division rounds it: a quotient that is within an ulp becomes
+// the correctly rounded one by its exact remainder times y (P. Markstein,
+// Computation of elementary functions on the IBM RISC System/6000 processor,
+// 1990). x y is within two ulp, the first correction brings it within one. Five
+// FP64 instructions.
+GBEES_HD double div_round(double x, double h, double y) {
+    const double q0 = x * y;
+    const double q1 = fma(fma(-q0, h, x), y, q0);
+    return fma(fma(-q1, h, x), y, q1);
 }
 
 }  // namespace gbees

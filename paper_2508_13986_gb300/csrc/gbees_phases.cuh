@@ -343,30 +343,92 @@ __device__ __forceinline__ void halo_body(const Model& m, const Bufs& b, const S
 
 // ------------------------------------------------------------------ link
 
+// f_j with component j of the state replaced by yj (y: the cell's centre): the
+// operations of drift, in its order.
+template <int N, int DYN>
+__device__ __forceinline__ double drift_at(const Model& m, const double* y, int j, double yj) {
+    using A = Ar;
+    auto at = [&](int k) { return k == j ? yj : y[k]; };
+    if constexpr (DYN == DYN_CONSTANT) {
+        return m.a[j];
+    } else if constexpr (DYN == DYN_LINEAR) {
+        double s = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) s = A::add(s, A::mul(m.a[j * N + k], at(k)));
+        return A::add(s, m.a[N * N + j]);
+    } else if constexpr (DYN == DYN_LORENZ63 && N == 3) {
+        if (j == 0) return A::mul(m.a[0], A::sub(at(1), at(0)));
+        if (j == 1) return A::sub(A::mul(at(0), A::sub(m.a[1], at(2))), at(1));
+        return A::sub(A::mul(at(0), at(1)), A::mul(m.a[2], at(2)));
+    } else if constexpr (DYN == DYN_LORENZ63_SHIFTED && N == 3) {
+        if (j == 0) return A::mul(m.a[0], A::sub(at(1), at(0)));
+        if (j == 1) return A::sub(-at(1), A::mul(at(0), at(2)));
+        return A::sub(A::add(A::mul(-m.a[1], at(2)), A::mul(at(0), at(1))), A::mul(m.a[1], m.a[2]));
+    } else if constexpr (DYN == DYN_LORENZ96 && N >= 4) {
+        return A::add(A::sub(A::mul(A::sub(at((j + 1) % N), at((j + N - 2) % N)), at((j + N - 1) % N)), at(j)), m.a[0]);
+    } else {
+        return 0.0;
+    }
+}
+
+// x > 0 without the FP64 pipe (false for NaN, as the comparison).
+__device__ __forceinline__ bool above0(double x) {
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7FF0000000000000ll;
+}
+
 // Face velocities, outward mask and CFL rate of entry c of generation g (cell
 // I; Eq. 7, Eq. 8 with |f|): bit 2j+1 of the mask when the flow leaves through the
 // upper j-face (f_j at the upper face > 0), bit 2j when it leaves through the lower
 // one (f_j < 0). The velocities and the rate are stored, the mask and the rate
-// returned.
-template <int N, typename T>
-__device__ __forceinline__ double entry_velocities(const Model& m, const Bufs& b, int g, long long c, const int* I,
-                                                   unsigned& msk) {
-    T* U = static_cast<T*>(b.u[g]);
+// returned. The FP64 pipe bounds the pass over many new entries, so each model has
+// its own straight code (one branch for all faces), the faces of a cell share its
+// index in double and what the drift has in common, and the signs are read from
+// the bits: 110 to 130 FP64 instructions per entry of Lorenz '96 6-D (493 with the
+// models selected face by face and divisions).
+template <int N, int DYN, typename T>
+__device__ __forceinline__ double entry_velocities_of(const Model& m, const Bufs& b, int g, long long c, const int* I,
+                                                      unsigned& msk) {
+    double di[N], y[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        di[k] = (double)I[k];
+        y[k] = __dadd_rn(m.x0[k], __dmul_rn(di[k], m.h[k]));
+    }
     double r = 0.0;
     msk = 0;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        int J[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) J[k] = I[k] + (k == j ? 1 : 0);
-        const double ul = face_velocity64<N>(m, I, j);
-        if (face_velocity64<N>(m, J, j) > 0.0) msk |= 1u << (2 * j + 1);
-        if (ul < 0.0) msk |= 1u << (2 * j);
-        U[j * m.cap + c] = (T)ul;
-        r = __dadd_rn(r, div_h(m, fabs(ul), j));
+        // x0 + (i -+ 1/2) h (i + 1/2 is exact, as (i + 1) - 1/2)
+        const double lo = __dadd_rn(m.x0[j], __dmul_rn(__dsub_rn(di[j], 0.5), m.h[j]));
+        const double hi = __dadd_rn(m.x0[j], __dmul_rn(__dadd_rn(di[j], 0.5), m.h[j]));
+        const double ul = drift_at<N, DYN>(m, y, j, lo);
+        if (above0(drift_at<N, DYN>(m, y, j, hi))) msk |= 1u << (2 * j + 1);
+        if (above0(-ul)) msk |= 1u << (2 * j);
+        static_cast<T*>(b.u[g])[j * m.cap + c] = (T)ul;
+        r = __dadd_rn(r, div_h(m, abs_bits(ul), j));
     }
     b.rate[g][c] = r;
     return r;
+}
+template <int N, typename T>
+__device__ __forceinline__ double entry_velocities(const Model& m, const Bufs& b, int g, long long c, const int* I,
+                                                   unsigned& msk) {
+    switch (m.dyn) {
+        case DYN_CONSTANT: return entry_velocities_of<N, DYN_CONSTANT, T>(m, b, g, c, I, msk);
+        case DYN_LINEAR: return entry_velocities_of<N, DYN_LINEAR, T>(m, b, g, c, I, msk);
+        case DYN_LORENZ63:
+            if constexpr (N == 3) return entry_velocities_of<N, DYN_LORENZ63, T>(m, b, g, c, I, msk);
+            break;
+        case DYN_LORENZ63_SHIFTED:
+            if constexpr (N == 3) return entry_velocities_of<N, DYN_LORENZ63_SHIFTED, T>(m, b, g, c, I, msk);
+            break;
+        case DYN_LORENZ96:
+            if constexpr (N >= 4) return entry_velocities_of<N, DYN_LORENZ96, T>(m, b, g, c, I, msk);
+            break;
+    }
+    msk = 0;
+    return 0.0;
 }
 
 // Face velocities and outward masks of the new entries [lo, hi) (the mask is
@@ -394,33 +456,172 @@ __device__ __forceinline__ double link_masks(const Model& m, const Bufs& b, long
     return rmax;
 }
 
-// Entries [lo, hi) are new: look up their 2n face neighbours (one probe per
-// thread and direction), write the reverse links into the neighbours, and set
-// their outward masks; returns this thread's largest CFL rate among the active
-// ones.
+// f_j at the lower (up = 0) or upper (up = 1) j-face of the cell with packed
+// key k: drift_at with j known at run time, out of line (the code of a
+// small grid's step loop runs once per step from the instruction caches, so what
+// is not a matter of a few instructions is kept in one place).
+template <int N>
+__device__ __noinline__ double face_velocity_key(const Model& m, unsigned long long k, int j, int up) {
+    using A = Ar;
+    const int bits = m.key_bits;
+    const long long bias = 1ll << (bits - 1);
+    const unsigned long long mask = (1ull << bits) - 1;
+    auto y = [&](int a) -> double {
+        const int i = (int)((long long)((k >> (bits * (N - 1 - a))) & mask) - bias);
+        const double s = a == j ? __dsub_rn((double)(i + up), 0.5) : (double)i;
+        return __dadd_rn(m.x0[a], __dmul_rn(s, m.h[a]));
+    };
+    if (m.dyn == DYN_CONSTANT) return m.a[j];
+    if (m.dyn == DYN_LINEAR) {
+        double s = 0;
+#pragma unroll 1
+        for (int a = 0; a < N; ++a) s = A::add(s, A::mul(m.a[j * N + a], y(a)));
+        return A::add(s, m.a[N * N + j]);
+    }
+    if (m.dyn == DYN_LORENZ96) {
+        const int jp = j + 1 < N ? j + 1 : j + 1 - N, jm1 = j >= 1 ? j - 1 : j + N - 1, jm2 = j >= 2 ? j - 2 : j + N - 2;
+        return A::add(A::sub(A::mul(A::sub(y(jp % N), y(jm2 % N)), y(jm1 % N)), y(j)), m.a[0]);
+    }
+    if constexpr (N == 3) {
+        const double y0 = y(0), y1 = y(1), y2 = y(2);
+        if (m.dyn == DYN_LORENZ63) {
+            if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
+            if (j == 1) return A::sub(A::mul(y0, A::sub(m.a[1], y2)), y1);
+            return A::sub(A::mul(y0, y1), A::mul(m.a[2], y2));
+        }
+        if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
+        if (j == 1) return A::sub(-y1, A::mul(y0, y2));
+        return A::sub(A::add(A::mul(-m.a[1], y2), A::mul(y0, y1)), A::mul(m.a[1], m.a[2]));
+    }
+    return 0.0;
+}
+
+// New entries of a warp, 2N lanes per entry (on: this lane has one; index c, key
+// k and flags the same in its lanes), one face each: face velocities, outward
+// mask, CFL rate (an FP64 instruction holds a warp scheduler for 64 cycles
+// whatever its active lanes, so one lane with all faces of its entry takes 2N
+// times as long), and with look the links to the neighbours in the table, both
+// ways. All lanes must call it. Returns the entry's rate.
+template <int N, typename T>
+__device__ __noinline__ double complete_group(const Model& m, const Bufs& b, int g, bool on, int c,
+                                              unsigned long long k, unsigned flags, bool look) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int F = 2 * N;
+    const long long cap = m.cap;
+    const int lane = threadIdx.x & 31;
+    const int s = lane / F, e = lane - s * F;
+    double u = 0.0, term = 0.0;
+    if (on) {
+        // the neighbour in direction e: one field of the key up or down, unless
+        // at its end; its first probe is in flight beside the velocity
+        const int shift = m.key_bits * (N - 1 - (e >> 1));
+        const unsigned long long last = (1ull << m.key_bits) - 1, field = (k >> shift) & last;
+        const bool end = field == ((e & 1) ? last : 0ull);
+        const unsigned long long nk = (e & 1) ? k + (1ull << shift) : k - (1ull << shift);
+        ulonglong2 first = make_ulonglong2(EMPTY_KEY, ~0ull);
+        if (look && !end) first = __ldcg(reinterpret_cast<const ulonglong2*>(b.table + table_home(nk, m.tmask)));
+        u = face_velocity_key<N>(m, k, e >> 1, e & 1);
+        if (!(e & 1)) {
+            (static_cast<T*>(b.u[g]) + (e >> 1) * cap)[c] = (T)u;
+            term = div_h(m, abs_bits(u), e >> 1);
+        }
+        if (look) {
+            int nbr = -1;
+            if (first.x == nk) nbr = (int)(long long)first.y;
+            else if (first.x != EMPTY_KEY) nbr = table_find(m, b.table, nk);
+            (b.link[g] + e * cap)[c] = nbr;
+            if (nbr >= 0) (b.link[g] + (e ^ 1) * cap)[nbr] = c;
+        }
+    }
+    // outward: upper face and u > 0, lower face and u < 0
+    const unsigned out = __ballot_sync(full, on && ((e & 1) ? u : -u) > 0.0);
+    double r = 0.0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) r = __dadd_rn(r, __shfl_sync(full, term, (s * F + 2 * j) & 31));
+    if (on && e == 0) {
+        b.om[g][c] = (unsigned short)(flags | ((out >> lane) & ((1u << F) - 1u)));
+        b.rate[g][c] = r;
+    }
+    return r;
+}
+
+// link_body for few new entries: 2N lanes per entry (complete_group). One thread's
+// chain of 2N lookups and FP64 drift evaluations takes about 10 us however few the
+// entries are; this takes 1.6 times the FP64 issue slots of link_body, which
+// counts only when there are many.
+template <int N, typename T>
+__device__ __forceinline__ double link_few_body(const Model& m, const Bufs& b, long long lo, long long hi, int g,
+                                                int nb, int bi) {
+    constexpr int F = 2 * N, G = 32 / F;  // entries per warp
+    const int total = (int)(hi - lo);
+    const int lane = threadIdx.x & 31, s = lane / F;
+    double rmax = 0.0;
+    for (Runs r((total + G - 1) / G, nb, bi); r.next();) {
+        const int q = r.k * G + s;
+        const bool on = s < G && q < total;
+        const int c = on ? (int)lo + q : 0;
+        const unsigned long long k = on ? b.key[g][c] : 0ull;
+        const unsigned f = on ? b.om[g][c] : OM_GHOST;
+        const double rate = complete_group<N, T>(m, b, g, on, c, k, f, true);
+        if (on && !(f & OM_GHOST)) rmax = fmax(rmax, rate);
+    }
+    return rmax;
+}
+
+// Entries [lo, hi) are new: their 2n links by hashtable lookups, the reverse
+// links of the entries below lo (two new entries find one another by their own
+// lookups), velocities, masks and rates. Returns this thread's largest CFL rate
+// among the active ones. One thread per entry, the first probes of N directions
+// in flight together: a probe of a table larger than L2 takes a microsecond, and
+// one per thread left the memory idle. Paper's 6-D case, 3.1e6 entries at init:
+// 1.01 ms (5.7 ms with one thread per (entry, direction), the models selected face
+// by face and single slots hashed); 2.1e6 entries in its first step: 0.78 ms.
 template <int N, typename T>
 __device__ __forceinline__ double link_body(const Model& m, const Bufs& b, long long lo, long long hi, int g, int nb,
                                              int bi) {
-    const unsigned long long* key = b.key[g];
-    int* link = b.link[g];
     const long long cap = m.cap;
-    const long long work = (hi - lo) * 2 * N;
+    const unsigned long long last = (1ull << m.key_bits) - 1;
+    double rmax = 0.0;
+    for (WarpRuns wr(hi - lo, nb, bi); wr.next();) {
+        const long long c = lo + wr.c;
+        const bool on = c < hi;
+        const unsigned long long k = on ? b.key[g][c] : 0ull;
 #pragma unroll 1
-    for (WarpRuns wr(work, nb, bi); wr.next();) {
-        const long long wi = wr.c;
-        if (wi >= work) continue;
-        const long long c = lo + wi / (2 * N);
-        const int dir = (int)(wi % (2 * N));
-        const int j = dir >> 1, s = dir & 1;
-        int I[N];
-        unpack_key<N>(m, key[c], I);
-        I[j] += s ? 1 : -1;
-        unsigned long long k;
-        const int nbr = pack_key<N>(m, I, k) ? table_find(m, b.table, k) : -1;
-        link[(long long)dir * cap + c] = nbr;
-        if (nbr >= 0) link[(long long)(2 * j + (1 - s)) * cap + nbr] = (int)c;
+        for (int up = 0; up < 2; ++up) {
+            unsigned long long nk[N];
+            ulonglong2 first[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                // one field of the key up or down, unless it is at its end
+                const int shift = m.key_bits * (N - 1 - j);
+                const unsigned long long field = (k >> shift) & last;
+                nk[j] = field == (up ? last : 0ull) ? EMPTY_KEY : up ? k + (1ull << shift) : k - (1ull << shift);
+                first[j] = __ldcg(reinterpret_cast<const ulonglong2*>(b.table + table_home(nk[j], m.tmask)));
+            }
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                int nbr = -1;
+                if (on && nk[j] != EMPTY_KEY && first[j].x != EMPTY_KEY)
+                    nbr = first[j].x == nk[j] ? (int)(long long)first[j].y : table_find(m, b.table, nk[j]);
+                if (on) b.link[g][(2 * j + up) * cap + c] = nbr;
+                if (nbr >= 0 && nbr < lo) b.link[g][(2 * j + 1 - up) * cap + nbr] = (int)c;
+            }
+            // the look-ups leave the warp in pieces, and it would stay so through the
+            // FP64 part (four times its instructions)
+            __syncwarp();
+        }
+        if (on) {
+            int I[N];
+            unpack_key<N>(m, k, I);
+            unsigned msk;
+            const double r = entry_velocities<N, T>(m, b, g, c, I, msk);
+            const unsigned short f = b.om[g][c];
+            b.om[g][c] = (unsigned short)(f | msk);
+            if (!(f & OM_GHOST)) rmax = fmax(rmax, r);
+        }
+        __syncwarp();
     }
-    return link_masks<N, T>(m, b, lo, hi, g, nb, bi);
+    return rmax;
 }
 
 // Cooperative variant: W lanes probe W consecutive slots together.
@@ -967,95 +1168,6 @@ struct GrowQueue {
     unsigned char code[GROW_QUEUE];
 };
 
-// f_j at the lower (up = 0) or upper (up = 1) j-face of the cell with packed
-// key k: face_velocity64 with j known at run time, out of line. The step loop's
-// code runs once per step and phase from the instruction caches, so what is not
-// a matter of a few instructions is kept in one place.
-template <int N>
-__device__ __noinline__ double face_velocity_key(const Model& m, unsigned long long k, int j, int up) {
-    using A = Ar<double>;
-    const int bits = m.key_bits;
-    const long long bias = 1ll << (bits - 1);
-    const unsigned long long mask = (1ull << bits) - 1;
-    auto y = [&](int a) -> double {
-        const int i = (int)((long long)((k >> (bits * (N - 1 - a))) & mask) - bias);
-        const double s = a == j ? __dsub_rn((double)(i + up), 0.5) : (double)i;
-        return __dadd_rn(m.x0[a], __dmul_rn(s, m.h[a]));
-    };
-    if (m.dyn == DYN_CONSTANT) return m.a[j];
-    if (m.dyn == DYN_LINEAR) {
-        double s = 0;
-#pragma unroll 1
-        for (int a = 0; a < N; ++a) s = A::add(s, A::mul(m.a[j * N + a], y(a)));
-        return A::add(s, m.a[N * N + j]);
-    }
-    if (m.dyn == DYN_LORENZ96) {
-        const int jp = j + 1 < N ? j + 1 : j + 1 - N, jm1 = j >= 1 ? j - 1 : j + N - 1, jm2 = j >= 2 ? j - 2 : j + N - 2;
-        return A::add(A::sub(A::mul(A::sub(y(jp % N), y(jm2 % N)), y(jm1 % N)), y(j)), m.a[0]);
-    }
-    if constexpr (N == 3) {
-        const double y0 = y(0), y1 = y(1), y2 = y(2);
-        if (m.dyn == DYN_LORENZ63) {
-            if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
-            if (j == 1) return A::sub(A::mul(y0, A::sub(m.a[1], y2)), y1);
-            return A::sub(A::mul(y0, y1), A::mul(m.a[2], y2));
-        }
-        if (j == 0) return A::mul(m.a[0], A::sub(y1, y0));
-        if (j == 1) return A::sub(-y1, A::mul(y0, y2));
-        return A::sub(A::add(A::mul(-m.a[1], y2), A::mul(y0, y1)), A::mul(m.a[1], m.a[2]));
-    }
-    return 0.0;
-}
-
-// New entries of a warp, 2N lanes per entry (on: this lane has one; index c, key
-// k and flags the same in its lanes), one face each: face velocities, outward
-// mask, CFL rate (an FP64 instruction holds a warp scheduler for 64 cycles
-// whatever its active lanes, so one lane with all faces of its entry takes 2N
-// times as long), and with look the links to the neighbours in the table, both
-// ways. All lanes must call it. Returns the entry's rate.
-template <int N, typename T>
-__device__ __noinline__ double complete_group(const Model& m, const Bufs& b, int g, bool on, int c,
-                                              unsigned long long k, unsigned flags, bool look) {
-    constexpr unsigned full = 0xffffffffu;
-    constexpr int F = 2 * N;
-    const long long cap = m.cap;
-    const int lane = threadIdx.x & 31;
-    const int s = lane / F, e = lane - s * F;
-    double u = 0.0, term = 0.0;
-    if (on) {
-        // the neighbour in direction e: one field of the key up or down, unless
-        // at its end; its first probe is in flight beside the velocity
-        const int shift = m.key_bits * (N - 1 - (e >> 1));
-        const unsigned long long last = (1ull << m.key_bits) - 1, field = (k >> shift) & last;
-        const bool end = field == ((e & 1) ? last : 0ull);
-        const unsigned long long nk = (e & 1) ? k + (1ull << shift) : k - (1ull << shift);
-        ulonglong2 first = make_ulonglong2(EMPTY_KEY, ~0ull);
-        if (look && !end) first = __ldcg(reinterpret_cast<const ulonglong2*>(b.table + (mix64(nk) & m.tmask)));
-        u = face_velocity_key<N>(m, k, e >> 1, e & 1);
-        if (!(e & 1)) {
-            (static_cast<T*>(b.u[g]) + (e >> 1) * cap)[c] = (T)u;
-            term = div_h(m, abs_bits(u), e >> 1);
-        }
-        if (look) {
-            int nbr = -1;
-            if (first.x == nk) nbr = (int)(long long)first.y;
-            else if (first.x != EMPTY_KEY) nbr = table_find(m, b.table, nk);
-            (b.link[g] + e * cap)[c] = nbr;
-            if (nbr >= 0) (b.link[g] + (e ^ 1) * cap)[nbr] = c;
-        }
-    }
-    // outward: upper face and u > 0, lower face and u < 0
-    const unsigned out = __ballot_sync(full, on && ((e & 1) ? u : -u) > 0.0);
-    double r = 0.0;
-#pragma unroll
-    for (int j = 0; j < N; ++j) r = __dadd_rn(r, __shfl_sync(full, term, (s * F + 2 * j) & 31));
-    if (on && e == 0) {
-        b.om[g][c] = (unsigned short)(flags | ((out >> lane) & ((1u << F) - 1u)));
-        b.rate[g][c] = r;
-    }
-    return r;
-}
-
 // A warp's grow requests: neighbour `code` of cell cc (made active as
 // grow_candidate does it, with the marks of the step loop, and the inserted
 // cells' velocities formed at once). rate_now: the largest CFL rate known; only a larger one is written (it
@@ -1259,14 +1371,14 @@ __device__ __forceinline__ void grow_drain(const Model& m, const Bufs& b, const 
 // Compare-and-swap at once: most keys asked for here are new.
 __device__ __forceinline__ int table_claim_or_find(const Model& m, Slot* T, unsigned long long key,
                                                    unsigned long long* slot) {
-    unsigned long long h = mix64(key) & m.tmask;
+    unsigned long long h = table_home(key, m.tmask);
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
         const unsigned long long k = atomicCAS(&T[h].key, EMPTY_KEY, key);
         *slot = h;
         if (k == EMPTY_KEY) return 1;
         if (k == key) return 0;
-        h = (h + 1) & m.tmask;
+        h = table_next(h, probe, m.tmask);
     }
     return -1;
 }
