@@ -463,8 +463,7 @@ void launch_list(gbees_ctx* ctx, void* const* f, const int* grids, int nf) {
 // survivors are sorted into the configured storage order (key or Morton order
 // of the cell indices), which keeps the neighbour gathers of a sweep close
 // together; a grid that fits in L2 keeps its order (stream compaction).
-constexpr int kSortPasses = 8;                          // 8-bit digits of the 64-bit sort key
-constexpr int kPruneKernelsSorted = 3 + 1 + 3 * kSortPasses + 1 + 2;
+constexpr int kPruneKernelsSorted = 3 + 1 + 3 * SORT_PASSES + 1 + 2;
 constexpr int kPruneKernelsPlain = 3 + 1 + 1;
 constexpr long long kSortMinEntries = 1ll << 18;        // smaller pools are not sorted
 
@@ -494,10 +493,10 @@ void launch_prune(gbees_ctx* ctx) {
         k_prune_count<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
         if (sorted) {
             k_sort_init<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-            for (int pass = 0; pass < kSortPasses; ++pass) {
-                k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass & 1, 8 * pass);
-                k_sort_scan<<<1, SCAN_THREADS, 0, s>>>(ctx->m, ctx->b, Gs);
-                k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass & 1, 8 * pass);
+            for (int pass = 0; pass < SORT_PASSES; ++pass) {
+                k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass);
+                k_sort_scan<<<256, THREADS, 0, s>>>(ctx->m, ctx->b, Gs, pass);
+                k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass);
             }
             k_sort_map<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_prune_compact_sorted<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
@@ -611,20 +610,17 @@ void graph_nodes(gbees_ctx* ctx, GraphBuilder& gb, cudaGraph_t body, cudaGraphCo
     int nblk = G;
     void* relink_args[] = {m, b, &nblk};
     const int Gs = std::min(G, SORT_BLOCKS);
-    static int srcs[2] = {0, 1};
-    static int shifts[kSortPasses] = {0, 8, 16, 24, 32, 40, 48, 56};
-    static int nsort = 0;
-    nsort = Gs;
+    int nsort = Gs;
     cudaGraphNode_t q = gb.add(pb, nullptr, (void*)k_prune_mark<T>, G, THREADS, mb);
     q = gb.add(pb, q, (void*)k_prune_scatter<N, T>, G, THREADS, mb);
     q = gb.add(pb, q, (void*)k_prune_count<N>, G, THREADS, mb);
     if (sorts(ctx)) {
         q = gb.add(pb, q, (void*)k_sort_init, G, THREADS, mb);
-        for (int pass = 0; pass < kSortPasses; ++pass) {
-            void* pass_args[] = {m, b, &srcs[pass & 1], &shifts[pass]};
-            void* scan_args[] = {m, b, &nsort};
+        for (int pass = 0; pass < SORT_PASSES; ++pass) {
+            void* pass_args[] = {m, b, &pass};
+            void* scan_args[] = {m, b, &nsort, &pass};
             q = gb.add(pb, q, (void*)k_sort_hist, Gs, THREADS, pass_args);
-            q = gb.add(pb, q, (void*)k_sort_scan, 1, SCAN_THREADS, scan_args);
+            q = gb.add(pb, q, (void*)k_sort_scan, 256, THREADS, scan_args);
             q = gb.add(pb, q, (void*)k_sort_scatter, Gs, THREADS, pass_args);
         }
         q = gb.add(pb, q, (void*)k_sort_map, G, THREADS, mb);

@@ -97,7 +97,8 @@ struct alignas(256) DevScalars {
     double step_dt;       // dt of the step being taken
     double step_t_new;    // time after it
     int step_last;        // the step lands on t_target
-    int step_pad;
+    int sort_passes;      // 8-bit digits of the current sort's codes
+    unsigned sort_lo[MAXN], sort_hi[MAXN];  // range of the key fields to sort
     double coef_dth[MAXN];  // dt / h_j
     long long mom[28][NDIG];     // exact sums for moments
     double mom_mean[MAXN];       // mean, input of the covariance pass

@@ -625,6 +625,10 @@ __device__ __forceinline__ bool prune_due(const DevScalars* sc) {
 template <typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_mark(const Model m, Bufs b) {
     if (!prune_due(b.sc)) return;
+    if (blockIdx.x == 0 && threadIdx.x < MAXN) {  // read and added to from the status pass on
+        b.sc->sort_lo[threadIdx.x] = ~0u;
+        b.sc->sort_hi[threadIdx.x] = 0u;
+    }
     prune_mark_body<T>(m, b, view_of(m, b.sc));
 }
 
@@ -641,7 +645,7 @@ __global__ void __launch_bounds__(THREADS) k_prune_scatter(const Model m, Bufs b
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_prune_count(const Model m, Bufs b) {
     if (!prune_due(b.sc)) return;
-    prune_count_body<N>(m, b, view_of(m, b.sc));
+    prune_count_body<N, true>(m, b, view_of(m, b.sc));
 }
 
 // Prune, pass 4: write the survivors into the other buffer set in the order

@@ -166,133 +166,199 @@ __global__ void k_set_count(DevScalars* sc, long long count, long long step0) {
     sc->step = step0;
 }
 
-// ------------------------------------------------------------------ storage order at a prune
+// ------------------------------------------------------------------ sorting
 // The prune of a large grid gives the survivors a new storage order with a
-// stable LSD radix sort of (order key, old index), 8 bits per pass: the
-// lexicographic order of the cell indices (the packed key itself, dimension 0
-// most significant), so that the face neighbours of a warp's consecutive cells
+// stable LSD radix sort of (order code, old index), 8 bits per pass: the
+// lexicographic order of the cell indices (the packed key, dimension 0 most
+// significant), so that the face neighbours of a warp's consecutive cells
 // in any dimension are consecutive too and the neighbour gathers coalesce, or
 // the Morton order of the indices. Scratch: the other generation's key/slot
 // arrays (A) and its link/value arrays (B), free until the compaction writes
 // them.
+// A key's fields are mostly empty (10 bits of index per dimension in six
+// dimensions, of which a grid uses 5 or 6): the code holds each field less its
+// smallest value, in as many bits as the range needs, which sorts alike. 36 bits in
+// place of 60 and five passes in place of eight on the 6-D grids; a pass beyond
+// the code's digits returns at once.
 
 constexpr int SORT_BLOCKS = 1024;  // blocks of the sort kernels at most (histogram rows)
-constexpr int SCAN_THREADS = 1024; // threads of the histogram scan
+constexpr int SORT_PASSES = 8;     // digits of a full code
 
 struct SortBufs {
     unsigned long long* key[2];
     unsigned int* val[2];
 };
 
-__device__ __forceinline__ SortBufs sort_bufs(const Bufs& b, const StepView& v) {
+__device__ __forceinline__ SortBufs sort_bufs(const Bufs& b, int g, int pb) {
     SortBufs s;
-    s.key[0] = b.key[v.g ^ 1];
-    s.key[1] = reinterpret_cast<unsigned long long*>(b.link[v.g ^ 1]);
-    s.val[0] = b.slot[v.g ^ 1];
-    s.val[1] = static_cast<unsigned int*>(b.q[v.pb ^ 1]);
+    s.key[0] = b.key[g ^ 1];
+    s.key[1] = reinterpret_cast<unsigned long long*>(b.link[g ^ 1]);
+    s.val[0] = b.slot[g ^ 1];
+    s.val[1] = static_cast<unsigned int*>(b.q[pb ^ 1]);
     return s;
 }
 
+// The compact code of a key: bits per field from the ranges in the scalars.
+struct KeyCode {
+    unsigned lo[MAXN];
+    int bits[MAXN], total;
+    __device__ __forceinline__ KeyCode(const Model& m, const DevScalars* sc) {
+        total = 0;
+        for (int j = 0; j < m.n; ++j) {
+            lo[j] = sc->sort_lo[j];
+            const unsigned hi = sc->sort_hi[j];
+            bits[j] = hi > lo[j] ? 32 - __clz(hi - lo[j]) : 0;
+            total += bits[j];
+        }
+    }
+    __device__ __forceinline__ unsigned long long operator()(const Model& m, unsigned long long k) const {
+        const unsigned long long mask = (1ull << m.key_bits) - 1;
+        unsigned long long out = 0;
+        for (int j = 0; j < m.n; ++j)
+            out = (out << bits[j]) | (unsigned)(((k >> (m.key_bits * (m.n - 1 - j))) & mask) - lo[j]);
+        return out;
+    }
+};
+
 // keep[c] = status (0 drop, 1 active, 2 halo, from the status pass in map);
-// A = (order key, c): active cells first, then the halo (each in the order of
+// A = (order code, c): active cells first, then the halo (each in the order of
 // the configured code), or both interleaved in key order; dropped entries
 // last (every result is independent of the storage order; only the speed
-// depends on it). A live entry's order key
-// is below 2^63: keys use at most 63 bits, and only an all-ones key has an
-// all-ones Morton code, a key no cell that survives a prune has.
+// depends on it). A survivor's full code is below 2^63: keys use at most 63 bits,
+// and only an all-ones key has an all-ones Morton code, a key no cell that
+// survives a prune has.
 __global__ void __launch_bounds__(THREADS) k_sort_init(const Model m, Bufs b) {
     if (!prune_due(b.sc)) return;
     const StepView v = view_of(m, b.sc);
-    const SortBufs sb = sort_bufs(b, v);
+    const SortBufs sb = sort_bufs(b, v.g, v.pb);
     const unsigned long long* key = b.key[v.g];
     long long c0, c1;
     block_chunk(v.N, c0, c1);
     const int order = m.sort_order;        // GBEES_ORDER_*
     const bool mixed = order == 3;          // halo cells among the active ones
+    const KeyCode code(m, b.sc);
+    const bool compact = (order == 0 || mixed) && code.total <= 62;
+    const int region_bit = compact ? code.total : 63;
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.sc->sort_passes = compact ? (code.total + 2 + 7) / 8 : SORT_PASSES;
     for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
         const int st = b.map[c];
         b.keep[c] = (unsigned char)st;
-        const unsigned long long region = (st == 2 && !mixed) ? (1ull << 63) : 0ull;
-        const unsigned long long code = order == 1   ? morton_code(key[c], m.n, m.key_bits)
-                                        : order == 4 ? row_morton_code(key[c], m.n, m.key_bits)
-                                                     : key[c];
-        sb.key[0][c] = st == 0 ? ~0ull : (region | code);
+        const unsigned long long k = key[c];
+        const unsigned long long x = compact      ? code(m, k)
+                                     : order == 1 ? morton_code(k, m.n, m.key_bits)
+                                     : order == 4 ? row_morton_code(k, m.n, m.key_bits)
+                                                  : k;
+        const unsigned long long region = (st == 2 && !mixed) ? (1ull << region_bit) : 0ull;
+        const unsigned long long drop = compact ? 3ull << region_bit : ~0ull;
+        sb.key[0][c] = st == 0 ? drop : (region | x);
         sb.val[0][c] = (unsigned int)c;
     }
 }
 
+// The entries of a sort: the pool of a due prune. False: nothing to do in this pass.
+__device__ __forceinline__ bool sort_pass(const Model& m, const Bufs& b, int pass, long long& n, SortBufs& sb) {
+    if (!prune_due(b.sc) || pass >= *(volatile int*)&b.sc->sort_passes) return false;
+    n = min(*(volatile long long*)&b.sc->N, m.cap);
+    sb = sort_bufs(b, *(volatile int*)&b.sc->gen, *(volatile int*)&b.sc->pbuf);
+    return true;
+}
+
 // Pass histogram: sorthist[d * nblk + block] = entries of this block's chunk
-// whose digit (key >> shift) & 255 is d.
-__global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, int src, int shift) {
-    if (!prune_due(b.sc)) return;
+// whose digit is d. (One shared atomic per digit that occurs in a warp: the high
+// digits of neighbouring entries are mostly alike.)
+__global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, int pass) {
+    long long n;
+    SortBufs sb;
+    if (!sort_pass(m, b, pass, n, sb)) return;
     __shared__ unsigned int cnt[256];
-    const StepView v = view_of(m, b.sc);
-    const SortBufs sb = sort_bufs(b, v);
+    const unsigned long long* in = sb.key[pass & 1];
     for (int d = threadIdx.x; d < 256; d += blockDim.x) cnt[d] = 0;
     __syncthreads();
     long long c0, c1;
-    block_chunk(v.N, c0, c1);
-    for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x)
-        atomicAdd(&cnt[(unsigned)(sb.key[src][c] >> shift) & 255u], 1u);
+    block_chunk(n, c0, c1);
+    const int lane = threadIdx.x & 31;
+    for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
+        const long long c = t0 + threadIdx.x;
+        const int d = c < c1 ? (int)((in[c] >> (8 * pass)) & 255u) : 256;
+        const unsigned same = __match_any_sync(0xffffffffu, d);
+        if (d < 256 && (same & ((1u << lane) - 1u)) == 0) atomicAdd(&cnt[d], (unsigned)__popc(same));
+    }
     __syncthreads();
     for (int d = threadIdx.x; d < 256; d += blockDim.x) b.sorthist[(long long)d * gridDim.x + blockIdx.x] = cnt[d];
 }
 
-// Exclusive scan of the 256 x nblk histogram in place (one block of
-// SCAN_THREADS threads: each sums a run of counters, a block-wide scan of the
-// run totals, then each writes its run's offsets).
-__global__ void __launch_bounds__(SCAN_THREADS) k_sort_scan(const Model m, Bufs b, int nblk) {
-    if (!prune_due(b.sc)) return;
-    __shared__ unsigned long long s_warp[SCAN_THREADS / 32];
-    unsigned int* hist = b.sorthist;
-    const long long total = 256ll * nblk;
-    const long long per = (total + blockDim.x - 1) / blockDim.x;
-    const long long i0 = min(total, threadIdx.x * per), i1 = min(total, i0 + per);
-    unsigned long long sum = 0;
-    for (long long i = i0; i < i1; ++i) sum += hist[i];
-    // inclusive scan of the run totals: within the warp, then over the warps
+// Exclusive prefixes of the histogram, block d along digit d's row of nblk (at
+// most 4 THREADS) counters, in place; the row's total goes to the reductions'
+// partials (free during a sort). The digits' offsets follow from the totals in the
+// scatter. (256 blocks: 3 us; one block over all rows took 427 us, eight times
+// the rest of the pass.)
+__global__ void __launch_bounds__(THREADS) k_sort_scan(const Model m, Bufs b, int nblk, int pass) {
+    long long n;
+    SortBufs sb;
+    if (!sort_pass(m, b, pass, n, sb)) return;
+    static_assert(SORT_BLOCKS <= 4 * THREADS, "a row has at most four counters per thread");
+    __shared__ unsigned int s_w[WARPS];
+    unsigned int* row = b.sorthist + (long long)blockIdx.x * nblk;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long x = sum;
+    unsigned v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = (int)threadIdx.x * 4 + k;
+        v[k] = i < nblk ? row[i] : 0u;
+        sum += v[k];
+    }
+    unsigned x = sum;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, off);
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, off);
         if (lane >= off) x += y;
     }
-    if (lane == 31) s_warp[wid] = x;
+    if (lane == 31) s_w[wid] = x;
     __syncthreads();
-    if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        unsigned long long w = lane < nw ? s_warp[lane] : 0ull;
+    unsigned before = x - sum, total = 0;
+    for (int w = 0; w < WARPS; ++w) {
+        if (w < wid) before += s_w[w];
+        total += s_w[w];
+    }
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, w, off);
-            if (lane >= off) w += y;
-        }
-        if (lane < nw) s_warp[lane] = w;
+    for (int k = 0; k < 4; ++k) {
+        const int i = (int)threadIdx.x * 4 + k;
+        if (i < nblk) row[i] = before;
+        before += v[k];
     }
-    __syncthreads();
-    unsigned long long run = x - sum + (wid > 0 ? s_warp[wid - 1] : 0ull);
-    for (long long i = i0; i < i1; ++i) {
-        const unsigned int c = hist[i];
-        hist[i] = (unsigned int)run;
-        run += c;
-    }
+    if (threadIdx.x == 0) reinterpret_cast<unsigned int*>(b.part)[blockIdx.x] = total;
 }
 
 // Stable scatter of a pass: every block walks its chunk in tiles of one
 // element per thread; an element's place is its digit's offset for the block,
 // plus the elements of that digit in earlier tiles, earlier warps of the tile
 // and earlier lanes of its warp.
-__global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b, int src, int shift) {
-    if (!prune_due(b.sc)) return;
+__global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b, int pass) {
+    long long n;
+    SortBufs sb;
+    if (!sort_pass(m, b, pass, n, sb)) return;
+    static_assert(THREADS == 256, "one thread per digit");
     __shared__ unsigned int base[256];
     __shared__ unsigned int wcnt[WARPS][256];
-    const StepView v = view_of(m, b.sc);
-    const SortBufs sb = sort_bufs(b, v);
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) base[d] = b.sorthist[(long long)d * gridDim.x + blockIdx.x];
+    __shared__ unsigned int s_w[WARPS];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, src = pass & 1, shift = 8 * pass;
+    {
+        // the digits' offsets: exclusive prefix of the rows' totals
+        const unsigned tot = reinterpret_cast<const unsigned int*>(b.part)[threadIdx.x];
+        unsigned x = tot;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) s_w[wid] = x;
+        __syncthreads();
+        unsigned before = x - tot;
+        for (int w = 0; w < wid; ++w) before += s_w[w];
+        base[threadIdx.x] = before + b.sorthist[(long long)threadIdx.x * gridDim.x + blockIdx.x];
+    }
     long long c0, c1;
-    block_chunk(v.N, c0, c1);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    block_chunk(n, c0, c1);
     for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
         for (int i = threadIdx.x; i < WARPS * 256; i += blockDim.x) (&wcnt[0][0])[i] = 0;
         __syncthreads();
@@ -331,9 +397,10 @@ __global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b,
 __global__ void __launch_bounds__(THREADS) k_sort_map(const Model m, Bufs b) {
     if (!prune_due(b.sc)) return;
     const StepView v = view_of(m, b.sc);
-    const SortBufs sb = sort_bufs(b, v);
+    const SortBufs sb = sort_bufs(b, v.g, v.pb);
+    const unsigned int* val = sb.val[b.sc->sort_passes & 1];
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < v.N; r += (long long)gridDim.x * blockDim.x) {
-        const unsigned int c = sb.val[0][r];
+        const unsigned int c = val[r];
         b.map[c] = b.keep[c] ? (int)r : -1;
     }
 }

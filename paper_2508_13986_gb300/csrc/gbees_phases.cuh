@@ -1689,12 +1689,58 @@ __device__ __forceinline__ long long block_count(int cnt) {
     return t;
 }
 
+// Range of the key fields of the entries a thread has seen, folded into the
+// scalars (for the sort's codes). All threads of the block must call fold.
+template <int N>
+struct FieldRange {
+    unsigned lo[N], hi[N];
+    __device__ __forceinline__ FieldRange() {
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            lo[j] = ~0u;
+            hi[j] = 0u;
+        }
+    }
+    __device__ __forceinline__ void see(const Model& m, unsigned long long k) {
+        const unsigned long long mask = (1ull << m.key_bits) - 1;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const unsigned f = (unsigned)((k >> (m.key_bits * (N - 1 - j))) & mask);
+            lo[j] = min(lo[j], f);
+            hi[j] = max(hi[j], f);
+        }
+    }
+    __device__ __forceinline__ void fold(DevScalars* sc) {
+        __shared__ unsigned s_lo[N], s_hi[N];
+        if (threadIdx.x < N) {
+            s_lo[threadIdx.x] = ~0u;
+            s_hi[threadIdx.x] = 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const unsigned l = __reduce_min_sync(0xffffffffu, lo[j]), h = __reduce_max_sync(0xffffffffu, hi[j]);
+            if ((threadIdx.x & 31) == 0 && l <= h) {
+                atomicMin(&s_lo[j], l);
+                atomicMax(&s_hi[j], h);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < N && s_lo[threadIdx.x] <= s_hi[threadIdx.x]) {
+            atomicMin(&sc->sort_lo[threadIdx.x], s_lo[threadIdx.x]);
+            atomicMax(&sc->sort_hi[threadIdx.x], s_hi[threadIdx.x]);
+        }
+    }
+};
+
 // Status of every entry into map: 1 active and kept, 2 halo of a kept cell
 // (not kept, with a kept face neighbour), 0 dropped. The block's counts of
 // both go to blk and blk2; the table slots of the current entries are emptied
-// for the rehash (the table holds nothing else).
-template <int N>
+// for the rehash (the table holds nothing else). RANGE: the range of the
+// survivors' key fields too.
+template <int N, bool RANGE = false>
 __device__ __forceinline__ void prune_count_body(const Model& m, const Bufs& b, const StepView& v) {
+    FieldRange<N> range;
     const int* link = b.link[v.g];
     const unsigned short* om = b.om[v.g];
     const long long cap = m.cap;
@@ -1716,7 +1762,9 @@ __device__ __forceinline__ void prune_count_body(const Model& m, const Bufs& b, 
         b.map[c] = st;
         na += st == 1;
         ng += st == 2;
+        if (RANGE && st) range.see(m, b.key[v.g][c]);
     }
+    if (RANGE) range.fold(b.sc);
     const long long ta = block_count(na);
     const long long tg = block_count(ng);
     if (threadIdx.x == 0) {
