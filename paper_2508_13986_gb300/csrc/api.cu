@@ -7,7 +7,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <numeric>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -494,9 +493,9 @@ void launch_prune(gbees_ctx* ctx) {
         if (sorted) {
             k_sort_init<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             for (int pass = 0; pass < SORT_PASSES; ++pass) {
-                k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass);
-                k_sort_scan<<<256, THREADS, 0, s>>>(ctx->m, ctx->b, Gs, pass);
-                k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass);
+                k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, -1);
+                k_sort_scan<<<256, THREADS, 0, s>>>(ctx->m, ctx->b, Gs, pass, -1);
+                k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, -1);
             }
             k_sort_map<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_prune_compact_sorted<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
@@ -518,6 +517,44 @@ void launch_readout(gbees_ctx* ctx, int* d_idx, double* d_p) {
         using T = decltype(TT);
         k_readout<NC, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, d_idx, d_p);
     });
+}
+
+// The same in lexicographic order of the cell indices; the number of kernels
+// launched, or -1 on an error (recorded). The host's copy of the scalars is current
+// (every call ends with it).
+int launch_readout_sorted(gbees_ctx* ctx, int* d_idx, double* d_p) {
+    const int G = ctx->grid;
+    const long long N = ctx->hs.N, NA = ctx->hs.NA;
+    cudaStream_t s = ctx->stream;
+    if (N <= RANK_MAX) {
+        const int Gr = (int)((N * RANK_LANES + THREADS - 1) / THREADS);
+        with_nt(ctx, [&](auto NN, auto TT) {
+            k_readout_rank<decltype(NN)::value, decltype(TT)><<<Gr, THREADS, 0, s>>>(ctx->m, ctx->b, d_idx, d_p);
+        });
+        return 1;
+    }
+    DevScalars* sc = ctx->b.sc;
+    if (!cuda_ok(ctx, cudaMemsetAsync(sc->sort_lo, 0xff, sizeof sc->sort_lo, s), "read_cells") ||
+        !cuda_ok(ctx, cudaMemsetAsync(sc->sort_hi, 0, sizeof sc->sort_hi, s), "read_cells"))
+        return -1;
+    with_nt(ctx, [&](auto NN, auto) { k_readout_range<decltype(NN)::value><<<G, THREADS, 0, s>>>(ctx->m, ctx->b); });
+    k_readout_count<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+    k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap);
+    k_readout_keys<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+    if (!sync_scalars(ctx, "read_cells")) return -1;
+    int bits = 0;
+    for (int j = 0; j < ctx->cfg.n; ++j)
+        for (unsigned r = ctx->hs.sort_hi[j] - ctx->hs.sort_lo[j]; r; r >>= 1) ++bits;
+    const int passes = (bits + 7) / 8, Gs = sort_blocks(NA);
+    for (int pass = 0; pass < passes; ++pass) {
+        k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, NA);
+        k_sort_scan<<<256, THREADS, 0, s>>>(ctx->m, ctx->b, Gs, pass, NA);
+        k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, NA);
+    }
+    with_nt(ctx, [&](auto NN, auto TT) {
+        k_readout_order<decltype(NN)::value, decltype(TT)><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, passes, NA, d_idx, d_p);
+    });
+    return 5 + 3 * passes;
 }
 
 // One time step: grow, halo, link the new entries, flux update (the last block of the
@@ -617,8 +654,9 @@ void graph_nodes(gbees_ctx* ctx, GraphBuilder& gb, cudaGraph_t body, cudaGraphCo
     if (sorts(ctx)) {
         q = gb.add(pb, q, (void*)k_sort_init, G, THREADS, mb);
         for (int pass = 0; pass < SORT_PASSES; ++pass) {
-            void* pass_args[] = {m, b, &pass};
-            void* scan_args[] = {m, b, &nsort, &pass};
+            long long pool = -1;
+            void* pass_args[] = {m, b, &pass, &pool};
+            void* scan_args[] = {m, b, &nsort, &pass, &pool};
             q = gb.add(pb, q, (void*)k_sort_hist, Gs, THREADS, pass_args);
             q = gb.add(pb, q, (void*)k_sort_scan, 256, THREADS, scan_args);
             q = gb.add(pb, q, (void*)k_sort_scatter, Gs, THREADS, pass_args);
@@ -1306,11 +1344,11 @@ int gbees_correct_gaussian(gbees_ctx* ctx, const double* y, const double* R, con
     return GBEES_OK;
 }
 
+// (The host's copy of the scalars is current: every call ends with it.)
 int gbees_count(gbees_ctx* ctx, int64_t* n_cells) {
     int st = guard(ctx, true);
     if (st) return st;
     if (!n_cells) return GBEES_EINVAL;
-    if (!sync_scalars(ctx, "count")) return ctx->status;
     *n_cells = ctx->hs.NA;
     return GBEES_OK;
 }
@@ -1318,7 +1356,6 @@ int gbees_count(gbees_ctx* ctx, int64_t* n_cells) {
 int gbees_get_stats(gbees_ctx* ctx, gbees_stats* stats) {
     int st = guard(ctx, true);
     if (st) return st;
-    if (!sync_scalars(ctx, "get_stats")) return ctx->status;
     fill_stats(ctx, stats);
     return GBEES_OK;
 }
@@ -1326,39 +1363,35 @@ int gbees_get_stats(gbees_ctx* ctx, gbees_stats* stats) {
 int gbees_read_cells(gbees_ctx* ctx, int32_t* idx, double* p, int64_t cap, int64_t* n_cells, int32_t sorted) {
     int st = guard(ctx, true);
     if (st) return st;
-    if (!sync_scalars(ctx, "read_cells")) return ctx->status;
-    const long long N = ctx->hs.NA;
+    const long long N = ctx->hs.NA;  // (current: every call ends with the scalars read back)
     if (n_cells) *n_cells = N;
     if (N == 0) return GBEES_OK;
     if ((!idx || !p) && cap > 0) return GBEES_EINVAL;
     const int n = ctx->cfg.n;
     const int g = ctx->hs.gen;
-    int* d_idx = ctx->b.link[g ^ 1];
-    double* d_p = reinterpret_cast<double*>(ctx->b.key[g ^ 1]);
+    // results in the other generation's arrays, free outside a prune; a sort uses others of them
+    int* d_idx = sorted ? (int*)ctx->b.u[g ^ 1] : ctx->b.link[g ^ 1];
+    double* d_p = sorted ? ctx->b.rate[g ^ 1] : reinterpret_cast<double*>(ctx->b.key[g ^ 1]);
     cudaStream_t s = ctx->stream;
     {
         Phase ph(ctx, GBEES_PHASE_OTHER, 3);
-        launch_readout(ctx, d_idx, d_p);
-    }
-    std::vector<int32_t> hidx((size_t)N * n);
-    std::vector<double> hp((size_t)N);
-    if (!cuda_ok(ctx, cudaMemcpyAsync(hidx.data(), d_idx, sizeof(int32_t) * n * N, cudaMemcpyDeviceToHost, s), "read_cells"))
-        return ctx->status;
-    if (!cuda_ok(ctx, cudaMemcpyAsync(hp.data(), d_p, sizeof(double) * N, cudaMemcpyDeviceToHost, s), "read_cells"))
-        return ctx->status;
-    if (!cuda_ok(ctx, cudaStreamSynchronize(s), "read_cells")) return ctx->status;
-    std::vector<long long> order((size_t)N);
-    std::iota(order.begin(), order.end(), 0ll);
-    if (sorted) {
-        std::sort(order.begin(), order.end(), [&](long long a, long long c) {
-            return std::lexicographical_compare(&hidx[a * n], &hidx[a * n] + n, &hidx[c * n], &hidx[c * n] + n);
-        });
+        if (sorted) {
+            ph.kernels = launch_readout_sorted(ctx, d_idx, d_p);
+            if (ph.kernels < 0) {
+                ph.kernels = 0;
+                return ctx->status;
+            }
+        } else {
+            launch_readout(ctx, d_idx, d_p);
+        }
     }
     const long long w = std::min<long long>(N, cap);
-    for (long long r = 0; r < w; ++r) {
-        std::memcpy(idx + r * n, &hidx[order[r] * n], sizeof(int32_t) * n);
-        p[r] = hp[order[r]];
-    }
+    if (w > 0 &&
+        (!cuda_ok(ctx, cudaMemcpyAsync(idx, d_idx, sizeof(int32_t) * n * w, cudaMemcpyDeviceToHost, s), "read_cells") ||
+         !cuda_ok(ctx, cudaMemcpyAsync(p, d_p, sizeof(double) * w, cudaMemcpyDeviceToHost, s), "read_cells")))
+        return ctx->status;
+    if (!cuda_ok(ctx, cudaStreamSynchronize(s), "read_cells") || !cuda_ok(ctx, cudaGetLastError(), "read_cells"))
+        return ctx->status;
     return N > cap ? GBEES_EINVAL : GBEES_OK;
 }
 

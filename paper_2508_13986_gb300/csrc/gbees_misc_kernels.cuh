@@ -255,10 +255,15 @@ __global__ void __launch_bounds__(THREADS) k_sort_init(const Model m, Bufs b) {
     }
 }
 
-// The entries of a sort: the pool of a due prune. False: nothing to do in this pass.
-__device__ __forceinline__ bool sort_pass(const Model& m, const Bufs& b, int pass, long long& n, SortBufs& sb) {
-    if (!prune_due(b.sc) || pass >= *(volatile int*)&b.sc->sort_passes) return false;
-    n = min(*(volatile long long*)&b.sc->N, m.cap);
+// The entries of a sort: count of them, or (count < 0) the pool of a due prune.
+// False: nothing to do in this pass.
+__device__ __forceinline__ bool sort_pass(const Model& m, const Bufs& b, int pass, long long count, long long& n,
+                                          SortBufs& sb) {
+    if (count < 0) {
+        if (!prune_due(b.sc) || pass >= *(volatile int*)&b.sc->sort_passes) return false;
+        count = min(*(volatile long long*)&b.sc->N, m.cap);
+    }
+    n = count;
     sb = sort_bufs(b, *(volatile int*)&b.sc->gen, *(volatile int*)&b.sc->pbuf);
     return true;
 }
@@ -266,10 +271,10 @@ __device__ __forceinline__ bool sort_pass(const Model& m, const Bufs& b, int pas
 // Pass histogram: sorthist[d * nblk + block] = entries of this block's chunk
 // whose digit is d. (One shared atomic per digit that occurs in a warp: the high
 // digits of neighbouring entries are mostly alike.)
-__global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, int pass) {
+__global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, int pass, long long count) {
     long long n;
     SortBufs sb;
-    if (!sort_pass(m, b, pass, n, sb)) return;
+    if (!sort_pass(m, b, pass, count, n, sb)) return;
     __shared__ unsigned int cnt[256];
     const unsigned long long* in = sb.key[pass & 1];
     for (int d = threadIdx.x; d < 256; d += blockDim.x) cnt[d] = 0;
@@ -292,10 +297,11 @@ __global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, in
 // partials (free during a sort). The digits' offsets follow from the totals in the
 // scatter. (256 blocks: 3 us; one block over all rows took 427 us, eight times
 // the rest of the pass.)
-__global__ void __launch_bounds__(THREADS) k_sort_scan(const Model m, Bufs b, int nblk, int pass) {
+__global__ void __launch_bounds__(THREADS) k_sort_scan(const Model m, Bufs b, int nblk, int pass,
+                                                       long long count) {
     long long n;
     SortBufs sb;
-    if (!sort_pass(m, b, pass, n, sb)) return;
+    if (!sort_pass(m, b, pass, count, n, sb)) return;
     static_assert(SORT_BLOCKS <= 4 * THREADS, "a row has at most four counters per thread");
     __shared__ unsigned int s_w[WARPS];
     unsigned int* row = b.sorthist + (long long)blockIdx.x * nblk;
@@ -333,10 +339,10 @@ __global__ void __launch_bounds__(THREADS) k_sort_scan(const Model m, Bufs b, in
 // element per thread; an element's place is its digit's offset for the block,
 // plus the elements of that digit in earlier tiles, earlier warps of the tile
 // and earlier lanes of its warp.
-__global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b, int pass) {
+__global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b, int pass, long long count) {
     long long n;
     SortBufs sb;
-    if (!sort_pass(m, b, pass, n, sb)) return;
+    if (!sort_pass(m, b, pass, count, n, sb)) return;
     static_assert(THREADS == 256, "one thread per digit");
     __shared__ unsigned int base[256];
     __shared__ unsigned int wcnt[WARPS][256];
@@ -416,6 +422,106 @@ __global__ void __launch_bounds__(THREADS) k_readout_count(const Model m, Bufs b
     for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x) cnt += !is_halo(om, c);
     const long long t = block_count(cnt);
     if (threadIdx.x == 0) b.blk[blockIdx.x] = t;
+}
+
+// ------------------------------------------------------------------ sorted read-out
+// The active cells in lexicographic order of their indices, on the device: a sort
+// on the host of the cells of one grid took longer than all the rest of a small
+// grid's read-out (5 * 10^3 cells: 0.5 ms, 5.5 * 10^4: 1.5 ms).
+
+// A pool of up to RANK_MAX entries: each active cell's place is the number of
+// active cells with smaller keys, counted by RANK_LANES lanes per cell against all
+// keys, staged through shared memory (no passes and no other launch; 27 us at
+// 1.6 * 10^4 entries, where the sort's launches take about 60).
+constexpr long long RANK_MAX = 1ll << 14;
+constexpr int RANK_LANES = 8;
+template <int N, typename T>
+__global__ void __launch_bounds__(THREADS) k_readout_rank(const Model m, Bufs b, int* __restrict__ idx,
+                                                          double* __restrict__ p) {
+    constexpr int TILE = 1024;
+    __shared__ unsigned long long s_key[TILE];
+    DevScalars* sc = b.sc;
+    const int ncell = (int)min(*(volatile long long*)&sc->N, m.cap);
+    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const unsigned short* om = b.om[g];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = t / RANK_LANES, sub = t % RANK_LANES;
+    const bool on = c < ncell && !is_halo(om, c);
+    const unsigned long long k = on ? b.key[g][c] : 0ull;
+    int rank = 0;
+    for (int t0 = 0; t0 < ncell; t0 += TILE) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < TILE; i += blockDim.x) {
+            const int e = t0 + i;
+            s_key[i] = e < ncell && !is_halo(om, e) ? b.key[g][e] : ~0ull;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int i = sub; i < TILE; i += RANK_LANES) rank += s_key[i] < k;
+    }
+#pragma unroll
+    for (int off = RANK_LANES / 2; off > 0; off >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
+    if (on && sub == 0) {
+        int I[N];
+        unpack_key<N>(m, k, I);
+#pragma unroll
+        for (int j = 0; j < N; ++j) idx[(long long)rank * N + j] = I[j];
+        p[rank] = __ddiv_rn((double)static_cast<const T*>(b.q[pb])[c], *(volatile double*)&sc->w);
+    }
+}
+
+// A larger pool: the ranges of the active cells' key fields (beside the counts),
+// then (code, entry) of every active cell for the sort, and the read-out in the
+// sorted order.
+template <int N>
+__global__ void __launch_bounds__(THREADS) k_readout_range(const Model m, Bufs b) {
+    DevScalars* sc = b.sc;
+    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
+    const int g = *(volatile int*)&sc->gen;
+    FieldRange<N> range;
+    for (WarpRuns r(ncell); r.next();)
+        if (r.c < ncell && !is_halo(b.om[g], r.c)) range.see(m, b.key[g][r.c]);
+    range.fold(sc);
+}
+
+__global__ void __launch_bounds__(THREADS) k_readout_keys(const Model m, Bufs b) {
+    DevScalars* sc = b.sc;
+    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
+    const int g = *(volatile int*)&sc->gen;
+    const SortBufs sb = sort_bufs(b, g, *(volatile int*)&sc->pbuf);
+    const KeyCode code(m, sc);
+    long long c0, c1;
+    block_chunk(ncell, c0, c1);
+    long long base = b.blk[blockIdx.x];
+    for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
+        const long long c = t0 + threadIdx.x;
+        const int f = c < c1 && !is_halo(b.om[g], c);
+        int total;
+        const int pos = block_exclusive_scan(f, total);
+        if (f) {
+            sb.key[0][base + pos] = code(m, b.key[g][c]);
+            sb.val[0][base + pos] = (unsigned)c;
+        }
+        base += total;
+    }
+}
+
+template <int N, typename T>
+__global__ void __launch_bounds__(THREADS) k_readout_order(const Model m, Bufs b, int passes, long long count,
+                                                           int* __restrict__ idx, double* __restrict__ p) {
+    DevScalars* sc = b.sc;
+    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const unsigned int* val = sort_bufs(b, g, pb).val[passes & 1];
+    const double w = *(volatile double*)&sc->w;
+    for (WarpRuns r(count); r.next();) {
+        if (r.c >= count) continue;
+        const unsigned c = val[r.c];
+        int I[N];
+        unpack_key<N>(m, b.key[g][c], I);
+#pragma unroll
+        for (int j = 0; j < N; ++j) idx[r.c * N + j] = I[j];
+        p[r.c] = __ddiv_rn((double)static_cast<const T*>(b.q[pb])[c], w);
+    }
 }
 
 // Zero the exact accumulators of the moments.
