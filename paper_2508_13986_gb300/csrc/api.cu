@@ -405,11 +405,19 @@ void* link_kernel(int probe_width) {
     }
 }
 
-// step != 0: the link of a time step (its last block also fixes dt).
+// Blocks for work over that many items of 256 threads each, at most G: a small
+// grid's kernels take longer to start and to elect their last block on the whole
+// GPU than to do their work.
+int blocks_for(long long items, int G) {
+    return (int)std::max(1ll, std::min<long long>(G, (items + THREADS - 1) / THREADS));
+}
+
+// step > 0: the link of a time step (its last block also fixes dt); else of a new
+// grid (its last block ends it) of at most `entries` entries.
 template <int N, typename T>
-void launch_link(gbees_ctx* ctx, int step) {
+void launch_link(gbees_ctx* ctx, int step, long long entries = 1ll << 40) {
     void* args[] = {&ctx->m, &ctx->b, &step};
-    const int G = ctx->link_grid > 0 ? ctx->link_grid : ctx->grid;
+    const int G = blocks_for(entries * 2 * N, ctx->link_grid > 0 ? ctx->link_grid : ctx->grid);
     cudaLaunchKernel(link_kernel<N, T>(ctx->m.probe_width), dim3(G), dim3(ctx->step_threads), args, 0, ctx->stream);
 }
 
@@ -476,12 +484,12 @@ int sort_blocks(long long N) {
 }
 
 void launch_prune(gbees_ctx* ctx) {
-    const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
     // the host's copy of the pool size (possibly a few steps old: it only
     // decides the storage order, which no result depends on)
     const long long N = ctx->hs.N;
     const bool sorted = sorts(ctx) && N > kSortMinEntries;
+    const int G = blocks_for(N, ctx->grid);
     const int Gs = sort_blocks(N);
     Phase ph(ctx, GBEES_PHASE_PRUNE, sorted ? kPruneKernelsSorted : kPruneKernelsPlain);
     with_nt(ctx, [&](auto NN, auto TT) {
@@ -508,10 +516,10 @@ void launch_prune(gbees_ctx* ctx) {
 
 // The active cells (indices, densities) into d_idx / d_p in storage order.
 void launch_readout(gbees_ctx* ctx, int* d_idx, double* d_p) {
-    const int G = ctx->grid;
+    const int G = blocks_for(ctx->hs.N, ctx->grid);
     cudaStream_t s = ctx->stream;
     k_readout_count<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-    k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap);
+    k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap, 0);
     with_nt(ctx, [&](auto NN, auto TT) {
         constexpr int NC = decltype(NN)::value;
         using T = decltype(TT);
@@ -523,7 +531,7 @@ void launch_readout(gbees_ctx* ctx, int* d_idx, double* d_p) {
 // launched, or -1 on an error (recorded). The host's copy of the scalars is current
 // (every call ends with it).
 int launch_readout_sorted(gbees_ctx* ctx, int* d_idx, double* d_p) {
-    const int G = ctx->grid;
+    const int G = blocks_for(ctx->hs.N, ctx->grid);
     const long long N = ctx->hs.N, NA = ctx->hs.NA;
     cudaStream_t s = ctx->stream;
     if (N <= RANK_MAX) {
@@ -539,7 +547,7 @@ int launch_readout_sorted(gbees_ctx* ctx, int* d_idx, double* d_p) {
         return -1;
     with_nt(ctx, [&](auto NN, auto) { k_readout_range<decltype(NN)::value><<<G, THREADS, 0, s>>>(ctx->m, ctx->b); });
     k_readout_count<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-    k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap);
+    k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, G, ctx->m.cap, 0);
     k_readout_keys<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
     if (!sync_scalars(ctx, "read_cells")) return -1;
     int bits = 0;
@@ -896,21 +904,33 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
     }
     const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
+    resolve_update_kernels(ctx);
     {
-        Phase ph(ctx, GBEES_PHASE_OTHER, 3);
-        k_reset<<<1, 1, 0, s>>>(ctx->b.sc, t0);
-        k_table_clear<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-        with_nt(ctx, [&](auto NN, auto) {
-            constexpr int N = decltype(NN)::value;
-            k_init_max<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
-        });
+        Phase ph(ctx, GBEES_PHASE_OTHER, 1);
+        k_new_grid<<<blocks_for((long long)ctx->m.tmask + 1, G), THREADS, 0, s>>>(ctx->m, ctx->b, t0, 0, 0);
     }
-    if (!sync_scalars(ctx, "init_gaussian")) return ctx->status;
-    unsigned long long ordk = ctx->hs.tmp_ord;
-    double gmax = 0.0;
-    if (ordk) {
-        unsigned long long bits = (ordk >> 63) ? (ordk & 0x7FFFFFFFFFFFFFFFull) : ~ordk;
-        std::memcpy(&gmax, &bits, 8);
+    // the largest density: that of cell 0 when its centre is the mean (exactly 1, and
+    // none is larger where the quadratic form is a sum of squares), else from a sweep
+    // of the box
+    bool centred = true;
+    for (int k = 0; k < n; ++k) centred = centred && mean[k] == ctx->cfg.x0[k];
+    for (int k = 0; k < n * n; ++k)
+        if (k / n != k % n && ((bx.nonzero >> k) & 1ull)) centred = false;
+    double gmax = centred ? 1.0 : 0.0;
+    if (!centred) {
+        {
+            Phase ph(ctx, GBEES_PHASE_OTHER, 1);
+            with_nt(ctx, [&](auto NN, auto) {
+                constexpr int N = decltype(NN)::value;
+                k_init_max<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
+            });
+        }
+        if (!sync_scalars(ctx, "init_gaussian")) return ctx->status;
+        const unsigned long long ordk = ctx->hs.tmp_ord;
+        if (ordk) {
+            unsigned long long bits = (ordk >> 63) ? (ordk & 0x7FFFFFFFFFFFFFFFull) : ~ordk;
+            std::memcpy(&gmax, &bits, 8);
+        }
     }
     if (!(gmax > 0.0)) {
         set_err(ctx, GBEES_EDEGENERATE, "initial density underflows on the grid");
@@ -923,26 +943,20 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         return GBEES_EINVAL;
     }
     {
-        Phase ph(ctx, GBEES_PHASE_OTHER, 7);
+        Phase ph(ctx, GBEES_PHASE_OTHER, 5);
         // the set's rows lie in the middle of the box: smaller chunks than one per
         // resident block even out a large one
         const long long rows = bx.total / bx.dims[n - 1];
-        const int Gi = (int)std::max<long long>(G, std::min<long long>(std::min(8 * G, GRID_MAX), rows / 256));
+        const int Gi = (int)std::max<long long>(blocks_for(bx.total, G), std::min<long long>(std::min(8 * G, GRID_MAX), rows / 256));
         with_nt(ctx, [&](auto NN, auto TT) {
             constexpr int N = decltype(NN)::value;
             using T = decltype(TT);
             k_init_count<N><<<Gi, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
-            k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, Gi, ctx->m.cap);
+            k_scan_blocks<<<1, THREADS, 0, s>>>(ctx->b, Gi, ctx->m.cap, 1);
             k_init_write<N, T><<<Gi, THREADS, 0, s>>>(ctx->m, ctx->b, bx);
+            k_halo<N, T, 0><<<blocks_for(bx.total * 2 * N, std::min(2 * G, GRID_MAX)), THREADS, 0, s>>>(ctx->m, ctx->b);
+            launch_link<N, T>(ctx, 0, bx.total);
         });
-        k_set_count_from_new<<<1, 1, 0, s>>>(ctx->b.sc);
-        with_nt(ctx, [&](auto NN, auto TT) {
-            constexpr int N = decltype(NN)::value;
-            using T = decltype(TT);
-            k_halo<N, T, 0><<<std::min(2 * G, GRID_MAX), THREADS, 0, s>>>(ctx->m, ctx->b);
-            launch_link<N, T>(ctx, 0);
-        });
-        k_finalise<<<1, 1, 0, s>>>(ctx->m, ctx->b.sc, 0);
     }
     if (!sync_scalars(ctx, "init_gaussian")) return ctx->status;
     ctx->has_grid = true;
@@ -965,9 +979,9 @@ int gbees_init_cells(gbees_ctx* ctx, const int32_t* idx, const double* p, int64_
     }
     cudaStream_t s = ctx->stream;
     const int G = ctx->grid;
-    Phase ph(ctx, GBEES_PHASE_OTHER, N > 0 ? 7 : 6);
-    k_reset<<<1, 1, 0, s>>>(ctx->b.sc, t0);
-    k_table_clear<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+    Phase ph(ctx, GBEES_PHASE_OTHER, N > 0 ? 4 : 3);
+    resolve_update_kernels(ctx);
+    k_new_grid<<<blocks_for((long long)ctx->m.tmask + 1, G), THREADS, 0, s>>>(ctx->m, ctx->b, t0, N, step0);
     // stage the inputs in the second buffer set (unused outside a prune)
     int* d_idx = ctx->b.link[1];
     double* d_p = reinterpret_cast<double*>(ctx->b.key[1]);
@@ -980,16 +994,10 @@ int gbees_init_cells(gbees_ctx* ctx, const int32_t* idx, const double* p, int64_
     with_nt(ctx, [&](auto NN, auto TT) {
         constexpr int NC = decltype(NN)::value;
         using T = decltype(TT);
-        if (N > 0) k_init_cells<NC, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, d_idx, d_p, N);
+        if (N > 0) k_init_cells<NC, T><<<blocks_for(N, G), THREADS, 0, s>>>(ctx->m, ctx->b, d_idx, d_p, N);
+        k_halo<NC, T, 0><<<blocks_for(N * 2 * NC, std::min(2 * G, GRID_MAX)), THREADS, 0, s>>>(ctx->m, ctx->b);
+        launch_link<NC, T>(ctx, -1, N * (2 * NC + 1));
     });
-    k_set_count<<<1, 1, 0, s>>>(ctx->b.sc, N, step0);
-    with_nt(ctx, [&](auto NN, auto TT) {
-        constexpr int NC = decltype(NN)::value;
-        using T = decltype(TT);
-        k_halo<NC, T, 0><<<std::min(2 * G, GRID_MAX), THREADS, 0, s>>>(ctx->m, ctx->b);
-        launch_link<NC, T>(ctx, 0);
-    });
-    k_finalise<<<1, 1, 0, s>>>(ctx->m, ctx->b.sc, 2);
     if (!sync_scalars(ctx, "init_cells")) return ctx->status;
     ctx->has_grid = true;
     return GBEES_OK;
@@ -1015,11 +1023,19 @@ int gbees_propagate(gbees_ctx* ctx, double t_end, gbees_stats* stats) {
         return GBEES_EINVAL;
     }
     cudaStream_t s = ctx->stream;
+    // what k_begin does, on the host's copy of the scalars (current after every call)
+    ctx->hs.t_target = t_end;
+    ctx->hs.done = !(ctx->hs.t < t_end);
+    ctx->hs.steps_call = 0;
+    ctx->hs.updates_call = 0;
+    if (ctx->hs.done) {
+        fill_stats(ctx, stats);
+        return GBEES_OK;
+    }
     {
         Phase ph(ctx, GBEES_PHASE_OTHER, 1);
         k_begin<<<1, 1, 0, s>>>(ctx->b.sc, t_end);
     }
-    if (!sync_scalars(ctx, "propagate")) return ctx->status;
     // Persistent path: one cooperative launch runs up to kPersistSteps steps
     // with grid barriers between the phases (small grids).
     resolve_update_kernels(ctx);
@@ -1044,8 +1060,9 @@ int gbees_propagate(gbees_ctx* ctx, double t_end, gbees_stats* stats) {
             void* args[] = {&ctx->m, &ctx->b, &max_steps, &max_pool};
             cudaEventRecord(ctx->pev[0], s);
             const int pg = ctx->persist_blocks > 0 ? std::min(ctx->persist_blocks, ctx->persist_grid) : ctx->persist_grid;
-            // the kernel's barriers count arrivals from zero
-            if (!cuda_ok(ctx, cudaMemsetAsync(&ctx->b.sc->bar_seq, 0, sizeof(unsigned long long), s), "propagate"))
+            // the kernel's barriers count arrivals from zero (k_begin cleared the counter)
+            if (before > 0 &&
+                !cuda_ok(ctx, cudaMemsetAsync(&ctx->b.sc->bar_seq, 0, sizeof(unsigned long long), s), "propagate"))
                 return ctx->status;
             if (!cuda_ok(ctx, cudaLaunchCooperativeKernel(ctx->kern.persist, dim3(pg), dim3(PERSIST_THREADS), args, 0, s),
                          "propagate"))
@@ -1329,7 +1346,7 @@ int gbees_correct_gaussian(gbees_ctx* ctx, const double* y, const double* R, con
     }
     for (int k = 0; k < m * m; ++k)
         if (ms.Rinv[k] != 0.0) ms.nonzero |= 1ull << k;
-    const int G = ctx->grid;
+    const int G = blocks_for(ctx->hs.N, ctx->grid);
     cudaStream_t s = ctx->stream;
     {
         Phase ph(ctx, GBEES_PHASE_CORRECT, 1);
@@ -1400,24 +1417,16 @@ int gbees_moments(gbees_ctx* ctx, double* mean, double* cov) {
     if (st) return st;
     if (!mean || !cov) return GBEES_EINVAL;
     const int n = ctx->cfg.n;
-    const int G = ctx->grid;
+    const int G = blocks_for(ctx->hs.N, ctx->grid);
     cudaStream_t s = ctx->stream;
-    DevScalars* sc = ctx->b.sc;
-    Phase ph(ctx, GBEES_PHASE_OTHER, 6);
-    k_moments_clear<<<1, THREADS, 0, s>>>(sc);
+    Phase ph(ctx, GBEES_PHASE_OTHER, 2);
     with_nt(ctx, [&](auto NN, auto TT) {
         constexpr int NC = decltype(NN)::value;
         using T = decltype(TT);
-        k_moments<NC, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, 0, sc->mom_mean);
+        constexpr int rows = (mom_slots<NC, 1>() + MOM_SUMS - 1) / MOM_SUMS;
+        k_moments<NC, T, 0><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+        k_moments<NC, T, 1><<<dim3(G, rows), THREADS, 0, s>>>(ctx->m, ctx->b);
     });
-    k_moments_final<<<1, 32, 0, s>>>(ctx->m, sc, sc->mom_mean, n);
-    k_moments_clear<<<1, THREADS, 0, s>>>(sc);
-    with_nt(ctx, [&](auto NN, auto TT) {
-        constexpr int NC = decltype(NN)::value;
-        using T = decltype(TT);
-        k_moments<NC, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, 1, sc->mom_mean);
-    });
-    k_moments_final<<<1, 32, 0, s>>>(ctx->m, sc, sc->mom_out, n * (n + 1) / 2);
     if (!sync_scalars(ctx, "moments")) return ctx->status;
     for (int a = 0; a < n; ++a) mean[a] = ctx->hs.mom_mean[a];
     int slot = 0;

@@ -669,7 +669,7 @@ __device__ __forceinline__ bool last_block(DevScalars* sc) {
     if (threadIdx.x == 0) {
         __threadfence();
         unsigned int t = atomicAdd(&sc->ticket, 1u);
-        s_last = (t == gridDim.x - 1);
+        s_last = (t == gridDim.x * gridDim.y - 1);
         if (s_last) __threadfence();
     }
     __syncthreads();
@@ -754,42 +754,48 @@ __device__ __forceinline__ void block_partial(Partial* part, long long (&d)[NDIG
     block_partial(part, d, mx, rate, blockIdx.x);
 }
 
+// Sum of the digits over a warp: the six digits (padded to eight) together, each
+// exchange halves the values a lane carries, 9 shuffles of 64 bits instead of 30.
+// Lane l returns the sum of digit l / 4 (0 of the padding).
+__device__ __forceinline__ long long warp_sum_digits(const long long (&d)[NDIG]) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    long long a[4];
+    const bool up = lane & 16;
+    const long long hi[4] = {d[4], d[5], 0, 0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const long long got = __shfl_xor_sync(full, up ? d[i] : hi[i], 16);
+        a[i] = (up ? hi[i] : d[i]) + got;
+    }
+    const bool up2 = lane & 8;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const long long got = __shfl_xor_sync(full, up2 ? a[i] : a[i + 2], 8);
+        a[i] = (up2 ? a[i + 2] : a[i]) + got;
+    }
+    const bool up4 = lane & 4;
+    const long long got = __shfl_xor_sync(full, up4 ? a[0] : a[1], 4);
+    a[0] = (up4 ? a[1] : a[0]) + got;
+    a[0] += __shfl_xor_sync(full, a[0], 2);
+    a[0] += __shfl_xor_sync(full, a[0], 1);
+    return a[0];
+}
+
 // The block's digits and maximum value folded into global accumulators with
 // atomics. Integer sums and maxima: the totals do not depend on the order of
-// the blocks. Within a warp the six digits (padded to eight) are summed
-// together: each exchange halves the values a lane carries, 9 shuffles of 64
-// bits instead of 30.
+// the blocks.
 __device__ __forceinline__ void block_atomics(long long* acc, unsigned long long* maxq, const long long (&d)[NDIG],
                                               double mx) {
     __shared__ long long s_acc[MAX_WARPS][8];
     __shared__ unsigned long long s_mx[MAX_WARPS];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    long long a[4];
-    {
-        const bool up = lane & 16;
-        const long long hi[4] = {d[4], d[5], 0, 0};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const long long got = __shfl_xor_sync(full, up ? d[i] : hi[i], 16);
-            a[i] = (up ? hi[i] : d[i]) + got;
-        }
-        const bool up2 = lane & 8;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const long long got = __shfl_xor_sync(full, up2 ? a[i] : a[i + 2], 8);
-            a[i] = (up2 ? a[i + 2] : a[i]) + got;
-        }
-        const bool up4 = lane & 4;
-        const long long got = __shfl_xor_sync(full, up4 ? a[0] : a[1], 4);
-        a[0] = (up4 ? a[1] : a[0]) + got;
-        a[0] += __shfl_xor_sync(full, a[0], 2);
-        a[0] += __shfl_xor_sync(full, a[0], 1);
-    }
+    const long long mine = warp_sum_digits(d);
     const unsigned long long mk = mx > -INFINITY ? ord_key(mx) : 0ull;
     const unsigned top = __reduce_max_sync(full, (unsigned)(mk >> 32));
     const unsigned low = __reduce_max_sync(full, (unsigned)(mk >> 32) == top ? (unsigned)mk : 0u);
-    if ((lane & 3) == 0) s_acc[wid][lane >> 2] = a[0];
+    if ((lane & 3) == 0) s_acc[wid][lane >> 2] = mine;
     if (lane == 0) s_mx[wid] = ((unsigned long long)top << 32) | low;
     __syncthreads();
     const int q = threadIdx.x, nw = (int)(blockDim.x >> 5);

@@ -13,10 +13,8 @@ __global__ void k_begin(DevScalars* sc, double t_target) {
     sc->done = !(sc->t < t_target) || sc->error != 0;
     sc->steps_call = 0;
     sc->updates_call = 0;
+    sc->bar_seq = 0;
 }
-
-// Normalisation scalars of a new grid (one thread).
-__global__ void k_finalise(const Model m, DevScalars* sc, int mode) { finalise_norm(m, sc, mode); }
 
 // Start a batched propagate call: k_begin for every grid of the batch.
 __global__ void k_batch_begin(const BatchItem* items, int count) {
@@ -69,17 +67,10 @@ __global__ void k_loop_ctl(DevScalars* sc, cudaGraphConditionalHandle h_while, c
     cudaGraphSetConditional(h_while, (!sc->done && !err && it < max_iter) ? 1u : 0u);
 }
 
-// Empty every hashtable slot.
-__global__ void k_table_clear(const Model m, Bufs b) {
-    const unsigned long long T = m.tmask + 1;
-    for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s < T;
-         s += (unsigned long long)gridDim.x * blockDim.x) {
-        reinterpret_cast<ulonglong2*>(b.table)[s] = make_ulonglong2(EMPTY_KEY, ~0ull);
-    }
-}
-
-// Exclusive scan of blk[0..nblk) by one block; the total goes to sc->N_new.
-__global__ void k_scan_blocks(Bufs b, int nblk, long long cap) {
+// Exclusive scan of blk[0..nblk) by one block; the total goes to sc->N_new, and
+// with count also becomes the pool of a new grid (its active cells; the halo
+// kernel adds their halo).
+__global__ void k_scan_blocks(Bufs b, int nblk, long long cap, int count) {
     __shared__ long long s_part[THREADS];
     const int per = (nblk + THREADS - 1) / THREADS;
     const int i0 = threadIdx.x * per;
@@ -95,6 +86,12 @@ __global__ void k_scan_blocks(Bufs b, int nblk, long long cap) {
             run += v;
         }
         b.sc->N_new = run;
+        if (count) {
+            b.sc->N = run;
+            b.sc->NA = run;
+            b.sc->N_prev = 0;
+            b.sc->n_act = 0;
+        }
         if (run > cap) set_error(b.sc, ST_ECAPACITY);
     }
     __syncthreads();
@@ -106,8 +103,8 @@ __global__ void k_scan_blocks(Bufs b, int nblk, long long cap) {
     }
 }
 
-// Reset the grid scalars before an init.
-__global__ void k_reset(DevScalars* sc, double t0) {
+// Reset the grid scalars.
+__device__ __forceinline__ void reset_scalars(DevScalars* sc, double t0) {
     sc->N = 0;
     sc->N_prev = 0;
     sc->N_new = 0;
@@ -145,25 +142,29 @@ __global__ void k_reset(DevScalars* sc, double t0) {
         for (int q = 0; q < NDIG; ++q) sc->loop_acc[e][q] = 0;
     }
     for (int q = 0; q < 8; ++q) sc->phase_cycles[q] = 0;
+    for (int k = 0; k < 28; ++k)
+        for (int q = 0; q < NDIG; ++q) sc->mom[k][q] = 0;
     sc->phase_steps = 0;
 }
 
-// Initial grid: the active cells written so far are the whole pool; the halo
-// kernel adds their halo next.
-__global__ void k_set_count_from_new(DevScalars* sc) {
-    sc->N = sc->N_new;
-    sc->NA = sc->N_new;
-    sc->N_prev = 0;
-    sc->n_act = 0;
-}
+// A new context's scalars.
+__global__ void k_reset(DevScalars* sc, double t0) { reset_scalars(sc, t0); }
 
-// Counts and step number of a grid loaded from explicit cells.
-__global__ void k_set_count(DevScalars* sc, long long count, long long step0) {
-    sc->N = count;
-    sc->NA = count;
-    sc->N_prev = 0;
-    sc->n_act = 0;
-    sc->step = step0;
+// A new grid: scalars reset (count > 0: loaded from that many cells, after step0
+// steps), every hashtable slot emptied.
+__global__ void __launch_bounds__(THREADS) k_new_grid(const Model m, Bufs b, double t0, long long count,
+                                                      long long step0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        reset_scalars(b.sc, t0);
+        b.sc->N = count;
+        b.sc->NA = count;
+        b.sc->step = step0;
+    }
+    const unsigned long long T = m.tmask + 1;
+    for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s < T;
+         s += (unsigned long long)gridDim.x * blockDim.x) {
+        reinterpret_cast<ulonglong2*>(b.table)[s] = make_ulonglong2(EMPTY_KEY, ~0ull);
+    }
 }
 
 // ------------------------------------------------------------------ sorting
@@ -522,17 +523,6 @@ __global__ void __launch_bounds__(THREADS) k_readout_order(const Model m, Bufs b
         for (int j = 0; j < N; ++j) idx[r.c * N + j] = I[j];
         p[r.c] = __ddiv_rn((double)static_cast<const T*>(b.q[pb])[c], w);
     }
-}
-
-// Zero the exact accumulators of the moments.
-__global__ void k_moments_clear(DevScalars* sc) {
-    for (int i = threadIdx.x; i < 28 * NDIG; i += blockDim.x) (&sc->mom[0][0])[i] = 0;
-}
-
-// Convert the moment sums to doubles times prod h: out[slot].
-__global__ void k_moments_final(const Model m, DevScalars* sc, double* out, int nslots) {
-    int s = threadIdx.x;
-    if (s < nslots) out[s] = __dmul_rn(m.prod_h, acc_to_double(sc->mom[s]));
 }
 
 }  // namespace gbees
