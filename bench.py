@@ -270,9 +270,9 @@ def fp64_flops_per_update(kernel: str, n: int) -> int:
     two): the flux pass evaluates the n lower faces of the cell, 11 flops each
     (the transverse sum, donor cell and corrections: 2 + 2 + 1; the limited
     high-resolution term: 1 + 2 + 1 + 2); the wave pass 7 per dimension (two
-    jumps, the entering wave 1 + 2, its share of tg 2); the update pass 3 per
+    jumps, the entering wave 1 + 2, its share of their sum 2); the update pass 3 per
     dimension plus 3 (difference and FMA per face, then the rescale)."""
-    return {"k_faces": 11 * n, "k_waves_list": 7 * n, "k_apply": 3 * n + 3}[kernel]
+    return {"k_faces": 11 * n, "k_waves": 7 * n, "k_apply": 3 * n + 3}[kernel]
 
 
 def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None):
@@ -379,9 +379,11 @@ def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None
     else:
         per_cell = {k: prof["ms"][k] for k in ("grow", "faces", "apply")}
         top = max(per_cell, key=per_cell.get)
-        kernel = {"grow": "k_waves_list", "faces": "k_faces", "apply": "k_apply"}[top]
+        # (FP32 forms the fluxes and the update in one kernel; the grow phase has two
+        # timed brackets per step, the grow's and the waves')
+        kernel = {"grow": "k_waves", "faces": "k_faces" if precision == "f64" else "k_update", "apply": "k_apply"}[top]
         timing = "CUDA events around each launch of that kernel in a profiled pass of the same runs"
-        launches_k = max(prof["timed"][top], 1)
+        launches_k = max(prof["timed"][top] // (2 if top == "grow" else 1), 1)
         units = prof_updates
         avg_us = per_cell[top] * 1e3 / launches_k
     units_per_launch = units / max(launches_k, 1)
@@ -405,7 +407,7 @@ def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None
         "avg_launch_us": avg_us,
     }
     kname = kernel.split(" ")[0]
-    if precision == "f64" and kname in ("k_faces", "k_waves_list", "k_apply"):
+    if precision == "f64" and kname in ("k_faces", "k_waves", "k_apply"):
         # FP64 step kernels are bound by the FP64 pipe on this chip (ncu: the
         # flux pass keeps it 64 % busy at 29 % of DRAM bandwidth):
         # the roofline is the FP64 arithmetic peak; the HBM figures stay beside it

@@ -472,7 +472,6 @@ void launch_list(gbees_ctx* ctx, void* const* f, const int* grids, int nf) {
 // together; a grid that fits in L2 keeps its order (stream compaction).
 constexpr int kPruneKernelsSorted = 3 + 1 + 3 * SORT_PASSES + 1 + 2;
 constexpr int kPruneKernelsPlain = 3 + 1 + 1;
-constexpr long long kSortMinEntries = 1ll << 18;        // smaller pools are not sorted
 
 bool sorts(const gbees_ctx* ctx) { return ctx->cfg.storage_order != GBEES_ORDER_NONE; }
 
@@ -488,7 +487,7 @@ void launch_prune(gbees_ctx* ctx) {
     // the host's copy of the pool size (possibly a few steps old: it only
     // decides the storage order, which no result depends on)
     const long long N = ctx->hs.N;
-    const bool sorted = sorts(ctx) && N > kSortMinEntries;
+    const bool sorted = sorts(ctx) && N > SORT_MIN_ENTRIES;
     const int G = blocks_for(N, ctx->grid);
     const int Gs = sort_blocks(N);
     Phase ph(ctx, GBEES_PHASE_PRUNE, sorted ? kPruneKernelsSorted : kPruneKernelsPlain);
@@ -585,11 +584,17 @@ void launch_step(gbees_ctx* ctx) {
         });
     }
     {
-        Phase ph(ctx, GBEES_PHASE_FACES, 1);
+        Phase ph(ctx, GBEES_PHASE_GROW, 1);
         launch_list(ctx, ctx->kern.post, ctx->post_grid, 1);
     }
-    Phase ph(ctx, GBEES_PHASE_APPLY, 1);
-    launch_list(ctx, ctx->kern.post + 1, ctx->post_grid + 1, 1);
+    {
+        Phase ph(ctx, GBEES_PHASE_FACES, 1);
+        launch_list(ctx, ctx->kern.post + 1, ctx->post_grid + 1, 1);
+    }
+    if (ctx->kern.npost > 2) {
+        Phase ph(ctx, GBEES_PHASE_APPLY, 1);
+        launch_list(ctx, ctx->kern.post + 2, ctx->post_grid + 2, 1);
+    }
 }
 
 // ---- the step loop as a CUDA graph
@@ -1109,11 +1114,14 @@ int gbees_propagate(gbees_ctx* ctx, double t_end, gbees_stats* stats) {
     const int K = ctx->cfg.prune_interval;
     long long host_step = ctx->hs.step;
     long long batch = 4;
+    bool first = true;
     while (!ctx->hs.done) {
         for (long long i = 0; i < batch; ++i) {
             ++host_step;
             launch_step(ctx);
-            if (K > 0 && host_step % K == 0) launch_prune(ctx);
+            // (after the first step of a call a grown pool may be due for a sort)
+            if ((K > 0 && host_step % K == 0) || (sorts(ctx) && first)) launch_prune(ctx);
+            first = false;
         }
         if (!sync_scalars(ctx, "propagate")) return ctx->status;
         host_step = ctx->hs.step;

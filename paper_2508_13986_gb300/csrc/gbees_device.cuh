@@ -58,6 +58,7 @@ struct alignas(256) DevScalars {
     long long n_halo;     // halo cells appended by the current halo phase
     long long n_act;      // halo cells made active by the current grow (listed in map)
     long long n_glist;    // cells listed for the current grow (listed form)
+    long long N_sorted;   // entries that the last sort put in order
     double t;             // time
     double t_target;      // end of the current propagate call
     double dt;            // last step
@@ -75,7 +76,7 @@ struct alignas(256) DevScalars {
     int gen;              // current key/link buffer
     int done;             // t reached t_target
     int error;            // first error status (0 = none)
-    int prune_now;        // the step just taken is a prune step
+    int prune_now;        // the step just taken is a prune step (1), or its pool is to be sorted (RESORT)
     unsigned int ticket;  // last-block election
     unsigned long long tmp_ord;  // scratch maximum (init)
     long long loop_iter;  // iterations of the device-side step loop in the current graph launch
@@ -188,6 +189,11 @@ struct Bufs {
     Partial* part;   // GRID_MAX per-block partials
 };
 
+
+constexpr int RESORT = 2;                            // DevScalars::prune_now
+constexpr int RESORT_STEPS = 5;                      // steps that a re-sort has to serve at least
+constexpr long long RESORT_MIN_ENTRIES = 1ll << 21;
+constexpr long long SORT_MIN_ENTRIES = 1ll << 18;    // smaller pools (they fit in L2) are not sorted
 
 constexpr unsigned short OM_COMPLETE = 0x8000;
 constexpr unsigned short OM_GHOST = 0x4000;
@@ -388,24 +394,32 @@ __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fma
 __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 
-// Sign tests, positive and negative parts. FP64 arithmetic is scarce on this
-// chip, so for doubles they work on the bit pattern in the integer pipe (a
-// finite double is > 0 exactly when its bits, read as a signed integer, are
-// > 0; -0 reads as the smallest integer).
-__device__ __forceinline__ bool gt0(double x) { return __double_as_longlong(x) > 0; }
+// Sign tests, absolute value and negation. FP64 arithmetic is scarce on this
+// chip, so for doubles they work on the two words of the bit pattern in the integer
+// pipe. (The words, not the pattern as one 64-bit integer: the compiler knows that
+// the pattern without its sign bit is the absolute value, and that the pattern
+// shifted left by one is zero for a zero, and would put the FP64 instructions back;
+// they were 8 of 13 per face of the flux pass and a third of the wave pass.)
+__device__ __forceinline__ bool gt0(double x) {
+    const int hi = __double2hiint(x);
+    return hi > 0 || (hi == 0 && __double2loint(x) != 0);
+}
 __device__ __forceinline__ bool lt0(double x) {
-    const long long b = __double_as_longlong(x);
-    return b < 0 && (b << 1) != 0;
+    const int hi = __double2hiint(x);
+    return hi < 0 && ((hi & 0x7fffffff) | __double2loint(x)) != 0;
 }
 __device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool lt0(float x) { return x < 0.0f; }
-template <typename T>
-__device__ __forceinline__ T pos_part(T x) { return gt0(x) ? x : (T)0; }
-template <typename T>
-__device__ __forceinline__ T neg_part(T x) { return lt0(x) ? x : (T)0; }
+__device__ __forceinline__ bool nonzero(double x) { return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 __device__ __forceinline__ double abs_bits(double x) {
-    return __longlong_as_double(__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll);
+    return __hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x));
 }
+// v >= 0 with the sign of s
+__device__ __forceinline__ double with_sign(double v, double s) {
+    return __hiloint2double(__double2hiint(v) | (__double2hiint(s) & (int)0x80000000), __double2loint(v));
+}
+__device__ __forceinline__ float with_sign(float v, float s) { return copysignf(v, s); }
 __device__ __forceinline__ float abs_bits(float x) { return fabsf(x); }
 // min of two non-negative finite values (integer order of the bits for doubles)
 __device__ __forceinline__ double min_nonneg(double a, double b) {
@@ -470,7 +484,7 @@ __device__ __forceinline__ T limited_wave(int lim, T W, T Wup) {
     if ((gt0(W) && gt0(Wup)) || (lt0(W) && lt0(Wup))) {
         const T aW = abs_bits(W), aU = abs_bits(Wup);
         const T v = min_nonneg(min_nonneg(half_nonneg(aW + aU), twice_nonneg(aW)), twice_nonneg(aU));
-        return gt0(W) ? v : -v;
+        return with_sign(v, W);
     }
     return (T)0;
 }

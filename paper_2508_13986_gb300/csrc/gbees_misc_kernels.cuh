@@ -113,6 +113,7 @@ __device__ __forceinline__ void reset_scalars(DevScalars* sc, double t0) {
     sc->n_halo = 0;
     sc->n_act = 0;
     sc->n_glist = 0;
+    sc->N_sorted = 0;
     sc->t = t0;
     sc->t_target = t0;
     sc->dt = 0.0;

@@ -12,9 +12,10 @@
 //   grow       directional grow of the significant cells (Sec. 3.3, Algorithm 2)
 //   halo       the missing face neighbours of the newly active cells, as halo cells
 //   link       neighbour links, outward mask and CFL rate of the new entries (Sec. 4.1)
-//   waves      per-entry velocities u_d and entering waves G_d
+//   waves      per-entry jumps and transverse terms
 //   faces      one flux per face (Eq. 7 + Algorithm 1 gathered + HR term)
 //   apply      P -= sum_j dt/h_j (F_hi - F_lo), normalised, reduced
+//              (faces and apply in one pass on large FP32 grids)
 //   prune      mark S, mark D(S), status, compact, relink and rehash (Algorithm 3)
 //
 // The pool holds the active cells and, as halo cells with p = 0, every face
@@ -193,8 +194,8 @@ __device__ __forceinline__ long long insert_cell(const Model& m, const Bufs& b, 
 //
 // The candidates of a cell (2n faces, 4 C(n,2) edges, those that are not
 // downwind skipped at once) are independent chains of dependent loads and
-// atomics, spread over many threads: for large grids the wave pass lists the
-// growing cells (grow_list_mark) and a kernel of its own spreads every (cell,
+// atomics, spread over many threads: for large grids a sweep lists the
+// growing cells (grow_list_mark) and a second kernel spreads every (cell,
 // candidate) pair of the list over the grid (grow_list_body); the step loop of
 // a small grid has grow_detect and grow_act.
 struct GrowWork {
@@ -267,9 +268,8 @@ __device__ __forceinline__ bool grows(const unsigned short* om, const T* Q, cons
     return !(f & (OM_COMPLETE | OM_GHOST)) && out;
 }
 
-// First half: cell c (of the wave pass's sweep) joins the
-// step's grow list (in the flux scratch, free until the flux pass) when it
-// grows.
+// First half: cell c joins the step's grow list (in the flux scratch, free until
+// the flux pass) when it grows.
 template <typename T>
 __device__ __forceinline__ void grow_list_mark(const Bufs& b, const StepView& v, const Above<T>& above, long long c) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
@@ -371,11 +371,13 @@ __device__ __forceinline__ double drift_at(const Model& m, const double* y, int 
     }
 }
 
-// x > 0 without the FP64 pipe (false for NaN, as the comparison).
-__device__ __forceinline__ bool above0(double x) {
-    const long long b = __double_as_longlong(x);
-    return b > 0 && b <= 0x7FF0000000000000ll;
+// x > 0 and x < 0 without the FP64 pipe (false for NaN, as the comparisons).
+__device__ __forceinline__ bool is_number(double x) {
+    const int a = __double2hiint(x) & 0x7fffffff;
+    return a < 0x7ff00000 || (a == 0x7ff00000 && __double2loint(x) == 0);
 }
+__device__ __forceinline__ bool above0(double x) { return gt0(x) && is_number(x); }
+__device__ __forceinline__ bool below0(double x) { return lt0(x) && is_number(x); }
 
 // Face velocities, outward mask and CFL rate of entry c of generation g (cell
 // I; Eq. 7, Eq. 8 with |f|): bit 2j+1 of the mask when the flow leaves through the
@@ -404,7 +406,7 @@ __device__ __forceinline__ double entry_velocities_of(const Model& m, const Bufs
         const double hi = __dadd_rn(m.x0[j], __dmul_rn(__dadd_rn(di[j], 0.5), m.h[j]));
         const double ul = drift_at<N, DYN>(m, y, j, lo);
         if (above0(drift_at<N, DYN>(m, y, j, hi))) msk |= 1u << (2 * j + 1);
-        if (above0(-ul)) msk |= 1u << (2 * j);
+        if (below0(ul)) msk |= 1u << (2 * j);
         static_cast<T*>(b.u[g])[j * m.cap + c] = (T)ul;
         r = __dadd_rn(r, div_h(m, abs_bits(ul), j));
     }
@@ -534,7 +536,7 @@ __device__ __noinline__ double complete_group(const Model& m, const Bufs& b, int
         }
     }
     // outward: upper face and u > 0, lower face and u < 0
-    const unsigned out = __ballot_sync(full, on && ((e & 1) ? u : -u) > 0.0);
+    const unsigned out = __ballot_sync(full, on && ((e & 1) ? above0(u) : below0(u)));
     double r = 0.0;
 #pragma unroll
     for (int j = 0; j < N; ++j) r = __dadd_rn(r, __shfl_sync(full, term, (s * F + 2 * j) & 31));
@@ -652,7 +654,7 @@ __device__ __forceinline__ double link_body_tile(const Model& m, const Bufs& b, 
     return link_masks<N, T>(m, b, lo, hi, g, nb, bi);
 }
 
-// ------------------------------------------------------------------ three-pass update
+// ------------------------------------------------------------------ update
 
 template <typename T>
 __device__ __forceinline__ T q_or_zero(const T* Q, int i) {
@@ -664,118 +666,96 @@ __device__ __forceinline__ bool is_halo(const unsigned short* om, long long i) {
 // 0 - x as IEEE subtraction gives it, without FP64 arithmetic for doubles:
 // the sign flips, except that both zeros give +0.
 __device__ __forceinline__ double zero_minus(double x) {
-    const long long b = __double_as_longlong(x);
-    return __longlong_as_double((b << 1) == 0 ? 0ll : (b ^ (long long)0x8000000000000000ull));
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    return __hiloint2double(((hi & 0x7fffffff) | lo) == 0 ? 0 : hi ^ (int)0x80000000, lo);
 }
 __device__ __forceinline__ float zero_minus(float x) { return 0.0f - x; }
 
-// The entering wave of entry y in dimension d,
+// Per entry y and dimension d the update works with the jump across the lower face,
+//   wl_d(y) = P_y - P_{y-e_d},
+// and the entering wave
 //   G_d(y) = max(u_lo, 0) (P_y - P_{y-e_d}) + min(u_hi, 0) (P_{y+e_d} - P_y),
 // u_lo, u_hi the velocities at its lower and upper d-face (the upper one is the
 // lower one of the neighbour above; a missing neighbour above of a halo cell
-// leaves both P at 0), with the jump across the lower face in wlo. VOTE: the
-// warp's lanes run this together (the wave pass), so terms that no lane needs
-// are skipped by a warp vote.
-template <int N, typename T, bool VOTE = false>
-__device__ __forceinline__ T wave_of(const T* Q, const T* U, long long cap, const int* L, long long y, T Py, int d,
-                                     T& wlo) {
-    const int dn = L[2 * d], up = L[2 * d + 1];
-    const T Pm = q_or_zero<T>(Q, dn);
-    const T Pp = q_or_zero<T>(Q, up);
-    const T ul = U[d * cap + y];
-    const T uh = up >= 0 ? U[d * cap + up] : (T)0;
-    wlo = Py - Pm;
-    // one product in the usual case (flow through the cell, or out of it on one
-    // side only); a cell that both faces flow into takes the second term too.
-    // The flow direction varies slowly: when no lane of the warp takes flow in
-    // through the upper face, the upper jump and the second term are skipped.
-    const bool in_lo = gt0(ul), in_hi = lt0(uh);
-    if constexpr (VOTE) {
-        const unsigned act = __activemask();
-        if (!__any_sync(act, in_hi)) return (in_lo ? ul : (T)0) * wlo;
-        const T G = (in_lo ? ul : (in_hi ? uh : (T)0)) * (in_lo ? wlo : Pp - Py);
-        if (!__any_sync(act, in_lo && in_hi)) return G;
-        return (in_lo && in_hi) ? fmadd(uh, Pp - Py, G) : G;
-    } else {
-        const T G = (in_lo ? ul : (in_hi ? uh : (T)0)) * (in_lo ? wlo : Pp - Py);
-        return (in_lo && in_hi) ? fmadd(uh, Pp - Py, G) : G;
-    }
-}
+// leaves both P at 0). The corrections that Algorithm 1 scatters onto the lower
+// j-face of X add up to -u_j(X) dt sum_{d != j} G_d(Y) / (2 h_d), Y the cell upwind
+// of the face, so that donor cell and corrections together are u_j(X) base_j(Y),
+//   base_j(y) = P_y - dt sum_{d != j} G_d(y) / (2 h_d).
+//
+// Large grids, pass 1, one thread per entry (active and halo, the step's new ones
+// too: their neighbours have no density, so theirs come out as 0): (wl_j, base_j)
+// as a pair per dimension. The pass runs when dt is known, after the links, so
+// that a face needs one pair of its own cell and one of a neighbour (four gathers
+// with the waves and their sum in separate arrays, formed before dt). Six
+// dimensions, 5.0e6 entries in storage order: 0.42 ms in FP64, 81 % of the FP64
+// pipe; 0.14 ms in FP32, bound by the gathers' sectors.
+template <typename T>
+struct alignas(2 * sizeof(T)) Wave {
+    T wl, base;
+};
 
-// wave_of for a halo entry, whose value is +0: the same results (0 - P_m and
-// P_p - 0 are exact) without the two subtractions.
 template <int N, typename T>
-__device__ __forceinline__ T wave_of_halo(const T* Q, const T* U, long long cap, const int* L, long long y, int d,
-                                          T& wlo) {
-    const int dn = L[2 * d], up = L[2 * d + 1];
-    const T Pm = q_or_zero<T>(Q, dn);
-    const T Pp = q_or_zero<T>(Q, up);
-    const T ul = U[d * cap + y];
-    const T uh = up >= 0 ? U[d * cap + up] : (T)0;
-    wlo = zero_minus(Pm);
-    const bool in_lo = gt0(ul), in_hi = lt0(uh);
-    const T G = (in_lo ? ul : (in_hi ? uh : (T)0)) * (in_lo ? wlo : Pp);
-    if (!__any_sync(__activemask(), in_lo && in_hi)) return G;
-    return (in_lo && in_hi) ? fmadd(uh, Pp, G) : G;
-}
-
-// Pass 1, one thread per entry c of [0, ncell) (active and halo), all
-// dimensions d: the jump wl[d] = P - P_{-e_d}, the entering wave wg[d] and
-// tg = sum_d wg[d] / (2 h_d). Entries added by this step's grow and halo phases
-// are left out: they have p = 0, and their waves are formed on the spot. Runs
-// beside grow: a cell that grow or halo adds has p = 0 like the missing cell it
-// replaces, so these waves do not change.
-template <int N, typename T, bool LIST_GROW = false>
-__device__ __forceinline__ void waves_body(const Model& m, const Bufs& b, const StepView& v, long long ncell) {
+__device__ __forceinline__ void waves_body(const Model& m, const Bufs& b, const StepView& v) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
     const int* link = b.link[v.g];
     const T* U = static_cast<const T*>(b.u[v.g]);
-    // the outputs alias no input (restrict: loads may be scheduled ahead of the
+    // the output aliases no input (restrict: loads may be scheduled ahead of the
     // stores; no read-only cache path is implied)
-    T* __restrict__ wl = static_cast<T*>(b.wl);
-    T* __restrict__ wg = static_cast<T*>(b.wg);
-    T* __restrict__ tg = static_cast<T*>(b.tg);
+    Wave<T>* __restrict__ wave = static_cast<Wave<T>*>(b.wl);
     const long long cap = m.cap;
+    const T ndt = -(T)v.dt;
     T i2h[N];  // 1 / (2 h_d) in the arithmetic type, converted once
 #pragma unroll
     for (int d = 0; d < N; ++d) i2h[d] = (T)m.inv_2h[d];
-    const Above<T> above(m.thr_rel * v.maxq);
-#pragma unroll 1
-    for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
+    for (WarpRuns wr(v.N, v.nb, v.bi); wr.next();) {
         const long long c = wr.c;
-        if (c >= ncell) continue;
-        if (LIST_GROW) grow_list_mark<T>(b, v, above, c);
+        if (c >= v.N) continue;
+        const unsigned act = __activemask();
         int L[2 * N];
         load_links<N>(link, cap, c, L);
         const T P0 = Q[c];
-        T t = (T)0;
-        // a warp of halo entries (the pool keeps them together after a
-        // prune) takes the form without the subtractions
-        if (__all_sync(__activemask(), is_halo(b.om[v.g], c))) {
+        // the gathers of all dimensions in flight together, in two steps (the jump
+        // across the upper face is needed only where the flow comes in through it)
+        T ul[N], uh[N], Pm[N], Pp[N];
 #pragma unroll
-            for (int d = 0; d < N; ++d) {
-                T wlo;
-                const T G = wave_of_halo<N, T>(Q, U, cap, L, c, d, wlo);
-                wl[d * cap + c] = wlo;
-                wg[d * cap + c] = G;
-                t = fmadd(G, i2h[d], t);
-            }
-        } else {
-#pragma unroll
-            for (int d = 0; d < N; ++d) {
-                T wlo;
-                const T G = wave_of<N, T, true>(Q, U, cap, L, c, P0, d, wlo);
-                wl[d * cap + c] = wlo;
-                wg[d * cap + c] = G;
-                t = fmadd(G, i2h[d], t);
-            }
+        for (int d = 0; d < N; ++d) {
+            ul[d] = U[d * cap + c];
+            Pm[d] = q_or_zero<T>(Q, L[2 * d]);
+            uh[d] = L[2 * d + 1] >= 0 ? U[d * cap + L[2 * d + 1]] : (T)0;
         }
-        tg[c] = t;
+#pragma unroll
+        for (int d = 0; d < N; ++d) Pp[d] = lt0(uh[d]) ? Q[L[2 * d + 1]] : (T)0;
+        // a warp of halo entries (P = 0; the pool keeps them together after a
+        // prune) needs no subtraction: 0 - P_m and P_p - 0 are exact
+        const bool zeros = __all_sync(act, !nonzero(P0));
+        T G[N], wl[N], t = (T)0;
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            const bool in_lo = gt0(ul[d]), in_hi = lt0(uh[d]);
+            wl[d] = zeros ? zero_minus(Pm[d]) : P0 - Pm[d];
+            // one product in the usual case (flow through the cell, or out of it on
+            // one side only); the flow direction varies slowly: when no lane of the
+            // warp takes flow in through a face, that face's term is skipped
+            G[d] = (T)0;
+            if (__any_sync(act, in_lo)) G[d] = (in_lo ? ul[d] : (T)0) * wl[d];
+            if (__any_sync(act, in_hi)) {
+                const T wh = zeros ? Pp[d] : Pp[d] - P0;
+                if (in_hi) G[d] = in_lo ? fmadd(uh[d], wh, G[d]) : uh[d] * wh;
+            }
+            t = fmadd(G[d], i2h[d], t);
+        }
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            Wave<T> w;
+            w.wl = wl[d];
+            w.base = fmadd(ndt, fmadd(-i2h[d], G[d], t), P0);
+            wave[d * cap + c] = w;
+        }
     }
 }
 
-// The same for the step loop of a small grid, in less code: one form for active
-// and halo entries, 32-bit indices.
+// The waves of the step loop of a small grid, formed beside the grow (before dt),
+// in little code: wl, G and tg = sum_d G_d / (2 h_d) of the existing entries.
 template <int N, typename T>
 __device__ __forceinline__ void waves_small_body(const Model& m, const Bufs& b, const StepView& v) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
@@ -808,7 +788,6 @@ __device__ __forceinline__ void waves_small_body(const Model& m, const Bufs& b, 
         T t = (T)0;
 #pragma unroll
         for (int d = 0; d < N; ++d) {
-            // wave_of with the warp's votes
             const T wlo = P0 - Pm[d];
             const bool in_lo = gt0(ul[d]), in_hi = lt0(uh[d]);
             T G = (in_lo ? ul[d] : (T)0) * wlo;
@@ -824,37 +803,6 @@ __device__ __forceinline__ void waves_small_body(const Model& m, const Bufs& b, 
     }
 }
 
-// sum_{d != j} G_d(y) / (2 h_d) of a new pool entry y (p = 0, no pass-1 values),
-// formed on the spot from its links.
-template <int N, typename T>
-__device__ __forceinline__ T waves_new(const Model& m, const T* Q, const T* U, const int* link, long long y, int j) {
-    const long long cap = m.cap;
-    int L[2 * N];
-    load_links<N>(link, cap, y, L);
-    T S = (T)0;
-#pragma unroll
-    for (int d = 0; d < N; ++d) {
-        if (d == j) continue;
-        T wlo;
-        S = fmadd(wave_of<N, T>(Q, U, cap, L, y, (T)0, d, wlo), (T)m.inv_2h[d], S);
-    }
-    return S;
-}
-
-// The flux pass's view of the step (pointers and constants in the arithmetic type).
-template <int N, typename T>
-struct FaceCtx {
-    const T* Q;
-    const int* link;
-    const T* U;
-    const T* wl;
-    const T* wg;
-    const T* tg;
-    long long cap, nold;
-    int lim;
-    T dt, i2h[N], dth[N];
-};
-
 // a[j] of a short array in registers, j known at run time only.
 template <int N, typename T, int M>
 __device__ __forceinline__ T pick_of(const T (&a)[M], int j) {
@@ -864,172 +812,88 @@ __device__ __forceinline__ T pick_of(const T (&a)[M], int j) {
     return x;
 }
 
-template <int N, typename T>
-__device__ __forceinline__ FaceCtx<N, T> face_ctx(const Model& m, const Bufs& b, const StepView& v) {
-    FaceCtx<N, T> fc;
-    fc.Q = static_cast<const T*>(b.q[v.pb]);
-    fc.link = b.link[v.g];
-    fc.U = static_cast<const T*>(b.u[v.g]);
-    fc.wl = static_cast<const T*>(b.wl);
-    fc.wg = static_cast<const T*>(b.wg);
-    fc.tg = static_cast<const T*>(b.tg);
-    fc.cap = m.cap;
-    fc.nold = v.N_prev;
-    fc.lim = m.limiter;
-    fc.dt = (T)v.dt;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {  // converted once
-        fc.i2h[j] = (T)m.inv_2h[j];
-        fc.dth[j] = (T)v.dth[j];
-    }
-    return fc;
+// The flux through a face with velocity u != 0: Eq. 7 and the corrections of
+// Algorithm 1 (u times the upwind cell's base), and the limited high-resolution
+// term 1/2 |u| (1 - dt |u| / h_j) phi W of the jump W across the face, Wup the jump
+// across the face beyond the upwind cell.
+template <typename T>
+__device__ __forceinline__ T flux_of(int lim, T u, T base, T W, T Wup, T dth) {
+    if (!nonzero(u)) return (T)0;
+    const T f = u * base;
+    if (lim == LIM_NONE || !nonzero(W)) return f;
+    const T au = abs_bits(u);
+    return fmadd(half_nonneg(au) * fmadd(-dth, au, (T)1), limited_wave<T>(lim, W, Wup), f);
 }
 
-// The flux through the lower j-face of pool entry X (Eq. 7, the corrections of
-// Algorithm 1 gathered onto the face, the limited HR term), X's value P0. The
-// corrections that Algorithm 1 scatters onto face (X, j) add up to
-//   -u_j(X) dt sum_{d != j} G_d(Y) / (2 h_d),  Y the cell upwind of the face,
-// with sum_{d != j} = tg(Y) - G_j(Y) / (2 h_j). Entries added by this step's
-// grow and halo phases (index >= nold) have no pass-1 values; theirs are formed
-// on the spot.
-template <int N, typename T>
-__device__ __forceinline__ T face_flux(const Model& m, const FaceCtx<N, T>& fc, long long X, T P0, int j) {
-    const long long cap = fc.cap;
-    const T u = fc.U[j * cap + X];
-    if (!(gt0(u) || lt0(u))) return (T)0;
-    const int Llo = fc.link[(long long)(2 * j) * cap + X];
-    const bool up = gt0(u);  // the flow crosses the face upwards: the upwind cell is Llo
-    const bool old_x = X < fc.nold;
-    const T PL = (up || !old_x) ? q_or_zero<T>(fc.Q, Llo) : (T)0;
-    const T W = old_x ? fc.wl[j * cap + X] : P0 - PL;
-    // transverse sum of the cell upwind of the face
-    const long long y = up ? (long long)Llo : X;
-    T S;
-    if (y < fc.nold) {
-        S = fmadd(-fc.i2h[j], fc.wg[j * cap + y], fc.tg[y]);
-    } else {
-        S = waves_new<N, T>(m, fc.Q, fc.U, fc.link, y, j);
-    }
-    // Eq. 7 (donor cell) and the corrections of Algorithm 1, gathered
-    T f = u * fmadd(-fc.dt, S, up ? PL : P0);
-    if (fc.lim != LIM_NONE && (gt0(W) || lt0(W))) {
-        T Wup;
-        if (up) {  // jump across the lower face of Llo
-            Wup = Llo < fc.nold ? fc.wl[j * cap + Llo]
-                                : PL - q_or_zero<T>(fc.Q, fc.link[(long long)(2 * j) * cap + Llo]);
-        } else {  // jump across the upper face of X
-            const int Lup = fc.link[(long long)(2 * j + 1) * cap + X];
-            Wup = (Lup >= 0 && Lup < fc.nold) ? fc.wl[j * cap + Lup]
-                  : (Lup >= 0 ? fc.Q[Lup] - P0 : zero_minus(P0));
-        }
-        // the limited high-resolution term 1/2 |u| (1 - dt |u| / h_j) phi W
-        const T au = abs_bits(u);
-        f = fmadd(half_nonneg(au) * fmadd(-fc.dth[j], au, (T)1), limited_wave<T>(fc.lim, W, Wup), f);
-    }
-    return f;
-}
-
-// face_flux for the faces whose values all come from pass 1: X and the cell
-// upwind of the face were in the pool before this step's grow, and so was the
-// upper neighbour whose jump the limiter reads. The same operations on the
-// same values as face_flux gives those faces; returns false, with nothing
-// evaluated, for any other face (new entries are few, and their waves are
-// formed on the spot by face_flux later, with all lanes of a warp).
-template <int N, typename T>
-__device__ __forceinline__ bool face_flux_old(const FaceCtx<N, T>& fc, long long X, T P0, int j, T& f) {
-    const long long cap = fc.cap;
-    const T u = fc.U[j * cap + X];
-    if (!(gt0(u) || lt0(u))) {
-        f = (T)0;
-        return true;
-    }
-    const int Llo = fc.link[(long long)(2 * j) * cap + X];
-    const bool up = gt0(u);
-    const int Lup = up ? -1 : fc.link[(long long)(2 * j + 1) * cap + X];
-    const long long y = up ? (long long)Llo : X;
-    if (X >= fc.nold || y >= fc.nold || Lup >= fc.nold) return false;
-    const T PL = up ? q_or_zero<T>(fc.Q, Llo) : (T)0;
-    const T W = fc.wl[j * cap + X];
-    const T S = fmadd(-fc.i2h[j], fc.wg[j * cap + y], fc.tg[y]);
-    f = u * fmadd(-fc.dt, S, up ? PL : P0);
-    if (fc.lim != LIM_NONE && (gt0(W) || lt0(W))) {
-        const T Wup = up ? fc.wl[j * cap + Llo] : (Lup >= 0 ? fc.wl[j * cap + Lup] : zero_minus(P0));
-        const T au = abs_bits(u);
-        f = fmadd(half_nonneg(au) * fmadd(-fc.dth[j], au, (T)1), limited_wave<T>(fc.lim, W, Wup), f);
-    }
-    return true;
-}
-
-// Pass 2: the flux through every face with an active cell on at least one
-// side, stored as the lower face of the entry above it: all n lower faces of
-// an active cell, and the lower faces of a halo cell whose neighbour below is
+// Large FP64 grids, pass 2: the flux through every face with an active cell on at
+// least one side, stored as the lower face of the entry above it: all n lower faces
+// of an active cell, and the lower faces of a halo cell whose neighbour below is
 // active. Each warp takes runs of 32 consecutive entries, queues their needed
 // faces (entry, j) in shared memory, dimension by dimension, and evaluates
-// them 32 at a time, so that the lanes of a warp all work although a halo cell
-// needs only the few faces it shares with active cells. The upper face of an active cell
-// is the lower face of its upper neighbour, which is in the pool (active or
-// halo).
+// them 64 at a time, two per lane with their loads in flight together, so that the
+// lanes of a warp all work although a halo cell needs only the few faces it shares
+// with active cells. The upper face of an active cell is the lower face of its upper
+// neighbour, which is in the pool (active or halo). Five FP64 instructions per face
+// (13 with the compiler's, see gt0); 5.0e6 entries in six dimensions: 0.34 ms (0.58
+// ms), 50 % of the FP64 pipe. One active cell per lane with all its faces unrolled
+// was slower (0.35 ms: fewer warps fit).
 template <int N, typename T>
 __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const StepView& v) {
+    constexpr int E = 2;  // faces per lane and evaluation
     const long long ncell = v.N;
     const long long cap = m.cap;
     const unsigned short* om = b.om[v.g];
+    const int* link = b.link[v.g];
+    const T* U = static_cast<const T*>(b.u[v.g]);
+    const Wave<T>* wave = static_cast<const Wave<T>*>(b.wl);
     T* __restrict__ fl = static_cast<T*>(b.fl);  // aliases no input
-    const FaceCtx<N, T> fc = face_ctx<N, T>(m, b, v);
-    // The warp's needed faces wait in a queue in shared memory (entry, j) and
-    // are evaluated 32 at a time once that many are queued, whatever runs
-    // they come from; the rest at the end.
-    constexpr int QCAP = 32 * N + 32;
+    const int lim = m.limiter;
+    constexpr int QCAP = 32 * N + 32 * E;
     __shared__ int s_qx[WARPS][QCAP];
     __shared__ unsigned char s_qj[WARPS][QCAP];
-    // FP64 (the pipe bounds it): faces that touch a new entry wait in a second
-    // queue, so that face_flux's longer path runs with all lanes too
-    constexpr bool DEFER = sizeof(T) == 8;
-    __shared__ int s_lx[WARPS][DEFER ? 64 : 1];
-    __shared__ unsigned char s_lj[WARPS][DEFER ? 64 : 1];
+    __shared__ T s_dth[N];  // dt / h_j, read with a face's j
+    if (threadIdx.x < N) s_dth[threadIdx.x] = (T)v.dth[threadIdx.x];
+    __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    int n_q = 0, n_later = 0;  // the same in every lane
-    auto later_flush = [&](int k) {  // the top k deferred faces, one per lane
-        n_later -= k;
-        if (lane < k) {
-            const long long X = s_lx[wid][n_later + lane];
-            const int jj = s_lj[wid][n_later + lane];
-            fl[jj * cap + X] = face_flux<N, T>(m, fc, X, fc.Q[X], jj);
-        }
-        __syncwarp();
-    };
-    auto eval = [&](int k) {  // the top k queued faces, one per lane
+    int n_q = 0;  // the same in every lane
+    auto eval = [&](int k) {  // the top k queued faces
         n_q -= k;
-        bool later = false;
-        long long X = 0;
-        int jj = 0;
-        if (lane < k) {
-            X = s_qx[wid][n_q + lane];
-            jj = s_qj[wid][n_q + lane];
-            if constexpr (DEFER) {
-                T f;
-                if (face_flux_old<N, T>(fc, X, fc.Q[X], jj, f)) fl[jj * cap + X] = f;
-                else later = true;
-            } else {
-                fl[jj * cap + X] = face_flux<N, T>(m, fc, X, fc.Q[X], jj);
-            }
+        long long X[E];
+        int j[E], lo[E], up[E];
+        T u[E];
+        Wave<T> own[E], other[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int at = lane + 32 * e;
+            X[e] = at < k ? s_qx[wid][n_q + at] : -1;
+            j[e] = at < k ? s_qj[wid][n_q + at] : 0;
         }
-        if constexpr (DEFER) {
-            const unsigned bal = __ballot_sync(0xffffffffu, later);
-            if (later) {
-                const int at = n_later + __popc(bal & lt);
-                s_lx[wid][at] = (int)X;
-                s_lj[wid][at] = (unsigned char)jj;
-            }
-            n_later += __popc(bal);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (X[e] < 0) continue;
+            u[e] = U[j[e] * cap + X[e]];
+            lo[e] = link[(long long)(2 * j[e]) * cap + X[e]];
+            up[e] = link[(long long)(2 * j[e] + 1) * cap + X[e]];
+            own[e] = wave[j[e] * cap + X[e]];
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (X[e] < 0) continue;
+            // the cell below (upwind when the flow crosses upwards), else the one above,
+            // whose lower face is the one beyond (missing only above a halo cell: no jump)
+            const int z = gt0(u[e]) ? lo[e] : up[e];
+            other[e].wl = other[e].base = (T)0;
+            if (z >= 0) other[e] = wave[j[e] * cap + z];
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (X[e] < 0) continue;
+            fl[j[e] * cap + X[e]] =
+                flux_of<T>(lim, u[e], gt0(u[e]) ? other[e].base : own[e].base, own[e].wl, other[e].wl, s_dth[j[e]]);
         }
         __syncwarp();
-        if constexpr (DEFER) {
-            if (n_later >= 32) later_flush(32);
-        }
     };
-#pragma unroll 1
     for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
         const long long c = wr.c;
         unsigned need = 0;
@@ -1039,7 +903,7 @@ __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const 
             } else {
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
-                    const int Llo = fc.link[(long long)(2 * j) * cap + c];
+                    const int Llo = link[(long long)(2 * j) * cap + c];
                     if (Llo >= 0 && !is_halo(om, Llo)) need |= 1u << j;
                 }
             }
@@ -1055,20 +919,16 @@ __device__ __forceinline__ void faces_body(const Model& m, const Bufs& b, const 
             n_q += __popc(bal);
         }
         __syncwarp();
-        while (n_q >= 32) eval(32);
+        while (n_q >= 32 * E) eval(32 * E);
     }
     if (n_q > 0) eval(n_q);
-    if constexpr (DEFER) {
-        if (n_later > 0) later_flush(n_later);
-    }
 }
 
-// Pass 3: the conservative update of the active cells with the previous
-// normalisation applied (halo cells stay 0); adds this thread's new values to
-// its digits and maximum. FP64: each warp queues the active cells of its runs in
+// Large FP64 grids, pass 3: the conservative update of the active cells with the
+// previous normalisation applied (halo cells stay 0); adds this thread's new values
+// to its digits and maximum. Each warp queues the active cells of its runs in
 // shared memory and updates them 32 at a time, so the FP64 lanes all work where
-// halo and active entries mix (after growth); FP32 is bound by load latency and
-// updates in place.
+// halo and active entries mix (after growth).
 template <int N, typename T>
 __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const StepView& v, long long (&dacc)[NDIG],
                                            double& mx, int& err) {
@@ -1085,55 +945,113 @@ __device__ __forceinline__ void apply_body(const Model& m, const Bufs& b, const 
     for (int k = 0; k < N; ++k) dth[k] = (T)v.dth[k];
     T tmax = -INFINITY;
     auto update = [&](long long c) {
-        int L[2 * N];
-        load_links<N>(link, cap, c, L);
+        int up[N];
+        T lo[N], hi[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) up[j] = link[(long long)(2 * j + 1) * cap + c];
+#pragma unroll
+        for (int j = 0; j < N; ++j) lo[j] = fl[j * cap + c];
+#pragma unroll
+        for (int j = 0; j < N; ++j) hi[j] = up[j] >= 0 ? fl[j * cap + up[j]] : (T)0;
         T upd = (T)0;
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const int up = L[2 * j + 1];
-            const T Fhi = up >= 0 ? fl[j * cap + up] : (T)0;
-            upd = fmadd(dth[j], Fhi - fl[j * cap + c], upd);
-        }
+        for (int j = 0; j < N; ++j) upd = fmadd(dth[j], hi[j] - lo[j], upd);
         const T qn = (Q[c] - upd) * scale;
         Qn[c] = qn;
         acc_add(dacc, qn, err);
         tmax = vmax(tmax, qn);
     };
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll 1
-        for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
-            const long long c = wr.c;
-            if (c >= ncell) continue;
-            if (is_halo(om, c)) {
-                Qn[c] = (T)0;
-                continue;
-            }
-            update(c);
+    __shared__ int s_ac[WARPS][64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    int n_a = 0;  // the same in every lane
+    for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
+        const long long c = wr.c;
+        bool act = false;
+        if (c < ncell) {
+            if (is_halo(om, c)) Qn[c] = (T)0;
+            else act = true;
         }
-    } else {
-        __shared__ int s_ac[WARPS][64];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        const unsigned lt = (1u << lane) - 1u;
-        int n_a = 0;  // the same in every lane
-#pragma unroll 1
-        for (WarpRuns wr(ncell, v.nb, v.bi); wr.next();) {
-            const long long c = wr.c;
-            bool act = false;
-            if (c < ncell) {
-                if (is_halo(om, c)) Qn[c] = (T)0;
-                else act = true;
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, act);
-            if (act) s_ac[wid][n_a + __popc(bal & lt)] = (int)c;
-            n_a += __popc(bal);
+        const unsigned bal = __ballot_sync(0xffffffffu, act);
+        if (act) s_ac[wid][n_a + __popc(bal & lt)] = (int)c;
+        n_a += __popc(bal);
+        __syncwarp();
+        if (n_a >= 32) {
+            n_a -= 32;
+            update(s_ac[wid][n_a + lane]);
             __syncwarp();
-            if (n_a >= 32) {
-                n_a -= 32;
-                update(s_ac[wid][n_a + lane]);
-                __syncwarp();
+        }
+    }
+    if (lane < n_a) update(s_ac[wid][lane]);
+    if (tmax > -INFINITY) mx = fmax(mx, (double)tmax);
+}
+
+// Large FP32 grids, passes 2 and 3 in one: every active cell forms the fluxes of
+// all its 2n faces itself (those of its upper faces as the lower faces of the
+// neighbours above: the same operations on the same values on both sides of a
+// face) and is updated at once. Each flux is formed twice, which single precision
+// has room for, while the fluxes' way through memory, the faces of the halo and a
+// sweep over the pool go; the loads of a cell's dimensions are all independent. Six
+// dimensions, 3.2e6 active cells: 0.28 ms in storage order (two kernels, flux and
+// update: 0.64 ms with the pool partly out of order, where this takes 0.50 ms).
+template <int N, typename T>
+__device__ __forceinline__ void update_body(const Model& m, const Bufs& b, const StepView& v, long long (&dacc)[NDIG],
+                                            double& mx, int& err) {
+    const long long cap = m.cap;
+    const T* Q = static_cast<const T*>(b.q[v.pb]);
+    T* __restrict__ Qn = static_cast<T*>(b.q[v.pb ^ 1]);  // aliases no input
+    const int* link = b.link[v.g];
+    const unsigned short* om = b.om[v.g];
+    const T* U = static_cast<const T*>(b.u[v.g]);
+    const Wave<T>* wave = static_cast<const Wave<T>*>(b.wl);
+    const T scale = (T)v.scale;
+    const int lim = m.limiter;
+    T tmax = -INFINITY;
+    for (WarpRuns wr(v.N, v.nb, v.bi); wr.next();) {
+        const long long c = wr.c;
+        if (c >= v.N) continue;
+        if (is_halo(om, c)) {
+            Qn[c] = (T)0;
+            continue;
+        }
+        int L[2 * N];
+        load_links<N>(link, cap, c, L);  // (an active cell has all its face neighbours)
+        T ul[N], uh[N];
+        Wave<T> own[N], above[N], other[N];
+        T beyond[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            ul[j] = U[j * cap + c];
+            own[j] = wave[j * cap + c];
+            above[j] = wave[j * cap + L[2 * j + 1]];
+            uh[j] = U[j * cap + L[2 * j + 1]];
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            // lower face: the cell below when the flow crosses upwards
+            other[j].wl = other[j].base = (T)0;
+            if (gt0(ul[j])) other[j] = wave[j * cap + L[2 * j]];
+            // upper face, flow downwards: the jump beyond the cell above
+            beyond[j] = (T)0;
+            if (lt0(uh[j])) {
+                const int z = link[(long long)(2 * j + 1) * cap + L[2 * j + 1]];
+                if (z >= 0) beyond[j] = wave[j * cap + z].wl;
             }
         }
-        if (lane < n_a) update(s_ac[wid][lane]);
+        T upd = (T)0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const T dth = (T)v.dth[j];
+            const T lo = flux_of<T>(lim, ul[j], gt0(ul[j]) ? other[j].base : own[j].base, own[j].wl,
+                                    gt0(ul[j]) ? other[j].wl : above[j].wl, dth);
+            const T hi = flux_of<T>(lim, uh[j], gt0(uh[j]) ? own[j].base : above[j].base, above[j].wl,
+                                    gt0(uh[j]) ? own[j].wl : beyond[j], dth);
+            upd = fmadd(dth, hi - lo, upd);
+        }
+        const T qn = (Q[c] - upd) * scale;
+        Qn[c] = qn;
+        acc_add(dacc, qn, err);
+        tmax = vmax(tmax, qn);
     }
     if (tmax > -INFINITY) mx = fmax(mx, (double)tmax);
 }
@@ -1486,7 +1404,7 @@ __device__ __forceinline__ void faces_old_body(const Model& m, const Bufs& b, co
         if (Llo < 0 || Llo >= nold) continue;
         if ((fX & OM_GHOST) && is_halo(om, Llo)) continue;
         T f = (T)0;
-        if (gt0(u) || lt0(u)) {
+        if (nonzero(u)) {
             const bool up = gt0(u);  // the upwind cell is Llo, else X
             const int y = up ? Llo : X;
             // the jump across the face beyond the upwind cell
@@ -1495,7 +1413,7 @@ __device__ __forceinline__ void faces_old_body(const Model& m, const Bufs& b, co
             const T Py = up ? Q[Llo] : P0;
             const T S = fmadd(-(T)m.inv_2h[j], (static_cast<const T*>(b.wg) + j * cap)[y], tg[y]);
             f = u * fmadd(-dt, S, Py);
-            if (lim != LIM_NONE && (gt0(W) || lt0(W))) {
+            if (lim != LIM_NONE && nonzero(W)) {
                 const T au = abs_bits(u);
                 f = fmadd(half_nonneg(au) * fmadd(-(T)pick_of<N>(v.dth, j), au, (T)1), limited_wave<T>(lim, W, Wb), f);
             }
@@ -1616,9 +1534,10 @@ __device__ __forceinline__ void clear_marks(const Bufs& b, const StepView& v, lo
 
 // ------------------------------------------------------------------ prune
 
-// keep[c] = (p_c > p*) for the active cells: the significant cells S.
+// keep[c] = (p_c > p*) for the active cells: the significant cells S. (all: a
+// re-sort, which keeps every active cell and, with them, every halo cell.)
 template <typename T>
-__device__ __forceinline__ void prune_mark_body(const Model& m, const Bufs& b, const StepView& v) {
+__device__ __forceinline__ void prune_mark_body(const Model& m, const Bufs& b, const StepView& v, bool all = false) {
     const double pstar = m.thr_rel * v.maxq;
     const Above<T> above(pstar);
     const T* Q = static_cast<const T*>(b.q[v.pb]);
@@ -1626,7 +1545,7 @@ __device__ __forceinline__ void prune_mark_body(const Model& m, const Bufs& b, c
 #pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
-        if (c < v.N) b.keep[c] = !is_halo(om, c) && above(Q[c]);
+        if (c < v.N) b.keep[c] = !is_halo(om, c) && (all || above(Q[c]));
     }
 }
 
@@ -1832,10 +1751,12 @@ __device__ __forceinline__ void copy_velocities(const Model& m, const Bufs& b, i
 // power of two that brings the maximum into [1, 2) (their ratios do not
 // change, and the exact sum stays in its window even after a very unlikely
 // measurement); halo cells hold 0. Adds the active cells' digits, maximum and
-// CFL rates.
+// CFL rates. (resort: the order alone changes, not the values, nor what is known to
+// be complete.)
 template <int N, typename T>
 __device__ __forceinline__ void prune_compact_body(const Model& m, const Bufs& b, const StepView& v, Survivors sv,
-                                                   long long (&d)[NDIG], double& mx, double& rmax, int& err) {
+                                                   long long (&d)[NDIG], double& mx, double& rmax, int& err,
+                                                   bool resort = false) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
     T* Qo = static_cast<T*>(b.q[v.pb ^ 1]);
     const unsigned long long* key = b.key[v.g];
@@ -1843,7 +1764,8 @@ __device__ __forceinline__ void prune_compact_body(const Model& m, const Bufs& b
     const unsigned short* om = b.om[v.g];
     unsigned short* omo = b.om[v.g ^ 1];
     const double mq = v.maxq;
-    const double s2 = (mq > 0.0 && isfinite(mq)) ? ldexp(1.0, -ilogb(mq)) : 1.0;
+    const double s2 = (mq > 0.0 && isfinite(mq) && !resort) ? ldexp(1.0, -ilogb(mq)) : 1.0;
+    const unsigned kept_flags = resort ? 0xfffu | OM_COMPLETE : 0xfffu;
     long long ba = sv.base_a, bg = sv.base_g;
     long long c0, c1;
     block_chunk(v.N, c0, c1, v.nb, v.bi);
@@ -1861,7 +1783,7 @@ __device__ __forceinline__ void prune_compact_body(const Model& m, const Bufs& b
                 const T val = (T)((double)Q[c] * s2);
                 keyo[nc] = k;
                 Qo[nc] = val;
-                omo[nc] = (unsigned short)(om[c] & 0xfffu);
+                omo[nc] = (unsigned short)(om[c] & kept_flags);
                 copy_velocities<N, T>(m, b, v.g, c, nc);
                 b.map[c] = (int)nc;
                 acc_add(d, (double)val, err);
@@ -1889,7 +1811,7 @@ __device__ __forceinline__ void prune_compact_body(const Model& m, const Bufs& b
 template <int N, typename T>
 __device__ __forceinline__ void prune_compact_sorted_body(const Model& m, const Bufs& b, const StepView& v,
                                                           long long (&d)[NDIG], double& mx, double& rmax,
-                                                          int& err) {
+                                                          int& err, bool resort) {
     const T* Q = static_cast<const T*>(b.q[v.pb]);
     T* Qo = static_cast<T*>(b.q[v.pb ^ 1]);
     const unsigned long long* key = b.key[v.g];
@@ -1897,7 +1819,8 @@ __device__ __forceinline__ void prune_compact_sorted_body(const Model& m, const 
     const unsigned short* om = b.om[v.g];
     unsigned short* omo = b.om[v.g ^ 1];
     const double mq = v.maxq;
-    const double s2 = (mq > 0.0 && isfinite(mq)) ? ldexp(1.0, -ilogb(mq)) : 1.0;
+    const double s2 = (mq > 0.0 && isfinite(mq) && !resort) ? ldexp(1.0, -ilogb(mq)) : 1.0;
+    const unsigned kept_flags = resort ? 0xfffu | OM_COMPLETE : 0xfffu;
 #pragma unroll 1
     for (WarpRuns r(v.N, v.nb, v.bi); r.next();) {
         const long long c = r.c;
@@ -1911,7 +1834,7 @@ __device__ __forceinline__ void prune_compact_sorted_body(const Model& m, const 
         if (st == 1) {
             const T val = (T)((double)Q[c] * s2);
             Qo[nc] = val;
-            omo[nc] = (unsigned short)(om[c] & 0xfffu);
+            omo[nc] = (unsigned short)(om[c] & kept_flags);
             acc_add(d, (double)val, err);
             mx = fmax(mx, (double)val);
             rmax = fmax(rmax, b.rate[v.g][c]);

@@ -31,13 +31,19 @@ void GBEES_ENTRY(Kernels* k) {
     constexpr int N = GBEES_DIM;
     k->persist = (void*)k_persistent<N, Real>;
     k->batch = (void*)k_batch<N, Real>;
-    k->pre[0] = (void*)k_waves_list<N, Real>;
+    k->pre[0] = (void*)k_grow_mark<Real>;
     k->pre[1] = (void*)k_grow_list<N, Real>;
     k->pre[2] = (void*)k_halo<N, Real, 1>;
     k->npre = 3;
-    k->post[0] = (void*)k_faces<N, Real>;
-    k->post[1] = (void*)k_apply<N, Real>;
+    k->post[0] = (void*)k_waves<N, Real>;
+#if GBEES_PREC == 64
+    k->post[1] = (void*)k_faces<N, Real>;
+    k->post[2] = (void*)k_apply<N, Real>;
+    k->npost = 3;
+#else
+    k->post[1] = (void*)k_update<N, Real>;
     k->npost = 2;
+#endif
 }
 
 }  // namespace gbees
