@@ -48,8 +48,10 @@ struct alignas(16) Slot {
     long long val;  // cell index (low 32 bits used)
 };
 
-// Scalars that live on the device so that a whole step needs no host round trip.
-struct alignas(256) DevScalars {
+// The part of the state that the kernels of a step read when they start: two
+// lines of memory, the counters that a step adds to by atomics and the words that
+// stay as they are while a kernel runs. Copied by each block as a whole (block_head).
+struct alignas(256) StepHead {
     long long N;          // pool entries, active cells and halo cells (grows during grow)
     long long N_prev;     // pool entries before the current grow
     long long N_new;      // pool entries surviving the current prune
@@ -59,26 +61,38 @@ struct alignas(256) DevScalars {
     long long n_act;      // halo cells made active by the current grow (listed in map)
     long long n_glist;    // cells listed for the current grow (listed form)
     long long N_sorted;   // entries that the last sort put in order
-    double t;             // time
-    double t_target;      // end of the current propagate call
-    double dt;            // last step
-    unsigned long long maxrate_bits;      // max CFL rate over the cells (non-negative double bits)
-    unsigned long long maxq_ord;          // order key of the running max of Q
-    double maxq;          // max of Q after the last finalisation
-    double w;             // (prod h) * sum Q at the last finalisation
-    double scale;         // 1 / w, applied by the next step
-    long long acc[NDIG];  // exact sum of Q
-    long long step;       // steps since init
-    long long steps_call; // steps of the current propagate call
+    unsigned long long maxrate_bits;  // max CFL rate over the cells (non-negative double bits)
+    unsigned long long maxq_ord;      // order key of the running max of Q
+    unsigned long long tmp_ord;       // scratch maximum (init)
+    long long steps_call;    // steps of the current propagate call
     long long updates_call;  // cell updates of the current propagate call
-    long long lookups_fallback;  // hashtable lookups of the flux update (none: every stencil cell is linked)
+    long long step;          // steps since init
+    unsigned int ticket;  // last-block election
+    int step_last;        // the step lands on t_target
+
     int pbuf;             // current Q buffer
     int gen;              // current key/link buffer
     int done;             // t reached t_target
     int error;            // first error status (0 = none)
     int prune_now;        // the step just taken is a prune step (1), or its pool is to be sorted (RESORT)
-    unsigned int ticket;  // last-block election
-    unsigned long long tmp_ord;  // scratch maximum (init)
+    int sort_passes;      // 8-bit digits of the current sort's codes
+    double maxq;          // max of Q after the last finalisation
+    double w;             // (prod h) * sum Q at the last finalisation
+    double scale;         // 1 / w, applied by the next step
+    // the current step (written by the last block of the link kernel)
+    double step_dt;         // dt of the step being taken
+    double step_t_new;      // time after it
+    double coef_dth[MAXN];  // dt / h_j
+    double t;               // time
+    double t_target;        // end of the current propagate call
+};
+static_assert(sizeof(StepHead) == 256, "copied as 32 words of 8 bytes");
+
+// Scalars that live on the device so that a whole step needs no host round trip.
+struct DevScalars : StepHead {
+    double dt;            // last step
+    long long acc[NDIG];  // exact sum of Q
+    long long lookups_fallback;  // hashtable lookups of the flux update (none: every stencil cell is linked)
     long long loop_iter;  // iterations of the device-side step loop in the current graph launch
     long long graph_kernels;  // kernels executed by graph launches (counted on the device)
     // grid barrier of the persistent kernel and of a team of a batched launch:
@@ -94,17 +108,26 @@ struct alignas(256) DevScalars {
     // halo, link, faces, apply, prune, step scalars) and the steps they cover
     long long phase_cycles[8];
     long long phase_steps;
-    // the current step (written by the last block of the link kernel)
-    double step_dt;       // dt of the step being taken
-    double step_t_new;    // time after it
-    int step_last;        // the step lands on t_target
-    int sort_passes;      // 8-bit digits of the current sort's codes
     unsigned sort_lo[MAXN], sort_hi[MAXN];  // range of the key fields to sort
-    double coef_dth[MAXN];  // dt / h_j
     long long mom[28][NDIG];     // exact sums for moments
     double mom_mean[MAXN];       // mean, input of the covariance pass
     double mom_out[28];          // moments times prod h
 };
+static_assert(sizeof(DevScalars) == 2304, "part of every workspace");
+
+// The head of the state as it was when the block began, for all its threads. One
+// warp of each block reads it, two lines in one load. With every thread reading the
+// dozen scalars that it needs, the 10^4 warps of a resident wave queued at the one L2
+// slice that holds them, 25 to 40 us in each of a step's kernels (6.5e5 entries in
+// six dimensions: the sweep of k_grow_mark took 43 us, now 7.5; k_halo 54, now 13).
+__device__ __forceinline__ const StepHead& block_head(const DevScalars* sc) {
+    __shared__ StepHead h;
+    if (threadIdx.x < sizeof(StepHead) / 8)
+        reinterpret_cast<unsigned long long*>(&h)[threadIdx.x] =
+            reinterpret_cast<const volatile unsigned long long*>(static_cast<const StepHead*>(sc))[threadIdx.x];
+    __syncthreads();
+    return h;
+}
 
 // Everything a kernel needs to know about the model and the grid (by value).
 struct Model {

@@ -43,9 +43,9 @@ template <int N, int W, typename T>
 __global__ void __launch_bounds__(THREADS, 4) k_link(const __grid_constant__ Model m, const __grid_constant__ Bufs b,
                                                      int step) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->error) return;
-    if (step > 0 && *(volatile int*)&sc->done) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (h.error || (step > 0 && h.done)) return;
+    const StepView v = view_of(m, &h);
     double r;
     if constexpr (W == 1) {
         // few: at most four rounds of all warps with one or a few entries each
@@ -317,7 +317,8 @@ template <int N, typename T>
 __global__ void __launch_bounds__(THREADS, 4) k_init_write(const __grid_constant__ Model m, Bufs b,
                                                         const __grid_constant__ InitBox bx) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->error) return;
+    const StepHead& h = block_head(sc);
+    if (h.error) return;
     __shared__ double s_tab[AXIS_MAX];
     const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     long long c0, c1;
@@ -473,10 +474,10 @@ __device__ __forceinline__ void grow_rates(DevScalars* sc, double r) {
 template <int N, typename T, int STEP>
 __global__ void __launch_bounds__(THREADS) k_halo(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->error) return;
-    if (STEP && *(volatile int*)&sc->done) return;
-    const StepView v = view_of(m, sc);
-    halo_body<N, T>(m, b, v, v.N_prev, v.N, *(volatile long long*)&sc->n_act);
+    const StepHead& h = block_head(sc);
+    if (h.error || (STEP && h.done)) return;
+    const StepView v = view_of(m, &h);
+    halo_body<N, T>(m, b, v, v.N_prev, v.N, h.n_act);
     if (last_block(sc)) {
         if (threadIdx.x == 0) {
             sc->N = min(sc->N + sc->n_halo, m.cap);
@@ -530,8 +531,9 @@ __device__ __forceinline__ void finish_step(const Model& m, DevScalars* sc, cons
 template <typename T>
 __global__ void __launch_bounds__(THREADS) k_grow_mark(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    const StepView v = view_of(m, &h);
     const Above<T> above(m.thr_rel * v.maxq);
     for (WarpRuns wr(v.N_prev, v.nb, v.bi); wr.next();)
         if (wr.c < v.N_prev) grow_list_mark<T>(b, v, above, wr.c);
@@ -540,25 +542,28 @@ __global__ void __launch_bounds__(THREADS) k_grow_mark(const Model m, Bufs b) {
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_grow_list(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    const StepView v = view_of(m, sc);
-    grow_rates(sc, grow_list_body<N, T>(m, b, v));
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    const StepView v = view_of(m, &h);
+    grow_rates(sc, grow_list_body<N, T>(m, b, v, h.n_glist));
 }
 
 // Update, pass 1 (after the links, with dt): jumps and transverse terms.
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS, sizeof(T) == 8 ? 2 : 3) k_waves(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    waves_body<N, T>(m, b, view_of(m, sc));
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    waves_body<N, T>(m, b, view_of(m, &h));
 }
 
 // Update, pass 2 (FP64): the flux through every face that touches an active cell.
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS, 3) k_faces(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    faces_body<N, T>(m, b, view_of(m, sc));
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    faces_body<N, T>(m, b, view_of(m, &h));
 }
 
 // The end of an update: exact per-block partial sums and maximum for the next
@@ -578,8 +583,9 @@ __device__ __forceinline__ void end_update(const Model& m, const Bufs& b, const 
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_apply(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    const StepView v = view_of(m, &h);
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
     double mx = -INFINITY;
     int err = 0;
@@ -591,8 +597,9 @@ __global__ void __launch_bounds__(THREADS) k_apply(const Model m, Bufs b) {
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS, 2) k_update(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->done | *(volatile int*)&sc->error) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (h.done | h.error) return;
+    const StepView v = view_of(m, &h);
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
     double mx = -INFINITY;
     int err = 0;
@@ -616,9 +623,10 @@ template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_correct(const __grid_constant__ Model m, Bufs b,
                                                      const __grid_constant__ Meas ms) {
     DevScalars* sc = b.sc;
-    if (*(volatile int*)&sc->error) return;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const StepHead& h = block_head(sc);
+    if (h.error) return;
+    const long long ncell = min(h.N, m.cap);
+    const int g = h.gen, pb = h.pbuf;
     T* Q = static_cast<T*>(b.q[pb]);
     const unsigned long long* key = b.key[g];
     T tmax = -INFINITY;
@@ -660,38 +668,39 @@ __global__ void __launch_bounds__(THREADS) k_correct(const __grid_constant__ Mod
 
 // ------------------------------------------------------------------ prune
 
-__device__ __forceinline__ bool prune_due(const DevScalars* sc) {
-    return *(volatile int*)&sc->prune_now && !*(volatile int*)&sc->error;
-}
+__device__ __forceinline__ bool prune_due(const StepHead& h) { return h.prune_now && !h.error; }
 
 // The prune kernels run to re-sort a grown pool, keeping every cell (finish_step).
-__device__ __forceinline__ bool resort_due(const DevScalars* sc) { return *(volatile int*)&sc->prune_now == RESORT; }
+__device__ __forceinline__ bool resort_due(const StepHead& h) { return h.prune_now == RESORT; }
 
 // Prune (Algorithm 3), pass 1: mark the significant cells S.
 template <typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_mark(const Model m, Bufs b) {
-    if (!prune_due(b.sc)) return;
+    const StepHead& h = block_head(b.sc);
+    if (!prune_due(h)) return;
     if (blockIdx.x == 0 && threadIdx.x < MAXN) {  // read and added to from the status pass on
         b.sc->sort_lo[threadIdx.x] = ~0u;
         b.sc->sort_hi[threadIdx.x] = 0u;
     }
-    prune_mark_body<T>(m, b, view_of(m, b.sc), resort_due(b.sc));
+    prune_mark_body<T>(m, b, view_of(m, &h), resort_due(h));
 }
 
 // Prune, pass 2: mark the downwind set D(S) of every significant cell (the
 // directional rule of Sec. 3.3).
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_scatter(const Model m, Bufs b) {
-    if (!prune_due(b.sc) || resort_due(b.sc)) return;
-    prune_scatter_body<N, T>(m, b, view_of(m, b.sc));
+    const StepHead& h = block_head(b.sc);
+    if (!prune_due(h) || resort_due(h)) return;
+    prune_scatter_body<N, T>(m, b, view_of(m, &h));
 }
 
 // Prune, pass 3: the status of every entry (active, halo or dropped) and the
 // per-block counts of the survivors.
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_prune_count(const Model m, Bufs b) {
-    if (!prune_due(b.sc)) return;
-    prune_count_body<N, true>(m, b, view_of(m, b.sc));
+    const StepHead& h = block_head(b.sc);
+    if (!prune_due(h)) return;
+    prune_count_body<N, true>(m, b, view_of(m, &h));
 }
 
 // Prune, pass 4: write the survivors into the other buffer set in the order
@@ -700,8 +709,9 @@ __global__ void __launch_bounds__(THREADS) k_prune_count(const Model m, Bufs b) 
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_compact_sorted(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (!prune_due(sc)) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (!prune_due(h)) return;
+    const StepView v = view_of(m, &h);
     const Survivors sv = block_offsets(b, v.nb, v.bi);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->N_new = sv.total_a + sv.total_g;
@@ -710,7 +720,7 @@ __global__ void __launch_bounds__(THREADS) k_prune_compact_sorted(const Model m,
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
     double mx = -INFINITY, rmax = 0.0;
     int err = 0;
-    prune_compact_sorted_body<N, T>(m, b, v, d, mx, rmax, err, resort_due(sc));
+    prune_compact_sorted_body<N, T>(m, b, v, d, mx, rmax, err, resort_due(h));
     if (err) set_error(sc, ST_EDEGENERATE);
     block_partial(b.part, d, mx, rmax);
 }
@@ -721,8 +731,9 @@ __global__ void __launch_bounds__(THREADS) k_prune_compact_sorted(const Model m,
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_compact(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
-    if (!prune_due(sc)) return;
-    const StepView v = view_of(m, sc);
+    const StepHead& h = block_head(sc);
+    if (!prune_due(h)) return;
+    const StepView v = view_of(m, &h);
     const Survivors sv = block_offsets(b, v.nb, v.bi);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->N_new = sv.total_a + sv.total_g;
@@ -731,7 +742,7 @@ __global__ void __launch_bounds__(THREADS) k_prune_compact(const Model m, Bufs b
     long long d[NDIG] = {0, 0, 0, 0, 0, 0};
     double mx = -INFINITY, rmax = 0.0;
     int err = 0;
-    prune_compact_body<N, T>(m, b, v, sv, d, mx, rmax, err, resort_due(sc));
+    prune_compact_body<N, T>(m, b, v, sv, d, mx, rmax, err, resort_due(h));
     if (err) set_error(sc, ST_EDEGENERATE);
     block_partial(b.part, d, mx, rmax);
 }
@@ -764,11 +775,12 @@ __device__ __forceinline__ void finish_prune(const Model& m, DevScalars* sc, con
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_prune_relink(const Model m, Bufs b, int nblk_compact) {
     DevScalars* sc = b.sc;
-    if (!prune_due(sc)) return;
-    prune_relink_body<N>(m, b, view_of(m, sc));
+    const StepHead& h = block_head(sc);
+    if (!prune_due(h)) return;
+    prune_relink_body<N>(m, b, view_of(m, &h));
     if (last_block(sc)) {
         Combined cp = combine_partials(b.part, nblk_compact);
-        if (threadIdx.x == 0) finish_prune(m, sc, cp, *(volatile long long*)&sc->N_new);
+        if (threadIdx.x == 0) finish_prune(m, sc, cp, h.N_new);
     }
 }
 
@@ -780,12 +792,12 @@ __global__ void __launch_bounds__(THREADS) k_prune_relink(const Model m, Bufs b,
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_readout(const Model m, Bufs b, int* __restrict__ idx,
                                                      double* __restrict__ p) {
-    DevScalars* sc = b.sc;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const StepHead& h = block_head(b.sc);
+    const long long ncell = min(h.N, m.cap);
+    const int g = h.gen, pb = h.pbuf;
     const T* Q = static_cast<const T*>(b.q[pb]);
     const unsigned short* om = b.om[g];
-    const double w = *(volatile double*)&sc->w;
+    const double w = h.w;
     long long c0, c1;
     block_chunk(ncell, c0, c1);
     long long base = b.blk[blockIdx.x];
@@ -821,10 +833,11 @@ __global__ void __launch_bounds__(THREADS) k_moments(const Model m, Bufs b) {
     constexpr int SLOTS = mom_slots<N, PASS>(), ROWS = (SLOTS + MOM_SUMS - 1) / MOM_SUMS;
     constexpr int K = SLOTS < MOM_SUMS ? SLOTS : MOM_SUMS;
     DevScalars* sc = b.sc;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const StepHead& h = block_head(sc);
+    const long long ncell = min(h.N, m.cap);
+    const int g = h.gen, pb = h.pbuf;
     const T* Q = static_cast<const T*>(b.q[pb]);
-    const double w = *(volatile double*)&sc->w;
+    const double w = h.w;
     const int row = ROWS > 1 ? blockIdx.y : 0;
     double mean[N];
 #pragma unroll

@@ -230,8 +230,9 @@ struct KeyCode {
 // and only an all-ones key has an all-ones Morton code, a key no cell that
 // survives a prune has.
 __global__ void __launch_bounds__(THREADS) k_sort_init(const Model m, Bufs b) {
-    if (!prune_due(b.sc)) return;
-    const StepView v = view_of(m, b.sc);
+    const StepHead& h = block_head(b.sc);
+    if (!prune_due(h)) return;
+    const StepView v = view_of(m, &h);
     const SortBufs sb = sort_bufs(b, v.g, v.pb);
     const unsigned long long* key = b.key[v.g];
     long long c0, c1;
@@ -261,12 +262,13 @@ __global__ void __launch_bounds__(THREADS) k_sort_init(const Model m, Bufs b) {
 // False: nothing to do in this pass.
 __device__ __forceinline__ bool sort_pass(const Model& m, const Bufs& b, int pass, long long count, long long& n,
                                           SortBufs& sb) {
+    const StepHead& h = block_head(b.sc);
     if (count < 0) {
-        if (!prune_due(b.sc) || pass >= *(volatile int*)&b.sc->sort_passes) return false;
-        count = min(*(volatile long long*)&b.sc->N, m.cap);
+        if (!prune_due(h) || pass >= h.sort_passes) return false;
+        count = min(h.N, m.cap);
     }
     n = count;
-    sb = sort_bufs(b, *(volatile int*)&b.sc->gen, *(volatile int*)&b.sc->pbuf);
+    sb = sort_bufs(b, h.gen, h.pbuf);
     return true;
 }
 
@@ -403,10 +405,11 @@ __global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b,
 // New index of every survivor: its rank in the sorted order (survivors sort
 // before the dropped entries); -1 for the dropped.
 __global__ void __launch_bounds__(THREADS) k_sort_map(const Model m, Bufs b) {
-    if (!prune_due(b.sc)) return;
-    const StepView v = view_of(m, b.sc);
+    const StepHead& h = block_head(b.sc);
+    if (!prune_due(h)) return;
+    const StepView v = view_of(m, &h);
     const SortBufs sb = sort_bufs(b, v.g, v.pb);
-    const unsigned int* val = sb.val[b.sc->sort_passes & 1];
+    const unsigned int* val = sb.val[h.sort_passes & 1];
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < v.N; r += (long long)gridDim.x * blockDim.x) {
         const unsigned int c = val[r];
         b.map[c] = b.keep[c] ? (int)r : -1;
@@ -415,9 +418,9 @@ __global__ void __launch_bounds__(THREADS) k_sort_map(const Model m, Bufs b) {
 
 // Per-block counts of the active cells (read-out, first pass).
 __global__ void __launch_bounds__(THREADS) k_readout_count(const Model m, Bufs b) {
-    DevScalars* sc = b.sc;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const unsigned short* om = b.om[*(volatile int*)&sc->gen];
+    const StepHead& h = block_head(b.sc);
+    const long long ncell = min(h.N, m.cap);
+    const unsigned short* om = b.om[h.gen];
     long long c0, c1;
     block_chunk(ncell, c0, c1);
     int cnt = 0;
@@ -442,9 +445,9 @@ __global__ void __launch_bounds__(THREADS) k_readout_rank(const Model m, Bufs b,
                                                           double* __restrict__ p) {
     constexpr int TILE = 1024;
     __shared__ unsigned long long s_key[TILE];
-    DevScalars* sc = b.sc;
-    const int ncell = (int)min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const StepHead& h = block_head(b.sc);
+    const int ncell = (int)min(h.N, m.cap);
+    const int g = h.gen, pb = h.pbuf;
     const unsigned short* om = b.om[g];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = t / RANK_LANES, sub = t % RANK_LANES;
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(THREADS) k_readout_rank(const Model m, Bufs b,
         unpack_key<N>(m, k, I);
 #pragma unroll
         for (int j = 0; j < N; ++j) idx[(long long)rank * N + j] = I[j];
-        p[rank] = __ddiv_rn((double)static_cast<const T*>(b.q[pb])[c], *(volatile double*)&sc->w);
+        p[rank] = __ddiv_rn((double)static_cast<const T*>(b.q[pb])[c], h.w);
     }
 }
 
@@ -477,21 +480,21 @@ __global__ void __launch_bounds__(THREADS) k_readout_rank(const Model m, Bufs b,
 // sorted order.
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_readout_range(const Model m, Bufs b) {
-    DevScalars* sc = b.sc;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen;
+    const StepHead& h = block_head(b.sc);
+    const long long ncell = min(h.N, m.cap);
+    const int g = h.gen;
     FieldRange<N> range;
     for (WarpRuns r(ncell); r.next();)
         if (r.c < ncell && !is_halo(b.om[g], r.c)) range.see(m, b.key[g][r.c]);
-    range.fold(sc);
+    range.fold(b.sc);
 }
 
 __global__ void __launch_bounds__(THREADS) k_readout_keys(const Model m, Bufs b) {
-    DevScalars* sc = b.sc;
-    const long long ncell = min(*(volatile long long*)&sc->N, m.cap);
-    const int g = *(volatile int*)&sc->gen;
-    const SortBufs sb = sort_bufs(b, g, *(volatile int*)&sc->pbuf);
-    const KeyCode code(m, sc);
+    const StepHead& h = block_head(b.sc);
+    const long long ncell = min(h.N, m.cap);
+    const int g = h.gen;
+    const SortBufs sb = sort_bufs(b, g, h.pbuf);
+    const KeyCode code(m, b.sc);
     long long c0, c1;
     block_chunk(ncell, c0, c1);
     long long base = b.blk[blockIdx.x];
@@ -511,10 +514,10 @@ __global__ void __launch_bounds__(THREADS) k_readout_keys(const Model m, Bufs b)
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_readout_order(const Model m, Bufs b, int passes, long long count,
                                                            int* __restrict__ idx, double* __restrict__ p) {
-    DevScalars* sc = b.sc;
-    const int g = *(volatile int*)&sc->gen, pb = *(volatile int*)&sc->pbuf;
+    const StepHead& h = block_head(b.sc);
+    const int g = h.gen, pb = h.pbuf;
     const unsigned int* val = sort_bufs(b, g, pb).val[passes & 1];
-    const double w = *(volatile double*)&sc->w;
+    const double w = h.w;
     for (WarpRuns r(count); r.next();) {
         if (r.c >= count) continue;
         const unsigned c = val[r.c];

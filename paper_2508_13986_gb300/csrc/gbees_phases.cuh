@@ -41,16 +41,17 @@ struct StepView {
     unsigned fresh;    // flag of the halo cells that this step makes active (step loop of a small grid)
 };
 
-__device__ __forceinline__ StepView view_of(const Model& m, DevScalars* sc) {
+// (volatile: the step loop reads the state itself, which other blocks change)
+__device__ __forceinline__ StepView view_of(const Model& m, const volatile StepHead* h) {
     StepView v;
-    v.N = min(*(volatile long long*)&sc->N, m.cap);
-    v.N_prev = min(*(volatile long long*)&sc->N_prev, m.cap);
-    v.pb = *(volatile int*)&sc->pbuf;
-    v.g = *(volatile int*)&sc->gen;
-    v.maxq = *(volatile double*)&sc->maxq;
-    v.scale = *(volatile double*)&sc->scale;
-    for (int j = 0; j < MAXN; ++j) v.dth[j] = *(volatile double*)&sc->coef_dth[j];
-    v.dt = *(volatile double*)&sc->step_dt;
+    v.N = min((long long)h->N, m.cap);
+    v.N_prev = min((long long)h->N_prev, m.cap);
+    v.pb = h->pbuf;
+    v.g = h->gen;
+    v.maxq = h->maxq;
+    v.scale = h->scale;
+    for (int j = 0; j < MAXN; ++j) v.dth[j] = h->coef_dth[j];
+    v.dt = h->step_dt;
     v.nb = gridDim.x;
     v.bi = blockIdx.x;
     v.fresh = OM_NEW;
@@ -284,11 +285,10 @@ __device__ __forceinline__ void grow_list_mark(const Bufs& b, const StepView& v,
 // threads of the grid; the thread of a cell's first candidate marks it
 // complete (only its own flag bit, and nothing else writes that word now).
 template <int N, typename T>
-__device__ __forceinline__ double grow_list_body(const Model& m, const Bufs& b, const StepView& v) {
+__device__ __forceinline__ double grow_list_body(const Model& m, const Bufs& b, const StepView& v, long long nl) {
     constexpr int K = GROW_K<N>;
     const int* glist = static_cast<const int*>(b.fl);
     unsigned short* om = b.om[v.g];
-    const long long nl = *(volatile long long*)&b.sc->n_glist;
     GrowWork gw;
     const long long items = nl * K;
     const long long tid = (long long)v.bi * blockDim.x + threadIdx.x;
