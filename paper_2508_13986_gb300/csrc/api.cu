@@ -470,15 +470,15 @@ void launch_list(gbees_ctx* ctx, void* const* f, const int* grids, int nf) {
 // survivors are sorted into the configured storage order (key or Morton order
 // of the cell indices), which keeps the neighbour gathers of a sweep close
 // together; a grid that fits in L2 keeps its order (stream compaction).
-constexpr int kPruneKernelsSorted = 3 + 1 + 3 * SORT_PASSES + 1 + 2;
+constexpr int kPruneKernelsSorted = 3 + 1 + 3 * SORT_PASSES + 1 + 1;
 constexpr int kPruneKernelsPlain = 3 + 1 + 1;
 
 bool sorts(const gbees_ctx* ctx) { return ctx->cfg.storage_order != GBEES_ORDER_NONE; }
 
-// Blocks of the sort kernels for a pool of N entries: about 16 tiles of
-// THREADS entries per block, at most SORT_BLOCKS.
+// Blocks of the sort kernels for a pool of N entries: two tiles per block (a tile is
+// a chain of dependent work: the fewer in a row, the better), at most SORT_BLOCKS.
 int sort_blocks(long long N) {
-    const long long per = (long long)THREADS * 16;
+    const long long per = SORT_TILE * 2;
     return (int)std::max(1ll, std::min<long long>(SORT_BLOCKS, (N + per - 1) / per));
 }
 
@@ -505,11 +505,11 @@ void launch_prune(gbees_ctx* ctx) {
                 k_sort_scatter<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, -1);
             }
             k_sort_map<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-            k_prune_compact_sorted<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+            k_prune_move<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
         } else {
             k_prune_compact<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
+            k_prune_relink<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, G);
         }
-        k_prune_relink<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, G);
     });
 }
 
@@ -675,11 +675,11 @@ void graph_nodes(gbees_ctx* ctx, GraphBuilder& gb, cudaGraph_t body, cudaGraphCo
             q = gb.add(pb, q, (void*)k_sort_scatter, Gs, THREADS, pass_args);
         }
         q = gb.add(pb, q, (void*)k_sort_map, G, THREADS, mb);
-        q = gb.add(pb, q, (void*)k_prune_compact_sorted<N, T>, G, THREADS, mb);
+        gb.add(pb, q, (void*)k_prune_move<N, T>, G, THREADS, mb);
     } else {
         q = gb.add(pb, q, (void*)k_prune_compact<N, T>, G, THREADS, mb);
+        gb.add(pb, q, (void*)k_prune_relink<N>, G, THREADS, relink_args);
     }
-    gb.add(pb, q, (void*)k_prune_relink<N>, G, THREADS, relink_args);
 }
 
 // Build and instantiate the step-loop graph of this context. False if the

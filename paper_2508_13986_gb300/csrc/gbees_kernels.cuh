@@ -703,31 +703,9 @@ __global__ void __launch_bounds__(THREADS) k_prune_count(const Model m, Bufs b) 
     prune_count_body<N, true>(m, b, view_of(m, &h));
 }
 
-// Prune, pass 4: write the survivors into the other buffer set in the order
-// of the radix sort (Morton order of the cell indices), active cells first, with exact partial
-// sums, maximum and CFL rates for the step scalars.
-template <int N, typename T>
-__global__ void __launch_bounds__(THREADS) k_prune_compact_sorted(const Model m, Bufs b) {
-    DevScalars* sc = b.sc;
-    const StepHead& h = block_head(sc);
-    if (!prune_due(h)) return;
-    const StepView v = view_of(m, &h);
-    const Survivors sv = block_offsets(b, v.nb, v.bi);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        sc->N_new = sv.total_a + sv.total_g;
-        sc->NA_new = sv.total_a;
-    }
-    long long d[NDIG] = {0, 0, 0, 0, 0, 0};
-    double mx = -INFINITY, rmax = 0.0;
-    int err = 0;
-    prune_compact_sorted_body<N, T>(m, b, v, d, mx, rmax, err, resort_due(h));
-    if (err) set_error(sc, ST_EDEGENERATE);
-    block_partial(b.part, d, mx, rmax);
-}
-
 // Prune, pass 4 without a sort: write the survivors into the other buffer set
 // in storage order, active cells first, then the halo (stream compaction), with
-// the same partials as the sorted form.
+// exact partial sums, maximum and CFL rates for the step scalars.
 template <int N, typename T>
 __global__ void __launch_bounds__(THREADS) k_prune_compact(const Model m, Bufs b) {
     DevScalars* sc = b.sc;
@@ -781,6 +759,31 @@ __global__ void __launch_bounds__(THREADS) k_prune_relink(const Model m, Bufs b,
     if (last_block(sc)) {
         Combined cp = combine_partials(b.part, nblk_compact);
         if (threadIdx.x == 0) finish_prune(m, sc, cp, h.N_new);
+    }
+}
+
+// Prune, passes 4 and 5 after a sort, in one: the survivors move into the other
+// buffer set in the order of the sort, with their links and hashtable entries; the
+// same partials, and the last block ends the prune.
+template <int N, typename T>
+__global__ void __launch_bounds__(THREADS) k_prune_move(const Model m, Bufs b) {
+    DevScalars* sc = b.sc;
+    const StepHead& h = block_head(sc);
+    if (!prune_due(h)) return;
+    const StepView v = view_of(m, &h);
+    const Survivors sv = block_offsets(b, v.nb, v.bi);
+    long long d[NDIG] = {0, 0, 0, 0, 0, 0};
+    double mx = -INFINITY, rmax = 0.0;
+    int err = 0;
+    prune_move_body<N, T>(m, b, v, sv.total_a + sv.total_g, d, mx, rmax, err, resort_due(h));
+    if (err) set_error(sc, ST_EDEGENERATE);
+    block_partial(b.part, d, mx, rmax);
+    if (last_block(sc)) {
+        Combined cp = combine_partials(b.part, gridDim.x);
+        if (threadIdx.x == 0) {
+            sc->NA_new = sv.total_a;
+            finish_prune(m, sc, cp, sv.total_a + sv.total_g);
+        }
     }
 }
 

@@ -185,6 +185,8 @@ __global__ void __launch_bounds__(THREADS) k_new_grid(const Model m, Bufs b, dou
 
 constexpr int SORT_BLOCKS = 1024;  // blocks of the sort kernels at most (histogram rows)
 constexpr int SORT_PASSES = 8;     // digits of a full code
+constexpr int SORT_ITEMS = 4;      // elements per thread of a tile
+constexpr int SORT_TILE = THREADS * SORT_ITEMS;
 
 struct SortBufs {
     unsigned long long* key[2];
@@ -285,12 +287,19 @@ __global__ void __launch_bounds__(THREADS) k_sort_hist(const Model m, Bufs b, in
     __syncthreads();
     long long c0, c1;
     block_chunk(n, c0, c1);
-    const int lane = threadIdx.x & 31;
-    for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
-        const long long c = t0 + threadIdx.x;
-        const int d = c < c1 ? (int)((in[c] >> (8 * pass)) & 255u) : 256;
-        const unsigned same = __match_any_sync(0xffffffffu, d);
-        if (d < 256 && (same & ((1u << lane) - 1u)) == 0) atomicAdd(&cnt[d], (unsigned)__popc(same));
+    const int lane = threadIdx.x & 31, shift = 8 * pass;
+    for (long long t0 = c0 + threadIdx.x; t0 - threadIdx.x < c1; t0 += SORT_TILE) {
+        int d[SORT_ITEMS];
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            const long long c = t0 + i * THREADS;
+            d[i] = c < c1 ? (int)((in[c] >> shift) & 255u) : 256;
+        }
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            const unsigned same = __match_any_sync(0xffffffffu, d[i]);
+            if (d[i] < 256 && (same & ((1u << lane) - 1u)) == 0) atomicAdd(&cnt[d[i]], (unsigned)__popc(same));
+        }
     }
     __syncthreads();
     for (int d = threadIdx.x; d < 256; d += blockDim.x) b.sorthist[(long long)d * gridDim.x + blockIdx.x] = cnt[d];
@@ -339,19 +348,22 @@ __global__ void __launch_bounds__(THREADS) k_sort_scan(const Model m, Bufs b, in
     if (threadIdx.x == 0) reinterpret_cast<unsigned int*>(b.part)[blockIdx.x] = total;
 }
 
-// Stable scatter of a pass: every block walks its chunk in tiles of one
-// element per thread; an element's place is its digit's offset for the block,
-// plus the elements of that digit in earlier tiles, earlier warps of the tile
-// and earlier lanes of its warp.
+// Stable scatter of a pass: every block walks its chunk in tiles of SORT_ITEMS
+// elements per thread (each warp a row of consecutive ones); an element's place is its
+// digit's offset for the block, plus the elements of that digit in earlier tiles, in
+// earlier warps of the tile, and before it in its warp's row. Bound by the chain of a
+// tile (load, count, block barriers): one element per thread and tile, and sixteen tiles
+// to a block, took 44 us at 6.5e5 entries, now 22 (k_sort_hist 22, now 13), and 0.14 ms
+// at 4.9e6, now 0.10.
 __global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b, int pass, long long count) {
     long long n;
     SortBufs sb;
     if (!sort_pass(m, b, pass, count, n, sb)) return;
     static_assert(THREADS == 256, "one thread per digit");
-    __shared__ unsigned int base[256];
     __shared__ unsigned int wcnt[WARPS][256];
     __shared__ unsigned int s_w[WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, src = pass & 1, shift = 8 * pass;
+    unsigned int base;  // place of the next element with digit threadIdx.x
     {
         // the digits' offsets: exclusive prefix of the rows' totals
         const unsigned tot = reinterpret_cast<const unsigned int*>(b.part)[threadIdx.x];
@@ -365,45 +377,54 @@ __global__ void __launch_bounds__(THREADS) k_sort_scatter(const Model m, Bufs b,
         __syncthreads();
         unsigned before = x - tot;
         for (int w = 0; w < wid; ++w) before += s_w[w];
-        base[threadIdx.x] = before + b.sorthist[(long long)threadIdx.x * gridDim.x + blockIdx.x];
+        base = before + b.sorthist[(long long)threadIdx.x * gridDim.x + blockIdx.x];
     }
     long long c0, c1;
     block_chunk(n, c0, c1);
-    for (long long t0 = c0; t0 < c1; t0 += blockDim.x) {
-        for (int i = threadIdx.x; i < WARPS * 256; i += blockDim.x) (&wcnt[0][0])[i] = 0;
-        __syncthreads();
-        const long long c = t0 + threadIdx.x;
-        const bool ok = c < c1;
-        unsigned long long k = 0;
-        unsigned int val = 0;
-        int d = 256 + lane;  // distinct dummies for lanes past the end
-        if (ok) {
-            k = sb.key[src][c];
-            val = sb.val[src][c];
-            d = (int)((k >> shift) & 255u);
+    for (long long t0 = c0; t0 < c1; t0 += SORT_TILE) {
+        unsigned long long k[SORT_ITEMS];
+        unsigned int val[SORT_ITEMS], rank[SORT_ITEMS];
+        int d[SORT_ITEMS];
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            const long long c = t0 + wid * (32 * SORT_ITEMS) + i * 32 + lane;
+            k[i] = c < c1 ? sb.key[src][c] : 0;
+            val[i] = c < c1 ? sb.val[src][c] : 0;
+            d[i] = c < c1 ? (int)((k[i] >> shift) & 255u) : 256;  // 256: past the end
         }
-        const unsigned same = __match_any_sync(0xffffffffu, d);
-        const int rank = __popc(same & ((1u << lane) - 1u));
-        if (ok && rank == 0) wcnt[wid][d] = __popc(same);
-        __syncthreads();
-        if (ok) {
-            unsigned int off = base[d] + rank;
-            for (int w = 0; w < wid; ++w) off += wcnt[w][d];
-            sb.key[src ^ 1][off] = k;
-            sb.val[src ^ 1][off] = val;
-        }
-        __syncthreads();
-        for (int dd = threadIdx.x; dd < 256; dd += blockDim.x) {
-            unsigned int tot = 0;
-            for (int w = 0; w < WARPS; ++w) tot += wcnt[w][dd];
-            base[dd] += tot;
+        for (int i = lane; i < 256; i += 32) wcnt[wid][i] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            const unsigned same = __match_any_sync(0xffffffffu, d[i]);
+            const int in_row = __popc(same & ((1u << lane) - 1u));
+            const unsigned before = d[i] < 256 ? wcnt[wid][d[i]] : 0u;
+            rank[i] = before + in_row;
+            __syncwarp();
+            if (d[i] < 256 && in_row == 0) wcnt[wid][d[i]] = before + __popc(same);
+            __syncwarp();
         }
         __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {  // counts -> places, digit threadIdx.x
+            const unsigned c = wcnt[w][threadIdx.x];
+            wcnt[w][threadIdx.x] = base;
+            base += c;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            if (d[i] == 256) continue;
+            const unsigned int off = wcnt[wid][d[i]] + rank[i];
+            sb.key[src ^ 1][off] = k[i];
+            sb.val[src ^ 1][off] = val[i];
+        }
+        __syncwarp();  // (a warp clears its own row only)
     }
 }
 
 // New index of every survivor: its rank in the sorted order (survivors sort
-// before the dropped entries); -1 for the dropped.
+// before the dropped entries), -1 for the dropped; and the survivors in that order.
 __global__ void __launch_bounds__(THREADS) k_sort_map(const Model m, Bufs b) {
     const StepHead& h = block_head(b.sc);
     if (!prune_due(h)) return;
@@ -412,7 +433,9 @@ __global__ void __launch_bounds__(THREADS) k_sort_map(const Model m, Bufs b) {
     const unsigned int* val = sb.val[h.sort_passes & 1];
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < v.N; r += (long long)gridDim.x * blockDim.x) {
         const unsigned int c = val[r];
-        b.map[c] = b.keep[c] ? (int)r : -1;
+        const bool kept = b.keep[c] != 0;
+        b.map[c] = kept ? (int)r : -1;
+        if (kept) sorted_order(b)[r] = (int)c;
     }
 }
 
