@@ -496,8 +496,8 @@ void launch_prune(gbees_ctx* ctx) {
         using T = decltype(TT);
         k_prune_mark<T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
         k_prune_scatter<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
-        k_prune_count<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
         if (sorted) {
+            k_prune_count<N, true><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_sort_init<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             for (int pass = 0; pass < SORT_PASSES; ++pass) {
                 k_sort_hist<<<Gs, THREADS, 0, s>>>(ctx->m, ctx->b, pass, -1);
@@ -507,6 +507,7 @@ void launch_prune(gbees_ctx* ctx) {
             k_sort_map<<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_prune_move<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
         } else {
+            k_prune_count<N, false><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_prune_compact<N, T><<<G, THREADS, 0, s>>>(ctx->m, ctx->b);
             k_prune_relink<N><<<G, THREADS, 0, s>>>(ctx->m, ctx->b, G);
         }
@@ -663,8 +664,8 @@ void graph_nodes(gbees_ctx* ctx, GraphBuilder& gb, cudaGraph_t body, cudaGraphCo
     int nsort = Gs;
     cudaGraphNode_t q = gb.add(pb, nullptr, (void*)k_prune_mark<T>, G, THREADS, mb);
     q = gb.add(pb, q, (void*)k_prune_scatter<N, T>, G, THREADS, mb);
-    q = gb.add(pb, q, (void*)k_prune_count<N>, G, THREADS, mb);
     if (sorts(ctx)) {
+        q = gb.add(pb, q, (void*)k_prune_count<N, true>, G, THREADS, mb);
         q = gb.add(pb, q, (void*)k_sort_init, G, THREADS, mb);
         for (int pass = 0; pass < SORT_PASSES; ++pass) {
             long long pool = -1;
@@ -677,6 +678,7 @@ void graph_nodes(gbees_ctx* ctx, GraphBuilder& gb, cudaGraph_t body, cudaGraphCo
         q = gb.add(pb, q, (void*)k_sort_map, G, THREADS, mb);
         gb.add(pb, q, (void*)k_prune_move<N, T>, G, THREADS, mb);
     } else {
+        q = gb.add(pb, q, (void*)k_prune_count<N, false>, G, THREADS, mb);
         q = gb.add(pb, q, (void*)k_prune_compact<N, T>, G, THREADS, mb);
         gb.add(pb, q, (void*)k_prune_relink<N>, G, THREADS, relink_args);
     }

@@ -696,11 +696,11 @@ __global__ void __launch_bounds__(THREADS) k_prune_scatter(const Model m, Bufs b
 
 // Prune, pass 3: the status of every entry (active, halo or dropped) and the
 // per-block counts of the survivors.
-template <int N>
+template <int N, bool SORTED>
 __global__ void __launch_bounds__(THREADS) k_prune_count(const Model m, Bufs b) {
     const StepHead& h = block_head(b.sc);
     if (!prune_due(h)) return;
-    prune_count_body<N, true>(m, b, view_of(m, &h));
+    prune_count_body<N, SORTED>(m, b, view_of(m, &h));
 }
 
 // Prune, pass 4 without a sort: write the survivors into the other buffer set
