@@ -15,13 +15,29 @@ namespace gbees {
 
 // ------------------------------------------------------------------ links
 
-// Finish a step's time after the link phase: the maximum CFL rate over all
-// cells (old maximum and the new cells' partials) and dt with its coefficients.
+// The CFL rates of the cells that a kernel made active join the running maximum
+// (known: the maximum when the kernel began; rates are compared as the words of
+// non-negative doubles, off the FP64 pipe). All threads of the block.
+__device__ __forceinline__ void join_rates(DevScalars* sc, double rate, unsigned long long known) {
+    __shared__ unsigned long long s_r[MAX_WARPS];
+    long long x = __double_as_longlong(rate);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x = max(x, __shfl_down_sync(0xffffffffu, x, off));
+    if ((threadIdx.x & 31) == 0) s_r[threadIdx.x >> 5] = x > 0 ? (unsigned long long)x : 0ull;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long r = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = max(r, s_r[w]);
+        if (r > known) atomicMax(&sc->maxrate_bits, r);
+    }
+}
+
+// Finish a step's time after the link phase: dt from the maximum CFL rate over all
+// cells, with its coefficients.
 // step: 1 of a time step; 0 and -1 of a new grid, whose normalisation follows
 // (-1: cells taken as given).
-__device__ __forceinline__ void finish_link(const Model& m, DevScalars* sc, const Combined& cr, int step) {
-    unsigned long long r = max(sc->maxrate_bits, cr.rate_bits);
-    sc->maxrate_bits = r;
+__device__ __forceinline__ void finish_link(const Model& m, DevScalars* sc, int step) {
+    const unsigned long long r = *(volatile unsigned long long*)&sc->maxrate_bits;
     if (step <= 0) {
         finalise_norm(m, sc, step < 0 ? 2 : 0);
         sc->N_sorted = step < 0 ? 0 : sc->NA;  // a Gaussian's cells are written in key order
@@ -55,12 +71,11 @@ __global__ void __launch_bounds__(THREADS, 4) k_link(const __grid_constant__ Mod
     } else {
         r = link_body_tile<N, W, T>(m, b, v.N_prev, v.N, v.g, v.nb, v.bi);
     }
-    long long zero[NDIG] = {0, 0, 0, 0, 0, 0};
-    block_partial(b.part, zero, -INFINITY, r);
-    if (last_block(sc)) {
-        Combined cr = combine_partials(b.part, gridDim.x);
-        if (threadIdx.x == 0) finish_link(m, sc, cr, step);
-    }
+    // (the rate alone, by an atomic: as one of the sums and maxima that the last block
+    // folds from every block's partials it took 5 us more, 31 of a step of 6.5e5 entries
+    // that links a few thousand, now 26)
+    join_rates(sc, r, h.maxrate_bits);
+    if (last_block(sc) && threadIdx.x == 0) finish_link(m, sc, step);
 }
 
 // ------------------------------------------------------------------ initial Gaussian
@@ -461,12 +476,6 @@ __global__ void __launch_bounds__(THREADS) k_init_cells(const Model m, Bufs b, c
 
 // ------------------------------------------------------------------ grow
 
-// The CFL rates of the halo cells that grow made active join the running maximum.
-__device__ __forceinline__ void grow_rates(DevScalars* sc, double r) {
-    r = block_max(r);
-    if (threadIdx.x == 0 && r > 0.0) atomicMax(&sc->maxrate_bits, (unsigned long long)__double_as_longlong(r));
-}
-
 // Halo cells around the cells that grow made active (inserted ones: [N_prev, N)
 // at entry; activated ones: the n_act entries listed in map). With STEP == 0
 // (initial grid) it runs whatever the done flag says. The last block appends
@@ -545,7 +554,7 @@ __global__ void __launch_bounds__(THREADS) k_grow_list(const Model m, Bufs b) {
     const StepHead& h = block_head(sc);
     if (h.done | h.error) return;
     const StepView v = view_of(m, &h);
-    grow_rates(sc, grow_list_body<N, T>(m, b, v, h.n_glist));
+    join_rates(sc, grow_list_body<N, T>(m, b, v, h.n_glist), h.maxrate_bits);
 }
 
 // Update, pass 1 (after the links, with dt): jumps and transverse terms.
