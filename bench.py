@@ -70,8 +70,8 @@ PAPER_CELLS_PER_S = {
 # cases run at the threshold that reproduces the burden of Table 2).
 PAPER_CONTEXT = {}
 DEVICE_SOURCES = [os.path.join(ROOT, "paper_2508_13986_gb300", "csrc", f)
-                  for f in ("gbees_keys.cuh", "gbees_device.cuh", "gbees_phases.cuh", "gbees_kernels.cuh",
-                            "gbees_misc_kernels.cuh", "gbees_persistent.cuh")]
+                  for f in ("gbees_keys.cuh", "gbees_rows.cuh", "gbees_device.cuh", "gbees_phases.cuh",
+                            "gbees_kernels.cuh", "gbees_misc_kernels.cuh", "gbees_persistent.cuh")]
 
 
 def parse():

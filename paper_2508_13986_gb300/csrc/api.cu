@@ -891,7 +891,7 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         return GBEES_EINVAL;
     }
     for (int k = 0; k < n * n; ++k) {
-        bx.icovf[k] = (float)bx.icov[k];
+        bx.icovc[k] = (float)(bx.icov[k] * ctx->cfg.h[k / n] * ctx->cfg.h[k % n]);
         if (bx.icov[k] != 0.0) bx.nonzero |= 1ull << k;
     }
     const double thr = ctx->cfg.thr_rel > 0.0 ? ctx->cfg.thr_rel : 1e-300;
@@ -899,15 +899,20 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         ctx->err = "initial box too large";
         return GBEES_EINVAL;
     }
+    auto slack_of = [&](int k) {
+        const double far = std::max(std::fabs((double)bx.lo[k]), std::fabs((double)bx.lo[k] + (double)bx.dims[k]));
+        return centre_slack(ctx->cfg.x0[k], ctx->cfg.h[k], far);
+    };
     {  // q of the cell nearest the mean: no cell with a larger one has the maximum
-        double dx[6], q = 0.0;
+        double dx[6], slack[6];
         for (int k = 0; k < n; ++k) {
             const double i = std::round((mean[k] - ctx->cfg.x0[k]) / ctx->cfg.h[k]);
-            dx[k] = ctx->cfg.x0[k] + i * ctx->cfg.h[k] - mean[k];
+            dx[k] = (ctx->cfg.x0[k] + i * ctx->cfg.h[k] - mean[k]) / ctx->cfg.h[k];
+            slack[k] = slack_of(k);
         }
-        for (int a = 0; a < n; ++a)
-            for (int c = 0; c < n; ++c) q += dx[a] * bx.icov[a * n + c] * dx[c];
-        bx.qlim = (float)q;
+        bx.qlim = (float)form_above(n, bx.icov, ctx->cfg.h, dx, slack);
+        bx.slack = (float)slack[n - 1];
+        bx.rows = 1;
     }
     const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
@@ -944,11 +949,13 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         return ctx->status;
     }
     bx.pstar = ctx->cfg.thr_rel * gmax;
-    bx.qlim = bx.pstar > 0.0 ? (float)(-2.0 * std::log(bx.pstar)) : INFINITY;
+    bx.rows = bx.pstar >= ROWS_MIN_PSTAR;
+    bx.qlim = bx.rows ? (float)(-2.0 * std::log(bx.pstar)) : INFINITY;
     if (!box_for(ctx, mean, cov, -2.0 * std::log(thr * gmax), &bx)) {
         ctx->err = "initial box too large";
         return GBEES_EINVAL;
     }
+    bx.slack = (float)slack_of(n - 1);
     {
         Phase ph(ctx, GBEES_PHASE_OTHER, 5);
         // the set's rows lie in the middle of the box: smaller chunks than one per

@@ -6,6 +6,7 @@
 #pragma once
 
 #include "gbees_phases.cuh"
+#include "gbees_rows.cuh"
 
 namespace gbees {
 
@@ -87,37 +88,52 @@ struct InitBox {
     double mean[MAXN];
     double icov[MAXN * MAXN];
     double pstar;
-    float qlim;  // pass 1: q of the cell nearest the mean; then: -2 ln pstar
-    float icovf[MAXN * MAXN];
+    int rows;                // the rows may decide (pstar is no tiny number)
+    float qlim;              // pass 1: q of the cell nearest the mean, from above; then: -2 ln pstar
+    float slack;             // centre_slack of the last dimension
+    float icovc[MAXN * MAXN];  // icov in cells: icov[a][c] h_a h_c
     unsigned long long nonzero;  // bit a N + c: icov[a][c] != 0 (a comparison would take the FP64 pipe)
 };
 
 // Distance of the cells' centres from the mean, per dimension and index of the
-// box, formed once per block (four FP64 instructions per look otherwise).
+// box, and in cells, formed once per block (five FP64 instructions per look otherwise).
 constexpr int AXIS_MAX = 1024;  // entries; a box with longer axes forms them where they are used
+struct AxisTable {
+    double dx[AXIS_MAX];
+    float cells[AXIS_MAX];
+};
 template <int N>
 struct Axes {
-    const double* tab;  // null: not tabulated
-    int at[N];          // place of index lo_k of axis k, less lo_k
+    const AxisTable* tab;  // null: not tabulated
+    int at[N];             // place of index lo_k of axis k, less lo_k
+    static __device__ __forceinline__ double form(const Model& m, const InitBox& bx, int k, int i) {
+        return __dsub_rn(centre64(m, k, i), bx.mean[k]);
+    }
     __device__ __forceinline__ double dx(const Model& m, const InitBox& bx, int k, int i) const {
-        return tab ? tab[at[k] + i] : __dsub_rn(centre64(m, k, i), bx.mean[k]);
+        return tab ? tab->dx[at[k] + i] : form(m, bx, k, i);
+    }
+    __device__ __forceinline__ float cells(const Model& m, const InitBox& bx, int k, int i) const {
+        return tab ? tab->cells[at[k] + i] : (float)__dmul_rn(form(m, bx, k, i), m.inv_h[k]);
     }
 };
 // (all threads of the block)
 template <int N>
-__device__ __forceinline__ Axes<N> make_axes(const Model& m, const InitBox& bx, double* s_tab) {
+__device__ __forceinline__ Axes<N> make_axes(const Model& m, const InitBox& bx, AxisTable& s_tab) {
     Axes<N> ax;
     long long n = 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) n += bx.dims[k];
-    ax.tab = n <= AXIS_MAX ? s_tab : nullptr;
+    ax.tab = n <= AXIS_MAX ? &s_tab : nullptr;
     int off = 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         ax.at[k] = off - bx.lo[k];
         if (ax.tab) {
-            for (int i = threadIdx.x; i < (int)bx.dims[k]; i += blockDim.x)
-                s_tab[off + i] = __dsub_rn(centre64(m, k, bx.lo[k] + i), bx.mean[k]);
+            for (int i = threadIdx.x; i < (int)bx.dims[k]; i += blockDim.x) {
+                const double d = Axes<N>::form(m, bx, k, bx.lo[k] + i);
+                s_tab.dx[off + i] = d;
+                s_tab.cells[off + i] = (float)__dmul_rn(d, m.inv_h[k]);
+            }
             off += (int)bx.dims[k];
         }
     }
@@ -154,7 +170,7 @@ __device__ __noinline__ double gauss_at(const Model& m, const InitBox& bx, const
 // From three dimensions on, most of the box lies outside the ellipsoid of the
 // initial set (97 % of it in six), and FP64 is scarce: the box is swept by rows
 // along the last dimension, one thread per row, with the quadratic form q of each
-// cell in single precision and a bound of its error. Only a cell whose q lies
+// cell in single precision and a bound of its error (gbees_rows.cuh). Only a cell whose q lies
 // within that bound of the limit is decided in FP64, so the set is the one that
 // FP64 gives everywhere; the densities of the cells in the set are FP64. The
 // paper's 6-D case (2.0e6 cells in the set, a box of 6.4e7): 0.11 + 0.13 + 0.6 ms
@@ -166,7 +182,7 @@ __device__ __noinline__ double gauss_at(const Model& m, const InitBox& bx, const
 constexpr int INIT_ROW_MAX = 1024;
 template <int N>
 __device__ __forceinline__ bool by_rows(const InitBox& bx) {
-    return N >= 3 && bx.dims[N - 1] <= INIT_ROW_MAX;
+    return N >= 3 && bx.rows && bx.dims[N - 1] <= INIT_ROW_MAX;
 }
 // Rows [c0, c1) of this block, as even as possible: a small box spreads over all blocks.
 __device__ __forceinline__ void row_chunk(long long rows, long long& c0, long long& c1) {
@@ -174,12 +190,6 @@ __device__ __forceinline__ void row_chunk(long long rows, long long& c0, long lo
     c0 = min(rows, per * blockIdx.x);
     c1 = min(rows, c0 + per);
 }
-
-struct InitRow {
-    float A, B, C;     // q = A + B dx + C dx^2
-    float Aa, Ba;      // the same sums of absolute values
-    float dx0, h, err; // dx of the row's first cell, cell width, error bound of dx
-};
 
 template <int N>
 __device__ __forceinline__ void row_index(const InitBox& bx, long long row, int* I) {
@@ -202,50 +212,19 @@ __device__ __forceinline__ void row_index(const InitBox& bx, long long row, int*
 }
 
 template <int N>
-__device__ __forceinline__ InitRow row_form(const Model& m, const InitBox& bx, const Axes<N>& ax, const int* I) {
+__device__ __forceinline__ InitRow row_at(const Model& m, const InitBox& bx, const Axes<N>& ax, const int* I) {
     float dx[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) dx[k] = (float)ax.dx(m, bx, k, I[k]);
-    InitRow r;
-    r.A = r.Aa = r.B = r.Ba = 0.0f;
-#pragma unroll
-    for (int a = 0; a < N - 1; ++a) {
-#pragma unroll
-        for (int c = 0; c < N - 1; ++c) {
-            const float t = dx[a] * bx.icovf[a * N + c] * dx[c];
-            r.A += t;
-            r.Aa += fabsf(t);
-        }
-        const float t = dx[a] * (bx.icovf[a * N + N - 1] + bx.icovf[(N - 1) * N + a]);
-        r.B += t;
-        r.Ba += fabsf(t);
-    }
-    r.C = bx.icovf[N * N - 1];
-    r.h = (float)m.h[N - 1];
-    r.dx0 = dx[N - 1];
-    // dx of a cell of the row as dx0 + i h: two roundings and those of dx0 and h
-    r.err = 5e-7f * (fabsf(r.dx0) + (float)bx.dims[N - 1] * r.h);
-    return r;
-}
-
-// q of cell i of the row and a bound of its error: fewer than 64 roundings of
-// relative size 2^-24 on sums of absolute value S (1e-5 is 2.5 times that), and
-// the error of dx.
-__device__ __forceinline__ float row_q(const InitRow& r, int i, float& e) {
-    const float dx = r.dx0 + (float)i * r.h, ad = fabsf(dx);
-    e = 1e-5f * (r.Aa + (r.Ba + r.C * ad) * ad) + (r.Ba + 2.0f * r.C * (ad + r.err)) * r.err + 1e-6f;
-    return r.A + (r.B + r.C * dx) * dx;
+    for (int k = 0; k < N; ++k) dx[k] = ax.cells(m, bx, k, I[k]);
+    return row_form<N>(dx, bx.icovc, (float)bx.dims[N - 1], bx.slack);
 }
 
 // Whether cell i of the row at I is in the set p > pstar (qlim: -2 ln pstar).
 template <int N>
 __device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const Axes<N>& ax, const InitRow& r, int* I,
                                        int i) {
-    float e;
-    const float q = row_q(r, i, e), d = q - bx.qlim;
-    e += 1e-6f * fabsf(bx.qlim);
-    if (d > e) return false;
-    if (d < -e) return true;
+    const int side = row_side(r, i, bx.qlim);
+    if (side) return side < 0;
     I[N - 1] = bx.lo[N - 1] + i;  // too near the limit (or not a number)
     return gauss_at<N>(m, bx, ax, I) > bx.pstar;
 }
@@ -256,7 +235,7 @@ __device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const 
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_init_max(const __grid_constant__ Model m, Bufs b,
                                                         const __grid_constant__ InitBox bx) {
-    __shared__ double s_tab[AXIS_MAX];
+    __shared__ AxisTable s_tab;
     const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     double mx = 0.0;
     const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -267,11 +246,9 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const __grid_constant__ Mo
         for (long long row = first; row < rows; row += stride) {
             int I[N];
             row_index<N>(bx, row, I);
-            const InitRow r = row_form<N>(m, bx, ax, I);
+            const InitRow r = row_at<N>(m, bx, ax, I);
             for (int i = 0; i < len; ++i) {
-                float e;
-                const float q = row_q(r, i, e);
-                if (q - bx.qlim > e + 1e-6f * fabsf(bx.qlim)) continue;
+                if (row_side(r, i, bx.qlim) > 0) continue;
                 I[N - 1] = bx.lo[N - 1] + i;
                 mx = fmax(mx, gauss_at<N>(m, bx, ax, I));
             }
@@ -292,7 +269,7 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const __grid_constant__ Mo
 template <int N>
 __global__ void __launch_bounds__(THREADS) k_init_count(const __grid_constant__ Model m, Bufs b,
                                                         const __grid_constant__ InitBox bx) {
-    __shared__ double s_tab[AXIS_MAX];
+    __shared__ AxisTable s_tab;
     const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     long long c0, c1;
     long long cnt = 0;
@@ -302,7 +279,7 @@ __global__ void __launch_bounds__(THREADS) k_init_count(const __grid_constant__ 
         for (long long row = c0 + threadIdx.x; row < c1; row += blockDim.x) {
             int I[N];
             row_index<N>(bx, row, I);
-            const InitRow r = row_form<N>(m, bx, ax, I);
+            const InitRow r = row_at<N>(m, bx, ax, I);
             for (int i = 0; i < len; ++i) cnt += row_in<N>(m, bx, ax, r, I, i);
         }
     } else {
@@ -334,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_init_write(const __grid_constant
     DevScalars* sc = b.sc;
     const StepHead& h = block_head(sc);
     if (h.error) return;
-    __shared__ double s_tab[AXIS_MAX];
+    __shared__ AxisTable s_tab;
     const Axes<N> ax = make_axes<N>(m, bx, s_tab);
     long long c0, c1;
     long long base = b.blk[blockIdx.x];
@@ -368,7 +345,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_init_write(const __grid_constant
             if (row < c1) {
                 int I[N];
                 row_index<N>(bx, row, I);
-                const InitRow r = row_form<N>(m, bx, ax, I);
+                const InitRow r = row_at<N>(m, bx, ax, I);
                 for (int i = 0; i < len; ++i)
                     if (row_in<N>(m, bx, ax, r, I, i)) {
                         if (n_in == 0) i_first = i;
@@ -408,7 +385,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_init_write(const __grid_constant
                     row_index<N>(bx, t0 + lo, I);
                     int left = q - (lo > 0 ? s_end[lo - 1] : 0), i = s_first[lo] + left;
                     if (s_first[lo] < 0) {
-                        const InitRow r = row_form<N>(m, bx, ax, I);
+                        const InitRow r = row_at<N>(m, bx, ax, I);
                         for (i = 0; i < len; ++i)
                             if (row_in<N>(m, bx, ax, r, I, i) && left-- == 0) break;
                     }
