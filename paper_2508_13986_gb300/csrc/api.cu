@@ -1037,18 +1037,20 @@ int gbees_propagate(gbees_ctx* ctx, double t_end, gbees_stats* stats) {
         return GBEES_EINVAL;
     }
     cudaStream_t s = ctx->stream;
-    // what k_begin does, on the host's copy of the scalars (current after every call)
+    {
+        Phase ph(ctx, GBEES_PHASE_OTHER, 1);
+        k_begin<<<1, 1, 0, s>>>(ctx->b.sc, t_end);
+    }
+    // the same on the host's copy of the scalars (current after every call), without a
+    // read-back; a call without steps has cleared both copies' counters
     ctx->hs.t_target = t_end;
     ctx->hs.done = !(ctx->hs.t < t_end);
     ctx->hs.steps_call = 0;
     ctx->hs.updates_call = 0;
     if (ctx->hs.done) {
+        if (!cuda_ok(ctx, cudaGetLastError(), "propagate")) return ctx->status;
         fill_stats(ctx, stats);
         return GBEES_OK;
-    }
-    {
-        Phase ph(ctx, GBEES_PHASE_OTHER, 1);
-        k_begin<<<1, 1, 0, s>>>(ctx->b.sc, t_end);
     }
     // Persistent path: one cooperative launch runs up to kPersistSteps steps
     // with grid barriers between the phases (small grids).
