@@ -181,13 +181,14 @@ bool make_layout(const gbees_config* c, Layout* L) {
     L->keep = take(cap);
     L->map = take(4 * cap);
     L->table = take(sizeof(Slot) * slots);
-    // face velocities (two generations) and the scratch of the three-pass
-    // update, storage type, n values per entry (one for tg)
+    // face velocities (two generations) and the scratch of the update, storage type, n
+    // values per entry (one for tg). wl and wg are the two halves of one block: the
+    // large-grid update keeps its pairs (Wave, 2 n values per entry) in both, from wl on
     const size_t rows = S * (size_t)c->n * cap;
     for (int g = 0; g < 2; ++g) L->u[g] = take(rows);
     for (int g = 0; g < 2; ++g) L->rate[g] = take(8 * cap);
-    L->wl = take(rows);
-    L->wg = take(rows);
+    L->wl = take(align_up(rows) + rows);
+    L->wg = L->wl + align_up(rows);
     L->tg = take(S * cap);
     L->fl = take(rows);
     L->total = off;

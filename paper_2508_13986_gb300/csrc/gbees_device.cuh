@@ -185,11 +185,14 @@ struct alignas(64) Partial {
 // the entry is created (the drift does not depend on time) and carried along
 // by the prune's compaction.
 //
-// Update scratch of the three-pass flux update (storage type, dimension-major:
-// element d * cap + c, so that a warp's 32 consecutive entries read and write
-// whole sectors): wl[d] the jump P_c - P_{c-e_d} across the lower d-face, wg[d]
-// the d-direction wave entering the cell, tg the sum over d of wg[d] / (2 h_d)
-// (one value per entry), fl[j] the flux through the lower j-face.
+// Update scratch (storage type, dimension-major: element d * cap + c, so that a
+// warp's 32 consecutive entries read and write whole sectors). Step loop of a small
+// grid: wl[d] the jump P_c - P_{c-e_d} across the lower d-face, wg[d] the
+// d-direction wave entering the cell, tg the sum over d of wg[d] / (2 h_d) (one value
+// per entry), fl[j] the flux through the lower j-face. Large grids: one pair per
+// entry and dimension (Wave: the jump and the upwind base) from wl on, over wl and wg,
+// which follow one another in one block of 2 n cap values; fl the flux in FP64; tg
+// unused. The grow's list and a prune's new order are in fl meanwhile.
 struct Bufs {
     unsigned long long* key[2];
     void* q[2];
@@ -205,7 +208,7 @@ struct Bufs {
     unsigned int* sorthist;  // digit histograms of the prune's radix sort
     void* u[2];  // face velocities (two generations, like the keys)
     double* rate[2];  // CFL rate sum_j |f_j(x_{c-e_j/2})| / h_j of every entry (Eq. 8, FP64, fixed at creation)
-    void* wl;    // update scratch in the storage type
+    void* wl;    // update scratch in the storage type (wl and wg: one block)
     void* wg;
     void* tg;
     void* fl;
