@@ -296,8 +296,8 @@ int gbees_profile_read(gbees_ctx* ctx, gbees_profile* out);
 
 /* Bound of the device-side waits of the context's multi-block launches (the
  * grid barriers of the persistent kernel and of a batch's teams): a barrier
- * gives up after `spins` polls of its generation word (2^26 by default, about
- * two seconds), records GBEES_ETIMEOUT in the device scalars and every block
+ * gives up after `spins` polls of its arrival count (2^26 by default: about 15
+ * seconds, 0.23 us per poll), records GBEES_ETIMEOUT in the device scalars and every block
  * leaves the launch; the call then returns GBEES_ETIMEOUT with the context
  * poisoned until the next init, and the device stays usable.
  * extra_arrivals (0 in normal use) makes every grid barrier wait for that

@@ -921,7 +921,8 @@ __device__ __forceinline__ Combined combine_partials(const Partial* part, int nb
 
 // Grid-wide barrier of a cooperative launch (all blocks resident). The wait is
 // bounded: it gives up when another block has set an error or after
-// spin_limit polls (BARRIER_SPIN_LIMIT by default: about two seconds), sets
+// spin_limit polls (BARRIER_SPIN_LIMIT by default: about 15 seconds, a poll being one
+// load from L2 and, every 32nd time, the error word and a short sleep: 0.23 us), sets
 // ST_ETIMEOUT, and returns false; callers then leave.
 constexpr long long BARRIER_SPIN_LIMIT = 1ll << 26;
 
