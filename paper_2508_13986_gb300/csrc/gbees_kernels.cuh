@@ -109,11 +109,15 @@ struct Axes {
     static __device__ __forceinline__ double form(const Model& m, const InitBox& bx, int k, int i) {
         return __dsub_rn(centre64(m, k, i), bx.mean[k]);
     }
+    // (out of line: in line, its FP64 instructions were executed and dropped)
+    static __device__ __noinline__ float form_cells(const Model& m, const InitBox& bx, int k, int i) {
+        return (float)__dmul_rn(form(m, bx, k, i), m.inv_h[k]);
+    }
     __device__ __forceinline__ double dx(const Model& m, const InitBox& bx, int k, int i) const {
         return tab ? tab->dx[at[k] + i] : form(m, bx, k, i);
     }
     __device__ __forceinline__ float cells(const Model& m, const InitBox& bx, int k, int i) const {
-        return tab ? tab->cells[at[k] + i] : (float)__dmul_rn(form(m, bx, k, i), m.inv_h[k]);
+        return tab ? tab->cells[at[k] + i] : form_cells(m, bx, k, i);
     }
 };
 // (all threads of the block)
@@ -223,8 +227,10 @@ __device__ __forceinline__ InitRow row_at(const Model& m, const InitBox& bx, con
 template <int N>
 __device__ __forceinline__ bool row_in(const Model& m, const InitBox& bx, const Axes<N>& ax, const InitRow& r, int* I,
                                        int i) {
-    const int side = row_side(r, i, bx.qlim);
-    if (side) return side < 0;
+    float e;
+    const float d = row_gap(r, i, bx.qlim, e);
+    if (d > e) return false;
+    if (d < -e) return true;
     I[N - 1] = bx.lo[N - 1] + i;  // too near the limit (or not a number)
     return gauss_at<N>(m, bx, ax, I) > bx.pstar;
 }
@@ -248,7 +254,9 @@ __global__ void __launch_bounds__(THREADS) k_init_max(const __grid_constant__ Mo
             row_index<N>(bx, row, I);
             const InitRow r = row_at<N>(m, bx, ax, I);
             for (int i = 0; i < len; ++i) {
-                if (row_side(r, i, bx.qlim) > 0) continue;
+                float e;
+                const float d = row_gap(r, i, bx.qlim, e);
+                if (d > e) continue;
                 I[N - 1] = bx.lo[N - 1] + i;
                 mx = fmax(mx, gauss_at<N>(m, bx, ax, I));
             }

@@ -86,13 +86,12 @@ GBEES_ROWS_HD float row_q(const InitRow& r, int i, float& e) {
     return r.A + (r.B + r.C * dx) * dx;
 }
 
-// q of cell i against the limit qlim (rounded to float): 1 above it, -1 below it, 0 too
-// near it (or not a number).
-GBEES_ROWS_HD int row_side(const InitRow& r, int i, float qlim) {
-    float e;
-    const float q = row_q(r, i, e), d = q - qlim;
+// q of cell i less the limit qlim (rounded to float), and a bound of its error: above
+// the limit when d > e, below it when d < -e, else too near it (or not a number).
+GBEES_ROWS_HD float row_gap(const InitRow& r, int i, float qlim, float& e) {
+    const float q = row_q(r, i, e);
     e += 1e-6f * fabsf(qlim);
-    return d > e ? 1 : d < -e ? -1 : 0;
+    return q - qlim;
 }
 
 }  // namespace gbees

@@ -17,7 +17,11 @@ template <int N>
 static void rows_of(const float* dx, long rows, const float* w, int len, float slack, float qlim, signed char* side) {
     for (long r = 0; r < rows; ++r) {
         const InitRow f = row_form<N>(dx + r * N, w, (float)len, slack);
-        for (int i = 0; i < len; ++i) side[r * len + i] = (signed char)row_side(f, i, qlim);
+        for (int i = 0; i < len; ++i) {
+            float e;
+            const float d = row_gap(f, i, qlim, e);
+            side[r * len + i] = d > e ? 1 : d < -e ? -1 : 0;  // out, in, left to FP64
+        }
     }
 }
 extern "C" void sides(int n, const float* dx, long rows, const float* w, int len, float slack, float qlim,
