@@ -217,7 +217,6 @@ struct Bufs {
 
 
 constexpr int RESORT = 2;                            // DevScalars::prune_now
-constexpr int RESORT_STEPS = 5;                      // steps that a re-sort has to serve at least
 constexpr long long RESORT_MIN_ENTRIES = 1ll << 21;
 constexpr long long SORT_MIN_ENTRIES = 1ll << 18;    // smaller pools (they fit in L2) are not sorted
 

@@ -487,7 +487,8 @@ __global__ void __launch_bounds__(THREADS) k_halo(const Model m, Bufs b) {
 
 // Time, step count, buffers, prune schedule and normalisation after the flux
 // update of a step, from the combined partials of the update's blocks.
-__device__ __forceinline__ void finish_step(const Model& m, DevScalars* sc, const Combined& cs, int pb) {
+// fp64: of the storage type.
+__device__ __forceinline__ void finish_step(const Model& m, DevScalars* sc, const Combined& cs, int pb, bool fp64) {
     sc->dt = sc->step_dt;
     sc->t = sc->step_t_new;
     sc->step += 1;
@@ -497,16 +498,17 @@ __device__ __forceinline__ void finish_step(const Model& m, DevScalars* sc, cons
     sc->pbuf = pb ^ 1;
     const long long K = m.prune_interval, into = K > 0 ? sc->step % K : 0;
     sc->prune_now = K > 0 && into == 0;
-    // A large pool more than a quarter of which is out of order (appended by growth
-    // since the last sort; the halo of a new grid) is sorted at once, by the prune's
-    // kernels with every cell kept, when the next prune is at least RESORT_STEPS
-    // steps away: no result depends on the order. The paper's 6-D case, 4 to 6e6
-    // entries: a step's update passes take 0.41 ms in order and 0.73 ms with 60 % of
-    // the pool out of order, a sort takes 2.2 ms. (Pools below RESORT_MIN_ENTRIES
+    // A large pool much of which is out of order (appended by growth since the last sort;
+    // the halo of a new grid) is sorted at once, by the prune's kernels with every cell
+    // kept, when that pays over the steps until the next prune or the end of the call
+    // (resort_pays): no result depends on the order. (Pools below RESORT_MIN_ENTRIES
     // lose: a sort of 6.5e5 entries takes 0.5 ms and gains 0.02 ms per step.)
     if (!sc->prune_now && !sc->done && m.sort_order != 2 && sc->N > RESORT_MIN_ENTRIES &&
-        (sc->N - sc->N_sorted) * 4 > sc->N && (K == 0 || K - into >= RESORT_STEPS))
-        sc->prune_now = RESORT;
+        (sc->N - sc->N_sorted) * 4 > sc->N) {
+        double left = (sc->t_target - sc->t) / sc->dt;
+        if (K > 0) left = fmin(left, (double)(K - into));
+        if (resort_pays(sc->N, sc->N - sc->N_sorted, left, fp64)) sc->prune_now = RESORT;
+    }
     sc->N_prev = sc->N;
     const double w = m.prod_h * acc_to_double(cs.acc);
     sc->w = w;
@@ -562,13 +564,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_faces(const Model m, Bufs b) {
 
 // The end of an update: exact per-block partial sums and maximum for the next
 // normalisation; the last block ends the step.
+template <typename T>
 __device__ __forceinline__ void end_update(const Model& m, const Bufs& b, const StepView& v, long long (&d)[NDIG],
                                            double mx, int err) {
     if (err) set_error(b.sc, ST_EDEGENERATE);
     block_partial(b.part, d, mx, 0.0);
     if (last_block(b.sc)) {
         Combined cs = combine_partials(b.part, gridDim.x);
-        if (threadIdx.x == 0) finish_step(m, b.sc, cs, v.pb);
+        if (threadIdx.x == 0) finish_step(m, b.sc, cs, v.pb, sizeof(T) == 8);
     }
 }
 
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(THREADS) k_apply(const Model m, Bufs b) {
     double mx = -INFINITY;
     int err = 0;
     apply_body<N, T>(m, b, v, d, mx, err);
-    end_update(m, b, v, d, mx, err);
+    end_update<T>(m, b, v, d, mx, err);
 }
 
 // Update, passes 2 and 3 in one (FP32).
@@ -598,7 +601,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_update(const Model m, Bufs b) {
     double mx = -INFINITY;
     int err = 0;
     update_body<N, T>(m, b, v, d, mx, err);
-    end_update(m, b, v, d, mx, err);
+    end_update<T>(m, b, v, d, mx, err);
 }
 
 // ------------------------------------------------------------------ measurement update
