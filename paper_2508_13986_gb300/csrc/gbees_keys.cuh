@@ -44,6 +44,16 @@ GBEES_HD void unpack_key_bits(int b, unsigned long long k, int* I) {
     }
 }
 
+// Component j of I one step up or down. False when there is no such 32-bit index: in
+// one dimension an index takes all 32 bits, and a wrapped one would have a key (in more
+// dimensions the index is there and has no key).
+template <int N>
+GBEES_HD bool step_index(int* I, int j, int up) {
+    if (N == 1 && I[0] == (up ? 0x7fffffff : -0x7fffffff - 1)) return false;
+    I[j] += up ? 1 : -1;
+    return true;
+}
+
 // Morton (Z-order) code of a packed key of n fields of b bits: the bits of
 // the n indices interleaved, from the most significant bit of every field
 // down, dimension 0 first within each bit. A bijection of the n*b-bit keys

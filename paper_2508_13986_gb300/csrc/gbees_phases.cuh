@@ -338,7 +338,10 @@ __device__ __forceinline__ void halo_body(const Model& m, const Bufs& b, const S
         }
         int I[N];
         unpack_key<N>(m, key[x], I);
-        I[d >> 1] += (d & 1) ? 1 : -1;
+        if (!step_index<N>(I, d >> 1, d & 1)) {
+            set_error(b.sc, ST_EKEYRANGE);
+            continue;
+        }
         insert_cell<N, T>(m, b, v, I, OM_GHOST, &b.sc->n_halo, hi);
     }
 }
@@ -472,7 +475,7 @@ __device__ __noinline__ double face_velocity_key(const Model& m, unsigned long l
     const unsigned long long mask = (1ull << bits) - 1;
     auto y = [&](int a) -> double {
         const int i = (int)((long long)((k >> (bits * (N - 1 - a))) & mask) - bias);
-        const double s = a == j ? __dsub_rn((double)(i + up), 0.5) : (double)i;
+        const double s = a == j ? __dadd_rn((double)i, up ? 0.5 : -0.5) : (double)i;
         return __dadd_rn(m.x0[a], __dmul_rn(s, m.h[a]));
     };
     if (m.dyn == DYN_CONSTANT) return m.a[j];
@@ -645,9 +648,9 @@ __device__ __forceinline__ double link_body_tile(const Model& m, const Bufs& b, 
         const int j = dir >> 1, s = dir & 1;
         int I[N];
         unpack_key<N>(m, key[c], I);
-        I[j] += s ? 1 : -1;
         unsigned long long k;
-        const int nbr = pack_key<N>(m, I, k) ? table_find_tile<W>(m, b.table, k, tile) : -1;
+        const int nbr =
+            step_index<N>(I, j, s) && pack_key<N>(m, I, k) ? table_find_tile<W>(m, b.table, k, tile) : -1;
         if (tile.thread_rank() == 0) {
             link[(long long)dir * cap + c] = nbr;
             if (nbr >= 0) link[(long long)(2 * j + (1 - s)) * cap + nbr] = (int)c;
