@@ -265,14 +265,27 @@ def fp64_peak():
     return tf, f"derived: {sms} SMs x 2 FP64 FMA lanes/clock x 2 flops x {mhz:.0f} MHz"
 
 
+# The kernels of one time step that a timed phase of the library brackets (direct launches,
+# one pair of events per launch or pair of launches), by precision: the grow's two, the
+# flux pass's two (FP32: the second one makes the update too), the update's.
+STEP_KERNELS = {
+    "f64": {"grow": ("k_grow_mark", "k_grow_list"), "faces": ("k_waves", "k_faces"), "apply": ("k_apply",)},
+    "f32": {"grow": ("k_grow_mark", "k_grow_list"), "faces": ("k_waves", "k_update"), "apply": ()},
+}
+# brackets per time step of a phase
+BRACKETS = {"grow": 1, "faces": 2, "apply": 1}
+
+
 def fp64_flops_per_update(kernel: str, n: int) -> int:
     """Algorithmic FP64 flops of one cell update in a step kernel (an FMA counts
-    two): the flux pass evaluates the n lower faces of the cell, 11 flops each
-    (the transverse sum, donor cell and corrections: 2 + 2 + 1; the limited
-    high-resolution term: 1 + 2 + 1 + 2); the wave pass 7 per dimension (two
-    jumps, the entering wave 1 + 2, its share of their sum 2); the update pass 3 per
-    dimension plus 3 (difference and FMA per face, then the rescale)."""
-    return {"k_faces": 11 * n, "k_waves": 7 * n, "k_apply": 3 * n + 3}[kernel]
+    two): the wave pass 11 per dimension (two jumps, the entering wave 1 + 2, its
+    share of their sum 2, the upwind base without the dimension's own 2 + 2); the
+    flux pass 7 for each of the n lower faces of the cell (donor cell and
+    corrections in one product 1; the limited high-resolution term: 2 + 1, the sum
+    of the jumps 1, 2); the update pass 3 per dimension plus 2 (difference and FMA
+    per face, then the rescale). Signs, minima and factors of two are integer
+    operations."""
+    return {"k_waves": 11 * n, "k_faces": 7 * n, "k_apply": 3 * n + 2}[kernel]
 
 
 def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None):
@@ -371,6 +384,7 @@ def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None
     # library on its stream), otherwise the slowest per-cell step kernel of the
     # profiled pass (one launch per kernel, events around each)
     if pt["persist_launches"] and pt["persist_updates"] >= 0.5 * total_updates:
+        names = ("k_persistent",)
         kernel = "k_persistent (whole step loop, one cooperative launch per propagate segment)"
         timing = "CUDA events around every persistent launch on the library stream, timed region"
         launches_k = pt["persist_launches"]
@@ -379,17 +393,18 @@ def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None
     else:
         per_cell = {k: prof["ms"][k] for k in ("grow", "faces", "apply")}
         top = max(per_cell, key=per_cell.get)
-        # (FP32 forms the fluxes and the update in one kernel; the grow phase has two
-        # timed brackets per step, the grow's and the waves')
-        kernel = {"grow": "k_waves", "faces": "k_faces" if precision == "f64" else "k_update", "apply": "k_apply"}[top]
-        timing = "CUDA events around each launch of that kernel in a profiled pass of the same runs"
-        launches_k = max(prof["timed"][top] // (2 if top == "grow" else 1), 1)
+        names = STEP_KERNELS[precision][top]
+        kernel = " + ".join(names) + (f" ({len(names)} launches per time step)" if len(names) > 1 else "")
+        timing = ("CUDA events around every launch in a profiled pass of the same runs"
+                  + (", added up per time step" if len(names) > 1 else ""))
+        # one pass of these kernels per time step
+        launches_k = max(prof["timed"][top] // BRACKETS[top], 1)
         units = prof_updates
         avg_us = per_cell[top] * 1e3 / launches_k
     units_per_launch = units / max(launches_k, 1)
     achieved = bpc * units_per_launch / (avg_us * 1e-6) / 1e9 if avg_us > 0 else None
     traffic = None
-    rec = TRAFFIC_BYTES_PER_CELL.get(f"{w.name}/{precision}/{kernel.split(' ')[0]}")
+    rec = TRAFFIC_BYTES_PER_CELL.get(f"{w.name}/{precision}/{'+'.join(names)}")
     if rec and rec.get("src") == device_source_hash():
         traffic = rec["bytes_per_cell"] * units_per_launch
     roof = {
@@ -406,13 +421,12 @@ def time_precision(args, w, precision, dev, rank, world, steps=None, warmup=None
         "cell_updates_per_launch": units_per_launch,
         "avg_launch_us": avg_us,
     }
-    kname = kernel.split(" ")[0]
-    if precision == "f64" and kname in ("k_faces", "k_waves", "k_apply"):
-        # FP64 step kernels are bound by the FP64 pipe on this chip (ncu: the
-        # flux pass keeps it 64 % busy at 29 % of DRAM bandwidth):
+    if precision == "f64" and set(names) <= {"k_waves", "k_faces", "k_apply"}:
+        # FP64 step kernels are bound by the FP64 pipe on this chip (ncu: the wave
+        # pass keeps it 81 % busy, the flux pass 50 % at 60 % of DRAM bandwidth):
         # the roofline is the FP64 arithmetic peak; the HBM figures stay beside it
         tf, how = fp64_peak()
-        fpc = fp64_flops_per_update(kname, w.n)
+        fpc = sum(fp64_flops_per_update(k, w.n) for k in names)
         ach = fpc * units_per_launch / (avg_us * 1e-6) / 1e12 if avg_us > 0 else None
         roof = {"bound": "alu", "kernel": kernel, "timing": timing, "achieved": ach, "peak": tf,
                 "peak_source": how, "unit": "TFLOP/s", "frac": (ach / tf) if ach else None, "traffic": traffic,

@@ -257,12 +257,13 @@ int gbees_get_stats(gbees_ctx* ctx, gbees_stats* stats);
  * and its duration is added up; launches counts every kernel the library
  * issues, enabled or not. Phases: */
 enum {
-    GBEES_PHASE_GROW = 0,    /* directional grow (Sec. 3.3); the waves (timed apart: two brackets per step) */
+    GBEES_PHASE_GROW = 0,    /* directional grow (Sec. 3.3) */
     GBEES_PHASE_HALO = 1,    /* halo cells around the newly active cells */
     GBEES_PHASE_LINK = 2,    /* neighbour links of the new entries, CFL step (Sec. 4.1, Eq. 8) */
-    GBEES_PHASE_FACES = 3,   /* face fluxes: DCU + CTU + high-resolution term (Eq. 7, Algorithm 1); FP32: with the update */
+    GBEES_PHASE_FACES = 3,   /* face fluxes: DCU + CTU + high-resolution term (Eq. 7, Algorithm 1), the waves and
+                                the fluxes timed apart: two brackets per step; FP32: with the update */
     GBEES_PHASE_APPLY = 4,   /* conservative update, normalisation partials (FP64) */
-    GBEES_PHASE_PRUNE = 5,   /* mark, status, Morton-order sort (graph and direct launch modes),
+    GBEES_PHASE_PRUNE = 5,   /* mark, status, sort into the storage order (graph and direct launch modes),
                                 compaction, relink and rehash (Algorithm 3) */
     GBEES_PHASE_CORRECT = 6, /* Bayesian update (Eq. 4) */
     GBEES_PHASE_OTHER = 7,   /* init, read-out, moments */

@@ -585,13 +585,9 @@ void launch_step(gbees_ctx* ctx) {
             launch_link<N, decltype(TT)>(ctx, 1);
         });
     }
-    {
-        Phase ph(ctx, GBEES_PHASE_GROW, 1);
-        launch_list(ctx, ctx->kern.post, ctx->post_grid, 1);
-    }
-    {
+    for (int i = 0; i < 2; ++i) {  // the flux pass: waves, then fluxes (FP32: with the update)
         Phase ph(ctx, GBEES_PHASE_FACES, 1);
-        launch_list(ctx, ctx->kern.post + 1, ctx->post_grid + 1, 1);
+        launch_list(ctx, ctx->kern.post + i, ctx->post_grid + i, 1);
     }
     if (ctx->kern.npost > 2) {
         Phase ph(ctx, GBEES_PHASE_APPLY, 1);
