@@ -447,6 +447,10 @@ __device__ __forceinline__ double with_sign(double v, double s) {
 __device__ __forceinline__ float with_sign(float v, float s) { return copysignf(v, s); }
 __device__ __forceinline__ float abs_bits(float x) { return fabsf(x); }
 // min of two non-negative finite values (integer order of the bits for doubles)
+// Whether a face's velocity carries a flux: it is not zero. (In FP32 a velocity that is
+// no number carries none; in FP64 it does, and the step ends with ST_EDEGENERATE.)
+__device__ __forceinline__ bool flows(double u) { return nonzero(u); }
+__device__ __forceinline__ bool flows(float u) { return fabsf(u) > 0.0f; }
 __device__ __forceinline__ double min_nonneg(double a, double b) {
     return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
 }

@@ -823,7 +823,7 @@ __device__ __forceinline__ T pick_of(const T (&a)[M], int j) {
 // across the face beyond the upwind cell.
 template <typename T>
 __device__ __forceinline__ T flux_of(int lim, T u, T base, T W, T Wup, T dth) {
-    if (!nonzero(u)) return (T)0;
+    if (!flows(u)) return (T)0;
     const T f = u * base;
     if (lim == LIM_NONE || !nonzero(W)) return f;
     const T au = abs_bits(u);
@@ -1091,6 +1091,12 @@ struct GrowQueue {
     unsigned char code[GROW_QUEUE];
 };
 
+// A rate (as the word of a non-negative double) above the largest known; one that is no
+// number is none, as in the maxima of the other phases.
+__device__ __forceinline__ bool larger_rate(unsigned long long rb, unsigned long long known) {
+    return rb > known && rb <= 0x7ff0000000000000ull;
+}
+
 // A warp's grow requests: neighbour `code` of cell cc (made active as
 // grow_candidate does it, with the marks of the step loop, and the inserted
 // cells' velocities formed at once). rate_now: the largest CFL rate known; only a larger one is written (it
@@ -1120,7 +1126,7 @@ __device__ __noinline__ void grow_act(const Model& m, const Bufs& b, int g, int 
         if (act) {
             atomicOr(word, fresh << sh);
             const unsigned long long rb = (unsigned long long)__double_as_longlong(b.rate[g][e]);
-            if (rb > rate_now) atomicMax(rate, rb);
+            if (larger_rate(rb, rate_now)) atomicMax(rate, rb);
         }
     }
     const unsigned acts = __ballot_sync(full, act);
@@ -1178,7 +1184,7 @@ __device__ __noinline__ void grow_act(const Model& m, const Bufs& b, int g, int 
         const int co = __shfl_sync(full, (int)c, owner);
         const double r = complete_group<N, T>(m, b, g, on, co, ko, 0u, false);
         const unsigned long long rb = (unsigned long long)__double_as_longlong(r);
-        if (on && lane == s * F && rb > rate_now) atomicMax(rate, rb);
+        if (on && lane == s * F && larger_rate(rb, rate_now)) atomicMax(rate, rb);
 #pragma unroll 1
         for (int i = 0; i < G; ++i) todo &= todo - 1;
     }
@@ -1409,7 +1415,7 @@ __device__ __forceinline__ void faces_old_body(const Model& m, const Bufs& b, co
         if (Llo < 0 || Llo >= nold) continue;
         if ((fX & OM_GHOST) && is_halo(om, Llo)) continue;
         T f = (T)0;
-        if (nonzero(u)) {
+        if (flows(u)) {
             const bool up = gt0(u);  // the upwind cell is Llo, else X
             const int y = up ? Llo : X;
             // the jump across the face beyond the upwind cell
