@@ -352,9 +352,18 @@ __device__ __forceinline__ int table_find_tile(const Model& m, const Slot* __res
     return -1;
 }
 
+// A claim whose probes grow long looks at the error word now and then: a pool that has
+// run out of capacity goes on claiming keys until its phase ends and fills the table,
+// where every further claim would look at all slots (minutes on one block).
+constexpr unsigned long long CLAIM_LOOK = 64;
+__device__ __forceinline__ bool claim_hopeless(const DevScalars* sc, unsigned long long probe) {
+    return (probe & (CLAIM_LOOK - 1)) == CLAIM_LOOK - 1 && *(volatile const int*)&sc->error;
+}
+
 // Insert key if absent. Returns 1 and the slot when this thread claimed a new
-// slot, 0 when the key is present, -1 when the table is full.
-__device__ __forceinline__ int table_claim(const Model& m, Slot* T, unsigned long long key, unsigned long long* slot) {
+// slot, 0 when the key is present, -1 when the table is full (or an error is recorded).
+__device__ __forceinline__ int table_claim(const Model& m, Slot* T, const DevScalars* sc, unsigned long long key,
+                                           unsigned long long* slot) {
     unsigned long long h = table_home(key, m.tmask);
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
@@ -368,6 +377,7 @@ __device__ __forceinline__ int table_claim(const Model& m, Slot* T, unsigned lon
             }
             if (old == key) return 0;
         }
+        if (claim_hopeless(sc, probe)) return -1;
         h = table_next(h, probe, m.tmask);
     }
     return -1;
@@ -437,6 +447,10 @@ __device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool lt0(float x) { return x < 0.0f; }
 __device__ __forceinline__ bool nonzero(double x) { return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0; }
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
+// Whether a face's velocity carries a flux: it is not zero. (In FP32 a velocity that is
+// no number carries none; in FP64 it does, and the step ends with ST_EDEGENERATE.)
+__device__ __forceinline__ bool flows(double u) { return nonzero(u); }
+__device__ __forceinline__ bool flows(float u) { return fabsf(u) > 0.0f; }
 __device__ __forceinline__ double abs_bits(double x) {
     return __hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x));
 }
@@ -447,10 +461,6 @@ __device__ __forceinline__ double with_sign(double v, double s) {
 __device__ __forceinline__ float with_sign(float v, float s) { return copysignf(v, s); }
 __device__ __forceinline__ float abs_bits(float x) { return fabsf(x); }
 // min of two non-negative finite values (integer order of the bits for doubles)
-// Whether a face's velocity carries a flux: it is not zero. (In FP32 a velocity that is
-// no number carries none; in FP64 it does, and the step ends with ST_EDEGENERATE.)
-__device__ __forceinline__ bool flows(double u) { return nonzero(u); }
-__device__ __forceinline__ bool flows(float u) { return fabsf(u) > 0.0f; }
 __device__ __forceinline__ double min_nonneg(double a, double b) {
     return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
 }

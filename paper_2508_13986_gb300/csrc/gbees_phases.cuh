@@ -115,7 +115,7 @@ __device__ __forceinline__ void load_links(const int* link, long long cap, long 
 __device__ __forceinline__ void table_insert_new(const Model& m, const Bufs& b, unsigned long long k, long long c,
                                                  unsigned int* slots) {
     unsigned long long slot;
-    int r = table_claim(m, b.table, k, &slot);
+    int r = table_claim(m, b.table, b.sc, k, &slot);
     if (r == 1) {
         b.table[slot].val = c;
         slots[c] = (unsigned int)slot;
@@ -167,7 +167,7 @@ __device__ __forceinline__ long long insert_cell(const Model& m, const Bufs& b, 
         return -1;
     }
     unsigned long long slot;
-    const int r = table_claim(m, b.table, k, &slot);
+    const int r = table_claim(m, b.table, b.sc, k, &slot);
     if (r < 0) {
         set_error(sc, ST_ETABLE);
         return -1;
@@ -1154,7 +1154,7 @@ __device__ __noinline__ void grow_act(const Model& m, const Bufs& b, int g, int 
         } else {
             pack_key<N>(m, J, key);
             unsigned long long slot;
-            const int claim = table_claim(m, b.table, key, &slot);
+            const int claim = table_claim(m, b.table, sc, key, &slot);
             if (claim < 0) set_error(sc, ST_ETABLE);
             if (claim > 0) {
                 c = (long long)atomicAdd((unsigned long long*)&sc->N, 1ull);
@@ -1298,8 +1298,8 @@ __device__ __forceinline__ void grow_drain(const Model& m, const Bufs& b, const 
 
 // The slot of key: claimed (1, was free), found (0) or the table is full (-1).
 // Compare-and-swap at once: most keys asked for here are new.
-__device__ __forceinline__ int table_claim_or_find(const Model& m, Slot* T, unsigned long long key,
-                                                   unsigned long long* slot) {
+__device__ __forceinline__ int table_claim_or_find(const Model& m, Slot* T, const DevScalars* sc,
+                                                   unsigned long long key, unsigned long long* slot) {
     unsigned long long h = table_home(key, m.tmask);
 #pragma unroll 1
     for (unsigned long long probe = 0; probe <= m.tmask; ++probe) {
@@ -1307,6 +1307,7 @@ __device__ __forceinline__ int table_claim_or_find(const Model& m, Slot* T, unsi
         *slot = h;
         if (k == EMPTY_KEY) return 1;
         if (k == key) return 0;
+        if (claim_hopeless(sc, probe)) return -1;
         h = table_next(h, probe, m.tmask);
     }
     return -1;
@@ -1343,7 +1344,7 @@ __device__ __forceinline__ void halo_claim_body(const Model& m, const Bufs& b, c
         }
         k = (d & 1) ? k + (1ull << shift) : k - (1ull << shift);
         unsigned long long slot;
-        const int claim = table_claim_or_find(m, b.table, k, &slot);
+        const int claim = table_claim_or_find(m, b.table, sc, k, &slot);
         if (claim < 0) {
             set_error(sc, ST_ETABLE);
         } else if (claim == 0) {
