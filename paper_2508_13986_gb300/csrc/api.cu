@@ -909,7 +909,6 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         }
         bx.qlim = (float)form_above(n, bx.icov, ctx->cfg.h, dx, slack);
         bx.slack = (float)slack[n - 1];
-        bx.rows = 1;
     }
     const int G = ctx->grid;
     cudaStream_t s = ctx->stream;
@@ -946,8 +945,7 @@ int gbees_init_gaussian(gbees_ctx* ctx, const double* mean, const double* cov, d
         return ctx->status;
     }
     bx.pstar = ctx->cfg.thr_rel * gmax;
-    bx.rows = bx.pstar >= ROWS_MIN_PSTAR;
-    bx.qlim = bx.rows ? (float)(-2.0 * std::log(bx.pstar)) : INFINITY;
+    bx.qlim = bx.pstar >= ROWS_MIN_PSTAR ? (float)(-2.0 * std::log(bx.pstar)) : INFINITY;
     if (!box_for(ctx, mean, cov, -2.0 * std::log(thr * gmax), &bx)) {
         ctx->err = "initial box too large";
         return GBEES_EINVAL;

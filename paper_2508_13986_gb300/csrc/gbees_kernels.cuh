@@ -88,8 +88,7 @@ struct InitBox {
     double mean[MAXN];
     double icov[MAXN * MAXN];
     double pstar;
-    int rows;                // the rows may decide (pstar is no tiny number)
-    float qlim;              // pass 1: q of the cell nearest the mean, from above; then: -2 ln pstar
+    float qlim;              // pass 1: q of the cell nearest the mean, from above; then: -2 ln pstar (inf: FP64 decides)
     float slack;             // centre_slack of the last dimension
     float icovc[MAXN * MAXN];  // icov in cells: icov[a][c] h_a h_c
     unsigned long long nonzero;  // bit a N + c: icov[a][c] != 0 (a comparison would take the FP64 pipe)
@@ -186,7 +185,7 @@ __device__ __noinline__ double gauss_at(const Model& m, const InitBox& bx, const
 constexpr int INIT_ROW_MAX = 1024;
 template <int N>
 __device__ __forceinline__ bool by_rows(const InitBox& bx) {
-    return N >= 3 && bx.rows && bx.dims[N - 1] <= INIT_ROW_MAX;
+    return N >= 3 && bx.dims[N - 1] <= INIT_ROW_MAX;
 }
 // Rows [c0, c1) of this block, as even as possible: a small box spreads over all blocks.
 __device__ __forceinline__ void row_chunk(long long rows, long long& c0, long long& c1) {

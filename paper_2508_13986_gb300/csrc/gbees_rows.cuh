@@ -21,7 +21,8 @@
 namespace gbees {
 
 // The smallest pstar that the rows may decide on: below 2^-1022 a density loses bits,
-// and -2 ln pstar no longer tells which densities exceed pstar.
+// and -2 ln pstar no longer tells which densities exceed pstar. With an infinite limit
+// nothing is decided (FP64 decides on every cell).
 constexpr double ROWS_MIN_PSTAR = 1e-290;
 
 // Rounding of the cells' centres along an axis, in cells. A distance from the mean

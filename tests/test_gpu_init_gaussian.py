@@ -23,7 +23,7 @@ def _cov(n, sigma, corr):
     return C * np.outer(sigma, sigma)
 
 
-def _check(n, sigma, per, origin, shift, corr, prec):
+def _check(n, sigma, per, origin, shift, corr, prec, thr=THR):
     """per: cells per standard deviation; origin: x0 in standard deviations;
     shift: the mean's distance from x0 in cells."""
     sigma = np.asarray(sigma, dtype=np.float64)
@@ -32,9 +32,9 @@ def _check(n, sigma, per, origin, shift, corr, prec):
     mean = x0 + np.asarray(shift, dtype=np.float64) * h
     cov = _cov(n, sigma, corr)
     drift = [0.0] * n
-    o = Oracle(n, DYN_CONSTANT, drift, list(h), list(x0), THR, 0.9, 20, LIM_MC)
+    o = Oracle(n, DYN_CONSTANT, drift, list(h), list(x0), thr, 0.9, 20, LIM_MC)
     o.init_gaussian(mean, cov)
-    cfg = gbees.make_config(n, gbees.GBEES_DYN_CONSTANT, drift, h, x0, THR, precision=prec, max_cells=1 << 22)
+    cfg = gbees.make_config(n, gbees.GBEES_DYN_CONSTANT, drift, h, x0, thr, precision=prec, max_cells=1 << 22)
     g = gbees.Grid(cfg)
     g.init_gaussian(mean, cov)
     gi, gp = g.read_cells()
@@ -44,7 +44,9 @@ def _check(n, sigma, per, origin, shift, corr, prec):
     # the two inverses of cov differ by a few roundings times its condition (below 20),
     # the exponents (up to 14) by as much: 14 * 20 * 36 * 2^-53 < 2e-12; FP32 storage
     # rounds a density and their sum by 2^-24 each
-    tol = 2e-12 if prec == gbees.GBEES_FP64 else 2e-12 + 2.5 * 2.0 ** -24
+    tol = 2e-12 * max(1.0, -np.log(thr) / 14.0)  # (a smaller threshold: larger exponents)
+    if prec == gbees.GBEES_FP32:
+        tol += 2.5 * 2.0 ** -24
     assert np.max(np.abs(gp / op - 1.0)) <= tol
 
 
@@ -80,3 +82,12 @@ def test_an_origin_far_from_zero(origin, corr, prec):
 def test_long_axes_and_rows(per, prec):
     """Axes beyond the table of 1024 distances, rows around and beyond 1024 cells."""
     _check(3, [1.0, 1.0, 1.0], per, [0.0, 0.5, 0.0], [0.2, 0.0, -0.3], 0.3, prec)
+
+
+@PREC
+@pytest.mark.parametrize("thr,per", [(1e-285, 0.7), (1e-295, 0.7), (1e-290, 0.4)])
+def test_tiny_thresholds(thr, per, prec):
+    """Thresholds around the one below which FP64 decides on every cell (FP32 stores 0
+    below 1e-45)."""
+    _check(3, [1.0, 0.8, 1.2], per, [0.0, 0.5, -1.0], [0.1, -0.2, 0.0], 0.3, prec,
+           thr if prec == gbees.GBEES_FP64 else 1e-30)

@@ -63,7 +63,7 @@ def _prior(n, sigma, corr, g):
     return np.linalg.inv(C) / np.outer(sigma, sigma)
 
 
-def _sides(lib, n, sigma, per, origin, corr, seed, thr=THR, rows=1500):
+def _sides(lib, n, sigma, per, origin, corr, seed, thr=THR, rows=1500, qlim=None):
     """(side of every cell of some rows, whether FP64 puts it in the set, FP64's q)."""
     g = np.random.Generator(np.random.PCG64(seed))
     sigma = np.broadcast_to(np.asarray(sigma, dtype=np.float64), n)
@@ -71,9 +71,9 @@ def _sides(lib, n, sigma, per, origin, corr, seed, thr=THR, rows=1500):
     x0 = origin * sigma
     mean = x0 + g.uniform(-3.0, 3.0, n) * h
     icov = _prior(n, sigma, corr, g)
-    qlim = -2.0 * np.log(thr)
+    limit = -2.0 * np.log(thr)
     ctr = np.round((mean - x0) / h)
-    hw = np.ceil(np.sqrt(qlim) * sigma / h) + 1.0
+    hw = np.ceil(np.sqrt(limit) * sigma / h) + 1.0
     idx = ctr + np.round(g.uniform(-1.0, 1.0, (rows, n)) * hw)
     idx[: rows // 2] = ctr + np.round(g.uniform(-0.4, 0.4, (rows // 2, n)) * hw)
     idx[:, -1] = ctr[-1] - hw[-1]
@@ -83,7 +83,7 @@ def _sides(lib, n, sigma, per, origin, corr, seed, thr=THR, rows=1500):
         w = (icov * h[:, None] * h[None, :]).astype(np.float32)
     slack = lib.slack_of(x0[-1], h[-1], abs(ctr[-1]) + hw[-1] + 1)
     side = np.zeros((rows, length), dtype=np.int8)
-    lib.sides(n, dx.ctypes.data, rows, w.ctypes.data, length, slack, qlim, side.ctypes.data)
+    lib.sides(n, dx.ctypes.data, rows, w.ctypes.data, length, slack, limit if qlim is None else qlim, side.ctypes.data)
     cells = np.repeat(idx[:, None, :], length, axis=1)
     cells[:, :, -1] += np.arange(length)
     d = (x0 + cells * h) - mean
@@ -122,6 +122,11 @@ def test_rows_decide_as_fp64_far_from_zero(lib, n, per, origin, corr):
 def test_cells_far_wider_than_the_prior_are_decided_or_left_to_fp64(lib, per):
     side, inside, _ = _sides(lib, 3, 1.0, per, 0.0, 0.3, 4)
     assert not np.any(side[inside] > 0) and not np.any(side[~inside] < 0)
+
+
+def test_an_infinite_limit_leaves_every_cell_to_fp64(lib):
+    side, _, _ = _sides(lib, 4, 1.0, 2.0, 1.0, 0.4, 3, qlim=np.inf)
+    assert not side.any()
 
 
 @pytest.mark.parametrize("origin", [0.0, 1e13, 1e15])
