@@ -10,10 +10,6 @@
 
 namespace gbees {
 
-// ------------------------------------------------------------------ begin / finalise
-
-// ------------------------------------------------------------------ hashtable helpers
-
 // ------------------------------------------------------------------ links
 
 // The CFL rates of the cells that a kernel made active join the running maximum

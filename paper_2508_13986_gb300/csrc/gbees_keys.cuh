@@ -1,7 +1,7 @@
 // Packed cell keys, the hashtable's hash, the rule of the pool's order and the rounded
-// division by a cell width: pure functions that the device code uses and that a host compiler can build too (the host tests pin
-// them: round trip, key order, range limits, the probe sequence, and the probe
-// lengths at load factor 1/2, Sec. 4.2).
+// division by a cell width: pure functions that the device code uses and that a host
+// compiler can build too (the host tests pin them: round trip, key order, range limits,
+// the probe sequence, and the probe lengths at load factor 1/2, Sec. 4.2).
 //
 // A cell index I (N signed ints) packs into one u64: each component biased by
 // 2^(b-1) into b bits, dimension 0 in the most significant position, so that

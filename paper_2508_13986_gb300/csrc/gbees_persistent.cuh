@@ -9,9 +9,9 @@
 // What bounds a step is the longest chain of its phases and the instruction
 // fetch (L1 instruction cache 32 KB, beyond it straight code runs at a third of
 // the rate): the phases' code is kept small, rare work out of line. Lorenz '63,
-// h = 0.25, 5 * 10^3 to 5 * 10^4 pool entries: 26.0 us per FP64 step and 25.3 us per FP32
-// step (38.2 and 35.4 us with five phases, each work item's chain in one
-// thread, in 214 KB of code); h = 0.5, 7 * 10^3 entries: 23.0 us (35.3 us).
+// h = 0.25, 5 * 10^3 to 5 * 10^4 pool entries: 24.0 us per step in both precisions
+// (38.2 us in FP64 and 35.4 us in FP32 with five phases, each work item's chain in one
+// thread, in 214 KB of code); h = 0.5, 7 * 10^3 entries: 24 us (35.3 us).
 //
 // k_batch: many independent grids in one launch. With a team of blocks per grid
 // (all grids resident, a cooperative launch), or as a queue: each block takes a
